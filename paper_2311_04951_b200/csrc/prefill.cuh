@@ -589,8 +589,11 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
     uint8_t *qhi = smem, *qlo = smem + kPtQBytes, *kring = smem + 2 * kPtQBytes, *vring = kring + 2 * kPtKvBytes;
     uint64_t *bars = (uint64_t *)(vring + 2 * kPtKvBytes);
     uint64_t *k_full = bars, *k_free = bars + 2, *v_full = bars + 4, *v_free = bars + 6, *s_full = bars + 8;
-    uint64_t *p_ready = bars + 10, *o_done = bars + 11;
-    uint32_t *tmem_slot = (uint32_t *)(bars + 12);
+    // By chunk parity, like the score buffers: S of chunk c + 1 is issued before P V of chunk c, so a warp may be a whole
+    // chunk ahead of the slowest one.  With one barrier its arrival for c + 1 would count for c, and its wait for P V of
+    // the last chunk would pass on the phase before the previous chunk's.
+    uint64_t *p_ready = bars + 10, *o_done = bars + 12;
+    uint32_t *tmem_slot = (uint32_t *)(bars + 14);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
 
     constexpr int Dh = 128;
@@ -621,8 +624,10 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
     }
     if (tid == 0) {
         for (int i = 0; i < 10; ++i) mbar_init(&bars[i], 1);
-        mbar_init(p_ready, 128);
-        mbar_init(o_done, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&p_ready[i], 128);
+            mbar_init(&o_done[i], 1);
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -722,7 +727,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
             for (int c = 0; c < n_chunks && !*abort_flag; ++c) {
                 const int s = c & 1;
                 if (c + 1 < n_chunks) issue_s(c + 1);
-                wait(p_ready, c & 1);
+                wait(&p_ready[s], (c >> 1) & 1);
                 wait(&v_full[s], (c >> 1) & 1);
                 if (*abort_flag) break;
                 tc_fence_after();
@@ -733,7 +738,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)  // P lo
                     tc_mma_bf16_ta(tO, tP + 32 * (ks >> 1) + 16 + 8 * (ks & 1), umma_desc(va + ks * 2048, 16384, 1024), idO, 1u);
-                tc_commit(o_done);
+                tc_commit(&o_done[s]);
                 tc_commit(&v_free[s]);
             }
         }
@@ -788,7 +793,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
             // the accumulated O row moves to the new maximum, once P V of the previous chunk has written it; the
             // tensor-memory loads and stores are warp-wide, so the warp goes together (f = 1 where nothing moved)
             if (c > 0 && __any_sync(0xffffffffu, f != 1.f)) {
-                wait(o_done, (c - 1) & 1);
+                wait(&o_done[(c - 1) & 1], ((c - 1) >> 1) & 1);
                 tc_fence_after();
 #pragma unroll 1
                 for (int g = 0; g < 4; ++g) {
@@ -800,9 +805,9 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
                 }
             }
             tc_fence_before();
-            mbar_arrive(p_ready);
+            mbar_arrive(&p_ready[c & 1]);
         }
-        wait(o_done, (n_chunks - 1) & 1);
+        wait(&o_done[(n_chunks - 1) & 1], ((n_chunks - 1) >> 1) & 1);
         tc_fence_after();
         {
             const bool store = m < a.M && !*abort_flag;  // (the loads are warp-wide: every lane takes them)

@@ -128,3 +128,30 @@ def test_prompt_longer_than_the_cache_is_refused(many_row_mode):
     with pytest.raises(B.SsdError):
         B.kv_prefill(model, kv, prompts, lens, B.device_buffer(model.prefill_workspace_bytes(2, 80)))
     assert kv.lengths().tolist() == [0, 0]
+
+
+def test_many_row_prompt_pass_is_run_to_run_identical():
+    """Nothing in the many-row pass depends on an order of arrival: the projections own their output tiles and a query
+    row's softmax and output belong to one thread.  Repeated passes over the same prompts must agree bit for bit (the
+    tensor-core attention runs its warps up to a chunk apart; with several chunks per row tile and many CTAs a
+    hand-over that miscounts shows up as other bits within a few passes)."""
+    arch = synth.llama_like(2, 4096, 32, 512, 512)
+    model = B.Model(arch, B.upload_weights(arch, synth.gen_weights(arch, 31)))
+    Bn, P = 8, 1000
+    dev = "cuda"
+    kv = B.KV(model, Bn, P)
+    prompts = torch.from_numpy(synth.gen_prompt(32, Bn, P, arch.vocab)).to(dev)
+    n = torch.full((Bn,), P, dtype=torch.int32, device=dev)
+    zero = torch.zeros(Bn, dtype=torch.int32, device=dev)
+    ws = B.device_buffer(model.prefill_workspace_bytes(Bn, P))
+    ref = None
+    for _ in range(40):
+        B.kv_rollback(kv, zero)
+        kv.lengths()
+        B.kv_prefill(model, kv, prompts, n, ws)
+        got = kv.cache_view()
+        if ref is None:
+            ref = got.clone()
+        else:
+            assert torch.equal(got, ref)
+    assert kv.status() == 0
