@@ -1028,6 +1028,7 @@ int ssd_model_share_prefix(const ssd_model *target, int n_layers, ssd_model **dr
     if (!target->tm.empty()) {
         m->tm.assign(target->tm.begin(), target->tm.begin() + 4 * n_layers);
         m->tm.push_back(target->tm.back());
+        m->tm256.assign(target->tm256.begin(), target->tm256.begin() + 4 * n_layers);
     }
     *draft_out = m;
     return SSD_OK;

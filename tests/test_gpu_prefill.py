@@ -155,3 +155,23 @@ def test_many_row_prompt_pass_is_run_to_run_identical():
         else:
             assert torch.equal(got, ref)
     assert kv.status() == 0
+
+
+@pytest.mark.parametrize("name", ["llama_bf16", "neox_bf16_h80"])
+def test_layer_skip_draft_takes_the_many_row_form(name, many_row_mode):
+    """A draft that shares its target's first layers has the target's many-row pass: its cache equals those layers of
+    the target's cache bit for bit (the same kernels on the same tensors)."""
+    arch = ARCHS[name]
+    model = B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, 3, 6.0)))
+    draft = model.share_prefix(arch.n_layers - 1)
+    Bn, P = 2, 140
+    assert draft.prefill_workspace_bytes(Bn, P) == model.prefill_workspace_bytes(Bn, P) > 0
+    prompts = torch.from_numpy(synth.gen_prompt(33, Bn, P, arch.vocab)).to("cuda")
+    n = torch.tensor([P, P - 50], dtype=torch.int32, device="cuda")
+    caches = []
+    for m in (model, draft):
+        kv = B.KV(m, Bn, P + 4)
+        B.kv_prefill(m, kv, prompts, n, B.device_buffer(m.prefill_workspace_bytes(Bn, P)))
+        assert kv.status() == 0 and kv.lengths().tolist() == n.tolist()
+        caches.append(kv.cache_view().clone())
+    assert torch.equal(caches[0][:arch.n_layers - 1], caches[1])
