@@ -298,16 +298,11 @@ size_t verify_scratch_bytes(int batch, int K);
  * but cannot own CUDA buffers.  The paper has no counterpart of this call; it is a packaging of the
  * same tail for such callers.
  *
- * The statistics that the two tail kernels pass to each other are kept in a fixed array inside
- * the library (SSD_NOALLOC_MAX_ROWS entries of 16 bytes = 64 KB, present on every GPU that loads
- * the library, for the life of the process).  Inputs and outputs are still the caller's.
+ * The tail is one kernel that keeps what its rows hand to each other in shared memory, so the call needs no
+ * device memory of its own.  Inputs and outputs are the caller's.
  *   - batch * (K + 1) > SSD_NOALLOC_MAX_ROWS is refused with SSD_E_CAPACITY; nothing is launched.
  *   - The call never calls cudaMalloc / cudaFree or any allocating routine.
- *   - The first call on each device looks up the array's device address (a host-side query with
- *     that device current); make that first call outside any stream capture.
- *   - All calls on a device share the one array, and it keeps the previous call's contents.  Each
- *     call overwrites every entry it later reads, so stale contents are harmless; but two calls
- *     whose kernels overlap on the GPU (different streams, no ordering) race on it.  Order them.
+ *   - SSD_E_UNIMPL while a sampling restriction is set (its threshold search needs scratch).
  * Results are identical to verify_from_logits.
  */
 enum { SSD_NOALLOC_MAX_ROWS = 4096 };

@@ -307,9 +307,7 @@ def verify_from_logits_noalloc(logits: torch.Tensor, K: int, rows: torch.Tensor,
                                next_token: torch.Tensor, next_token_stride: int,
                                p_debug: Optional[torch.Tensor]) -> None:
     """The tail of a verification on supplied logits, for callers that may not allocate on the device:
-    same arguments as verify_from_logits minus the scratch buffer (the library keeps a fixed 64 KB
-    array for it, shared by all calls on a device; at most NOALLOC_MAX_ROWS logits rows per call;
-    calls that overlap on the GPU must be ordered by the caller)."""
+    same arguments as verify_from_logits minus the scratch buffer; at most NOALLOC_MAX_ROWS logits rows per call."""
     Bn, M, V = logits.shape
     assert M == K + 1 and logits.is_contiguous() and logits.dtype == torch.float32
     _check(load().verify_from_logits_noalloc(_p(logits), Bn, K, V, _p(rows), _p(q), _p(u), temperature,

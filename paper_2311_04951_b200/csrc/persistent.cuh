@@ -134,7 +134,7 @@ struct alignas(64) FwdParams {
     float *tp_m, *tp_s; int32_t *tp_a;             // per (sequence, CTA): max, sum of exp relative to it, argmax of the CTA's slice
     double *tp_mass;                               // per (sequence, CTA): mass of q in the CTA's slice
     int32_t *tail_hit;                             // [n_steps][B][2]: smallest index past u S (INT_MAX: none) / largest index with q > 0
-    unsigned long long *mailbox; unsigned mb_seq;  // the largest length, reported to the host at the end
+    unsigned long long *mailbox; unsigned mb_seq;  // the lengths, reported to the host at the end
 };
 
 struct GemmDesc {
@@ -2324,11 +2324,9 @@ __global__ void __launch_bounds__(kPersistThreads, 1) forward_kernel(const __gri
                 if (!(go = grid_sync(p, sh, epoch))) break;
             }
         }
-        if (go && p.tail && p.mailbox && blockIdx.x == 0 && threadIdx.x == 0) {  // the host's length bound follows (see report_max_len)
-            int m = 0;
-            for (int b = 0; b < p.B; ++b) m = max(m, __ldcg(p.len_rw + b));
-            *reinterpret_cast<volatile unsigned long long *>(p.mailbox) = ((unsigned long long)p.mb_seq << 32) | (unsigned)m;
-        }
+        if (go && p.tail && p.mailbox && blockIdx.x == 0 && (int)threadIdx.x < p.B)  // the host's length bound follows (see report_len)
+            *reinterpret_cast<volatile unsigned long long *>(p.mailbox + threadIdx.x) =
+                ((unsigned long long)p.mb_seq << 32) | (unsigned)__ldcg(p.len_rw + threadIdx.x);
         if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
             unsigned long long t;
             asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));

@@ -163,6 +163,7 @@ int init_device_once() {
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 8>, attn_smem<__nv_bfloat16, 8>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 16>, attn_smem<__nv_bfloat16, 16>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 32>, attn_smem<__nv_bfloat16, 32>(128));
+    rc |= set_smem(row_filter_kernel, (size_t)kFilterCache * 4);
     rc |= set_smem(prefill_gemm_kernel, kPfSmem);
     rc |= set_smem(prefill_attn_kernel, prefill_attn_smem(128));
     rc |= set_smem(prefill_attn_tc_kernel, kPtSmem);
@@ -195,7 +196,7 @@ struct ssd_kv {
     int len_ub;   // host-side upper bound of the committed lengths
     int last_rows;  // rows the last forward left uncommitted (upper bound bookkeeping)
     // The bound follows the device without a synchronisation: every kernel that changes the lengths writes
-    // (operation number << 32 | largest length) into this word of mapped host memory; the host adds what the
+    // (operation number << 32 | length) into the sequence's word of mapped host memory; the host adds what the
     // operations queued behind that number can add at most (growth_at[n & 255] = total growth bound after op n).
     unsigned long long *mailbox, *mailbox_dev;
     unsigned op_seq;
@@ -217,12 +218,15 @@ unsigned kv_note_op(ssd_kv *kv, int growth) {
 // Upper bound of the committed lengths once everything queued so far has run.
 int kv_bound(ssd_kv *kv) {
     if (kv->mailbox) {
-        const unsigned long long v = *reinterpret_cast<volatile unsigned long long *>(kv->mailbox);
-        const unsigned seq = (unsigned)(v >> 32);
-        if (seq != 0 && kv->op_seq - seq < 256u) {
+        long long most = 0;
+        for (int b = 0; b < kv->B; ++b) {
+            const unsigned long long v = reinterpret_cast<volatile unsigned long long *>(kv->mailbox)[b];
+            const unsigned seq = (unsigned)(v >> 32);
+            if (seq == 0 || kv->op_seq - seq >= 256u) return kv->len_ub;
             const long long ub = (long long)(unsigned)(v & 0xffffffffu) + kv->growth_total - kv->growth_at[seq & 255];
-            kv->len_ub = ub > kv->S ? kv->S : (int)ub;
+            if (ub > most) most = ub;
         }
+        kv->len_ub = most > kv->S ? kv->S : (int)most;
     }
     return kv->len_ub;
 }
@@ -1073,10 +1077,10 @@ int kv_init(const ssd_model *m, int batch, int max_len, void *dev_buf, size_t by
     kv->growth_total = 0;
     memset(kv->growth_at, 0, sizeof(kv->growth_at));
     kv->mailbox = kv->mailbox_dev = nullptr;
-    {   // eight bytes of mapped host memory (not device memory); without it the bound is only advanced
+    {   // eight bytes of mapped host memory per sequence (not device memory); without them the bound is only advanced
         void *h = nullptr, *d = nullptr;
-        if (cudaHostAlloc(&h, sizeof(unsigned long long), cudaHostAllocMapped) == cudaSuccess) {
-            *reinterpret_cast<unsigned long long *>(h) = 0;
+        if (cudaHostAlloc(&h, sizeof(unsigned long long) * batch, cudaHostAllocMapped) == cudaSuccess) {
+            memset(h, 0, sizeof(unsigned long long) * batch);
             if (cudaHostGetDevicePointer(&d, h, 0) == cudaSuccess) {
                 kv->mailbox = (unsigned long long *)h;
                 kv->mailbox_dev = (unsigned long long *)d;
@@ -1107,7 +1111,7 @@ int kv_init(const ssd_model *m, int batch, int max_len, void *dev_buf, size_t by
 
 void kv_destroy(ssd_kv *kv) {
     if (kv && kv->mailbox) {
-        // the word may still be written by queued kernels: wait for the device before it goes away
+        // the words may still be written by queued kernels: wait for the device before they go away
         cudaDeviceSynchronize();
         cudaFreeHost(kv->mailbox);
     }
@@ -1171,6 +1175,24 @@ int kv_prefill(ssd_model *m, ssd_kv *kv, const int32_t *dev_tokens, const int32_
     return SSD_OK;
 }
 
+// ---- vocabulary-wide tail ----
+// A piece of a row (1 / 256 of it) is held in 1, 4 or 8 registers per lane: the smallest that the row fills, so that no slot is
+// worked on for nothing; from 65537 entries a piece is read in several steps of 8.
+constexpr int kTailSmallV = 32 * kTailCluster * kTailWarps, kTailMediumV = 4 * kTailSmallV;
+
+static bool restricted(float temperature, int V) {  // (a greedy row is its own restriction)
+    return temperature > 0.f && ((g_top_k > 0 && g_top_k < V) || (g_top_p > 0.f && g_top_p < 1.f));
+}
+static int run_row_filter(const float *logits, int B, int M, int V, const int32_t *n_eff, float temperature, RowStat *stats,
+                          RowFilter *filt, float *p_out, cudaStream_t st) {
+    FilterArgs f;
+    f.logits = logits; f.M = M; f.V = V; f.n_eff = n_eff; f.inv_t = 1.0f / temperature;
+    f.top_k = g_top_k; f.top_p = g_top_p;
+    f.stats = stats; f.filt = filt; f.p_out = p_out;
+    LAUNCH(row_filter_kernel, dim3((n_eff ? 1 : M) * kFilterCluster, B), kTailThreads, filter_smem(V), st, f);
+    return SSD_OK;
+}
+
 int draft_step(ssd_model *draft, ssd_kv *dkv, const int32_t *dev_tokens_in, int tokens_stride, int rows_in,
                const int32_t *dev_n_in, float temperature, const float *dev_u, int u_stride, int32_t *dev_token_out,
                int token_out_stride, float *dev_q_out, size_t q_stride, void *dev_ws, size_t ws_bytes, void *stream) {
@@ -1188,10 +1210,19 @@ int draft_step(ssd_model *draft, ssd_kv *dkv, const int32_t *dev_tokens_in, int 
     t.u = dev_u; t.u_stride = u_stride;
     t.token_out = dev_token_out; t.token_stride = token_out_stride;
     t.q_out = dev_q_out; t.q_stride = q_stride;
-    t.top_k = g_top_k; t.top_p = g_top_p;
-    LAUNCH(draft_tail_kernel, dkv->B * kTailCluster, kTailThreads, 0, st, t);
-    const unsigned seq = kv_note_op(dkv, rows_in);
-    LAUNCH(kv_commit_rows_kernel, 1, 64, 0, st, dkv->len, w.ri.n_eff, dkv->B, dkv->mailbox_dev, seq);
+    t.stats = w.stats; t.filt = w.filt;
+    t.len = dkv->len; t.mailbox = dkv->mailbox_dev; t.seq = kv_note_op(dkv, rows_in);
+    const int B = dkv->B, V = t.V;
+    if (restricted(temperature, V)) {
+        if ((rc = run_row_filter(w.logits, B, rows_in, V, w.ri.n_eff, temperature, w.stats, w.filt, nullptr, st))) return rc;
+        if (V <= kTailSmallV) { LAUNCH((draft_tail_kernel<true, 1>), B * kTailCluster, kTailThreads, 0, st, t); }
+        else if (V <= kTailMediumV) { LAUNCH((draft_tail_kernel<true, 4>), B * kTailCluster, kTailThreads, 0, st, t); }
+        else { LAUNCH((draft_tail_kernel<true, 8>), B * kTailCluster, kTailThreads, 0, st, t); }
+    } else {
+        if (V <= kTailSmallV) { LAUNCH((draft_tail_kernel<false, 1>), B * kTailCluster, kTailThreads, 0, st, t); }
+        else if (V <= kTailMediumV) { LAUNCH((draft_tail_kernel<false, 4>), B * kTailCluster, kTailThreads, 0, st, t); }
+        else { LAUNCH((draft_tail_kernel<false, 8>), B * kTailCluster, kTailThreads, 0, st, t); }
+    }
     return SSD_OK;
 }
 
@@ -1204,8 +1235,8 @@ int draft_steps(ssd_model *draft, ssd_kv *dkv, int n_steps, const int32_t *dev_t
         q_stride < (size_t)n_steps * (size_t)draft->a.vocab)
         return SSD_E_ARG;
     if (!same_cache_shape(draft, dkv)) return SSD_E_ARG;
-    const bool restricted = g_top_k > 0 || (g_top_p > 0.f && g_top_p < 1.f);
-    if (!single_kernel_path(draft) || restricted) {
+    const bool restriction = g_top_k > 0 || (g_top_p > 0.f && g_top_p < 1.f);
+    if (!single_kernel_path(draft) || restriction) {
         // the same steps, one call each (fp32 models, head dimensions the single kernel does not cover, or a
         // sampling restriction, whose threshold search lives in the stand-alone tail kernel)
         for (int s = 0; s < n_steps; ++s) {
@@ -1245,10 +1276,18 @@ static int run_verify_tail(const float *logits, int B, int K, int V, const int32
     v.logits = logits; v.K = K; v.V = V; v.rows = rows; v.q = q; v.u = u;
     v.inv_t = temperature > 0.f ? 1.0f / temperature : 0.f;
     v.n_accepted = n_acc; v.next_token = next; v.next_stride = next_stride;
-    v.p_debug = p_debug; v.keep = keep; v.stats = stats;
-    v.filt = filt; v.top_k = filt ? g_top_k : 0; v.top_p = filt ? g_top_p : 1.0f;
-    LAUNCH(row_stats_kernel, dim3((K + 1) * kTailCluster, B), kTailThreads, 0, st, v);
-    LAUNCH(verify_kernel, B * kTailCluster, kTailThreads, 0, st, v);
+    v.p_debug = p_debug; v.keep = keep; v.stats = stats; v.filt = filt;
+    if (restricted(temperature, V)) {
+        const int rc = run_row_filter(logits, B, K + 1, V, nullptr, temperature, stats, filt, p_debug, st);
+        if (rc) return rc;
+        if (V <= kTailSmallV) { LAUNCH((verify_kernel<true, 1>), B * kTailCluster, kTailThreads, 0, st, v); }
+        else if (V <= kTailMediumV) { LAUNCH((verify_kernel<true, 4>), B * kTailCluster, kTailThreads, 0, st, v); }
+        else { LAUNCH((verify_kernel<true, 8>), B * kTailCluster, kTailThreads, 0, st, v); }
+    } else {
+        if (V <= kTailSmallV) { LAUNCH((verify_kernel<false, 1>), B * kTailCluster, kTailThreads, 0, st, v); }
+        else if (V <= kTailMediumV) { LAUNCH((verify_kernel<false, 4>), B * kTailCluster, kTailThreads, 0, st, v); }
+        else { LAUNCH((verify_kernel<false, 8>), B * kTailCluster, kTailThreads, 0, st, v); }
+    }
     return SSD_OK;
 }
 
@@ -1261,6 +1300,8 @@ int verify_from_logits(const float *dev_logits, int batch, int K, int vocab, con
         return SSD_E_ARG;
     if (K > 0 && !dev_q) return SSD_E_ARG;
     if (scratch_bytes < verify_scratch_bytes(batch, K)) return SSD_E_CAPACITY;
+    const int rc = init_device_once();  // (may be a program's first call)
+    if (rc) return rc;
     return run_verify_tail(dev_logits, batch, K, vocab, dev_rows, dev_q, dev_u, temperature, dev_n_accepted,
                            dev_next_token, next_token_stride, dev_p_debug, nullptr, (RowStat *)dev_scratch,
                            (RowFilter *)((uint8_t *)dev_scratch + align_up(sizeof(RowStat) * (size_t)batch * (K + 1), 256)),
@@ -1364,36 +1405,8 @@ int ssd_last_logits(const ssd_model *m, int batch, int rows_per_seq, const void 
     return SSD_OK;
 }
 
-// ---------------------------------------------------------------------------------------------
-// verify_from_logits for callers that cannot allocate device memory.
-//
-// The row statistics (max, normaliser, argmax of every logits row) that the two tail kernels hand
-// to each other live in a fixed array inside the library image instead of a caller buffer.  The
-// array is part of every context that loads the library (64 KB per GPU, held until exit).
-static __device__ __align__(256) RowStat g_noalloc_stats[SSD_NOALLOC_MAX_ROWS];
-
-namespace {
-constexpr int kMaxDevices = 64;
-RowStat *g_noalloc_ptr[kMaxDevices] = {nullptr};
-std::mutex g_noalloc_mu;
-
-// In host code `g_noalloc_stats` is only a handle for the runtime, not a device address: the real
-// address differs per device and has to be asked for with that device current.
-int noalloc_scratch(RowStat **out) {
-    int dev = -1;
-    CUDA_OK(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= kMaxDevices) return SSD_E_CAPACITY;
-    std::lock_guard<std::mutex> lk(g_noalloc_mu);
-    if (!g_noalloc_ptr[dev]) {
-        void *p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_noalloc_stats) != cudaSuccess || !p) return SSD_E_CUDA;
-        g_noalloc_ptr[dev] = (RowStat *)p;
-    }
-    *out = g_noalloc_ptr[dev];
-    return SSD_OK;
-}
-}  // namespace
-
+// verify_from_logits for callers that cannot allocate device memory: without a restriction the tail is one kernel that
+// keeps everything its rows hand to each other in shared memory.
 int verify_from_logits_noalloc(const float *dev_logits, int batch, int K, int vocab, const int32_t *dev_rows,
                                const float *dev_q, const float *dev_u, float temperature,
                                int32_t *dev_n_accepted, int32_t *dev_next_token, int next_token_stride,
@@ -1403,14 +1416,9 @@ int verify_from_logits_noalloc(const float *dev_logits, int batch, int K, int vo
         return SSD_E_ARG;
     if (K > 0 && !dev_q) return SSD_E_ARG;
     if ((long long)batch * (K + 1) > SSD_NOALLOC_MAX_ROWS) return SSD_E_CAPACITY;
-    if (g_top_k > 0 || (g_top_p > 0.f && g_top_p < 1.f)) return SSD_E_UNIMPL;  // its fixed array has no room for the restriction
-    RowStat *stats = nullptr;
-    int rc = noalloc_scratch(&stats);
-    if (rc) return rc;
-    // every entry a call reads is written earlier in the same call (row_stats_kernel fills
-    // stats[0 .. batch*(K+1)) before verify_kernel looks at them): nothing has to start at zero
+    if (g_top_k > 0 || (g_top_p > 0.f && g_top_p < 1.f)) return SSD_E_UNIMPL;  // a restriction needs scratch
     return run_verify_tail(dev_logits, batch, K, vocab, dev_rows, dev_q, dev_u, temperature, dev_n_accepted,
-                           dev_next_token, next_token_stride, dev_p_debug, nullptr, stats, nullptr, (cudaStream_t)stream);
+                           dev_next_token, next_token_stride, dev_p_debug, nullptr, nullptr, nullptr, (cudaStream_t)stream);
 }
 
 uint64_t ssd_launch_count(void) { return g_launches.load(); }

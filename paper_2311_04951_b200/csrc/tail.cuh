@@ -2,13 +2,16 @@
 // residual renormalise-and-resample or bonus draw, and the draft's "sample from q, export q".
 // (Section "Speculative Sampling", Figure 2: the target model passes or refuses each draft token in
 // turn and generates one token itself.)  No host round-trip: everything a decision
-// needs stays on the device; reductions use warp shuffles, prefix sums run in fp64.
+// needs stays on the device.
 //
-// One row of the vocabulary is worked on by a thread-block cluster of kTailCluster CTAs (one SM alone
-// is issue- and latency-bound on a 50 K-entry row: ncu shows 52 % issue slots busy on the statistics
-// and long-scoreboard stalls of 18 per issue on the draw).  CTA `rank` owns a contiguous slice of the
-// row; block results are published in shared memory and read by the other CTAs of the cluster through
-// distributed shared memory, always combined in rank order so that sums keep the index order.
+// A sequence's rows are worked on by a thread-block cluster of kTailCluster CTAs of 32 warps (one SM alone is issue-
+// and latency-bound on a 50 K-entry row).  Warp g of the cluster owns the contiguous piece [g * per, (g + 1) * per)
+// of every row and its lanes take consecutive entries of it, kStep / 32 loads in flight per lane (1, 4 or 8: what the
+// vocabulary fills); what the warps find meets once in shared memory and once, through distributed shared memory, across
+// the cluster, always combined in the same order.  What bounds it is instruction issue on the cluster's few SMs and that
+// chain of exchanges, not the bytes: hence one kernel per verification, which carries the statistics of ALL rows of a
+// sequence through one exchange (one sequence, 5 rows of 32000: 21.6 us a call back to back with a cluster per row and a
+// second launch for the draw, now 14.3).
 #pragma once
 #include <cooperative_groups.h>
 
@@ -19,22 +22,9 @@ namespace ssd {
 namespace cg = cooperative_groups;
 
 constexpr int kTailThreads = 1024;
+constexpr int kTailWarps = kTailThreads / 32;
 constexpr int kTailCluster = 8;
-
-// What a CTA publishes to its cluster.  Every exchange uses slots of its own, so one cluster barrier
-// per exchange suffices; a kernel ends with a cluster barrier (nobody leaves while its slots are read).
-struct ClusterSlots {
-    float v[2];
-    int i[6];
-    double d[4];
-};
-
-// CTA `rank`'s slice [lo, hi) of a row of V entries: whole rows of 32 indices, split evenly.
-__device__ __forceinline__ void tail_slice(int V, int rank, int &lo, int &hi) {
-    const int rows = (V + 31) >> 5, per = (rows + kTailCluster - 1) / kTailCluster;
-    lo = min(V, rank * per * 32);
-    hi = min(V, lo + per * 32);
-}
+constexpr int kTailMaxRows = kMaxRowsPerSeq;
 
 struct RowStat {
     float mx;      // max logit of the row
@@ -62,272 +52,535 @@ __device__ __forceinline__ float prob_f(float logit, const RowStat &st, const Ro
     return pr >= f.thr ? pr / f.mass : 0.f;
 }
 
-// Block-wide (max, lowest index of max).
-__device__ __forceinline__ void block_argmax(float v, int idx, float *sv, int *si, float &out_v, int &out_i) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+// Warp `g` of `pieces` warps owns this piece [lo, hi) of a row of V entries: whole lane rows.
+__device__ __forceinline__ void row_piece(int V, int pieces, int g, int &lo, int &hi) {
+    const int per = (((V + pieces - 1) / pieces) + 31) & ~31;
+    lo = min(V, g * per);
+    hi = min(V, lo + per);
+}
+__device__ __forceinline__ void tail_piece(int V, int rank, int &lo, int &hi) {
+    row_piece(V, kTailCluster * kTailWarps, rank * kTailWarps + (int)(threadIdx.x >> 5), lo, hi);
+}
+// Entries base + lane, base + lane + 32, ... of the piece; `fill` where it has ended.
+template <int IT>
+__device__ __forceinline__ void tail_load(const float *row, int base, int hi, float fill, float (&l)[IT]) {
+    const int j = base + (int)(threadIdx.x & 31);
+    if (base + 32 * IT <= hi) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float ov = __shfl_xor_sync(0xffffffffu, v, o);
-        int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-        if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-    }
-    __syncthreads();
-    if (lane == 0) { sv[w] = v; si[w] = idx; }
-    __syncthreads();
-    if (w == 0) {
-        v = lane < nw ? sv[lane] : -INFINITY;
-        idx = lane < nw ? si[lane] : 0x7fffffff;
+        for (int u = 0; u < IT; ++u) l[u] = __ldcg(row + j + 32 * u);
+    } else {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float ov = __shfl_xor_sync(0xffffffffu, v, o);
-            int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-            if (ov > v || (ov == v && oi < idx)) { v = ov; idx = oi; }
-        }
-        if (lane == 0) { sv[0] = v; si[0] = idx; }
+        for (int u = 0; u < IT; ++u) l[u] = j + 32 * u < hi ? __ldcg(row + j + 32 * u) : fill;
     }
-    __syncthreads();
-    out_v = sv[0];
-    out_i = si[0];
 }
 
-// Row statistics of logits[row, :] by the whole cluster; every thread of every CTA returns the same RowStat.
-__device__ __forceinline__ RowStat row_stats(const float *logits, int V, float inv_t, float *sv, int *si, double *sd,
-                                             ClusterSlots *pub, cg::cluster_group &cl) {
-    const int rank = (int)cl.block_rank();
-    int lo, hi;
-    tail_slice(V, rank, lo, hi);
-    float mx = -INFINITY;
-    int am = 0x7fffffff;
-    // eight loads in flight per thread: the row comes from L2, and one latency per element is the whole cost
-    for (int j0 = lo + threadIdx.x; j0 < hi; j0 += 8 * blockDim.x) {
-        float l[8];
+// max over the warp (an order-preserving map to signed integers, one reduction instruction); never of a NaN
+__device__ __forceinline__ float warp_max_redux(float v) {
+    const int b = __float_as_int(v);
+    const int m = __reduce_max_sync(0xffffffffu, b >= 0 ? b : b ^ 0x7fffffff);
+    return __int_as_float(m >= 0 ? m : m ^ 0x7fffffff);
+}
+
+// (max, argmax, sum of exp relative to the max) of a part of a row
+struct PartStat {
+    float mx;
+    int am;
+    double s;
+};
+// The statistics of W parts held by the W lanes of a group (W = 32: the warps of a CTA, else the CTAs of a cluster).
+template <int W>
+__device__ __forceinline__ PartStat join_parts(PartStat a, float inv_t) {
+    float m = a.mx;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int j = j0 + u * blockDim.x;
-            l[u] = j < hi ? __ldcg(logits + j) : -INFINITY;
-        }
+    for (int o = W / 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int am = a.mx == m ? a.am : 0x7fffffff;
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (l[u] > mx) { mx = l[u]; am = j0 + u * blockDim.x; }  // strided ascending: first maximum per thread
-    }
-    float bmx;
-    int bam;
-    block_argmax(mx, am, sv, si, bmx, bam);
-    if (threadIdx.x == 0) { pub->v[0] = bmx; pub->i[0] = bam; }
-    cl.sync();
-    RowStat st;
-    st.mx = -INFINITY;
-    st.amax = 0x7fffffff;
-    for (int r = 0; r < kTailCluster; ++r) {  // lowest index among the maxima
-        const ClusterSlots *o = cl.map_shared_rank(pub, r);
-        const float v = o->v[0];
-        const int i = o->i[0];
-        if (v > st.mx || (v == st.mx && i < st.amax)) { st.mx = v; st.amax = i; }
-    }
-    double z = 0.0;
+    for (int o = W / 2; o > 0; o >>= 1) am = min(am, __shfl_xor_sync(0xffffffffu, am, o));
+    double s = 0.0;
     if (inv_t != 0.f) {
-        float part = 0.f;
-        for (int j0 = lo + threadIdx.x; j0 < hi; j0 += 8 * blockDim.x) {
-            float l[8];
+        s = a.mx > -INFINITY ? a.s * (double)expf((a.mx - m) * inv_t) : 0.0;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int j = j0 + u * blockDim.x;
-                l[u] = j < hi ? __ldcg(logits + j) : -INFINITY;  // exp(-inf) = 0
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) part += expf((l[u] - st.mx) * inv_t);
-        }
-        const double zb = block_sum((double)part, sd);
-        if (threadIdx.x == 0) pub->d[0] = zb;
-        cl.sync();
-        for (int r = 0; r < kTailCluster; ++r) z += cl.map_shared_rank(pub, r)->d[0];
+        for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
-    st.z = (float)z;
+    PartStat r;
+    r.mx = m;
+    r.am = am;
+    r.s = s;
+    return r;
+}
+__device__ __forceinline__ RowStat row_stat(const PartStat &t) {
+    RowStat st;
+    st.mx = t.mx;
+    st.z = (float)t.s;
+    st.amax = t.am;
     st.pad = 0;
     return st;
 }
 
-// Shared memory of the threshold search below.
-struct FilterSmem {
-    unsigned cnt[256];
-    double mass[256];
-    unsigned tot_cnt[256];
-    double tot_mass[256];
-    unsigned sel, cnt_above;
-    double mass_above, total;
+struct StatSmem {
+    PartStat warp[kTailMaxRows][kTailWarps];  // of this CTA's warps
+    PartStat cta[kTailMaxRows];               // of this CTA, read by the others
+    RowStat row[kTailMaxRows];
 };
 
-// The threshold of a restriction, by the whole cluster: the largest probability value t such that the tokens
-// with p >= t (p >= lo only are looked at) number at least want_cnt (by_mass false) or weigh at least want_mass
-// (by_mass true); if no t reaches it, the smallest value present.  Tokens equal to the threshold all stay.  A
-// radix search over the fp32 bit pattern (probabilities are >= 0, so the patterns order like the values): four
-// passes of eight bits, each a 256-bin histogram of counts and masses of the tokens that match the bits fixed
-// so far, summed over the CTAs in rank order through distributed shared memory; the bins are walked from the
-// top.  Returns the threshold and, through *kept_mass, the mass at or above it (fp64 sums; the walk order
-// differs from a sorted running sum only in rounding).  The same result in every thread of the cluster.
-template <typename ProbFn>
-__device__ __forceinline__ float select_threshold(ProbFn prob, int V, float lo, bool by_mass, unsigned want_cnt,
-                                                  double want_frac, FilterSmem *fs, cg::cluster_group &cl,
-                                                  double *kept_mass) {
-    const int rank = (int)cl.block_rank();
-    int lo_i, hi_i;
-    tail_slice(V, rank, lo_i, hi_i);
-    unsigned prefix = 0;
-    int nb = 0;
-    double want_mass = 0.0;
-    if (threadIdx.x == 0) { fs->cnt_above = 0; fs->mass_above = 0.0; }
-    for (int pass = 0; pass < 4; ++pass) {
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) { fs->cnt[i] = 0; fs->mass[i] = 0.0; }
-        __syncthreads();
-        for (int j = lo_i + threadIdx.x; j < hi_i; j += blockDim.x) {
-            const float pr = prob(j);
-            const unsigned bits = __float_as_uint(pr);
-            if (pr >= lo && (nb == 0 || (bits >> (32 - nb)) == prefix)) {
-                const unsigned bin = (bits >> (24 - nb)) & 255u;
-                atomicAdd(&fs->cnt[bin], 1u);
-                atomicAdd(&fs->mass[bin], (double)pr);
-            }
+// Statistics of `rows` rows (row pitch V) by the whole cluster, left in ss->row of every CTA.  Where a piece fits one
+// step (hi - lo <= 32 IT) `l` returns its entries of the last row.
+template <int IT>
+__device__ __forceinline__ void cluster_stats(const float *logits, int rows, int V, float inv_t, StatSmem *ss,
+                                              cg::cluster_group &cl, float (&l)[IT]) {
+    constexpr int kStep = 32 * IT;
+    const int rank = (int)cl.block_rank(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int lo, hi;
+    tail_piece(V, rank, lo, hi);
+    const bool one = hi - lo <= kStep;
+    float nx[IT];
+    tail_load<IT>(logits, lo, hi, -INFINITY, nx);
+    for (int r = 0; r < rows; ++r) {
+        const float *lg = logits + (size_t)r * V;
+#pragma unroll
+        for (int u = 0; u < IT; ++u) l[u] = nx[u];
+        if (r + 1 < rows) tail_load<IT>(lg + V, lo, hi, -INFINITY, nx);  // the next row, under this one's arithmetic
+        float mx = -INFINITY;
+        int at = lo;  // the step that the lane's first maximum lies in
+        for (int b = lo;;) {
+            float m = l[0];
+#pragma unroll
+            for (int u = 1; u < IT; ++u) m = fmaxf(m, l[u]);
+            if (m > mx) { mx = m; at = b; }
+            b += kStep;
+            if (b >= hi) break;
+            tail_load<IT>(lg, b, hi, -INFINITY, l);
         }
-        __syncthreads();
-        cl.sync();  // every CTA's histogram is complete
-        for (int i = threadIdx.x; i < 256; i += blockDim.x) {
-            unsigned c = 0;
-            double m = 0.0;
-            for (int r = 0; r < kTailCluster; ++r) {
-                const FilterSmem *o = cl.map_shared_rank(fs, r);
-                c += o->cnt[i];
-                m += o->mass[i];
-            }
-            fs->tot_cnt[i] = c;
-            fs->tot_mass[i] = m;
+        const float m = warp_max_redux(mx);
+        int am = 0x7fffffff;
+        if (mx == m && m > -INFINITY) {
+            float x[IT];
+#pragma unroll
+            for (int u = 0; u < IT; ++u) x[u] = l[u];
+            if (!one) tail_load<IT>(lg, at, hi, -INFINITY, x);
+#pragma unroll
+            for (int u = IT - 1; u >= 0; --u)
+                if (x[u] == m) am = at + 32 * u + lane;  // the lowest index
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (pass == 0) {  // the mass of everything looked at: the base of a mass target
-                double t = 0.0;
-                for (int i = 255; i >= 0; --i) t += fs->tot_mass[i];
-                fs->total = t;
+        am = __reduce_min_sync(0xffffffffu, am);
+        double s = 0.0;
+        if (inv_t != 0.f && m > -INFINITY) {
+            float part = 0.f;
+            if (!one) tail_load<IT>(lg, lo, hi, -INFINITY, l);
+            for (int b = lo;;) {
+#pragma unroll
+                for (int u = 0; u < IT; ++u) part += expf((l[u] - m) * inv_t);  // exp(-inf) = 0
+                b += kStep;
+                if (b >= hi) break;
+                tail_load<IT>(lg, b, hi, -INFINITY, l);
             }
-            const double target = want_frac * fs->total;
-            unsigned c = fs->cnt_above;
-            double m = fs->mass_above;
-            int sel = -1, lowest = -1;
-            for (int i = 255; i >= 0; --i) {
-                if (fs->tot_cnt[i] == 0) continue;
-                lowest = i;
-                const bool met = by_mass ? (m + fs->tot_mass[i] >= target) : (c + fs->tot_cnt[i] >= want_cnt);
-                if (met) { sel = i; break; }
-                c += fs->tot_cnt[i];
-                m += fs->tot_mass[i];
-            }
-            if (sel < 0) {  // the target lies beyond everything there is: keep all (back off the last bin's sums)
-                sel = lowest < 0 ? 0 : lowest;
-                if (lowest >= 0) { c -= fs->tot_cnt[sel]; m -= fs->tot_mass[sel]; }
-            }
-            fs->sel = (unsigned)sel;
-            fs->cnt_above = c;
-            fs->mass_above = m;
+            s = warp_sum((double)part);
         }
-        __syncthreads();
-        prefix = (prefix << 8) | fs->sel;
-        nb += 8;
-        want_mass = fs->mass_above + fs->tot_mass[fs->sel];
-        cl.sync();  // all remote reads of this pass are done before the histograms are cleared
+        if (lane == 0) {
+            PartStat t;
+            t.mx = m;
+            t.am = am;
+            t.s = s;
+            ss->warp[r][warp] = t;
+        }
     }
-    *kept_mass = want_mass;
-    return __uint_as_float(prefix);
+    __syncthreads();
+    for (int r = warp; r < rows; r += kTailWarps) {
+        const PartStat t = join_parts<32>(ss->warp[r][lane], inv_t);
+        if (lane == 0) ss->cta[r] = t;
+    }
+    cl.sync();
+    for (int i = threadIdx.x; i < ((rows * kTailCluster + 31) & ~31); i += kTailThreads) {
+        const int r = min(i / kTailCluster, rows - 1);
+        const PartStat t = join_parts<kTailCluster>(*cl.map_shared_rank(&ss->cta[r], i % kTailCluster), inv_t);
+        if (i % kTailCluster == 0 && i / kTailCluster < rows) ss->row[r] = row_stat(t);
+    }
+    __syncthreads();
 }
 
-// The restriction of a row (top_k tokens, then the top_p nucleus of those), by the whole cluster.
-__device__ __forceinline__ RowFilter row_filter(const float *logits, int V, const RowStat &st, float inv_t, int top_k,
-                                                float top_p, FilterSmem *fs, cg::cluster_group &cl) {
+// ---- top-k / top-p ---------------------------------------------------------------------------------
+// The threshold of a restriction: the largest probability value t such that the tokens with p >= t number at least top_k,
+// or - of those that top-k kept - weigh at least top_p of their mass; if no t reaches it, the smallest value there is.
+// Tokens equal to the threshold all stay.
+//
+// Probabilities are >= 0, so their fp32 bit patterns order like the values.  A token's key is its pattern's distance
+// below the largest one's.  First pass: 1024 bins of 2^18 keys, 32 to a factor of two, so that a softmax row spreads over
+// hundreds of them (bins of the pattern's top eight bits put a whole row into a dozen: the histogram's atomic operations
+// queue up on a few addresses); the bins are walked from the top, and two or three more passes refine the one that the
+// target falls into.  A bin holds a count and the tokens' mass in units of 2^-62, in three native 32-bit words: integer
+// sums do not depend on their order and are finer than an fp64 running sum.  A thread joins consecutive tokens of one bin
+// before it touches the histogram (a row of equal values, or the tail of a peaked one, is one bin).  The first histogram
+// is kept: with the tokens that top-k took off its bin put aside, it is top-p's first pass too.
+//
+// A row is a cluster of TWO CTAs, its probabilities computed once and kept in their shared memory (up to kFilterCache of
+// them each): the histograms of two CTAs are joined with three remote loads per thread, where eight CTAs took 9 us per
+// pass for it and left most of 48 rows waiting for SMs.
+// 8 sequences x 6 rows x 50304 entries, top-k 50 and top-p 0.9, whole call: 573 us with byte-wide bins and fp64 atomics on
+// eight CTAs, 193 with these bins on eight, 55 on two.
+constexpr int kBins = 1024;
+constexpr int kFilterCluster = 2;
+constexpr int kFilterCache = 44 * 1024;     // probabilities a CTA keeps (176 KB)
+constexpr int kFilterBatch = 8;
+constexpr double kMassUnit = 4611686018427387904.0;  // 2^62
+struct FilterHist {
+    unsigned cnt[kBins], mlo[kBins], mhi[kBins];
+};
+struct FilterSmem {
+    PartStat warp[kTailWarps], cta;
+    FilterHist hist[3];         // [0] the first pass; [1], [2] in turn for the others, so that a pass needs one cluster barrier
+    unsigned wcnt[kTailWarps];
+    unsigned long long wmass[kTailWarps];
+    int first, last;            // first bin that meets the target, last bin that holds anything
+    unsigned above_cnt;         // of the chosen bin: what lies above it, and its own mass
+    unsigned long long above_mass, sel_mass;
+};
+__host__ __device__ constexpr size_t filter_smem(int V) {  // dynamic shared memory: the CTA's probabilities
+    const size_t n = (size_t)((V + kFilterCluster - 1) / kFilterCluster) + 32 * kTailWarps;
+    return n <= (size_t)kFilterCache ? n * 4 : 0;
+}
+
+__device__ __forceinline__ void bin_add(FilterHist &h, int bin, unsigned c, unsigned long long m) {
+    if (c == 0) return;
+    atomicAdd(&h.cnt[bin], c);
+    const unsigned lo = (unsigned)m, old = atomicAdd(&h.mlo[bin], lo);
+    const unsigned hi = (unsigned)(m >> 32) + (old + lo < old ? 1u : 0u);
+    if (hi) atomicAdd(&h.mhi[bin], hi);
+}
+
+// What a search has narrowed its threshold down to: the keys [d_lo, d_lo + 2^width) and what lies above them.
+struct KeyRange {
+    unsigned d_lo;
+    int width;
+    unsigned above_cnt;
+    unsigned long long above_mass, sel_mass;
+};
+
+// Choose the first bin (thread = bin, holding count c and mass m) that `met(inclusive count, inclusive mass)` holds at.
+template <typename MetFn>
+__device__ __forceinline__ int choose_bin(unsigned c, unsigned long long m, MetFn met, FilterSmem *fs, KeyRange &kr) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned ci = c;              // inclusive sums over the bins, from the largest keys down
+    unsigned long long mi = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned tc = __shfl_up_sync(0xffffffffu, ci, o);
+        const unsigned long long tm = __shfl_up_sync(0xffffffffu, mi, o);
+        if (lane >= o) { ci += tc; mi += tm; }
+    }
+    if (lane == 31) { fs->wcnt[warp] = ci; fs->wmass[warp] = mi; }
+    if (tid == 0) { fs->first = kBins; fs->last = -1; }
+    __syncthreads();
+    unsigned wc = lane < warp ? fs->wcnt[lane] : 0u;
+    unsigned long long wm = lane < warp ? fs->wmass[lane] : 0ull;
+    wc = __reduce_add_sync(0xffffffffu, wc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wm += __shfl_xor_sync(0xffffffffu, wm, o);
+    ci += wc;
+    mi += wm;
+    const unsigned met_mask = __ballot_sync(0xffffffffu, c > 0 && met(kr.above_cnt + ci, kr.above_mass + mi));
+    const unsigned any_mask = __ballot_sync(0xffffffffu, c > 0);
+    if (lane == 0) {
+        if (met_mask) atomicMin(&fs->first, tid + __ffs(met_mask) - 1);
+        if (any_mask) atomicMax(&fs->last, tid + 31 - __clz(any_mask));
+    }
+    __syncthreads();
+    const int sel = fs->first < kBins ? fs->first : max(fs->last, 0);  // (out of reach: keep everything there is)
+    if (tid == sel) {
+        fs->above_cnt = kr.above_cnt + ci - c;
+        fs->above_mass = kr.above_mass + mi - m;
+        fs->sel_mass = m;
+    }
+    __syncthreads();
+    kr.above_cnt = fs->above_cnt;
+    kr.above_mass = fs->above_mass;
+    kr.sel_mass = fs->sel_mass;
+    return sel;
+}
+
+// grid (kFilterCluster rows, B): statistics, restriction and p row of the rows that a restriction applies to.
+struct FilterArgs {
+    const float *logits;  // [B, M, V]
+    int M, V;
+    const int32_t *n_eff; // null: every row, grid.x = kFilterCluster M; else only row n_eff[b] - 1 of sequence b
+    float inv_t;
+    int top_k;
+    float top_p;
+    RowStat *stats;       // [B, grid.x / kFilterCluster]
+    RowFilter *filt;
+    float *p_out;         // [B, M, V] or null
+};
+__global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailThreads) row_filter_kernel(FilterArgs a) {
+    extern __shared__ float fcache[];
+    __shared__ FilterSmem sm;
+    FilterSmem *fs = &sm;
+    cg::cluster_group cl = cg::this_cluster();
+    constexpr int IT = kFilterBatch, kStep = 32 * IT;
+    const int b = blockIdx.y, i = blockIdx.x / kFilterCluster, V = a.V, n_rows = gridDim.x / kFilterCluster;
+    const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const float inv_t = a.inv_t;
+    const size_t row = (size_t)b * a.M + (a.n_eff ? max(a.n_eff[b] - 1, 0) : i);
+    const float *lg = a.logits + row * V;
+    int lo, hi;
+    row_piece(V, kFilterCluster * kTailWarps, rank * kTailWarps + warp, lo, hi);
+    const bool cached = filter_smem(V) > 0;
+    int cta_lo, unused;
+    row_piece(V, kFilterCluster * kTailWarps, rank * kTailWarps, cta_lo, unused);
+    float *mine = fcache - cta_lo;   // entry j of the row at mine[j]
+
+    // ---- statistics; the logits stay in shared memory ----
+    float mx = -INFINITY;
+    int at = 0x7fffffff;
+    for (int base = lo; base < hi; base += kStep) {
+        float x[IT];
+        tail_load<IT>(lg, base, hi, -INFINITY, x);
+#pragma unroll
+        for (int u = 0; u < IT; ++u) {
+            const int j = base + 32 * u + lane;
+            if (x[u] > mx) { mx = x[u]; at = j; }
+            if (cached && j < hi) mine[j] = x[u];
+        }
+    }
+    auto entry = [&](int j) { return cached ? mine[j] : __ldcg(lg + j); };
+    {
+        const float m = warp_max_redux(mx);
+        const int am = __reduce_min_sync(0xffffffffu, mx == m ? at : 0x7fffffff);
+        float part = 0.f;
+        if (m > -INFINITY)
+            for (int j = lo + lane; j < hi; j += 32) part += expf((entry(j) - m) * inv_t);
+        const double s = warp_sum((double)part);
+        if (lane == 0) {
+            PartStat t;
+            t.mx = m;
+            t.am = am;
+            t.s = s;
+            fs->warp[warp] = t;
+        }
+    }
+    for (int k = tid; k < 2 * 3 * kBins; k += kTailThreads) reinterpret_cast<unsigned *>(fs->hist)[k] = 0;
+    __syncthreads();
+    if (warp == 0) {
+        const PartStat t = join_parts<32>(fs->warp[lane], inv_t);
+        if (lane == 0) fs->cta = t;
+    }
+    cl.sync();
+    const RowStat st = row_stat(join_parts<kFilterCluster>(*cl.map_shared_rank(&fs->cta, lane % kFilterCluster), inv_t));
+    const unsigned kmax = __float_as_uint(prob_of(st.mx, st, inv_t, st.amax));
+
+    // ---- histogram of the keys in [d_lo, d_lo + bins << shift) with p >= p_min (open_end: the last bin takes all beyond) ----
+    auto count = [&](FilterHist &h, unsigned d_lo, int shift, int bins, bool open_end, float p_min, bool first) {
+        int bin = -1;
+        unsigned c = 0;
+        unsigned long long m = 0;
+        for (int j = lo + lane; j < hi; j += 32) {
+            float p;
+            if (first || !cached) {
+                p = prob_of(entry(j), st, inv_t, j);
+                if (cached) mine[j] = p;
+            } else {
+                p = mine[j];
+            }
+            if (!(p >= p_min)) continue;   // (a NaN is not looked at)
+            const unsigned bits = __float_as_uint(p), d = bits < kmax ? kmax - bits : 0u;
+            if (d < d_lo) continue;
+            unsigned k = (d - d_lo) >> shift;
+            if (k >= (unsigned)bins) {
+                if (!open_end) continue;
+                k = bins - 1;
+            }
+            if ((int)k != bin) {
+                bin_add(h, bin, c, m);
+                bin = (int)k;
+                c = 0;
+                m = 0;
+            }
+            ++c;
+            m += __double2ull_rz((double)fminf(p, 2.f) * kMassUnit);
+        }
+        bin_add(h, bin, c, m);
+    };
+    auto joined = [&](int h, unsigned &c, unsigned long long &m) {  // this thread's bin over the cluster
+        c = 0;
+        m = 0;
+#pragma unroll
+        for (int r = 0; r < kFilterCluster; ++r) {
+            const FilterHist *o = cl.map_shared_rank(&fs->hist[h], r);
+            c += o->cnt[tid];
+            m += (unsigned long long)o->mlo[tid] + ((unsigned long long)o->mhi[tid] << 32);
+        }
+    };
+    int turn = 0;
+    auto refine = [&](KeyRange &kr, float p_min, auto met) {  // down to one key
+        while (kr.width > 0) {
+            const int shift = max(0, kr.width - 10), h = 1 + (turn & 1);
+            ++turn;
+            count(fs->hist[h], kr.d_lo, shift, 1 << (kr.width - shift), false, p_min, false);
+            cl.sync();
+            unsigned c;
+            unsigned long long m;
+            joined(h, c, m);
+            for (int k = tid; k < 3 * kBins; k += kTailThreads) reinterpret_cast<unsigned *>(&fs->hist[3 - h])[k] = 0;  // (read by all before the barrier above)
+            const int sel = choose_bin(c, m, met, fs, kr);
+            kr.d_lo += (unsigned)sel << shift;
+            kr.width = shift;
+        }
+    };
+    constexpr int kShift0 = 18;
+    auto range_of = [&](int sel, KeyRange &kr) {
+        kr.d_lo = (unsigned)sel << kShift0;
+        kr.width = sel == kBins - 1 ? 30 : kShift0;
+    };
+    count(fs->hist[0], 0u, kShift0, kBins, true, 0.f, true);
+    cl.sync();
+    unsigned c0;
+    unsigned long long m0;
+    joined(0, c0, m0);
+
     RowFilter f;
     f.thr = 0.f;
     f.mass = 0.f;
-    const bool use_k = top_k > 0 && top_k < V, use_p = top_p > 0.f && top_p < 1.f;
-    if (inv_t == 0.f || (!use_k && !use_p)) return f;
-    auto prob = [&](int j) { return prob_of(__ldcg(logits + j), st, inv_t, j); };
     double mass = 0.0;
-    float thr = 0.f;
-    if (use_k) thr = select_threshold(prob, V, 0.f, false, (unsigned)top_k, 0.0, fs, cl, &mass);
-    if (use_p) thr = select_threshold(prob, V, thr, true, 0u, (double)top_p, fs, cl, &mass);
-    f.thr = thr;
-    f.mass = (float)mass;
-    return f;
-}
-
-// Inverse-CDF draw over V weights w(j) >= 0 by the whole cluster: the smallest j whose inclusive prefix
-// sum exceeds u * S; prefix sums in index order, fp64.  If rounding leaves none: the largest j with
-// w > 0.  Each CTA owns a slice, each thread a contiguous segment of it, so the prefix order is the
-// index order: thread sums are scanned inside the CTA, CTA totals in rank order across the cluster.
-// `slot` (0 or 1) selects the exchange slots, so that two draws in one kernel need no extra barrier.
-// Returns S via *total; S and the drawn index are the same in every thread of the cluster.  S <= 0
-// returns -1.
-template <typename WeightFn>
-__device__ __forceinline__ int inv_cdf_cluster(WeightFn w, int V, float u, double *sd, int *si, double *total,
-                                               ClusterSlots *pub, cg::cluster_group &cl, int slot) {
-    const int rank = (int)cl.block_rank();
-    int lo, hi;
-    tail_slice(V, rank, lo, hi);
-    const int seg = (hi - lo + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int j0 = min(hi, lo + (int)threadIdx.x * seg), j1 = min(hi, j0 + seg);
-    double local = 0.0;
-    int last_pos = -1;
-    for (int j = j0; j < j1; ++j) {
-        float wj = w(j);
-        local += (double)wj;
-        if (wj > 0.f) last_pos = j;
+    const bool use_k = a.top_k > 0 && a.top_k < V, use_p = a.top_p > 0.f && a.top_p < 1.f;
+    unsigned long long kept = ~0ull;  // mass of what top-k keeps
+    if (use_k) {
+        const unsigned want = (unsigned)a.top_k;
+        auto met = [&](unsigned c, unsigned long long) { return c >= want; };
+        KeyRange kr = {0u, 0, 0u, 0ull, 0ull};
+        const int sel = choose_bin(c0, m0, met, fs, kr);
+        const unsigned long long above = kr.above_mass;
+        range_of(sel, kr);
+        refine(kr, 0.f, met);
+        f.thr = __uint_as_float(kmax - min(kr.d_lo, kmax));
+        kept = kr.above_mass + kr.sel_mass;
+        mass = (double)kept / kMassUnit;
+        // top-p looks at what is left: whole bins above the chosen one, a part of it
+        if (tid == sel) m0 = kept - above;
+        if (tid > sel) { c0 = 0; m0 = 0; }
     }
-    // exclusive scan of the per-thread sums over the block (warp scan + scan of warp totals)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double incl = local;
+    if (use_p) {
+        if (kept == ~0ull) {  // (everything: the sum over the bins, once more through the exchange words)
+            unsigned long long w = m0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        double t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+            for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+            if (lane == 0) fs->wmass[warp] = w;
+            __syncthreads();
+            kept = 0;
+            for (int k = 0; k < kTailWarps; ++k) kept += fs->wmass[k];
+            __syncthreads();
+        }
+        const unsigned long long target = __double2ull_ru((double)a.top_p * (double)kept);
+        auto met = [&](unsigned, unsigned long long m) { return m >= target; };
+        KeyRange kr = {0u, 0, 0u, 0ull, 0ull};
+        const int sel = choose_bin(c0, m0, met, fs, kr);
+        range_of(sel, kr);
+        refine(kr, f.thr, met);
+        f.thr = __uint_as_float(kmax - min(kr.d_lo, kmax));
+        mass = (double)(kr.above_mass + kr.sel_mass) / kMassUnit;
     }
-    __syncthreads();
-    if (lane == 31) sd[wid] = incl;
-    if (threadIdx.x == 0) { si[0] = 0x7fffffff; si[1] = -1; }
-    __syncthreads();
-    double warp_off = 0.0, T = 0.0;
-    for (int k = 0; k < nw; ++k) {  // nw <= 32: short serial pass keeps the order fixed
-        double t = sd[k];
-        if (k < wid) warp_off += t;
-        T += t;
+    f.mass = (float)mass;
+    if (rank == 0 && tid == 0) {
+        a.stats[(size_t)b * n_rows + i] = st;
+        a.filt[(size_t)b * n_rows + i] = f;
     }
-    if (threadIdx.x == 0) pub->d[1 + slot] = T;
-    cl.sync();
-    double cta_off = 0.0, S = 0.0;
-    for (int r = 0; r < kTailCluster; ++r) {
-        const double t = cl.map_shared_rank(pub, r)->d[1 + slot];
-        if (r < rank) cta_off += t;
-        S += t;
-    }
-    *total = S;
-    if (!(S > 0.0)) return -1;  // the same decision in every CTA of the cluster
-    const double target = (double)u * S;
-    double run = cta_off + warp_off + (incl - local);
-    int hit = 0x7fffffff;
-    if (run + local > target || run > target) {
-        for (int j = j0; j < j1; ++j) {
-            const float wj = w(j);
-            run += (double)wj;
-            if (wj > 0.f && run > target) { hit = j; break; }  // a zero-weight index is never drawn
+    if (a.p_out) {
+        float *p = a.p_out + row * V;
+        for (int j = lo + lane; j < hi; j += 32) {
+            const float pr = cached ? mine[j] : prob_of(__ldcg(lg + j), st, inv_t, j);
+            p[j] = pr >= f.thr ? pr / f.mass : 0.f;   // (as prob_f)
         }
     }
-    if (hit != 0x7fffffff) atomicMin(&si[0], hit);
-    if (last_pos >= 0) atomicMax(&si[1], last_pos);
-    __syncthreads();
-    if (threadIdx.x == 0) { pub->i[1 + 2 * slot] = si[0]; pub->i[2 + 2 * slot] = si[1]; }
-    cl.sync();
-    int first = 0x7fffffff, last = -1;
-    for (int r = 0; r < kTailCluster; ++r) {
-        const ClusterSlots *o = cl.map_shared_rank(pub, r);
-        first = min(first, o->i[1 + 2 * slot]);
-        last = max(last, o->i[2 + 2 * slot]);
+    cl.sync();  // nobody leaves while its shared memory is read
+}
+
+// ---- inverse-CDF draw -------------------------------------------------------------------------------
+struct DrawSmem {
+    double tot[kTailWarps], incl[kTailWarps];  // the warps' sums, and their running sums
+    double cta[2];              // this CTA's total, by draw (a kernel draws at most twice)
+    float w[32 * 8];            // the owner warp's entries, handed from its load order to index order
+};
+
+// Inverse-CDF draw over V weights >= 0 by the whole cluster: the smallest j whose inclusive prefix sum (fp64, pieces in
+// index order) exceeds u * S.  `weights(base, w)` gives the piece's weights from `base` on, 0 beyond its end; it is
+// called again by the warp whose piece the draw falls into.  That warp is found without a vote: piece boundaries are the
+// same fp64 numbers on both sides (a piece ends where the next one starts), so exactly one piece holds u * S.  Inside it
+// a zero-weight index is never drawn; if rounding leaves no index, the piece's largest with weight > 0 is taken.
+// Returns the index in every lane of that warp and -1 elsewhere; *total = S everywhere (S <= 0: nothing was drawn).
+template <int IT, typename WeightFn>
+__device__ __forceinline__ int cluster_draw(WeightFn weights, int V, float u, DrawSmem *ds, cg::cluster_group &cl, int slot,
+                                            double *total) {
+    constexpr int kStep = 32 * IT;
+    const int rank = (int)cl.block_rank(), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int lo, hi;
+    tail_piece(V, rank, lo, hi);
+    double sum = 0.0;
+    float w[IT];
+    for (int b = lo; b < hi; b += kStep) {
+        weights(b, w);
+#pragma unroll
+        for (int k = 0; k < IT; ++k) sum += (double)w[k];
     }
-    return first != 0x7fffffff ? first : last;
+    sum = warp_sum(sum);
+    if (lane == 0) ds->tot[warp] = sum;
+    __syncthreads();
+    // Piece boundaries as running sums in index order: what one warp takes for its end is bit for bit the next one's beginning.
+    if (warp == 0) {
+        double T = 0.0;
+#pragma unroll
+        for (int k = 0; k < kTailWarps; ++k)
+            if (k <= lane) T += ds->tot[k];
+        ds->incl[lane] = T;
+        if (lane == 31) ds->cta[slot] = T;
+    }
+    cl.sync();
+    const double w_beg = warp ? ds->incl[warp - 1] : 0.0, w_end = ds->incl[warp];
+    const double one_cta = lane < kTailCluster ? *cl.map_shared_rank(&ds->cta[slot], lane) : 0.0;
+    double c_beg = 0.0, S = 0.0;
+#pragma unroll
+    for (int k = 0; k < kTailCluster; ++k) {
+        if (k == rank) c_beg = S;
+        S += __shfl_sync(0xffffffffu, one_cta, k);
+    }
+    *total = S;
+    if (!(S > 0.0)) return -1;
+    const double beg = c_beg + w_beg, end = c_beg + w_end;  // (the last warp's end is c_beg + T, where the next CTA begins)
+    const double target = (double)u * S;
+    if (!(beg <= target && target < end)) return -1;  // the same in all lanes
+    double run = beg;
+    int hit = -1, last = -1;
+    for (int b = lo; b < hi && hit < 0; b += kStep) {
+        weights(b, w);
+#pragma unroll
+        for (int k = 0; k < IT; ++k) ds->w[32 * k + lane] = w[k];
+        __syncwarp();
+        float v[IT];
+        double s = 0.0;
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            v[k] = ds->w[IT * lane + k];
+            s += (double)v[k];
+        }
+        double si = s;  // inclusive over the lanes
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double t = __shfl_up_sync(0xffffffffu, si, o);
+            if (lane >= o) si += t;
+        }
+        double r = run + (si - s);
+        int mine = 0x7fffffff, tail = -1;
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            r += (double)v[k];
+            if (v[k] > 0.f) {
+                tail = b + IT * lane + k;
+                if (mine == 0x7fffffff && r > target) mine = tail;
+            }
+        }
+        mine = __reduce_min_sync(0xffffffffu, mine);
+        last = max(last, __reduce_max_sync(0xffffffffu, tail));
+        if (mine != 0x7fffffff) hit = mine;
+        run += __shfl_sync(0xffffffffu, si, 31);
+        __syncwarp();
+    }
+    return hit >= 0 ? hit : last;
 }
 
 struct VerifyArgs {
@@ -342,82 +595,100 @@ struct VerifyArgs {
     int next_stride;
     float *p_debug;         // [B, K+1, V] or null
     int32_t *keep;          // [B] or null: n_accepted + 1 for kv_commit
-    RowStat *stats;         // scratch [B, K+1]
-    RowFilter *filt;        // scratch [B, K+1]
-    int top_k;              // restriction of the target rows (0 / 1.0: none); q arrives already restricted
-    float top_p;
+    const RowStat *stats;   // [B, K+1], only under a restriction of the target rows (q arrives already restricted)
+    const RowFilter *filt;
 };
 
-// grid (kTailCluster (K+1), B), one cluster per row: statistics of every row (+ optional export of the p row)
-__global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThreads) row_stats_kernel(VerifyArgs a) {
-    __shared__ float sv[32];
-    __shared__ int si[32];
-    __shared__ double sd[32];
-    __shared__ ClusterSlots pub;
-    __shared__ FilterSmem fs;
-    cg::cluster_group cl = cg::this_cluster();
-    const int i = blockIdx.x / kTailCluster, b = blockIdx.y;
-    const float *lg = a.logits + ((size_t)b * (a.K + 1) + i) * a.V;
-    RowStat st = row_stats(lg, a.V, a.inv_t, sv, si, sd, &pub, cl);
-    const RowFilter fl = row_filter(lg, a.V, st, a.inv_t, a.filt ? a.top_k : 0, a.top_p, &fs, cl);  // (no room for it: no restriction)
-    if (cl.block_rank() == 0 && threadIdx.x == 0) {
-        a.stats[b * (a.K + 1) + i] = st;
-        if (a.filt) a.filt[b * (a.K + 1) + i] = fl;
-    }
-    if (a.p_debug) {
-        int lo, hi;
-        tail_slice(a.V, (int)cl.block_rank(), lo, hi);
-        float *p = a.p_debug + ((size_t)b * (a.K + 1) + i) * a.V;
-        for (int j = lo + threadIdx.x; j < hi; j += blockDim.x) p[j] = prob_f(lg[j], st, fl, a.inv_t, j);
-    }
-    cl.sync();
-}
-
-// grid (kTailCluster B), one cluster per sequence: accept scan, then residual / bonus draw
+// grid (kTailCluster B), one cluster per sequence: row statistics (given by row_filter_kernel under a restriction), accept
+// scan, then residual / bonus draw.
+template <bool kGiven, int IT>
 __global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThreads) verify_kernel(VerifyArgs a) {
-    __shared__ double sd[32];
-    __shared__ int si[32];
+    __shared__ StatSmem ss;
+    __shared__ DrawSmem ds;
     __shared__ int s_acc;
-    __shared__ ClusterSlots pub;
     cg::cluster_group cl = cg::this_cluster();
-    const int b = blockIdx.x / kTailCluster, K = a.K, V = a.V;
-    const RowStat *st = a.stats + b * (K + 1);
+    constexpr int kStep = 32 * IT;
+    const int b = blockIdx.x / kTailCluster, K = a.K, V = a.V, lane = threadIdx.x & 31;
+    const float *logits = a.logits + (size_t)b * (K + 1) * V;
     const RowFilter none = {0.f, 0.f};
-    if (threadIdx.x == 0) {  // (every CTA of the cluster takes the same few steps)
-        int acc = 0;
-        for (int i = 0; i < K; ++i) {
-            int x = a.rows[b * (K + 1) + 1 + i];
-            x = max(0, min(x, V - 1));
-            const float px = prob_f(a.logits[((size_t)b * (K + 1) + i) * V + x], st[i], a.filt ? a.filt[b * (K + 1) + i] : none, a.inv_t, x);
-            const float qx = a.q[((size_t)b * K + i) * V + x];
-            // accept with probability min(1, p/q): u * q < p, one fp32 rounding of the product
-            if (__fmul_rn(a.u[b * (K + 1) + i], qx) < px) ++acc; else break;
+    const float inv_t = a.inv_t;
+    // what the accept scan needs of row i, in lane i of warp 0: on its way under the statistics
+    float xl = 0.f, xq = 0.f, xu = 0.f;
+    int x = 0;
+    if (threadIdx.x < K) {
+        x = max(0, min(a.rows[b * (K + 1) + 1 + lane], V - 1));
+        xl = __ldcg(logits + (size_t)lane * V + x);
+        xq = __ldcg(a.q + ((size_t)b * K + lane) * V + x);
+        xu = a.u[b * (K + 1) + lane];
+    }
+    const float u = a.u[b * (K + 1) + K];
+    if (kGiven) {
+        for (int i = threadIdx.x; i <= K; i += kTailThreads) ss.row[i] = a.stats[b * (K + 1) + i];
+        __syncthreads();
+    } else {
+        float l[IT];
+        cluster_stats<IT>(logits, K + 1, V, inv_t, &ss, cl, l);
+    }
+    if (threadIdx.x < 32) {  // (every CTA of the cluster takes the same few steps)
+        bool ok = false;
+        if (lane < K) {
+            const float px = prob_f(xl, ss.row[lane], kGiven ? a.filt[b * (K + 1) + lane] : none, inv_t, x);
+            ok = __fmul_rn(xu, xq) < px;  // accept with probability min(1, p/q): u * q < p, one fp32 rounding of the product
         }
-        s_acc = acc;
+        const unsigned refused = ~__ballot_sync(0xffffffffu, ok);  // (K <= 31: lane K always refuses)
+        if (lane == 0) s_acc = min(K, __ffs(refused) - 1);
     }
     __syncthreads();
     const int acc = s_acc;
-    const float *lg = a.logits + ((size_t)b * (K + 1) + acc) * V;
-    const RowStat rs = st[acc];
-    const RowFilter rf = a.filt ? a.filt[b * (K + 1) + acc] : none;
-    const float u = a.u[b * (K + 1) + K];
-    const float inv_t = a.inv_t;
-    double S;
+    const float *lg = logits + (size_t)acc * V;
+    const RowStat rs = ss.row[acc];
+    const RowFilter rf = kGiven ? a.filt[b * (K + 1) + acc] : none;
+    const int rank = (int)cl.block_rank();
+    int lo, hi;
+    tail_piece(V, rank, lo, hi);
+    double S = 0.0;
     int y = -1;
+    auto p_weights = [&](int base, float (&w)[IT]) {
+        tail_load<IT>(lg, base, hi, 0.f, w);
+#pragma unroll
+        for (int k = 0; k < IT; ++k) w[k] = base + lane + 32 * k < hi ? prob_f(w[k], rs, rf, inv_t, base + lane + 32 * k) : 0.f;
+    };
     if (acc < K) {
         const float *qr = a.q + ((size_t)b * K + acc) * V;
-        y = inv_cdf_cluster([&](int j) { return fmaxf(0.f, __fsub_rn(prob_f(lg[j], rs, rf, inv_t, j), qr[j])); }, V, u,
-                            sd, si, &S, &pub, cl, 0);
+        y = cluster_draw<IT>(
+            [&](int base, float (&w)[IT]) {
+                float qv[IT];
+                tail_load<IT>(qr, base, hi, 0.f, qv);
+                p_weights(base, w);
+#pragma unroll
+                for (int k = 0; k < IT; ++k) w[k] = fmaxf(0.f, __fsub_rn(w[k], qv[k]));
+            },
+            V, u, &ds, cl, 0, &S);
     }
-    if (y < 0)  // all accepted: bonus from p_{K+1}; or an all-zero residual: fall back to p
-        y = inv_cdf_cluster([&](int j) { return prob_f(lg[j], rs, rf, inv_t, j); }, V, u, sd, si, &S, &pub, cl, 1);
-    if (y < 0) y = rs.amax;  // a row whose probabilities all vanished (non-finite logits)
-    if (cl.block_rank() == 0 && threadIdx.x == 0) {
+    if (!(S > 0.0))  // all accepted: bonus from p_{K+1}; or an all-zero residual: fall back to p
+        y = cluster_draw<IT>(p_weights, V, u, &ds, cl, 1, &S);
+    const bool first = rank == 0 && threadIdx.x == 0;
+    if (!(S > 0.0) && first) y = rs.amax;  // a row whose probabilities all vanished (non-finite logits)
+    if (y >= 0 && lane == 0) a.next_token[(size_t)b * a.next_stride] = y;
+    if (first) {
         a.n_accepted[b] = acc;
-        a.next_token[(size_t)b * a.next_stride] = y;
         if (a.keep) a.keep[b] = acc + 1;
     }
-    cl.sync();
+    if (!kGiven && a.p_debug) {
+        for (int i = 0; i <= K; ++i) {
+            const RowStat st = ss.row[i];
+            const float *row = logits + (size_t)i * V;
+            float *p = a.p_debug + ((size_t)b * (K + 1) + i) * V;
+            for (int base = lo; base < hi; base += kStep) {
+                float l[IT];
+                tail_load<IT>(row, base, hi, 0.f, l);
+#pragma unroll
+                for (int k = 0; k < IT; ++k)
+                    if (base + lane + 32 * k < hi) p[base + lane + 32 * k] = prob_of(l[k], st, inv_t, base + lane + 32 * k);
+            }
+        }
+    }
+    cl.sync();  // nobody leaves while its shared memory is read
 }
 
 struct DraftTailArgs {
@@ -428,89 +699,112 @@ struct DraftTailArgs {
     const float *u; int u_stride;
     int32_t *token_out; int token_stride;
     float *q_out; size_t q_stride;
-    int top_k;            // restriction of q (0 / 1.0: none)
-    float top_p;
+    const RowStat *stats; // [B], only under a restriction: of the sampled rows, from row_filter_kernel
+    const RowFilter *filt;
+    int32_t *len;         // [B] committed lengths: the fed rows are committed here
+    unsigned long long *mailbox; unsigned seq;  // see report_len
 };
 
-// grid (kTailCluster B), one cluster per sequence: q = softmax(last row / T), exported; x~ = inverse-CDF(q, u)
+__device__ __forceinline__ void report_len(unsigned long long *mailbox, int b, unsigned seq, int len);
+
+// grid (kTailCluster B), one cluster per sequence: q = softmax(last row / T), exported; x~ = inverse-CDF(q, u); the fed
+// rows become part of the cache
+template <bool kGiven, int IT>
 __global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThreads) draft_tail_kernel(DraftTailArgs a) {
-    __shared__ float sv[32];
-    __shared__ int si[32];
-    __shared__ double sd[32];
-    __shared__ ClusterSlots pub;
-    __shared__ FilterSmem fs;
+    __shared__ StatSmem ss;
+    __shared__ DrawSmem ds;
     cg::cluster_group cl = cg::this_cluster();
-    const int b = blockIdx.x / kTailCluster;
-    int row = a.n_eff[b] - 1;
-    if (row < 0) row = 0;
+    constexpr int kStep = 32 * IT;
+    const int b = blockIdx.x / kTailCluster, rank = (int)cl.block_rank(), lane = threadIdx.x & 31;
+    const int fed = a.n_eff[b], row = max(fed - 1, 0);
+    const float u = a.u[(size_t)b * a.u_stride];
     const float *lg = a.logits + ((size_t)b * a.M + row) * a.V;
-    const RowStat st = row_stats(lg, a.V, a.inv_t, sv, si, sd, &pub, cl);
-    const RowFilter fl = row_filter(lg, a.V, st, a.inv_t, a.top_k, a.top_p, &fs, cl);
-    float *q = a.q_out + (size_t)b * a.q_stride;
     int lo, hi;
-    tail_slice(a.V, (int)cl.block_rank(), lo, hi);
-    for (int j = lo + threadIdx.x; j < hi; j += blockDim.x) q[j] = prob_f(lg[j], st, fl, a.inv_t, j);
-    __syncthreads();  // the draw below reads this CTA's own slice of q
+    tail_piece(a.V, rank, lo, hi);
+    float l[IT];
+    RowStat st;
+    RowFilter fl = {0.f, 0.f};
+    if (kGiven) {
+        tail_load<IT>(lg, lo, hi, 0.f, l);
+        st = a.stats[b];
+        fl = a.filt[b];
+    } else {
+        cluster_stats<IT>(lg, 1, a.V, a.inv_t, &ss, cl, l);
+        st = ss.row[0];
+    }
+    float *q = a.q_out + (size_t)b * a.q_stride;
+    const bool one = hi - lo <= kStep;
+    for (int base = lo; base < hi; base += kStep) {
+        if (!one) tail_load<IT>(lg, base, hi, 0.f, l);
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            const int j = base + lane + 32 * k;
+            l[k] = j < hi ? prob_f(l[k], st, fl, a.inv_t, j) : 0.f;
+            if (j < hi) q[j] = l[k];
+        }
+    }
     double S;
-    int y = inv_cdf_cluster([&](int j) { return q[j]; }, a.V, a.u[(size_t)b * a.u_stride], sd, si, &S, &pub, cl, 0);
-    if (y < 0) y = st.amax;
-    if (cl.block_rank() == 0 && threadIdx.x == 0) a.token_out[(size_t)b * a.token_stride] = y;
-    cl.sync();
+    int y = cluster_draw<IT>(
+        [&](int base, float (&w)[IT]) {
+            if (one) {
+#pragma unroll
+                for (int k = 0; k < IT; ++k) w[k] = l[k];
+            } else {
+                tail_load<IT>(q, base, hi, 0.f, w);  // (written by this very lane)
+            }
+        },
+        a.V, u, &ds, cl, 0, &S);
+    const bool first = rank == 0 && threadIdx.x == 0;
+    if (!(S > 0.0) && first) y = st.amax;
+    if (y >= 0 && lane == 0) a.token_out[(size_t)b * a.token_stride] = y;
+    if (first) {
+        const int n = a.len[b] + fed;  // fed is what the forward's set-up found to fit
+        a.len[b] = n;
+        report_len(a.mailbox, b, a.seq, n);
+    }
+    cl.sync();  // nobody leaves while its shared memory is read
 }
 
 // ---------------- cache length bookkeeping ----------------
-// Every kernel that changes the committed lengths runs as ONE block of 64 threads (at most 64 sequences)
-// and afterwards reports the largest length to the host through a word of mapped host memory, tagged with
-// the host's sequence number of the operation: (seq << 32) | max length.  The host plans attention splits
-// from an upper bound of the lengths; with this word the bound follows the real lengths without a
+// Every kernel that changes a committed length reports it to the host through the sequence's word of mapped host
+// memory, tagged with the host's number of the operation: (seq << 32) | length.  The host plans attention splits
+// from an upper bound of the lengths; with these words the bound follows the real lengths without a
 // synchronisation (it adds what the operations queued behind `seq` can add at most).
-__device__ __forceinline__ void report_max_len(int my_len, unsigned long long *mailbox, unsigned seq) {
-    __shared__ int s_max[2];
-    int v = my_len;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0 && mailbox) {
-        const unsigned m = (unsigned)max(s_max[0], s_max[1]);
-        *reinterpret_cast<volatile unsigned long long *>(mailbox) = ((unsigned long long)seq << 32) | m;
-    }
+__device__ __forceinline__ void report_len(unsigned long long *mailbox, int b, unsigned seq, int len) {
+    if (mailbox) *reinterpret_cast<volatile unsigned long long *>(mailbox + b) = ((unsigned long long)seq << 32) | (unsigned)len;
 }
 // Keep n_keep[b] more rows.  A length that would pass the capacity S is clamped and recorded as
 // SSD_E_CAPACITY in the sticky status word: rows that no forward wrote must not become context.
 __global__ void kv_commit_kernel(int32_t *len, const int32_t *n_keep, int B, int S, int32_t *status,
                                  unsigned long long *mailbox, unsigned seq) {
     const int b = threadIdx.x;
-    int v = 0;
     if (b < B) {
-        v = len[b] + max(0, n_keep[b]);
+        int v = len[b] + max(0, n_keep[b]);
         if (v > S) {
             v = S;
             set_status(status, -3);
         }
         len[b] = v;
+        report_len(mailbox, b, seq, v);
     }
-    report_max_len(v, mailbox, seq);
 }
 __global__ void kv_commit_rows_kernel(int32_t *len, const int32_t *n_eff, int B, unsigned long long *mailbox,
                                       unsigned seq) {
     const int b = threadIdx.x;
-    int v = 0;
     if (b < B) {
-        v = len[b] + n_eff[b];   // n_eff is what the forward's set-up found to fit
+        const int v = len[b] + n_eff[b];   // n_eff is what the forward's set-up found to fit
         len[b] = v;
+        report_len(mailbox, b, seq, v);
     }
-    report_max_len(v, mailbox, seq);
 }
 __global__ void kv_rollback_kernel(int32_t *len, const int32_t *new_len, int B, unsigned long long *mailbox,
                                    unsigned seq) {
     const int b = threadIdx.x;
-    int v = 0;
     if (b < B) {
-        v = max(0, min(len[b], new_len[b]));
+        const int v = max(0, min(len[b], new_len[b]));
         len[b] = v;
+        report_len(mailbox, b, seq, v);
     }
-    report_max_len(v, mailbox, seq);
 }
 // chunk c of a prompt pass: rows fed per sequence = clamp(n_tokens - c*C, 0, C)
 __global__ void prefill_rows_kernel(const int32_t *n_tokens, int chunk, int C, int32_t *n_rows, int B) {
@@ -526,11 +820,11 @@ struct AdvanceArgs {
     int next_stride;
     int32_t *out_tokens; int out_cap; int32_t *out_count;
     int32_t *draft_in, *draft_n_in;
-    unsigned long long *t_mailbox, *d_mailbox;  // see report_max_len
+    unsigned long long *t_mailbox, *d_mailbox;  // see report_len
     unsigned t_seq, d_seq;
 };
 
-__device__ __forceinline__ void spec_advance_one(const AdvanceArgs &a, int b, int &t_new, int &d_new) {
+__device__ __forceinline__ void spec_advance_one(const AdvanceArgs &a, int b) {
     const int K = a.K;
     int acc = max(0, min(a.n_accepted[b], K));
     const int y = a.next_token[(size_t)b * a.next_stride];
@@ -556,21 +850,18 @@ __device__ __forceinline__ void spec_advance_one(const AdvanceArgs &a, int b, in
             a.draft_n_in[b] = 1;
         }
     }
-    t_new = a.tlen[b] + acc + 1;
+    const int t_new = n + acc;
     a.tlen[b] = t_new;
+    report_len(a.t_mailbox, b, a.t_seq, t_new);
     if (a.dlen) {
-        d_new = min(a.dlen[b], K > 0 ? min(n + acc, n + K - 1) : n + acc);
+        const int d_new = min(a.dlen[b], K > 0 ? min(n + acc, n + K - 1) : n + acc);
         a.dlen[b] = d_new;
+        report_len(a.d_mailbox, b, a.d_seq, d_new);
     }
     row[0] = y;
 }
 __global__ void spec_advance_kernel(AdvanceArgs a) {  // one block of 64 threads
-    const int b = threadIdx.x;
-    int t_new = 0, d_new = 0;
-    if (b < a.B) spec_advance_one(a, b, t_new, d_new);
-    report_max_len(t_new, a.t_mailbox, a.t_seq);
-    __syncthreads();  // the exchange slots are reused
-    report_max_len(d_new, a.d_mailbox, a.d_seq);
+    if ((int)threadIdx.x < a.B) spec_advance_one(a, threadIdx.x);
 }
 
 }  // namespace ssd

@@ -193,3 +193,35 @@ def test_draft_and_verify_under_a_restriction_follow_the_oracle_loop():
     assert max(int((t["q"][0] > 0).sum()) for t in ref["trace"]) <= top_k     # the restriction was active
     n_out = int(eng.out_count.cpu()[0])
     assert eng.out_tokens.cpu().numpy()[0, :n_out].tolist() == ref["all_tokens"][len(prompt[0]):]
+
+
+@pytest.mark.parametrize("top_k,top_p", [(0, 1.0), (37, 0.9), (0, 0.9)])
+@pytest.mark.parametrize("V", [33, 255, 8193, 65535, 65537, 131100])
+def test_tail_at_the_edges_of_the_row_pieces(V, top_k, top_p):
+    """A cluster's 256 warps own pieces of whole 32-entry lane rows and hold 256 entries at a time: rows shorter than one
+    piece per warp, one entry past a whole number of lane rows, and (from 65537 entries) pieces read in two steps; under a
+    restriction, rows whose probabilities fit the two CTAs' shared memory and (from about 88000 entries) do not; with equal
+    values at the threshold, a flat row (one bin of the search), a row of two values and one with a far tail."""
+    T, K, Bn = 1.0, 3, 2
+    logits, rows, q, u = make_case(3000 + V, Bn, K, V, T, True)
+    logits[0, 1] = 0.25
+    logits[1, 0] = np.where(np.arange(V) % 3 == 0, 1.0, -30.0)
+    logits[1, 2] *= 20.0
+    q = np.stack([[osamp.filter_top_k_top_p(q[b, i], top_k, top_p) for i in range(K)] for b in range(Bn)])
+    rows[:, 1:] = synth.draw_tokens_from_rows(78, q.reshape(Bn * K, V)).reshape(Bn, K)
+    B.set_sampling(top_k, top_p)
+    try:
+        n_acc, nxt, p = run_tail(logits, rows, q, u, T)
+    finally:
+        B.set_sampling(0, 1.0)
+    for b in range(Bn):
+        for i in range(K + 1):
+            raw = osamp.softmax_t(logits[b, i], T)
+            ref = osamp.filter_top_k_top_p(raw, top_k, top_p)
+            odd = raw[(p[b, i] > 0) != (ref > 0)]
+            if odd.size:      # only values at the nucleus boundary, within the rounding of the running sums
+                assert np.ptp(odd) <= 1e-6 * odd.max()
+            else:
+                assert np.abs(p[b, i] - ref).max() <= gu.P_ATOL
+            assert abs(float(p[b, i].astype(np.float64).sum()) - 1.0) < 1e-5
+        gu.check_decisions_on_own_rows(p[b], q[b], rows[b, 1:], u[b, :K], u[b, K], int(n_acc[b]), int(nxt[b]))
