@@ -19,6 +19,7 @@
 #include "rowops.cuh"
 #include "tail.cuh"
 #include "prefill.cuh"
+#include "f32_forward.cuh"
 
 using namespace ssd;
 
@@ -164,6 +165,8 @@ int init_device_once() {
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 16>, attn_smem<__nv_bfloat16, 16>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 32>, attn_smem<__nv_bfloat16, 32>(128));
     rc |= set_smem(row_filter_kernel, (size_t)kFilterCache * 4);
+    rc |= set_smem(forward_f32_kernel<8>, kFfMaxSmem);
+    rc |= set_smem(forward_f32_kernel<kMaxRowsPerSeq>, kFfMaxSmem);
     rc |= set_smem(prefill_gemm_kernel, kPfSmem);
     rc |= set_smem(prefill_attn_kernel, prefill_attn_smem(128));
     rc |= set_smem(prefill_attn_tc_kernel, kPtSmem);
@@ -181,6 +184,7 @@ struct ssd_model {
     std::vector<CUtensorMap> tm;  // bf16 models: per layer {qkv, o, in, out}, then lm head
     std::vector<CUtensorMap> tm256;  // the same four per layer with 256-row boxes (many-row prompt pass)
     int d_in;
+    bool aligned16;  // every tensor starts on a 16-byte boundary
     const ModelDesc *dev_desc;    // bf16 models: the same maps + vector pointers in device memory (caller-owned)
 };
 
@@ -672,10 +676,57 @@ bool single_kernel_path(const ssd_model *m) {
            (a.pos == 0 || a.rotary_dim % 16 == 0);  // the MMA attention tiles heads by 16 and rotary halves by 8
 }
 
+// fp32 models whose row blocks fit shared memory, with contexts that one CTA walks quickly (see f32_forward.cuh)
+bool f32_kernel_path(const ssd_model *m, ssd_kv *kv, int M) {
+    const ssd_arch &a = m->a;
+    return a.dtype == 0 && g_persistent && a.n_layers <= kFfMaxLayers && a.d_ff % 4 == 0 && kv_bound(kv) + M <= kFfMaxCtx &&
+           ff_smem(a.d_model, a.d_ff, a.parallel_residual, M, a.head_dim) <= (size_t)kFfMaxSmem && m->aligned16;
+}
+
+int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int M, const int32_t *n_rows,
+                bool want_logits, const Workspace &w, cudaStream_t st) {
+    const ssd_arch &a = m->a;
+    FfParams p;
+    memset(&p, 0, sizeof(p));
+    p.n_layers = a.n_layers; p.d = a.d_model; p.H = a.n_heads; p.Dh = a.head_dim; p.F = a.d_ff; p.V = a.vocab;
+    p.norm_kind = a.norm; p.swiglu = a.act == 1; p.parallel = a.parallel_residual;
+    p.rotary_dim = a.pos == 1 ? a.rotary_dim : 0; p.learned_pos = a.pos == 0; p.pos_limit = a.pos == 0 ? a.max_pos : 0;
+    p.eps = a.norm_eps; p.rotary_base = a.rotary_base; p.scale = 1.0f / sqrtf((float)a.head_dim);
+    p.B = kv->B; p.M = M; p.R = kv->B * M; p.S = kv->S;
+    p.tokens = tokens; p.tok_stride = tok_stride; p.n_rows = n_rows;
+    p.tok_emb = (const float *)m->w[T_TOK]; p.pos_emb = (const float *)m->w[T_POS];
+    p.lnf_g = (const float *)fw(m, 0); p.lnf_b = (const float *)fw(m, 1); p.w_lm = (const float *)lm_matrix(m);
+    p.cache = (float *)kv->cache; p.layer_elems = kv->layer_bytes / 4;
+    p.len = kv->len; p.status = kv->status; p.ri = w.ri;
+    p.x = w.x; p.qkv = w.qkv; p.ao = w.ao.f32; p.act = w.act.f32; p.logits = w.logits;
+    p.gbar = w.sync;
+    p.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : kWaitCycles;
+    p.want_logits = want_logits ? 1 : 0;
+    for (int l = 0; l < a.n_layers; ++l) {
+        const float **dst = (const float **)&p.layer[l];
+        for (int i = 0; i < PER_LAYER; ++i) dst[i] = (const float *)lw(m, l, i);
+    }
+    // as many CTAs as the widest projection has columns for (a barrier costs less with fewer)
+    int widest = 3 * a.d_model > a.d_ff ? 3 * a.d_model : a.d_ff;
+    if (want_logits && a.vocab > widest) widest = a.vocab;
+    int grid = ceil_div(widest, kFfWarps);
+    if (grid < kv->B * a.n_heads) grid = kv->B * a.n_heads;
+    if (grid > g_num_sms) grid = g_num_sms;
+    const size_t smem = ff_smem(a.d_model, a.d_ff, a.parallel_residual, M, a.head_dim);
+    CUDA_OK(cudaMemsetAsync(w.sync, 0, 64, st));
+    void *args[] = {&p};
+    const void *k = M <= 8 ? (const void *)forward_f32_kernel<8> : (const void *)forward_f32_kernel<kMaxRowsPerSeq>;
+    CUDA_OK(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kFfThreads), args, smem, st));
+    g_launches.fetch_add(1, std::memory_order_relaxed);
+    kv->last_rows = M;
+    return SSD_OK;
+}
+
 int forward(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int M, const int32_t *n_rows,
             bool want_logits, const Workspace &w, cudaStream_t st) {
     const ssd_arch &a = m->a;
     if (single_kernel_path(m)) return forward_persistent(m, kv, tokens, tok_stride, M, n_rows, want_logits, w, st);
+    if (f32_kernel_path(m, kv, M)) return forward_f32(m, kv, tokens, tok_stride, M, n_rows, want_logits, w, st);
     const int B = kv->B, R = B * M, d = a.d_model, F = a.d_ff;
     GemmCall gc{m, st, R, (R + 7) / 8 * 8};
     int rc = run_setup(m, kv, M, n_rows, w, st);
@@ -961,6 +1012,8 @@ int ssd_model_create(const ssd_arch *arch, const void *const *dev_weights, int n
     m->a = *arch;
     m->w.assign(dev_weights, dev_weights + n_tensors);
     m->d_in = arch->act == 1 ? 2 * arch->d_ff : arch->d_ff;
+    m->aligned16 = true;
+    for (const void *t : m->w) m->aligned16 = m->aligned16 && ((uintptr_t)t & 15) == 0;
     if ((rc = build_maps(m))) {
         delete m;
         return rc;
@@ -1026,6 +1079,7 @@ int ssd_model_share_prefix(const ssd_model *target, int n_layers, ssd_model **dr
     m->a = target->a;
     m->a.n_layers = n_layers;
     m->d_in = target->d_in;
+    m->aligned16 = target->aligned16;
     m->dev_desc = target->dev_desc;  // LM head first, then the layers: a prefix of the layers is a prefix of the block
     m->w.assign(target->w.begin(), target->w.begin() + T_L0 + PER_LAYER * n_layers);
     m->w.insert(m->w.end(), target->w.end() - 3, target->w.end());

@@ -220,3 +220,44 @@ def test_prompt_pass_in_large_chunks_matches_oracle(name, Bn):
         tol = gu.LOGIT_RTOL * np.abs(r).max(axis=-1, keepdims=True) + gu.LOGIT_ATOL if arch.dtype else 1e-4
         bad = np.argwhere(np.abs(g - r) > tol)
         assert bad.shape[0] == 0, (b, bad[:8].tolist(), [(float(g[tuple(i)]), float(r[tuple(i)])) for i in bad[:8]])
+
+
+@pytest.mark.parametrize("arch,lens,M", [
+    (synth.neox_like(2, 72, 3, 132, 130, dtype=synth.DT_F32), [255, 3], 1),          # head 24: rows of 72, 132 and 130 columns
+    (synth.llama_like(2, 256, 2, 1028, 300, dtype=synth.DT_F32), [249, 260], 8),     # head 128; the context ends on / past a 256-position step
+    (synth.llama_like(2, 256, 4, 2100, 5000, dtype=synth.DT_F32), [511, 1, 0], 9),   # several columns per warp, 27 rows in four blocks
+    (synth.gpt2_like(3, 128, 16, 512, 200, 620, dtype=synth.DT_F32), [600, 40], 17),  # head 8
+])
+def test_fp32_forward_in_one_kernel_matches_oracle_and_stepwise(arch, lens, M):
+    """The single-kernel fp32 forward (prompt pass and verification rows) at the edges of its row blocks, column shares
+    and attention steps: logits and cache rows against the oracle and against one launch per step."""
+    ws_np = gu.scaled_weights(synth, arch, 41, 4.0)
+    omodel = od.Model(arch, ws_np)
+    model = B.Model(arch, B.upload_weights(arch, ws_np))
+    lens = np.array(lens, np.int32)
+    Bn, P, S = len(lens), int(lens.max()), int(lens.max()) + M + 3
+    prompts = synth.gen_prompt(42, Bn, P, arch.vocab)
+    rows = synth.gen_prompt(43, Bn, M, arch.vocab)
+    res = []
+    for one_kernel in (True, False):
+        B.set_persistent(one_kernel)
+        try:
+            kv = B.KV(model, Bn, S)
+            n0 = B.launch_count()
+            B.kv_prefill(model, kv, torch.from_numpy(prompts).to("cuda"), torch.from_numpy(lens).to("cuda"),
+                         model.new_workspace(Bn, min(32, 64 // Bn), S))
+            launches = B.launch_count() - n0
+            lg = gpu_logits(model, kv, model.new_workspace(Bn, M, S), rows, M - 1)
+            assert kv.status() == 0 and kv.lengths().tolist() == lens.tolist()
+            res.append((lg, kv.cache_view().cpu().numpy(), launches))
+        finally:
+            B.set_persistent(True)
+    assert res[0][2] < res[1][2]
+    assert np.abs(res[0][0] - res[1][0]).max() <= 1e-3
+    for b in range(Bn):
+        oc = omodel.new_cache(S)
+        if lens[b]:
+            oc.feed(prompts[b, :lens[b]], want_logits=False)
+        gu.assert_logits_close(res[0][0][b], oc.feed(rows[b], advance=False))
+        n = int(lens[b]) + M
+        assert np.abs(res[0][1][:, b, :, :, :n] - oc.kv[:, :, :, :n]).max() <= 1e-3
