@@ -8,7 +8,7 @@ namespace ssd {
 
 constexpr int kMaxRows = 64;        // rows of one forward (sequences x rows per sequence)
 constexpr int kMaxRowsPerSeq = 32;  // K + 1
-constexpr int kHeaderInts = 64;     // cache header: [0] status, [1] reserved ..., then len[], keep[]
+constexpr int kHeaderInts = 64;     // cache header: [0] status, [32] barrier counter, [40] finished attention CTAs, [48] CTAs that have left, then len[], keep[]
 
 // Sticky device-side status: first error wins.
 __device__ __forceinline__ void set_status(int32_t *status, int32_t code) {

@@ -47,9 +47,10 @@ struct FfParams {
     int32_t *status;
     RowInfo ri;
     float *x, *qkv, *ao, *act, *logits;
-    unsigned *gbar;      // zeroed before the launch
+    unsigned *gbar;      // see leave_grid
     long long wait_cycles;
     int want_logits;
+    unsigned long long *trace;  // optional: CTA 0 stamps the global timer at the start, after every grid barrier and at the end
     FfLayer layer[kFfMaxLayers];
 };
 
@@ -61,6 +62,14 @@ inline size_t ff_smem(int d, int F, int parallel, int M, int Dh) {
     return gemm > attn ? gemm : attn;
 }
 
+__device__ __forceinline__ void ff_stamp(const FfParams &p, unsigned i) {
+    if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        p.trace[i] = t;
+        p.trace[i + 1] = 0;
+    }
+}
 // All threads of the grid; false (everywhere in the CTA) once a wait has run out.
 __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, volatile int *ok) {
     __syncthreads();
@@ -80,6 +89,7 @@ __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, vola
             }
         }
         __threadfence();
+        ff_stamp(p, epoch);
     }
     __syncthreads();
     return *ok != 0;
@@ -172,17 +182,20 @@ __device__ __forceinline__ void ff_stage_norm(const FfParams &p, int rb, bool em
                 for (int i = lane; i < d / 4; i += 32) reinterpret_cast<float4 *>(xr)[i] = __ldcg(x4 + i);
             }
             __syncwarp();
-            double mean = 0.0, var = 0.0;
-            if (p.norm_kind == 0) {
-                double s = 0.0;
-                for (int i = lane; i < d; i += 32) s += (double)xr[i];
-                mean = warp_sum(s) / d;
-            }
+            double s1 = 0.0, s2 = 0.0;
             for (int i = lane; i < d; i += 32) {
-                const double c = (double)xr[i] - mean;
-                var += c * c;
+                const double v = (double)xr[i];
+                s1 += v;
+                s2 += v * v;
             }
-            var = warp_sum(var) / d;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+                s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+            }
+            const double mean = p.norm_kind == 0 ? s1 / d : 0.0;
+            double var = s2 / d - mean * mean;
+            if (var < 0.0) var = 0.0;
             const double rstd = rsqrt(var + (double)p.eps);
             for (int i = lane; i < d; i += 32) {
                 double y = ((double)xr[i] - mean) * rstd * (double)__ldg(g + i);
@@ -202,6 +215,23 @@ __device__ __forceinline__ void ff_stage(const FfParams &p, int rb, const float 
     for (int i = threadIdx.x; i < kFfRows * K4; i += kFfThreads)
         d4[i] = i < rows * K4 ? __ldcg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
+}
+
+// What a CTA will read behind the next barrier and nobody writes before it: into L1, under the wait.
+__device__ __forceinline__ void ff_prefetch_norm(const FfParams &p, const float *g, const float *b) {
+    for (int i = threadIdx.x * 32; i < p.d; i += kFfThreads * 32) {
+        prefetch_l1(g + i);
+        if (b) prefetch_l1(b + i);
+    }
+}
+__device__ __forceinline__ void ff_prefetch_cache(const FfParams &p, int layer, int item) {
+    if (item >= p.B * p.H) return;
+    const int b = item / p.H, h = item % p.H, n = min(p.len[b], kFfChunk) * p.Dh;  // (the committed positions of the first step)
+    const float *kc = p.cache + (size_t)layer * p.layer_elems + ((size_t)(b * 2) * p.H + h) * p.S * p.Dh, *vc = kc + (size_t)p.H * p.S * p.Dh;
+    for (int i = threadIdx.x * 32; i < n; i += kFfThreads * 32) {
+        prefetch_l1(kc + i);
+        prefetch_l1(vc + i);
+    }
 }
 
 // Attention of one (sequence, head): rotary, append, scores, softmax, P V.  MR bounds the rows per sequence.
@@ -329,10 +359,7 @@ __device__ __forceinline__ void ff_attention(const FfParams &p, int layer, int i
 }
 
 template <int MR>
-__global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid_constant__ FfParams p) {
-    extern __shared__ __align__(16) float ff_smem_[];
-    __shared__ volatile int ok;
-    float *xs = ff_smem_;
+__device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatile int &ok) {
     const float4 *xs4 = reinterpret_cast<const float4 *>(xs);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r8 = lane >> 2;
     const int d = p.d, F = p.F, d4 = d / 4, F4 = F / 4, blocks = (p.R + kFfRows - 1) / kFfRows;
@@ -383,6 +410,7 @@ __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid
         }
     };
 
+    ff_stamp(p, 0);
     fetch(p.layer[0].w_qkv, 3 * d, d4);
     // row bookkeeping and the rotary table (read behind the first barrier)
     {
@@ -428,8 +456,9 @@ __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid
                 mlp_in(L, rb, false);
             }
         }
+        ff_prefetch_cache(p, l, blockIdx.x);
         if (!ff_sync(p, epoch, &ok)) return;
-        for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention<MR>(p, l, item, last, ff_smem_);
+        for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention<MR>(p, l, item, last, xs);
         if (last) return;
         fetch(L.w_o, d, d4);
         if (!ff_sync(p, epoch, &ok)) return;
@@ -458,6 +487,7 @@ __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid
                 project(L.w_o, d, d4, xs4, rb == 0, [&](int n, int r, float v) { add_to_x(rb, n, r, v, L.b_o); });
             }
             fetch(L.w_in, F, d4);
+            ff_prefetch_norm(p, L.ln2_g, L.ln2_b);
             if (!ff_sync(p, epoch, &ok)) return;
             for (int rb = 0; rb < blocks; ++rb) {
                 if (rb) __syncthreads();
@@ -472,8 +502,13 @@ __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid
                 project(L.w_out, d, F4, xs4, rb == 0, [&](int n, int r, float v) { add_to_x(rb, n, r, v, L.b_out); });
             }
         }
-        if (l + 1 < p.n_layers) fetch(p.layer[l + 1].w_qkv, 3 * d, d4);
-        else fetch(p.w_lm, p.V, d4);
+        if (l + 1 < p.n_layers) {
+            fetch(p.layer[l + 1].w_qkv, 3 * d, d4);
+            ff_prefetch_norm(p, p.layer[l + 1].ln1_g, p.layer[l + 1].ln1_b);
+        } else {
+            fetch(p.w_lm, p.V, d4);
+            ff_prefetch_norm(p, p.lnf_g, p.lnf_b);
+        }
         if (!ff_sync(p, epoch, &ok)) return;
     }
     for (int rb = 0; rb < blocks; ++rb) {
@@ -483,6 +518,16 @@ __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid
             if (rb * kFfRows + r < p.R) p.logits[(size_t)(rb * kFfRows + r) * p.V + n] = v;
         });
     }
+    ff_stamp(p, epoch + 1);
+}
+
+template <int MR>
+__global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid_constant__ FfParams p) {
+    extern __shared__ __align__(16) float ff_smem_[];
+    __shared__ volatile int ok;
+    ff_forward<MR>(p, ff_smem_, ok);
+    __syncthreads();
+    if (threadIdx.x == 0) leave_grid(p.gbar);
 }
 
 }  // namespace ssd

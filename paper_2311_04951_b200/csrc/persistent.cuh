@@ -104,8 +104,8 @@ struct alignas(64) FwdParams {
     RowInfo ri;
     float *x, *qkv, *t_in, *logits;
     float *part_m, *part_l, *part_o;
-    unsigned *tickets;  // [B*H]
-    unsigned *gbar;     // grid barrier counter (zeroed before launch)
+    unsigned *tickets;  // [B*H]: zeroed by the set-up
+    unsigned *gbar;     // grid barrier counter (see leave_grid)
     int chunk, n_split;
     int want_logits;
     // Shared-memory ring: slots [0, stages_lo) hold weights at any time; slots [stages_lo, stages) share
@@ -469,8 +469,20 @@ __device__ __forceinline__ void grid_arrive(const FwdParams &p, Shared *sh, int 
     }
 }
 
-// Count of attention CTAs that have finished their items, over the layers of this pass (zeroed with the
-// barrier counter before the launch).  With few attention items in a parallel-residual block the CTAs
+// The barrier counter and its neighbours live in the cache's header, which kv_init zeroes; every launch leaves them at
+// zero again: one thread per CTA calls this as the CTA's last step, whatever way it came there, and the last one clears
+// them.  (A memset in front of every launch cost a stream operation of 2-3 us.)
+__device__ __forceinline__ void leave_grid(unsigned *gbar) {
+    __threadfence();
+    if (atomicAdd(gbar + 16, 1u) == gridDim.x - 1) {
+        atomicExch(gbar, 0u);
+        atomicExch(gbar + 8, 0u);
+        atomicExch(gbar + 16, 0u);
+    }
+}
+
+// Count of attention CTAs that have finished their items, over the layers of this pass (cleared with the
+// barrier counter).  With few attention items in a parallel-residual block the CTAs
 // without an item run the MLP-out GEMM beside the attention and go straight on to the out-projection:
 // its operand issuer waits for this count instead of a grid barrier.
 __device__ __forceinline__ unsigned *attn_done(const FwdParams &p) { return p.gbar + 8; }
@@ -666,6 +678,8 @@ __device__ __noinline__ void act_phase(const FwdParams &p) {
 }
 
 __device__ __noinline__ void setup_phase(const FwdParams &p) {
+    if (blockIdx.x == gridDim.x - 1)  // (they are used behind this phase's barrier; every user leaves its own at zero)
+        for (int i = threadIdx.x; i < p.B * p.H; i += kWorkThreads) p.tickets[i] = 0;
     // K not a multiple of 64: the last tile's unused columns must be finite (the weight copy zero-fills its own)
     for (int o = 0; o < 4; ++o) {
         const int K = p.op_ld[o], pad = (-K) & (kTileK - 1);
@@ -2348,6 +2362,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1) forward_kernel(const __gri
     }
     tc_fence_before();
     __syncthreads();
+    if (threadIdx.x == 0) leave_grid(p.gbar);
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");

@@ -193,6 +193,7 @@ struct ssd_kv {
     int B, S;
     uint8_t *buf;
     int32_t *status, *len, *keep;
+    unsigned *gbar;  // grid barrier counter and its neighbours (header ints 32 .. 48)
     uint8_t *cache;
     size_t layer_bytes, esize;
     CUtensorMap tm_rows;  // bf16 caches of head dim 128: every (layer, sequence, K|V, head, position) row, box 64 x 128
@@ -292,8 +293,7 @@ struct Workspace {
     float *part_m, *part_l, *part_o;
     int max_split;
     // persistent kernel
-    unsigned *sync;  // [0] grid barrier counter, [16..] attention tickets
-    size_t sync_bytes;
+    unsigned *tickets;  // [B * H]
     unsigned long long *trace;  // [kTraceSlots] phase time stamps (debug)
     int rows_k;      // rows the persistent kernel's tiles span (padded)
     size_t bytes;
@@ -342,8 +342,7 @@ Workspace carve(const ssd_model *m, int B, int M, uint8_t *base) {
     w.qkv = (float *)take(sizeof(float) * (size_t)R * 3 * d);
     w.qrot = (float *)take(sizeof(float) * (size_t)R * d);
     w.t_in = (float *)take(sizeof(float) * (size_t)R * m->d_in);
-    w.sync_bytes = sizeof(unsigned) * (16 + (size_t)B * a.n_heads);
-    w.sync = (unsigned *)take(w.sync_bytes);
+    w.tickets = (unsigned *)take(sizeof(unsigned) * (size_t)B * a.n_heads);
     w.trace = (unsigned long long *)take(sizeof(unsigned long long) * kTraceSlots);
     w.logits = (float *)take(sizeof(float) * (size_t)R * a.vocab);
     w.stats = (RowStat *)take(sizeof(RowStat) * R);
@@ -617,7 +616,7 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
     p.ri = w.ri;
     p.x = w.x; p.qkv = w.qkv; p.t_in = w.t_in; p.logits = w.logits;
     p.part_m = w.part_m; p.part_l = w.part_l; p.part_o = w.part_o;
-    p.gbar = w.sync; p.tickets = w.sync + 16;
+    p.gbar = kv->gbar; p.tickets = w.tickets;
     int ctx = kv_bound(kv) + M;
     if (ctx > kv->S) ctx = kv->S;
     // Tensor-core attention items stream 128 positions per ~2 us but cost ~8 us more to start than the
@@ -658,7 +657,6 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
         p.mailbox = kv->mailbox_dev; p.mb_seq = dl->mb_seq;
     }
     p.trace = (g_trace && 2 + p.n_steps * (barriers_needed(a) + 6) + 3 < kTraceSlots) ? w.trace : nullptr;
-    CUDA_OK(cudaMemsetAsync(w.sync, 0, w.sync_bytes, st));
     cudaEvent_t prof_stop;
     if (prof_begin(st, &prof_stop)) return SSD_E_CUDA;
     int rc = launch_forward_rows(p, Rk, w.ri.seq, w.bytes, st);
@@ -699,9 +697,10 @@ int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride,
     p.cache = (float *)kv->cache; p.layer_elems = kv->layer_bytes / 4;
     p.len = kv->len; p.status = kv->status; p.ri = w.ri;
     p.x = w.x; p.qkv = w.qkv; p.ao = w.ao.f32; p.act = w.act.f32; p.logits = w.logits;
-    p.gbar = w.sync;
+    p.gbar = kv->gbar;
     p.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : kWaitCycles;
     p.want_logits = want_logits ? 1 : 0;
+    p.trace = g_trace ? w.trace : nullptr;
     for (int l = 0; l < a.n_layers; ++l) {
         const float **dst = (const float **)&p.layer[l];
         for (int i = 0; i < PER_LAYER; ++i) dst[i] = (const float *)lw(m, l, i);
@@ -713,7 +712,6 @@ int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride,
     if (grid < kv->B * a.n_heads) grid = kv->B * a.n_heads;
     if (grid > g_num_sms) grid = g_num_sms;
     const size_t smem = ff_smem(a.d_model, a.d_ff, a.parallel_residual, M, a.head_dim);
-    CUDA_OK(cudaMemsetAsync(w.sync, 0, 64, st));
     void *args[] = {&p};
     const void *k = M <= 8 ? (const void *)forward_f32_kernel<8> : (const void *)forward_f32_kernel<kMaxRowsPerSeq>;
     CUDA_OK(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kFfThreads), args, smem, st));
@@ -1121,6 +1119,7 @@ int kv_init(const ssd_model *m, int batch, int max_len, void *dev_buf, size_t by
     kv->buf = (uint8_t *)dev_buf;
     kv->status = (int32_t *)dev_buf;
     kv->len = kv->status + kHeaderInts;
+    kv->gbar = (unsigned *)kv->status + 32;
     kv->keep = kv->len + batch;
     kv->cache = kv->buf + kv_header_bytes(batch);
     kv->esize = m->a.dtype ? 2 : 4;
