@@ -11,7 +11,7 @@
 //     first 1024 weights of the warp's first column are fetched into registers BEFORE the barrier in front of the phase;
 //   * attention: one CTA per (sequence, head): four lanes per position for the scores, a thread per (head column, position
 //     group) for P V; the CTA appends the pass's keys / values itself, so nothing else has to wait for them.
-// Generation with the four-layer 256-wide model (K = 4, 16 iterations): 13.2 ms as one launch per step, 6.5 as one
+// Generation with the four-layer 256-wide model (K = 4, 16 iterations): 13.2 ms as one launch per step, 5.7 as one
 // per forward.
 // Results as the stepwise path's up to fp32 summation order.  Every barrier wait is bounded.
 #pragma once
@@ -38,6 +38,7 @@ struct FfLayer {
 struct FfParams {
     int n_layers, d, H, Dh, F, V, norm_kind, swiglu, parallel, rotary_dim, learned_pos, pos_limit;
     float eps, rotary_base, scale;
+    double inv_d;  // 1 / d
     int B, M, R, S;
     const int32_t *tokens; int tok_stride;
     const int32_t *n_rows;
@@ -55,8 +56,8 @@ struct FfParams {
 };
 
 // dynamic shared memory of a pass
-inline size_t ff_smem(int d, int F, int parallel, int M, int Dh) {
-    const size_t gemm = (size_t)kFfRows * (parallel ? d + F : (d > F ? d : F)) * 4;
+inline size_t ff_smem(int d, int F, int M, int Dh) {
+    const size_t gemm = (size_t)kFfRows * (d > F ? d : F) * 4;
     const size_t groups = kFfThreads / Dh;
     const size_t attn = ((size_t)M * Dh + (size_t)M * kFfChunk + 3 * (size_t)M + groups * M * Dh) * 4;
     return gemm > attn ? gemm : attn;
@@ -72,8 +73,8 @@ __device__ __forceinline__ void ff_stamp(const FfParams &p, unsigned i) {
 }
 // All threads of the grid; false (everywhere in the CTA) once a wait has run out.
 __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, volatile int *ok) {
-    __syncthreads();
     ++epoch;
+    __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         red_release_add(p.gbar, 1u);
@@ -95,36 +96,53 @@ __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, vola
     return *ok != 0;
 }
 
-// the first 1024 entries of a weight row
-__device__ __forceinline__ void ff_fetch(const float4 *w, int K4, float4 (&v)[8]) {
+// A warp's weights on their way: 1024 / NF entries of each of NF columns' rows (columns `cols` apart; those from n_end on
+// are read as the last one and dropped by the caller).
+template <int NF>
+__device__ __forceinline__ void ff_fetch(const float *W, int n, int cols, int n_end, int K4, int k0, float4 (&v)[8]) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) v[i] = lane + 32 * i < K4 ? __ldg(w + lane + 32 * i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int j = 0; j < NF; ++j) {
+        const float4 *w = reinterpret_cast<const float4 *>(W) + (size_t)min(n + j * cols, n_end - 1) * K4;
+#pragma unroll
+        for (int i = 0; i < 8 / NF; ++i) {
+            const int k = k0 + lane + 32 * i;
+            v[j * (8 / NF) + i] = k < K4 ? __ldg(w + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
 }
-// sum_k w[k] x[r][k] for the eight staged rows; `v` holds the first 1024 entries of w (and is used up)
-__device__ __forceinline__ void ff_dot(const float4 *w, int K4, const float4 *xs, float4 (&v)[8], float (&acc)[kFfRows]) {
+// acc[j][r] = sum_k w_j[k] x[r][k] for NF columns and the `rows` staged rows; `v` holds the columns' first entries (and is used
+// up).  A staged row is read once for all NF columns: shared-memory reads bound the small projections.
+template <int NF>
+__device__ __forceinline__ void ff_dot(const float *W, int n, int cols, int n_end, int K4, const float4 *xs, int rows, float4 (&v)[8],
+                                       float (&acc)[NF][kFfRows]) {
     const int lane = threadIdx.x & 31;
+    constexpr int KC = 8 / NF;
 #pragma unroll
-    for (int r = 0; r < kFfRows; ++r) acc[r] = 0.f;
+    for (int j = 0; j < NF; ++j)
+#pragma unroll
+        for (int r = 0; r < kFfRows; ++r) acc[j][r] = 0.f;
     for (int k0 = 0;;) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int k = k0 + lane + 32 * i;
-            if (k0 + 32 * i >= K4) break;
-            if (k < K4) {
+        for (int r = 0; r < kFfRows; ++r) {
+            if (r < rows) {
 #pragma unroll
-                for (int r = 0; r < kFfRows; ++r) {
-                    const float4 x = xs[(size_t)r * K4 + k];
-                    acc[r] = fmaf(v[i].x, x.x, acc[r]);
-                    acc[r] = fmaf(v[i].y, x.y, acc[r]);
-                    acc[r] = fmaf(v[i].z, x.z, acc[r]);
-                    acc[r] = fmaf(v[i].w, x.w, acc[r]);
+                for (int i = 0; i < KC; ++i) {
+                    const int k = k0 + lane + 32 * i;
+                    if (k < K4) {
+                        const float4 x = xs[(size_t)r * K4 + k];
+#pragma unroll
+                        for (int j = 0; j < NF; ++j) {
+                            const float4 w = v[j * KC + i];
+                            acc[j][r] = fmaf(w.x, x.x, fmaf(w.y, x.y, fmaf(w.z, x.z, fmaf(w.w, x.w, acc[j][r]))));
+                        }
+                    }
                 }
             }
         }
-        k0 += 256;
+        k0 += 32 * KC;
         if (k0 >= K4) break;
-        ff_fetch(w + k0, K4 - k0, v);
+        ff_fetch<NF>(W, n, cols, n_end, K4, k0, v);
     }
 }
 // the sums over the warp: lane 4 r (and its three neighbours) returns row r's
@@ -145,15 +163,19 @@ __device__ __forceinline__ float ff_reduce(float (&a)[kFfRows]) {
     return v;
 }
 
-// Rows 8 rb .. of the residual stream, normalised, into xs [8][d]: a warp per row.  `embed`: they are embedding rows
+// Rows 8 rb .. of the residual stream, normalised, into xs [8][d]: a warp per row, everything it needs (row, gain, bias) on
+// its way together; rows of up to 256 columns stay in registers, wider ones are read again.  `embed`: they are embedding rows
 // (and their owner starts the residual stream with them).
 __device__ __forceinline__ void ff_stage_norm(const FfParams &p, int rb, bool embed, const float *g, const float *b, float *xs) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = rb * kFfRows + warp, d = p.d;
+    constexpr int NR = 2;  // float4 per lane held in registers
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r = rb * kFfRows + warp, d4 = p.d / 4;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
     if (warp < kFfRows) {
-        float *xr = xs + (size_t)warp * d;
+        float4 *xr = reinterpret_cast<float4 *>(xs) + (size_t)warp * d4;
         if (r >= p.R) {
-            for (int i = lane; i < d; i += 32) xr[i] = 0.f;
+            for (int i = lane; i < d4; i += 32) xr[i] = zero;
         } else {
+            const float4 *x4 = reinterpret_cast<const float4 *>(p.x + (size_t)r * p.d), *q4 = nullptr;
             if (embed) {
                 const int bs = r / p.M, j = r % p.M;
                 int n = p.n_rows ? p.n_rows[bs] : p.M;
@@ -165,43 +187,57 @@ __device__ __forceinline__ void ff_stage_norm(const FfParams &p, int rb, bool em
                 pos = min(pos, lim);
                 int tok = fits && j < n ? p.tokens[(size_t)bs * p.tok_stride + j] : 0;  // rows that are not fed read nothing
                 tok = max(0, min(tok, p.V - 1));
-                const float4 *e = reinterpret_cast<const float4 *>(p.tok_emb + (size_t)tok * d);
-                const float4 *q = p.learned_pos ? reinterpret_cast<const float4 *>(p.pos_emb + (size_t)pos * d) : nullptr;
-                for (int i = lane; i < d / 4; i += 32) {
-                    float4 v = __ldg(e + i);
-                    if (q) {
-                        const float4 w = __ldg(q + i);
-                        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-                    }
-                    reinterpret_cast<float4 *>(xr)[i] = v;
-                    if ((int)blockIdx.x == r % (int)gridDim.x) reinterpret_cast<float4 *>(p.x + (size_t)r * d)[i] = v;
+                x4 = reinterpret_cast<const float4 *>(p.tok_emb + (size_t)tok * p.d);
+                if (p.learned_pos) q4 = reinterpret_cast<const float4 *>(p.pos_emb + (size_t)pos * p.d);
+            }
+            auto entry = [&](int i) {
+                float4 v = __ldcg(x4 + i);
+                if (q4) {
+                    const float4 w = __ldg(q4 + i);
+                    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
                 }
-            } else {
-                const float4 *x4 = reinterpret_cast<const float4 *>(p.x + (size_t)r * d);
-#pragma unroll 4
-                for (int i = lane; i < d / 4; i += 32) reinterpret_cast<float4 *>(xr)[i] = __ldcg(x4 + i);
+                return v;
+            };
+            const float4 *g4 = reinterpret_cast<const float4 *>(g), *b4 = reinterpret_cast<const float4 *>(b);
+            float4 x[NR], gv[NR], bv[NR];
+#pragma unroll
+            for (int k = 0; k < NR; ++k) {
+                const int i = lane + 32 * k;
+                x[k] = i < d4 ? entry(i) : zero;
+                gv[k] = i < d4 ? __ldg(g4 + i) : zero;
+                bv[k] = i < d4 && b ? __ldg(b4 + i) : zero;
             }
-            __syncwarp();
             double s1 = 0.0, s2 = 0.0;
-            for (int i = lane; i < d; i += 32) {
-                const double v = (double)xr[i];
-                s1 += v;
-                s2 += v * v;
-            }
+            auto add = [&](const float4 &v) {
+                s1 += ((double)v.x + (double)v.y) + ((double)v.z + (double)v.w);
+                s2 += ((double)v.x * v.x + (double)v.y * v.y) + ((double)v.z * v.z + (double)v.w * v.w);
+            };
+#pragma unroll
+            for (int k = 0; k < NR; ++k) add(x[k]);
+            for (int i = lane + 32 * NR; i < d4; i += 32) add(entry(i));
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 s1 += __shfl_xor_sync(0xffffffffu, s1, o);
                 s2 += __shfl_xor_sync(0xffffffffu, s2, o);
             }
-            const double mean = p.norm_kind == 0 ? s1 / d : 0.0;
-            double var = s2 / d - mean * mean;
+            const double mean = p.norm_kind == 0 ? s1 * p.inv_d : 0.0;
+            double var = s2 * p.inv_d - mean * mean;
             if (var < 0.0) var = 0.0;
             const double rstd = rsqrt(var + (double)p.eps);
-            for (int i = lane; i < d; i += 32) {
-                double y = ((double)xr[i] - mean) * rstd * (double)__ldg(g + i);
-                if (b) y += (double)__ldg(b + i);
-                xr[i] = (float)y;
-            }
+            const bool owner = embed && (int)blockIdx.x == r % (int)gridDim.x;
+            auto emit = [&](int i, const float4 &v, const float4 &gg, const float4 &bb) {
+                float4 y;
+                y.x = (float)(((double)v.x - mean) * rstd * (double)gg.x + (double)bb.x);
+                y.y = (float)(((double)v.y - mean) * rstd * (double)gg.y + (double)bb.y);
+                y.z = (float)(((double)v.z - mean) * rstd * (double)gg.z + (double)bb.z);
+                y.w = (float)(((double)v.w - mean) * rstd * (double)gg.w + (double)bb.w);
+                xr[i] = y;
+                if (owner) reinterpret_cast<float4 *>(p.x + (size_t)r * p.d)[i] = v;
+            };
+#pragma unroll
+            for (int k = 0; k < NR; ++k)
+                if (lane + 32 * k < d4) emit(lane + 32 * k, x[k], gv[k], bv[k]);
+            for (int i = lane + 32 * NR; i < d4; i += 32) emit(i, entry(i), __ldg(g4 + i), b ? __ldg(b4 + i) : zero);
         }
     }
     __syncthreads();
@@ -215,23 +251,6 @@ __device__ __forceinline__ void ff_stage(const FfParams &p, int rb, const float 
     for (int i = threadIdx.x; i < kFfRows * K4; i += kFfThreads)
         d4[i] = i < rows * K4 ? __ldcg(s4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     __syncthreads();
-}
-
-// What a CTA will read behind the next barrier and nobody writes before it: into L1, under the wait.
-__device__ __forceinline__ void ff_prefetch_norm(const FfParams &p, const float *g, const float *b) {
-    for (int i = threadIdx.x * 32; i < p.d; i += kFfThreads * 32) {
-        prefetch_l1(g + i);
-        if (b) prefetch_l1(b + i);
-    }
-}
-__device__ __forceinline__ void ff_prefetch_cache(const FfParams &p, int layer, int item) {
-    if (item >= p.B * p.H) return;
-    const int b = item / p.H, h = item % p.H, n = min(p.len[b], kFfChunk) * p.Dh;  // (the committed positions of the first step)
-    const float *kc = p.cache + (size_t)layer * p.layer_elems + ((size_t)(b * 2) * p.H + h) * p.S * p.Dh, *vc = kc + (size_t)p.H * p.S * p.Dh;
-    for (int i = threadIdx.x * 32; i < n; i += kFfThreads * 32) {
-        prefetch_l1(kc + i);
-        prefetch_l1(vc + i);
-    }
 }
 
 // Attention of one (sequence, head): rotary, append, scores, softmax, P V.  MR bounds the rows per sequence.
@@ -358,60 +377,69 @@ __device__ __forceinline__ void ff_attention(const FfParams &p, int layer, int i
     __syncthreads();
 }
 
+// The steps of a pass.  Sequential layer: qkv | attention | out-projection | MLP in | MLP out; parallel-residual layer: qkv, MLP in |
+// attention | out-projection, MLP out (a bar is a grid barrier); at the end the LM head.  One loop over them, so that staging
+// and projection exist once in the code: a phase runs a few hundred instructions per warp, and fetching them would cost more.
+enum { FS_QKV = 0, FS_ATTN, FS_O, FS_IN, FS_OUT, FS_LM };
+struct FfStep {
+    const float *W, *bias, *src;  // projection: weights, bias, operand rows (null: the norm of the residual stream with g, b)
+    const float *g, *b;
+    int N, K4, kind;
+    bool barrier;                 // behind it
+};
+__device__ __forceinline__ FfStep ff_step(const FfParams &p, int i) {
+    FfStep s;
+    const int l = i / 5, e = i % 5;
+    if (l >= p.n_layers) {
+        s.kind = FS_LM;
+        s.W = p.w_lm; s.bias = nullptr; s.src = nullptr; s.g = p.lnf_g; s.b = p.lnf_b; s.N = p.V; s.K4 = p.d / 4; s.barrier = false;
+        return s;
+    }
+    const FfLayer &L = p.layer[l];
+    s.kind = !p.parallel ? e : e == 0 ? FS_QKV : e == 1 ? FS_IN : e == 2 ? FS_ATTN : e == 3 ? FS_O : FS_OUT;
+    s.barrier = !(p.parallel && (e == 0 || e == 3));
+    s.K4 = p.d / 4; s.src = nullptr; s.g = s.b = nullptr; s.W = nullptr; s.bias = nullptr; s.N = 0;
+    if (s.kind == FS_QKV) { s.W = L.w_qkv; s.bias = L.b_qkv; s.g = L.ln1_g; s.b = L.ln1_b; s.N = 3 * p.d; }
+    if (s.kind == FS_O) { s.W = L.w_o; s.bias = L.b_o; s.src = p.ao; s.N = p.d; }
+    if (s.kind == FS_IN) { s.W = L.w_in; s.bias = L.b_in; s.g = L.ln2_g; s.b = L.ln2_b; s.N = p.F; }
+    if (s.kind == FS_OUT) { s.W = L.w_out; s.bias = L.b_out; s.src = p.act; s.N = p.d; s.K4 = p.F / 4; }
+    return s;
+}
+// one projected value to where the step wants it
+__device__ __forceinline__ void ff_out(const FfParams &p, const FfStep &s, int n, int row, float v) {
+    if (s.bias) v += __ldg(s.bias + n);
+    if (s.kind == FS_QKV) p.qkv[(size_t)row * 3 * p.d + n] = v;
+    else if (s.kind == FS_IN) p.act[(size_t)row * p.F + n] = gelu_erf(v);
+    else if (s.kind == FS_LM) p.logits[(size_t)row * p.V + n] = v;
+    else {  // the residual stream: this thread owns the entry in both projections that add to it
+        float *x = p.x + (size_t)row * p.d + n;
+        *x = __ldcg(x) + v;
+    }
+}
+
 template <int MR>
 __device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatile int &ok) {
     const float4 *xs4 = reinterpret_cast<const float4 *>(xs);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r8 = lane >> 2;
-    const int d = p.d, F = p.F, d4 = d / 4, F4 = F / 4, blocks = (p.R + kFfRows - 1) / kFfRows;
-    const int gw = blockIdx.x * kFfWarps + warp, nw = gridDim.x * kFfWarps;  // this warp's first column, and the stride
+    const int blocks = (p.R + kFfRows - 1) / kFfRows;
+    const int gw = blockIdx.x * kFfWarps + warp, nw = gridDim.x * kFfWarps;  // this warp's columns: gw, gw + nw, ...
     unsigned epoch = 0;
     if (threadIdx.x == 0) ok = 1;
 
+    // Four columns at a time where a warp has several and their rows are short; gate and up together for SwiGLU; else one.
     float4 pre[8];
-    auto fetch = [&](const float *W, int N, int K4) {  // of the next phase's first column
-        if (gw < N) ff_fetch(reinterpret_cast<const float4 *>(W + (size_t)gw * K4 * 4), K4, pre);
-    };
-    // out(n, row in block, value) for every column n of W [N, K] and the staged rows
-    auto project = [&](const float *W, int N, int K4, const float4 *x4, bool fetched, auto out) {
-        for (int n = gw; n < N; n += nw) {
-            const float4 *w = reinterpret_cast<const float4 *>(W + (size_t)n * K4 * 4);
-            if (!fetched || n != gw) ff_fetch(w, K4, pre);
-            float acc[kFfRows];
-            ff_dot(w, K4, x4, pre, acc);
-            const float v = ff_reduce(acc);
-            if ((lane & 3) == 0) out(n, r8, v);
-        }
-    };
-    auto mlp_in = [&](const FfLayer &L, int rb, bool fetched) {
-        if (!p.swiglu) {
-            project(L.w_in, F, d4, xs4, fetched, [&](int n, int r, float v) {
-                if (rb * kFfRows + r < p.R) p.act[(size_t)(rb * kFfRows + r) * F + n] = gelu_erf(v + (L.b_in ? __ldg(L.b_in + n) : 0.f));
-            });
-        } else {
-            for (int n = gw; n < F; n += nw) {
-                const float4 *wg = reinterpret_cast<const float4 *>(L.w_in + (size_t)n * d), *wu = wg + (size_t)F * d4;
-                if (!fetched || n != gw) ff_fetch(wg, d4, pre);
-                float acc[kFfRows];
-                ff_dot(wg, d4, xs4, pre, acc);
-                ff_fetch(wu, d4, pre);
-                const float gv = ff_reduce(acc) + (L.b_in ? __ldg(L.b_in + n) : 0.f);
-                ff_dot(wu, d4, xs4, pre, acc);
-                const float uv = ff_reduce(acc) + (L.b_in ? __ldg(L.b_in + F + n) : 0.f);
-                const int r = rb * kFfRows + r8;
-                if ((lane & 3) == 0 && r < p.R) p.act[(size_t)r * F + n] = silu(gv) * uv;
-            }
-        }
-    };
-    auto add_to_x = [&](int rb, int n, int r, float v, const float *bias) {
-        const int row = rb * kFfRows + r;
-        if (row < p.R) {
-            float *x = p.x + (size_t)row * d + n;
-            *x = __ldcg(x) + (v + (bias ? __ldg(bias + n) : 0.f));
-        }
+    auto columns = [&](const FfStep &s) { return s.kind == FS_IN && p.swiglu ? 2 : s.N > nw && s.K4 <= 64 ? 4 : 1; };
+    auto fetch = [&](const FfStep &s, int n) {
+        const int nf = columns(s);
+        if (n >= s.N) return;
+        if (nf == 4) ff_fetch<4>(s.W, n, nw, s.N, s.K4, 0, pre);
+        else if (nf == 2) ff_fetch<2>(s.W, n, p.F, 2 * p.F, s.K4, 0, pre);
+        else ff_fetch<1>(s.W, n, nw, s.N, s.K4, 0, pre);
     };
 
     ff_stamp(p, 0);
-    fetch(p.layer[0].w_qkv, 3 * d, d4);
+    FfStep s = ff_step(p, 0);
+    fetch(s, gw);
     // row bookkeeping and the rotary table (read behind the first barrier)
     {
         const int half = p.rotary_dim / 2;
@@ -434,93 +462,70 @@ __device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatil
                 if (j == 0) p.ri.n_eff[b] = n;
             }
             for (int i = threadIdx.x; i < half; i += kFfThreads) {
-                double s, c;
-                sincos((double)pos * exp2(-2.0 * i / p.rotary_dim * log2((double)p.rotary_base)), &s, &c);
+                double sn, c;
+                sincos((double)pos * exp2(-2.0 * i / p.rotary_dim * log2((double)p.rotary_base)), &sn, &c);
                 p.ri.rope_cos[(size_t)r * half + i] = (float)c;
-                p.ri.rope_sin[(size_t)r * half + i] = (float)s;
+                p.ri.rope_sin[(size_t)r * half + i] = (float)sn;
             }
         }
     }
-    for (int l = 0; l < p.n_layers; ++l) {
-        const FfLayer &L = p.layer[l];
-        const bool last = l + 1 == p.n_layers && !p.want_logits;  // only its keys and values are wanted
-        for (int rb = 0; rb < blocks; ++rb) {
-            if (rb) __syncthreads();
-            ff_stage_norm(p, rb, l == 0, L.ln1_g, L.ln1_b, xs);
-            project(L.w_qkv, 3 * d, d4, xs4, rb == 0, [&](int n, int r, float v) {
-                if (rb * kFfRows + r < p.R) p.qkv[(size_t)(rb * kFfRows + r) * 3 * d + n] = v + (L.b_qkv ? __ldg(L.b_qkv + n) : 0.f);
-            });
-            if (p.parallel && !last) {
-                __syncthreads();
-                ff_stage_norm(p, rb, l == 0, L.ln2_g, L.ln2_b, xs);
-                mlp_in(L, rb, false);
-            }
-        }
-        ff_prefetch_cache(p, l, blockIdx.x);
-        if (!ff_sync(p, epoch, &ok)) return;
-        for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention<MR>(p, l, item, last, xs);
-        if (last) return;
-        fetch(L.w_o, d, d4);
-        if (!ff_sync(p, epoch, &ok)) return;
-        if (p.parallel) {
-            float *xf = xs + (size_t)kFfRows * d;
+    const int steps = 5 * p.n_layers + 1;
+#pragma unroll 1
+    for (int i = 0; i < steps; ++i) {
+        const bool last = i >= 5 * (p.n_layers - 1) && !p.want_logits;  // of the last layer only the keys and values are wanted
+        bool fetched = true;                                            // this warp's first columns
+        if (s.kind == FS_ATTN) {
+            for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention<MR>(p, i / 5, item, last, xs);
+            if (last) return;
+        } else if (!(last && s.kind == FS_IN)) {
+#pragma unroll 1
             for (int rb = 0; rb < blocks; ++rb) {
-                if (rb) __syncthreads();
-                ff_stage(p, rb, p.ao, d, xs);
-                ff_stage(p, rb, p.act, F, xf);
-                for (int n = gw; n < d; n += nw) {
-                    const float4 *wo = reinterpret_cast<const float4 *>(L.w_o + (size_t)n * d), *wf = reinterpret_cast<const float4 *>(L.w_out + (size_t)n * F);
-                    if (rb || n != gw) ff_fetch(wo, d4, pre);
-                    float acc[kFfRows];
-                    ff_dot(wo, d4, xs4, pre, acc);
-                    ff_fetch(wf, F4, pre);
-                    const float av = ff_reduce(acc);
-                    ff_dot(wf, F4, reinterpret_cast<const float4 *>(xf), pre, acc);
-                    const float fv = ff_reduce(acc) + (L.b_out ? __ldg(L.b_out + n) : 0.f);
-                    if ((lane & 3) == 0) add_to_x(rb, n, r8, av + fv, L.b_o);
+                __syncthreads();  // the staged rows of before have been read
+                if (s.src) ff_stage(p, rb, s.src, 4 * s.K4, xs);
+                else ff_stage_norm(p, rb, i < 5 && (s.kind == FS_QKV || p.parallel), s.g, s.b, xs);
+                const int rows = min(kFfRows, p.R - rb * kFfRows), row = rb * kFfRows + r8, nf = columns(s);
+                const bool writes = (lane & 3) == 0 && r8 < rows;
+#pragma unroll 1
+                for (int n = gw; n < s.N; n += nf == 4 ? 4 * nw : nw) {
+                    if (!fetched) fetch(s, n);
+                    fetched = false;
+                    if (nf == 4) {
+                        float acc[4][kFfRows];
+                        ff_dot<4>(s.W, n, nw, s.N, s.K4, xs4, rows, pre, acc);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float v = ff_reduce(acc[j]);
+                            if (writes && n + j * nw < s.N) ff_out(p, s, n + j * nw, row, v);
+                        }
+                    } else if (nf == 1) {
+                        float acc[1][kFfRows];
+                        ff_dot<1>(s.W, n, nw, s.N, s.K4, xs4, rows, pre, acc);
+                        const float v = ff_reduce(acc[0]);
+                        if (writes) ff_out(p, s, n, row, v);
+                    } else {
+                        float acc[2][kFfRows];
+                        ff_dot<2>(s.W, n, p.F, 2 * p.F, s.K4, xs4, rows, pre, acc);
+                        const float g = ff_reduce(acc[0]) + (s.bias ? __ldg(s.bias + n) : 0.f);
+                        const float u = ff_reduce(acc[1]) + (s.bias ? __ldg(s.bias + p.F + n) : 0.f);
+                        if (writes) p.act[(size_t)row * p.F + n] = silu(g) * u;
+                    }
                 }
-            }
-        } else {
-            for (int rb = 0; rb < blocks; ++rb) {
-                if (rb) __syncthreads();
-                ff_stage(p, rb, p.ao, d, xs);
-                project(L.w_o, d, d4, xs4, rb == 0, [&](int n, int r, float v) { add_to_x(rb, n, r, v, L.b_o); });
-            }
-            fetch(L.w_in, F, d4);
-            ff_prefetch_norm(p, L.ln2_g, L.ln2_b);
-            if (!ff_sync(p, epoch, &ok)) return;
-            for (int rb = 0; rb < blocks; ++rb) {
-                if (rb) __syncthreads();
-                ff_stage_norm(p, rb, false, L.ln2_g, L.ln2_b, xs);
-                mlp_in(L, rb, rb == 0);
-            }
-            fetch(L.w_out, d, F4);
-            if (!ff_sync(p, epoch, &ok)) return;
-            for (int rb = 0; rb < blocks; ++rb) {
-                if (rb) __syncthreads();
-                ff_stage(p, rb, p.act, F, xs);
-                project(L.w_out, d, F4, xs4, rb == 0, [&](int n, int r, float v) { add_to_x(rb, n, r, v, L.b_out); });
+                fetched = false;
             }
         }
-        if (l + 1 < p.n_layers) {
-            fetch(p.layer[l + 1].w_qkv, 3 * d, d4);
-            ff_prefetch_norm(p, p.layer[l + 1].ln1_g, p.layer[l + 1].ln1_b);
-        } else {
-            fetch(p.w_lm, p.V, d4);
-            ff_prefetch_norm(p, p.lnf_g, p.lnf_b);
+        const bool barrier = s.barrier;
+        if (i + 1 < steps) {
+            s = ff_step(p, i + 1);
+            if (s.kind != FS_ATTN) fetch(s, gw);  // ahead of the barrier
         }
-        if (!ff_sync(p, epoch, &ok)) return;
-    }
-    for (int rb = 0; rb < blocks; ++rb) {
-        if (rb) __syncthreads();
-        ff_stage_norm(p, rb, false, p.lnf_g, p.lnf_b, xs);
-        project(p.w_lm, p.V, d4, xs4, rb == 0, [&](int n, int r, float v) {
-            if (rb * kFfRows + r < p.R) p.logits[(size_t)(rb * kFfRows + r) * p.V + n] = v;
-        });
+        if (barrier && !ff_sync(p, epoch, &ok)) return;
     }
     ff_stamp(p, epoch + 1);
 }
 
+// (The same kernel as one cluster of 16 CTAs, with the cluster's hardware barrier instead of the counter in L2, gains what the
+// barriers cost and loses it again to 16 SMs' share of the projections: 124 us for four layers and 5 rows against 128 on 64
+// CTAs, 31 against 30 for one layer and one row.)
 template <int MR>
 __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid_constant__ FfParams p) {
     extern __shared__ __align__(16) float ff_smem_[];

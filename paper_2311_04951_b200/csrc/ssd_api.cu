@@ -678,7 +678,7 @@ bool single_kernel_path(const ssd_model *m) {
 bool f32_kernel_path(const ssd_model *m, ssd_kv *kv, int M) {
     const ssd_arch &a = m->a;
     return a.dtype == 0 && g_persistent && a.n_layers <= kFfMaxLayers && a.d_ff % 4 == 0 && kv_bound(kv) + M <= kFfMaxCtx &&
-           ff_smem(a.d_model, a.d_ff, a.parallel_residual, M, a.head_dim) <= (size_t)kFfMaxSmem && m->aligned16;
+           ff_smem(a.d_model, a.d_ff, M, a.head_dim) <= (size_t)kFfMaxSmem && m->aligned16;
 }
 
 int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int M, const int32_t *n_rows,
@@ -705,14 +705,15 @@ int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride,
         const float **dst = (const float **)&p.layer[l];
         for (int i = 0; i < PER_LAYER; ++i) dst[i] = (const float *)lw(m, l, i);
     }
+    p.inv_d = 1.0 / (double)a.d_model;
+    const size_t smem = ff_smem(a.d_model, a.d_ff, M, a.head_dim);
+    void *args[] = {&p};
     // as many CTAs as the widest projection has columns for (a barrier costs less with fewer)
     int widest = 3 * a.d_model > a.d_ff ? 3 * a.d_model : a.d_ff;
     if (want_logits && a.vocab > widest) widest = a.vocab;
     int grid = ceil_div(widest, kFfWarps);
     if (grid < kv->B * a.n_heads) grid = kv->B * a.n_heads;
     if (grid > g_num_sms) grid = g_num_sms;
-    const size_t smem = ff_smem(a.d_model, a.d_ff, a.parallel_residual, M, a.head_dim);
-    void *args[] = {&p};
     const void *k = M <= 8 ? (const void *)forward_f32_kernel<8> : (const void *)forward_f32_kernel<kMaxRowsPerSeq>;
     CUDA_OK(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kFfThreads), args, smem, st));
     g_launches.fetch_add(1, std::memory_order_relaxed);

@@ -199,19 +199,28 @@ class Engine:
         self.prefill(torch.from_numpy(np.ascontiguousarray(prompts, np.int32)).to(dev))
         iters = 0
         limit = max_iters if max_iters is not None else n_new
+        # The uniforms of a group of iterations go to the device in one copy from pinned memory, which nothing waits for: a
+        # copy per iteration from pageable memory held the host until the GPU had run dry.  The counter read at the end of a
+        # group is the point from which the pinned block is free again.
+        Bn, group = self.batch, min(check_every, max(limit, 1))
+        stage = torch.empty(group * Bn * (2 * K + 1), dtype=torch.float32, pin_memory=True)
+        block = torch.empty_like(stage, device=dev, pin_memory=False)
+        ud_h, uv_h = (stage.numpy()[:group * Bn * K].reshape(group, Bn, K), stage.numpy()[group * Bn * K:].reshape(group, Bn, K + 1))
+        ud, uv = block[:group * Bn * K].view(group, Bn, K), block[group * Bn * K:].view(group, Bn, K + 1)
         while iters < limit:
-            for _ in range(check_every):
-                if iters >= limit:
-                    break
-                u = np.stack([uniforms(s, iters) for s in range(self.batch)]).astype(np.float32)
+            n = min(group, limit - iters)
+            for i in range(n):
+                for s in range(Bn):
+                    u = np.asarray(uniforms(s, iters + i), np.float32)
+                    ud_h[i, s], uv_h[i, s] = u[:K], u[K:2 * K + 1]
+            block.copy_(stage, non_blocking=True)
+            for i in range(n):
                 if K == 0:
-                    self.ar_step(torch.from_numpy(u[:, :1].copy()).to(dev))
+                    self.ar_step(uv[i])
                 else:
-                    ud = torch.from_numpy(u[:, :K].copy()).to(dev)
-                    uv = torch.from_numpy(u[:, K:2 * K + 1].copy()).to(dev)
-                    self.spec_iteration(ud, uv)
+                    self.spec_iteration(ud[i], uv[i])
                     self.advance()
-                iters += 1
+            iters += n
             if int(self.out_count.min().item()) >= n_new:
                 break
         counts = self.out_count.cpu().numpy()
