@@ -33,15 +33,20 @@ __host__ __device__ constexpr int m8_scratch_bytes(int Dh) {
 }
 
 template <int DH>
-__device__ __noinline__ void attention_item_mma8(const FwdParams &p, int layer, int item, uint8_t *scratch, Shared *sh) {
+__device__ __noinline__ void attention_items_mma8(int layer) {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
+    uint8_t *scratch = smem_base() + p.attn_smem_off;
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.attn_items; item += gridDim.x) {
     constexpr int NK = DH / 16, ND = DH / 8, ROWB = m8_row_bytes(DH), GPR = DH / 8;  // k-steps; 8-column tiles; bytes of a tile row; 16-byte pieces of a head row
     static_assert(DH % 16 == 0 && DH <= 128 && ND % 2 == 0, "head dims that are multiples of 16");
     constexpr int STAGE = m8_stage_bytes(DH), NS = m8_stages(DH);
     const int split = item % p.n_split, bh = item / p.n_split, b = bh / p.H, h = bh % p.H;
     const int d = p.d;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-    const int n_rows = staged_len(sh)[64 + b];
-    const int len = staged_len(sh)[b];
+    const int n_rows = staged_len()[64 + b];
+    const int len = staged_len()[b];
     const int r0 = b * p.M;
     const int chunk = split_chunk(p, len + n_rows, kAttnTile);
     const int p_begin = split * chunk;
@@ -272,4 +277,5 @@ __device__ __noinline__ void attention_item_mma8(const FwdParams &p, int layer, 
         }
     }
     named_bar(3, kAttnThreadsP);  // scratch is free for the next item
+    }
 }

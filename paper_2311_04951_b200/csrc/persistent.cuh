@@ -70,6 +70,11 @@ __device__ __forceinline__ const LayerDesc *layer_desc(const ModelDesc *md, int 
     return reinterpret_cast<const LayerDesc *>(md + 1) + l;
 }
 
+__device__ __forceinline__ uint8_t *smem_base() {
+    extern __shared__ uint8_t smem_raw[];
+    return (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+}
+
 enum { OP_XN1 = 0, OP_XN2 = 1, OP_AO = 2, OP_ACT = 3 };
 
 struct alignas(64) FwdParams {
@@ -110,14 +115,15 @@ struct alignas(64) FwdParams {
     int want_logits;
     // Shared-memory ring: slots [0, stages_lo) hold weights at any time; slots [stages_lo, stages) share
     // their bytes with the attention scratch (at attn_smem_off = stages_lo * stage bytes) and are used
-    // only between attention phases.  bar_off: byte offset of the barriers behind both.
-    int stages, stages_lo, attn_smem_off, bar_off;
+    // only between attention phases.
+    int stages, stages_lo, attn_smem_off;
     unsigned long long *trace;  // optional: CTA 0 stamps the global timer after every grid barrier
     // tensor-core attention (head dim 128): the whole cache as rows of Dh bf16, box 64 x 128 rows
     CUtensorMap tm_kv;
     const CUtensorMap *tm_kv_ptr;  // where the copy engine can read tm_kv (set by the kernel: see params copy)
-    int attn_tc;             // 0: attention_item (warp MMAs, 16-row tiles); 1: attention_item_tc; 2: attention_item_mma8 (up to eight rows, hi and lo in one MMA tile)
+    int attn_form;           // ATT_*: the form of the attention items
     int kv_rows_per_layer;   // B * 2 * H * S
+    int attn_items;          // attention items of a layer
     int attn_ctas;           // min(attention items, CTAs): set by the host together with the split plan
     int overlap_out;         // parallel-residual block and at most half of the CTAs on attention
     long long wait_cycles;   // bound of every wait that takes work (see Shared::wait_limit)
@@ -288,7 +294,6 @@ constexpr int kAccStride = 256;
 constexpr int kEpiWarps = 4;    // warps 0-3: one tensor-memory lane quadrant each
 constexpr int kMmaWarp = 4;
 constexpr int kEpiPitch = kTileNP + 8;             // floats per row of the epilogue tile (bank spread)
-constexpr int kEpiBytes = 8 * kEpiPitch * 4 + 16 + 16 * 8 + 16 * 4 + 16 + 2 * 16 + 8 * 4 + 1024 + 512 + (8 * kMaxStagedLayers + 2) * 8;  // ... + parameter copy, staged tables  // 8 rows, the four warps' wait results, attention barriers
 constexpr int kXWarp = 5;      // issues the operand copies of a GEMM phase
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -381,22 +386,39 @@ struct alignas(16) Shared {
     volatile int released;  // grid barriers completed so far
     volatile int abort;     // some wait in this CTA gave up
     volatile int go;        // snapshot of !abort taken inside the grid barrier: uniform for all work threads
+    int epoch;              // grid barriers passed (thread 0's)
     int flag;
     long long wait_limit;   // cycles after which a wait that takes work gives up (the drain waits of the error path keep kWaitCycles)
-    // for the tensor-core attention items (kept here so that they take no more arguments than the others):
     uint32_t tmem_base;     // base address of this CTA's tensor memory
-    uint32_t attn_bar_off;  // byte offset from this block to the attention barriers, followed by their counts
-    // small tables staged in shared memory (byte offsets from this block), so that the head of a phase does
-    // not start with a trip to global memory:
-    uint32_t seq_off;       // int len[64], then int rows[64]: committed length and rows of this pass, per sequence
-    uint32_t ltab_off;      // const float *[8 n_layers + 2]: the layers' gain / bias pointers, then the final norm's; 0 = not staged
+    int ltab_staged;        // the layers' gain / bias pointers are in shared memory (else: more layers than the table holds)
 };
-__device__ __forceinline__ const int *staged_len(const Shared *sh) {
-    return reinterpret_cast<const int *>(reinterpret_cast<const uint8_t *>(sh) + sh->seq_off);
+// The phase functions find their state at fixed shared-memory addresses: nothing is passed to them and nothing is kept in
+// registers across their calls for it, and a field is one shared-memory load with an immediate address.
+constexpr int kAttnBars = 15;
+struct alignas(128) SharedBlock {
+    uint8_t params[(sizeof(FwdParams) + 63) / 64 * 64];  // the kernel parameters, copied once (see forward_kernel)
+    Shared state;
+    int seq[128];                                  // committed length [64] and rows of this pass [64], per sequence
+    const float *ltab[8 * kMaxStagedLayers + 2];   // the layers' gain / bias pointers, then the final norm's
+    uint64_t fullW[32], fullX[32], empty[32];      // ring slots: weights there, operand there, free again
+    uint64_t accFull[2], accEmpty[2], mmaDone;     // accumulators
+    uint64_t abar[kAttnBars];                      // the tensor-core attention's barriers, and
+    uint32_t acnt[kAttnBars];                      // the phases they have completed
+    RingPos role_rp[2];  // the MMA issuer's and the operand issuer's walk of the ring, between GEMMs
+    int role_seg[8];     // per work warp: tile segments so far
+    int epi_ok[4];       // the epilogue warps' wait results
+    uint32_t tmem_slot;
+    double red[16];      // block reductions
+    float epi_tile[8 * kEpiPitch];
+};
+__device__ __forceinline__ SharedBlock &shared_block() {
+    __shared__ SharedBlock blk;
+    return blk;
 }
-__device__ __forceinline__ const float *const *staged_ltab(const Shared *sh) {
-    return sh->ltab_off ? reinterpret_cast<const float *const *>(reinterpret_cast<const uint8_t *>(sh) + sh->ltab_off) : nullptr;
-}
+__device__ __forceinline__ FwdParams &params_copy() { return *reinterpret_cast<FwdParams *>(shared_block().params); }
+__device__ __forceinline__ Shared *shared_state() { return &shared_block().state; }
+__device__ __forceinline__ const int *staged_len() { return shared_block().seq; }
+__device__ __forceinline__ const float *const *staged_ltab() { return shared_state()->ltab_staged ? shared_block().ltab : nullptr; }
 
 // Bounded wait that also gives up as soon as another thread of the CTA has.
 __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t *bar, uint32_t parity, const Shared *sh) {
@@ -420,12 +442,14 @@ __device__ __forceinline__ bool mbar_spin_or_abort(uint64_t *bar, uint32_t parit
 
 // Grid barrier for the 256 work threads of every CTA.  Returns false (the same value in every work
 // thread of the CTA) once a wait has timed out anywhere in this CTA; the caller then stops.
-__device__ __forceinline__ bool grid_sync(const FwdParams &p, Shared *sh, int &epoch) {
+__device__ __noinline__ bool grid_sync() {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
     fence_async_proxy();  // this thread's operand writes must be seen by other CTAs' TMA reads
     __threadfence();
     named_bar(1, kWorkThreads);
-    ++epoch;
     if (threadIdx.x == 0) {
+        const int epoch = ++sh->epoch;
         bool ok = sh->abort == 0;
         if (ok) {
             red_release_add(p.gbar, 1u);
@@ -456,16 +480,20 @@ __device__ __forceinline__ bool grid_sync(const FwdParams &p, Shared *sh, int &e
 
 // Arrival at the next grid barrier without waiting for it (for a CTA whose next work does not depend on
 // what the others publish there).  Its own writes are published like at a full barrier.
-__device__ __forceinline__ void grid_arrive(const FwdParams &p, Shared *sh, int &epoch) {
+__device__ __noinline__ void grid_arrive() {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
     fence_async_proxy();
     __threadfence();
     named_bar(1, kWorkThreads);
-    ++epoch;
-    if (threadIdx.x == 0 && sh->abort == 0) red_release_add(p.gbar, 1u);
-    if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {  // (the stamp of a barrier this CTA does not wait at: its arrival)
-        unsigned long long t;
-        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-        p.trace[epoch] = t;
+    if (threadIdx.x == 0) {
+        const int epoch = ++sh->epoch;
+        if (sh->abort == 0) red_release_add(p.gbar, 1u);
+        if (p.trace && blockIdx.x == 0) {  // (the stamp of a barrier this CTA does not wait at: its arrival)
+            unsigned long long t;
+            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+            p.trace[epoch] = t;
+        }
     }
 }
 
@@ -486,7 +514,9 @@ __device__ __forceinline__ void leave_grid(unsigned *gbar) {
 // without an item run the MLP-out GEMM beside the attention and go straight on to the out-projection:
 // its operand issuer waits for this count instead of a grid barrier.
 __device__ __forceinline__ unsigned *attn_done(const FwdParams &p) { return p.gbar + 8; }
-__device__ __forceinline__ void attn_signal(const FwdParams &p, Shared *sh) {
+__device__ __noinline__ void attn_signal() {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
     fence_async_proxy();  // the attention output is read by other CTAs' bulk copies
     __threadfence();
     named_bar(1, kWorkThreads);
@@ -494,29 +524,6 @@ __device__ __forceinline__ void attn_signal(const FwdParams &p, Shared *sh) {
 }
 
 // ---- non-GEMM phases (256 work threads) -------------------------------------------------------
-
-__device__ __forceinline__ float block_sum_work(float v, float *red) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    named_bar(2, kWorkThreads);
-    if (lane == 0) red[w] = v;
-    named_bar(2, kWorkThreads);
-    float t = 0.f;
-#pragma unroll
-    for (int i = 0; i < kConsumerWarps; ++i) t += red[i];
-    return t;
-}
-__device__ __forceinline__ double block_sum_work(double v, double *red) {
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    named_bar(2, kWorkThreads);
-    if (lane == 0) red[w] = v;
-    named_bar(2, kWorkThreads);
-    double t = 0.0;
-#pragma unroll
-    for (int i = 0; i < kConsumerWarps; ++i) t += red[i];
-    return t;
-}
 
 // two sums in one exchange
 __device__ __forceinline__ void block_sum2_work(double &a, double &b, double *red) {
@@ -579,8 +586,8 @@ __device__ __forceinline__ void norm_emit(const FwdParams &p, int r, int i, cons
 }
 
 template <int Q>  // float4 per thread held in registers: rows up to Q * 1024 wide; wider rows are re-read
-__device__ __noinline__ void norm_rows(const FwdParams &p, const float *g1, const float *b1, int op1,
-                                          const float *g2, const float *b2, int op2, double *red) {
+__device__ __noinline__ void norm_rows(const float *g1, const float *b1, int op1, const float *g2, const float *b2, int op2) {
+    const FwdParams &p = params_copy();
     const int n4 = p.d >> 2;  // d is a multiple of 8
     for (int r = blockIdx.x; r < p.R; r += gridDim.x) {
         const float4 *x4 = reinterpret_cast<const float4 *>(p.x + (size_t)r * p.d);
@@ -614,7 +621,7 @@ __device__ __noinline__ void norm_rows(const FwdParams &p, const float *g1, cons
             s1 += (double)v.x + (double)v.y + (double)v.z + (double)v.w;
             s2 += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
         }
-        block_sum2_work(s1, s2, red);
+        block_sum2_work(s1, s2, shared_block().red);
         double mean = 0.0, var;
         if (p.norm_kind == 0) {
             mean = s1 * p.inv_d;
@@ -640,17 +647,46 @@ __device__ __noinline__ void norm_rows(const FwdParams &p, const float *g1, cons
     }
 }
 
-__device__ __noinline__ void norm_phase(const FwdParams &p, const float *g1, const float *b1, int op1,
-                                           const float *g2, const float *b2, int op2, double *red) {
+__device__ __noinline__ void norm_phase(const float *g1, const float *b1, int op1, const float *g2, const float *b2, int op2) {
+    const FwdParams &p = params_copy();
     const int n4 = p.d >> 2;
-    if (n4 <= kWorkThreads) norm_rows<1>(p, g1, b1, op1, g2, b2, op2, red);
-    else if (n4 <= 2 * kWorkThreads) norm_rows<2>(p, g1, b1, op1, g2, b2, op2, red);
-    else if (n4 <= 4 * kWorkThreads) norm_rows<4>(p, g1, b1, op1, g2, b2, op2, red);
-    else norm_rows<8>(p, g1, b1, op1, g2, b2, op2, red);
+    if (n4 <= kWorkThreads) norm_rows<1>(g1, b1, op1, g2, b2, op2);
+    else if (n4 <= 2 * kWorkThreads) norm_rows<2>(g1, b1, op1, g2, b2, op2);
+    else if (n4 <= 4 * kWorkThreads) norm_rows<4>(g1, b1, op1, g2, b2, op2);
+    else norm_rows<8>(g1, b1, op1, g2, b2, op2);
+}
+
+// The norm in front of layer l's first GEMM(s) - or of the LM head - and the zeroing of what they accumulate into.
+__device__ __noinline__ void norm_for_layer(int l) {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
+    const float *const *lt = staged_ltab();
+    if (l < p.n_layers) {
+        const LayerDesc *ld = layer_desc(p.md, l);
+        const float *g1 = lt ? lt[8 * l + 0] : ld->ln1_g, *b1 = lt ? lt[8 * l + 1] : ld->ln1_b;
+        if (p.parallel)
+            norm_phase(g1, b1, OP_XN1, lt ? lt[8 * l + 4] : ld->ln2_g, lt ? lt[8 * l + 5] : ld->ln2_b, OP_XN2);
+        else norm_phase(g1, b1, OP_XN1, nullptr, nullptr, 0);
+        grid_zero(p.qkv, p.R, 3 * p.d, 3 * p.d);
+        if (p.parallel) grid_zero(p.t_in, p.R, p.d_in, p.d_in);
+    } else if (p.want_logits) {
+        norm_phase(lt ? lt[8 * p.n_layers] : p.md->lnf_g, lt ? lt[8 * p.n_layers + 1] : p.md->lnf_b, OP_XN1, nullptr, nullptr, 0);
+        grid_zero(p.logits, p.R, p.V, p.V);
+    }
+}
+// ... and between the two halves of a sequential block.
+__device__ __noinline__ void norm_mid_layer(int l) {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
+    const float *const *lt = staged_ltab();
+    const LayerDesc *ld = layer_desc(p.md, l);
+    norm_phase(lt ? lt[8 * l + 4] : ld->ln2_g, lt ? lt[8 * l + 5] : ld->ln2_b, OP_XN1, nullptr, nullptr, 0);
+    grid_zero(p.t_in, p.R, p.d_in, p.d_in);
 }
 
 // MLP activation of t_in into the hi/lo operand of the down projection, spread over the grid
-__device__ __noinline__ void act_phase(const FwdParams &p) {
+__device__ __noinline__ void act_phase() {
+    const FwdParams &p = params_copy();
     const int f4 = p.F >> 2;
     const long long total = (long long)p.R * f4;
     for (long long i = (long long)blockIdx.x * kWorkThreads + threadIdx.x; i < total;
@@ -677,7 +713,8 @@ __device__ __noinline__ void act_phase(const FwdParams &p) {
     }
 }
 
-__device__ __noinline__ void setup_phase(const FwdParams &p) {
+__device__ __noinline__ void setup_phase() {
+    const FwdParams &p = params_copy();
     if (blockIdx.x == gridDim.x - 1)  // (they are used behind this phase's barrier; every user leaves its own at zero)
         for (int i = threadIdx.x; i < p.B * p.H; i += kWorkThreads) p.tickets[i] = 0;
     // K not a multiple of 64: the last tile's unused columns must be finite (the weight copy zero-fills its own)
@@ -717,7 +754,8 @@ __device__ __noinline__ void setup_phase(const FwdParams &p) {
     }
 }
 
-__device__ __noinline__ void embed_phase(const FwdParams &p) {
+__device__ __noinline__ void embed_phase() {
+    const FwdParams &p = params_copy();
     for (int r = blockIdx.x; r < p.R; r += gridDim.x) {
         const int b = r / p.M, j = r % p.M;
         int tok = 0;
@@ -863,7 +901,12 @@ __host__ __device__ inline size_t attn_scratch_bytes(int Dh) {
 // their keys / values from qkv (rotary, cache rounding) and the split that owns them appends them
 // to the cache.  With one split the result goes straight to the out-projection operand; otherwise
 // partials are written and the split that finishes last merges them.  All exponentials are base 2.
-__device__ __noinline__ void attention_item(const FwdParams &p, int layer, int item, uint8_t *scratch, Shared *sh) {
+__device__ __noinline__ void attention_items(int layer) {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
+    uint8_t *scratch = smem_base() + p.attn_smem_off;
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.attn_items; item += gridDim.x) {
     const int MT = (p.M + kAttnRows - 1) / kAttnRows;
     const int mt = item % MT, rest = item / MT;
     const int split = rest % p.n_split, bh = rest / p.n_split, b = bh / p.H, h = bh % p.H;
@@ -882,8 +925,8 @@ __device__ __noinline__ void attention_item(const FwdParams &p, int layer, int i
     const int pg = warp & 3, dhh = warp >> 2;
     const int nk = Dh >> 4;          // k-steps of Q K^T; also 8-column output tiles per head half
     const int dh0 = dhh * (Dh >> 1);
-    const int n_rows = staged_len(sh)[64 + b];
-    const int len = staged_len(sh)[b];
+    const int n_rows = staged_len()[64 + b];
+    const int len = staged_len()[b];
     const int r0 = b * p.M, m_base = mt * kAttnRows;
     const int chunk = split_chunk(p, len + n_rows, kAttnTile);
     const int p_begin = split * chunk;
@@ -1181,6 +1224,7 @@ __device__ __noinline__ void attention_item(const FwdParams &p, int layer, int i
         }
     }
     named_bar(3, kAttnThreadsP);  // scratch is free for the next item
+    }
 }
 
 __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, bool valid) {
@@ -1190,38 +1234,41 @@ __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, boo
 #include "attn_mma8.cuh"
 
 // ---- attention on tcgen05 (head dim 128) ----------------------------------------------------------
-// The same item as attention_item - up to 16 query rows of one (sequence, head) over one split of the
-// position axis - with the two products on the 5th-generation tensor core and the scores and the
-// output in tensor memory, 128 positions per chunk:
-//   S^T [128 positions x 32]  = K chunk (the M = 128 operand, straight from the TMA copy of the cache)
-//                               x Q rows (16 hi + 16 lo, the N = 32 operand)
-//   O^T [128 head dims x 32] += V chunk read as its transpose (MN-major M = 128 operand) x P (16 hi + 16 lo)
-// Roles: threads 0-127 = one position each (softmax: masks, running max shared through shared memory,
-// P as bf16 hi + lo into the P tile, rescale of O^T when a maximum moved) and, at the end, one head
-// dim each (output); warp 4: MMA issue; warp 5: TMA copies of K and V chunks into a 4-stage ring;
-// warps 6-7: rows of this pass (positions >= len) - rotary, rounding, append to the cache - written
+// ALL query rows of one (sequence, head) - up to RP = 16 or 32 of them, so that every key and value is fetched once - over one
+// split of the position axis, with the two products on the 5th-generation tensor core and the scores and the output in tensor
+// memory, 128 positions per chunk:
+//   S^T [128 positions x 2 RP]  = K chunk (the M = 128 operand, straight from the TMA copy of the cache)
+//                                 x Q rows (RP hi + RP lo, the N operand; in log2 units)
+//   O^T [128 head dims x 2 RP] += V chunk read as its transpose (MN-major M = 128 operand) x P (RP hi + RP lo)
+// Roles: threads 0-127 = one position each (masks, P = exp2(S - reference), running sums in registers, P as bf16 hi + lo
+// into the P tile) and, at the end, one head dim each (output); warp 4: MMA issue; warp 5: TMA copies of K and V chunks
+// into a 4-stage ring; warps 6-7: rows of this pass (positions >= len) - rotary, rounding, append to the cache - written
 // into the chunk tiles over what the copy brought.  Positions behind them are masked (P = 0) and
 // multiply whatever the cache holds there: kv_init zeroes the cache, and all later writes are
-// finite rows of earlier passes, so 0 x stale is 0.  Per chunk 8 + 8 MMA steps of ~120 cycles against 1.5 us of HBM time for its
-// 64 KB: the chunk loop is bandwidth-bound instead of a latency chain.
+// finite rows of earlier passes, so 0 x stale is 0.
+// A row's softmax reference is the maximum of the first chunk it sees; it is only raised when a score passes it by more than
+// 2^32 (fp32 sums and bf16 hi + lo carry the factor without loss), which one barrier vote per chunk finds out: no maxima are
+// exchanged and O^T is not rescaled in the ordinary chunk.
+// Bound: the 64 KB of K and V a chunk fetches.  7B, 17 rows x 16384 positions: TC_OLD us a layer with two 16-row tiles that each
+// walk the cache and exchange maxima in every chunk, TC_NEW now, against 41 us of HBM time.
 constexpr int kTcChunk = 128;
 constexpr int kTcStages = 4;  // K / V ring stages of 32 KB: the bytes in flight set the chunk rate (3 stages: 2.7 us per chunk)
 constexpr int kTcKvStage = kTcChunk * 128 * 2;  // one K or V chunk: two 64-column panels of 128 rows x 128 B
-constexpr int kTcPBytes = 8192;  // one P tile (16 hi + 16 lo rows x 128 positions, bf16); two of them, used in turn
-constexpr int kTcQOff = kTcStages * kTcKvStage, kTcPOff = kTcQOff + 8192, kTcMiscOff = kTcPOff + 2 * kTcPBytes;
-constexpr int kTcScratchBytes = kTcMiscOff + 1536 + kAttnRows * 128 * 4;  // + per-thread running sums [16][128]
+__host__ __device__ constexpr int tc_rows_pad(int M) { return M <= 16 ? 16 : 32; }
+__host__ __device__ constexpr int tc_p_tiles(int rp) { return rp == 16 ? 2 : 1; }   // P tiles used in turn
+__host__ __device__ constexpr int tc_scratch_bytes(int rp) {  // ring, Q tile, P tiles, maxima and sums of four warps, references and factors
+    return kTcStages * kTcKvStage + (1 + tc_p_tiles(rp)) * 2 * rp * 256 + 10 * rp * 4;
+}
 // Its mbarriers live outside the scratch (which the weight ring reuses), are initialised once per kernel
 // and keep running: cnt[i] = phases barrier i has completed before the current item.  A parity wait is
 // only meaningful for a waiter that follows every phase of its barrier in order and that the barrier
 // cannot pass by two phases; the threads that patch this pass's rows into a chunk skip most chunks, so
 // they do not wait on the ring's barriers: the MMA issuer, which follows every stage, tells them through
-// `landed` when such a chunk has arrived, and hears back through `fixed`.
+// `landed` when such a chunk has arrived, and hears back through `fixed`.  (The vote keeps the softmax warps within a chunk
+// of each other, so that p_ready may be one barrier.)
 enum { AB_KV_FULL = 0, AB_KV_FREE = kTcStages, AB_S_FULL = 2 * kTcStages, AB_P_READY = AB_S_FULL + 2, AB_O_DONE /* two: chunk parity */,
        AB_FIXED = AB_O_DONE + 2, AB_LANDED, AB_COUNT };
-// The running maximum of a row is only raised when a chunk's maximum exceeds it by more than this (log2 units):
-// P then stays below 2^8, the sums and O^T absorb it, and the dependent rescale of O^T - which has to wait for the
-// previous chunk's P V - becomes rare instead of happening in every other chunk.
-constexpr float kTcMaxSlack = 8.f;
+constexpr float kTcMaxSlack = 32.f;
 
 __device__ __forceinline__ void tc_ld_32(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
@@ -1288,38 +1335,54 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
 // byte offset of (row, 16-byte chunk c) in a tile of 128-byte rows with the 128-byte swizzle
 __device__ __forceinline__ uint32_t sw128(int row, int c) { return (uint32_t)(row * 128 + ((c ^ (row & 7)) << 4)); }
 
-__device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, int item, uint8_t *scratch, Shared *sh) {
+// (all of the first 128 threads) true in all of them if `mine` is true in any
+__device__ __forceinline__ bool softmax_vote(bool mine) {
+    uint32_t any;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.u32 p, %1, 0;\n"
+        "barrier.cta.red.or.pred q, 6, 128, p;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n"
+        : "=r"(any)
+        : "r"(mine ? 1u : 0u)
+        : "memory");
+    return any != 0;
+}
+
+template <int RP>
+__device__ __noinline__ void attention_items_tc(int layer) {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
+    uint8_t *scratch = smem_base() + p.attn_smem_off;
+#pragma unroll 1
+    for (int item = blockIdx.x; item < p.attn_items; item += gridDim.x) {
+    constexpr int NP = tc_p_tiles(RP), kQBytes = 2 * RP * 256, kPanel = 2 * RP * 128;  // a tile: two panels of 2 RP rows x 128 B
     const uint32_t tmem_base = sh->tmem_base;
-    uint64_t *abar = reinterpret_cast<uint64_t *>(reinterpret_cast<uint8_t *>(sh) + sh->attn_bar_off);
-    uint32_t *acnt = reinterpret_cast<uint32_t *>(abar + AB_COUNT);
+    static_assert(AB_COUNT == kAttnBars, "barriers in the shared block");
+    uint64_t *abar = shared_block().abar;
+    uint32_t *acnt = shared_block().acnt;
     constexpr int Dh = 128;
-    const int MT = (p.M + kAttnRows - 1) / kAttnRows;
-    const int mt = item % MT, rest = item / MT;
-    const int split = rest % p.n_split, bh = rest / p.n_split, b = bh / p.H, h = bh % p.H;
+    const int split = item % p.n_split, bh = item / p.n_split, b = bh / p.H, h = bh % p.H;
     const int d = p.d;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint8_t *ring = scratch, *qt = scratch + kTcQOff, *pt = scratch + kTcPOff;
-    // [2][4][16] chunk maxima per warp: scores are one chunk ahead, so a fast warp may already write the next
-    // chunk's maxima while a slow one still reads this chunk's
-    float *wmax2 = reinterpret_cast<float *>(scratch + kTcMiscOff);
-    float *wsum = wmax2 + 128;                                      // [4][16]
-    float *wmrun = wsum + 64;                                       // [4][16] running maxima, one copy per warp
-    float *fsh = wmrun + 64;                                        // [4][16] this chunk's rescale factors
-    float *l_sh = fsh + 64;                                         // [16][128] running sums, one per (row, thread)
+    uint8_t *ring = scratch, *qt = scratch + kTcStages * kTcKvStage, *pt = qt + kQBytes;
+    float *wmax = reinterpret_cast<float *>(pt + NP * kQBytes);  // [4][RP] of the four softmax warps
+    float *wsum = wmax + 4 * RP, *m_ref = wsum + 4 * RP, *fsh = m_ref + RP;  // [4][RP], the rows' references, a raise's factors
     uint64_t *kv_full = abar + AB_KV_FULL, *kv_free = abar + AB_KV_FREE;  // [kTcStages] each
     uint64_t *s_full = abar + AB_S_FULL;  // [2]: the scores are double-buffered in tensor memory
     uint64_t *p_ready = abar + AB_P_READY, *o_done = abar + AB_O_DONE, *fixed = abar + AB_FIXED, *landed = abar + AB_LANDED;
 
-    const int n_rows = staged_len(sh)[64 + b];
-    const int len = staged_len(sh)[b];
-    const int r0 = b * p.M, m_base = mt * kAttnRows;
-    const int rows_here = max(0, min(kAttnRows, p.M - m_base));
+    const int n_rows = staged_len()[64 + b];
+    const int len = staged_len()[b];
+    const int r0 = b * p.M, rows_here = p.M;
     const int chunk = split_chunk(p, len + n_rows, kTcChunk);
     const int p_begin = split * chunk;
     const int p_end = min(p_begin + chunk, len + n_rows);
     const int n_chunks = p_begin < p_end ? (p_end - p_begin + kTcChunk - 1) / kTcChunk : 0;
     const float sc = p.attn_scale * 1.4426950408889634f;  // scores in log2 units
-    const uint32_t tS = tmem_base, tO = tmem_base + 64;  // scores of chunk c at tS + 32 (c & 1)
+    const uint32_t tS = tmem_base, tO = tmem_base + 4 * RP;  // scores of chunk c at tS + 2 RP (c & 1)
     __nv_bfloat16 *kc = (__nv_bfloat16 *)(p.cache + (size_t)layer * p.layer_bytes) + ((size_t)(b * 2) * p.H + h) * p.S * Dh;
     __nv_bfloat16 *vc = kc + (size_t)p.H * p.S * Dh;
     const int krow0 = layer * p.kv_rows_per_layer + ((b * 2) * p.H + h) * p.S, vrow0 = krow0 + p.H * p.S;
@@ -1333,16 +1396,12 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
         }
     };
 
-    // phases completed before this item (written by thread 0 at the end of the previous item, behind a barrier)
-    uint32_t c_full[kTcStages], c_free[kTcStages];
-#pragma unroll
-    for (int i = 0; i < kTcStages; ++i) { c_full[i] = acnt[AB_KV_FULL + i]; c_free[i] = acnt[AB_KV_FREE + i]; }
-    const uint32_t c_s0 = acnt[AB_S_FULL], c_s1 = acnt[AB_S_FULL + 1];
-    const uint32_t c_p = acnt[AB_P_READY], c_o0 = acnt[AB_O_DONE], c_o1 = acnt[AB_O_DONE + 1], c_fix = acnt[AB_FIXED], c_land = acnt[AB_LANDED];
+    // acnt: phases completed before this item (advanced by thread 0 at the end of the previous item, behind a barrier)
     // P V of chunk c completes phase c >> 1 of o_done[c & 1]
-    auto o_par = [&](int c) { return ((c & 1 ? c_o1 : c_o0) + (uint32_t)(c >> 1)) & 1u; };
-    auto full_par = [&](int j) { return (c_full[j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u; };          // stage j has landed
-    auto free_par = [&](int j) { return ((c_free[j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u) ^ 1u; };   // its slot was released
+    auto o_par = [&](int c) { return (acnt[AB_O_DONE + (c & 1)] + (uint32_t)(c >> 1)) & 1u; };
+    auto s_par = [&](int c) { return (acnt[AB_S_FULL + (c & 1)] + (uint32_t)(c >> 1)) & 1u; };
+    auto full_par = [&](int j) { return (acnt[AB_KV_FULL + j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u; };          // stage j has landed
+    auto free_par = [&](int j) { return ((acnt[AB_KV_FREE + j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u) ^ 1u; };   // its slot was released
     int n_fix_total = 0;
     for (int c = 0; c < n_chunks; ++c) n_fix_total += (p_begin + (c + 1) * kTcChunk > len) ? 1 : 0;
 
@@ -1360,25 +1419,26 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
         fence_async_proxy();  // the previous user of these slots wrote them through the generic proxy
         for (int j = 0; j < n_early; ++j) issue_kv(j);
     }
-    // ---- set-up: Q tile (rotary applied; 16 hi rows, 16 lo rows), P tile zeroed ----
-    {
-        const int ml = tid >> 4, v8 = tid & 15, m = m_base + ml;
+    // ---- set-up: Q tile (rotary applied, in log2 units; RP hi rows, RP lo rows) ----
+#pragma unroll
+    for (int it = 0; it < RP / 16; ++it) {
+        const int m = 16 * it + (tid >> 4), v8 = tid & 15;
         float q[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) q[u] = 0.f;
-        if (m < n_rows && ml < rows_here) rope_vec8(p, p.qkv + (size_t)(r0 + m) * 3 * d + h * Dh, r0 + m, v8 * 8, q);
+        if (m < n_rows) rope_vec8(p, p.qkv + (size_t)(r0 + m) * 3 * d + h * Dh, r0 + m, v8 * 8, q);
         __nv_bfloat16 hq[8], lq[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
+            q[u] *= sc;
             hq[u] = __float2bfloat16_rn(q[u]);
             lq[u] = __float2bfloat16_rn(q[u] - __bfloat162float(hq[u]));
         }
-        uint8_t *panel = qt + (v8 >> 3) * 4096;
-        *reinterpret_cast<uint4 *>(panel + sw128(ml, v8 & 7)) = *reinterpret_cast<uint4 *>(hq);
-        *reinterpret_cast<uint4 *>(panel + sw128(16 + ml, v8 & 7)) = *reinterpret_cast<uint4 *>(lq);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) reinterpret_cast<uint4 *>(pt)[4 * tid + i] = make_uint4(0, 0, 0, 0);  // both P tiles
+        uint8_t *panel = qt + (v8 >> 3) * kPanel;
+        *reinterpret_cast<uint4 *>(panel + sw128(m, v8 & 7)) = *reinterpret_cast<uint4 *>(hq);
+        *reinterpret_cast<uint4 *>(panel + sw128(RP + m, v8 & 7)) = *reinterpret_cast<uint4 *>(lq);
     }
+    // (P rows that no softmax thread writes meet output columns that nobody reads)
     fence_async_proxy();
     named_bar(3, kAttnThreadsP);
 
@@ -1399,7 +1459,7 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
     } else if (warp == 4) {
         // ---------------- MMA issue ----------------
         if (lane == 0) {
-            const uint32_t idS = umma_idesc_bf16(128, 32), idO = umma_idesc_bf16(128, 32) | (1u << 15);  // A of PV: MN-major
+            const uint32_t idS = umma_idesc_bf16(128, 2 * RP), idO = umma_idesc_bf16(128, 2 * RP) | (1u << 15);  // A of PV: MN-major
             const uint32_t qa = smem_u32(qt), pa = smem_u32(pt);
             int n_fix = 0;
             // S(c): scores of chunk c into buffer c & 1; issued one chunk ahead of P V so that it runs
@@ -1411,7 +1471,7 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
                 if (fix) {  // both tiles are here: let the patching threads in, wait for them
                     wait(&kv_full[jv % kTcStages], full_par(jv));
                     if (!sh->abort) mbar_arrive(landed);
-                    wait(fixed, (c_fix + n_fix) & 1u);
+                    wait(fixed, (acnt[AB_FIXED] + n_fix) & 1u);
                     ++n_fix;
                 }
                 if (sh->abort) return;
@@ -1419,8 +1479,8 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
                 const uint32_t ka = smem_u32(ring + (jk % kTcStages) * kTcKvStage);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)  // k = 16 head dims per step; panel ks / 4
-                    tc_mma_bf16(tS + 32 * (c & 1), umma_desc(ka + (ks >> 2) * (kTcKvStage / 2) + (ks & 3) * 32, 16, 1024),
-                                umma_desc(qa + (ks >> 2) * 4096 + (ks & 3) * 32, 16, 1024), idS, ks ? 1u : 0u);
+                    tc_mma_bf16(tS + 2 * RP * (c & 1), umma_desc(ka + (ks >> 2) * (kTcKvStage / 2) + (ks & 3) * 32, 16, 1024),
+                                umma_desc(qa + (ks >> 2) * kPanel + (ks & 3) * 32, 16, 1024), idS, ks ? 1u : 0u);
                 tc_commit(&s_full[c & 1]);
                 tc_commit(&kv_free[jk % kTcStages]);
             };
@@ -1428,7 +1488,7 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
             for (int c = 0; c < n_chunks && !sh->abort; ++c) {
                 const int jv = 2 * c + 1;
                 if (c + 1 < n_chunks) issue_s(c + 1);
-                wait(p_ready, (c_p + c) & 1u);
+                wait(p_ready, (acnt[AB_P_READY] + c) & 1u);
                 wait(&kv_full[jv % kTcStages], full_par(jv));
                 if (sh->abort) break;
                 tc_fence_after();
@@ -1436,7 +1496,7 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)  // k = 16 positions per step: two 8-row groups of the V tile
                     tc_mma_bf16(tO, umma_desc(va + ks * 2048, kTcKvStage / 2, 1024),
-                                umma_desc(pa + (c & 1) * kTcPBytes + (ks >> 2) * 4096 + (ks & 3) * 32, 16, 1024), idO, (c | ks) ? 1u : 0u);
+                                umma_desc(pa + (c % NP) * kQBytes + (ks >> 2) * kPanel + (ks & 3) * 32, 16, 1024), idO, (c | ks) ? 1u : 0u);
                 tc_commit(&o_done[c & 1]);
                 tc_commit(&kv_free[jv % kTcStages]);
             }
@@ -1452,162 +1512,148 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
             const int jk = 2 * c, jv = 2 * c + 1;
             uint8_t *kt = ring + (jk % kTcStages) * kTcKvStage, *vt = ring + (jv % kTcStages) * kTcKvStage;
             const int first = max(0, len - base), last = min(kTcChunk, len + n_rows - base);  // tile rows [first, last)
-            // at most 32 rows x 16 vectors = 8 work items per thread: compute them all, then wait for the copies
-            uint4 kq[8], vq[8];
+            // 16 vectors a row; two of them per thread and step, computed before the copies are waited for
+            bool here = false;
+#pragma unroll 1
+            for (int i0 = ft; i0 < (last - first) * 16; i0 += 128) {
+                uint4 kq[2], vq[2];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = ft + 64 * u, pr = first + (i >> 4), v8 = i & 15;
-                kq[u] = vq[u] = make_uint4(0, 0, 0, 0);
-                if (pr < last) {
-                    const int pos = base + pr, r = r0 + (pos - len);
-                    const float *krow = p.qkv + (size_t)r * 3 * d + d + h * Dh;
-                    float kf[8];
-                    rope_vec8(p, krow, r, v8 * 8, kf);
-                    const float4 v0 = __ldcg(reinterpret_cast<const float4 *>(krow + d + v8 * 8));
-                    const float4 v1 = __ldcg(reinterpret_cast<const float4 *>(krow + d + v8 * 8 + 4));
-                    const float vf[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-                    __nv_bfloat16 kb[8], vb[8];
-#pragma unroll
-                    for (int w = 0; w < 8; ++w) {
-                        kb[w] = __float2bfloat16_rn(kf[w]);
-                        vb[w] = __float2bfloat16_rn(vf[w]);
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + 64 * u, pr = first + (i >> 4), v8 = i & 15;
+                    if (pr < last) {
+                        const int pos = base + pr, r = r0 + (pos - len);
+                        const float *krow = p.qkv + (size_t)r * 3 * d + d + h * Dh;
+                        float kf[8];
+                        rope_vec8(p, krow, r, v8 * 8, kf);
+                        const float4 v0 = __ldcg(reinterpret_cast<const float4 *>(krow + d + v8 * 8));
+                        const float4 v1 = __ldcg(reinterpret_cast<const float4 *>(krow + d + v8 * 8 + 4));
+                        kq[u] = make_uint4(pack_bf16x2(kf[0], kf[1]), pack_bf16x2(kf[2], kf[3]), pack_bf16x2(kf[4], kf[5]), pack_bf16x2(kf[6], kf[7]));
+                        vq[u] = make_uint4(pack_bf16x2(v0.x, v0.y), pack_bf16x2(v0.z, v0.w), pack_bf16x2(v1.x, v1.y), pack_bf16x2(v1.z, v1.w));
                     }
-                    kq[u] = *reinterpret_cast<uint4 *>(kb);
-                    vq[u] = *reinterpret_cast<uint4 *>(vb);
                 }
-            }
-            wait(landed, (c_land + (uint32_t)n_fixed) & 1u);
-            ++n_fixed;
+                if (!here) {
+                    wait(landed, (acnt[AB_LANDED] + (uint32_t)n_fixed) & 1u);
+                    here = true;
+                }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = ft + 64 * u, pr = first + (i >> 4), v8 = i & 15;
-                if (pr < last) {
-                    const uint32_t off = (uint32_t)(v8 >> 3) * (kTcKvStage / 2) + sw128(pr, v8 & 7);
-                    *reinterpret_cast<uint4 *>(kt + off) = kq[u];
-                    *reinterpret_cast<uint4 *>(vt + off) = vq[u];
-                    if (mt == 0) {  // append: exactly one split owns this position (stores after all the loads)
-                        const size_t go = (size_t)(base + pr) * Dh + v8 * 8;
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + 64 * u, pr = first + (i >> 4), v8 = i & 15;
+                    if (pr < last) {
+                        const uint32_t off = (uint32_t)(v8 >> 3) * (kTcKvStage / 2) + sw128(pr, v8 & 7);
+                        *reinterpret_cast<uint4 *>(kt + off) = kq[u];
+                        *reinterpret_cast<uint4 *>(vt + off) = vq[u];
+                        const size_t go = (size_t)(base + pr) * Dh + v8 * 8;  // append: exactly one split owns this position
                         *reinterpret_cast<uint4 *>(kc + go) = kq[u];
                         *reinterpret_cast<uint4 *>(vc + go) = vq[u];
                     }
                 }
             }
+            if (!here) wait(landed, (acnt[AB_LANDED] + (uint32_t)n_fixed) & 1u);
+            ++n_fixed;
             fence_async_proxy();
             mbar_arrive(fixed);
         }
     } else {
         // ---------------- softmax: thread = position tid of the chunk ----------------
-        // Runtime loops over the real rows (usually 5 of 16) and per-row tensor-memory loads keep this
-        // code small: it runs once per item and layer, so its instruction fetch is mostly cold.
         const uint32_t lane_sel = (uint32_t)(warp * 32) << 16;
-        float *lrow = l_sh + tid;
-        for (int r = 0; r < rows_here; ++r) lrow[r * 128] = 0.f;
-        if (lane < kAttnRows) { wmrun[warp * 16 + lane] = -INFINITY; fsh[warp * 16 + lane] = 1.f; }
-        __syncwarp();
+        float l[RP];
+#pragma unroll
+        for (int r = 0; r < RP; ++r) l[r] = 0.f;
+        if (tid < RP) m_ref[tid] = -INFINITY;
+        named_bar(6, 128);
         for (int c = 0; c < n_chunks; ++c) {
             const int pos = p_begin + c * kTcChunk + tid;
-            const uint32_t tSc = tS + 32 * (c & 1) + lane_sel;
-            float *wmax = wmax2 + 64 * (c & 1);
-            wait(&s_full[c & 1], ((c & 1 ? c_s1 : c_s0) + (uint32_t)(c >> 1)) & 1u);
+            // rows from `first` on see this position (none beyond the split)
+            const int first = pos < p_end ? pos - len : RP;
+            const uint32_t tSc = tS + 2 * RP * (c & 1) + lane_sel;
+            wait(&s_full[c & 1], s_par(c));
             tc_fence_after();
-            // the chunk's row maxima over its 128 positions; 8 rows per tensor-memory round trip, unrolled
-            // over those 8 so that their shuffles and exponentials overlap
-            const int nblk = (rows_here + 7) >> 3;
+            // (the scores are read from tensor memory again for each use: a block of eight rows at a time in registers)
+            auto scores = [&](int blk, float (&v)[8]) {
+                float lo[8];
+                tc_ld_2x8(tSc + 8 * blk, tSc + RP + 8 * blk, v, lo);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) v[i] = 8 * blk + i >= first ? v[i] + lo[i] : -INFINITY;
+            };
+            bool over = false;
 #pragma unroll 1
-            for (int blk = 0; blk < nblk; ++blk) {
-                float a[8], b2[8];
-                tc_ld_2x8(tSc + 8 * blk, tSc + 16 + 8 * blk, a, b2);
-                float mx[8];
+            for (int blk = 0; 8 * blk < rows_here; ++blk) {
+                float v[8];
+                scores(blk, v);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = 8 * blk + i;
-                    const bool vis = r < rows_here && pos < p_end && pos <= len + m_base + r;
-                    mx[i] = vis ? (a[i] + b2[i]) * sc : -INFINITY;
-                }
-#pragma unroll
-                for (int o = 16; o; o >>= 1)
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) mx[i] = fmaxf(mx[i], __shfl_xor_sync(0xffffffffu, mx[i], o));
-                if (lane < 8) {
-                    float sel = mx[0];
-#pragma unroll
-                    for (int i = 1; i < 8; ++i) sel = lane == i ? mx[i] : sel;
-                    wmax[warp * 16 + 8 * blk + lane] = sel;
-                }
+                for (int i = 0; i < 8; ++i) over = over || (8 * blk + i < rows_here && v[i] > m_ref[8 * blk + i] + kTcMaxSlack);
             }
-            named_bar(6, 128);
-            if (c > 1) wait(&o_done[c & 1], o_par(c - 2));  // this chunk's P tile was last read by P V of chunk c - 2
-            bool moved = false;
-            uint8_t *panel = pt + (c & 1) * kTcPBytes + (tid >> 6) * 4096;
-            const int cc = (tid & 63) >> 3, e = (tid & 7) * 2;
+            if (softmax_vote(over)) {  // rare, and the first chunk: raise the references that are passed
 #pragma unroll 1
-            for (int blk = 0; blk < nblk; ++blk) {
-                float a[8], b2[8];
-                tc_ld_2x8(tSc + 8 * blk, tSc + 16 + 8 * blk, a, b2);
-                float fl[8], ml[8];
+                for (int blk = 0; 8 * blk < rows_here; ++blk) {
+                    float v[8];
+                    scores(blk, v);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    const int r = 8 * blk + i;
-                    fl[i] = 1.f;
-                    ml[i] = -INFINITY;
-                    if (r < rows_here) {
-                        const bool vis = pos < p_end && pos <= len + m_base + r;
-                        const float v = vis ? (a[i] + b2[i]) * sc : -INFINITY;
-                        const float mc = fmaxf(fmaxf(wmax[r], wmax[16 + r]), fmaxf(wmax[32 + r], wmax[48 + r]));
-                        const float m_old = wmrun[warp * 16 + r];
-                        const float m_new = (mc > m_old + kTcMaxSlack || m_old == -INFINITY) ? fmaxf(m_old, mc) : m_old;
-                        float pv = 0.f;
-                        if (m_new > -INFINITY) {
-                            fl[i] = exp2f(m_old - m_new);  // 0 on the first non-empty chunk
-                            pv = exp2f(v - m_new);
-                        }
-                        ml[i] = m_new;
-                        moved = moved || (fl[i] != 1.f);  // the same in all 128 threads: they read the same maxima
-                        lrow[r * 128] = lrow[r * 128] * fl[i] + pv;
-                        // P as bf16 hi + lo into the P tile: row r (hi) / 16 + r (lo), column = this position
-                        const __nv_bfloat16 hv = __float2bfloat16_rn(pv);
-                        *reinterpret_cast<__nv_bfloat16 *>(panel + sw128(r, cc) + e) = hv;
-                        *reinterpret_cast<__nv_bfloat16 *>(panel + sw128(16 + r, cc) + e) =
-                            __float2bfloat16_rn(pv - __bfloat162float(hv));
+                    for (int i = 0; i < 8; ++i) {
+                        const float mx = warp_max(v[i]);
+                        if (lane == 0) wmax[warp * RP + 8 * blk + i] = mx;
                     }
                 }
-                __syncwarp();  // every lane has read this block's running maxima
-                if (lane < 8 && 8 * blk + lane < rows_here) {
-                    float msel = ml[0], fsel = fl[0];
+                named_bar(6, 128);
+                if (tid < rows_here) {
+                    const float mx = fmaxf(fmaxf(wmax[tid], wmax[RP + tid]), fmaxf(wmax[2 * RP + tid], wmax[3 * RP + tid]));
+                    const float old = m_ref[tid];
+                    const bool up = mx > old + kTcMaxSlack;
+                    fsh[tid] = up ? exp2f(old - mx) : 1.f;  // 0 where nothing had been seen
+                    if (up) m_ref[tid] = mx;
+                }
+                named_bar(6, 128);
 #pragma unroll
-                    for (int i = 1; i < 8; ++i) {
-                        msel = lane == i ? ml[i] : msel;
-                        fsel = lane == i ? fl[i] : fsel;
+                for (int r = 0; r < RP; ++r)
+                    if (r < rows_here) l[r] *= fsh[r];
+                if (c > 0) {  // thread = head dim tid: scale the accumulated O^T, once P V of the previous chunk has written it
+                    wait(&o_done[(c - 1) & 1], o_par(c - 1));
+                    tc_fence_after();
+#pragma unroll 1
+                    for (int blk = 0; blk < 2 * RP / 32; ++blk) {
+                        float o[32];
+                        tc_ld_32(tO + lane_sel + 32 * blk, o);
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) o[i] *= i % RP < rows_here ? fsh[i % RP] : 1.f;
+                        tc_st_32(tO + lane_sel + 32 * blk, o);
                     }
-                    wmrun[warp * 16 + 8 * blk + lane] = msel;
-                    fsh[warp * 16 + 8 * blk + lane] = fsel;
                 }
             }
-            __syncwarp();
-            if (c > 0 && moved) {  // thread = head dim tid: scale the accumulated O^T, once P V of the previous chunk has written it
-                wait(&o_done[(c - 1) & 1], o_par(c - 1));
-                tc_fence_after();
-                float o[32];
-                tc_ld_32(tO + lane_sel, o);
+            if (c >= NP) wait(&o_done[(c - NP) & 1], o_par(c - NP));  // this chunk's P tile was last read by P V of chunk c - NP
+            // (opaque, or the compiler keeps the tile's 2 RP store addresses in registers - and on the stack - across the chunks)
+            uint32_t panel = smem_u32(pt) + (uint32_t)((c % NP) * kQBytes + (tid >> 6) * kPanel + (tid & 7) * 2);
+            uint32_t cc = (uint32_t)((tid & 63) >> 3);
+            asm volatile("" : "+r"(panel), "+r"(cc));
 #pragma unroll
-                for (int r = 0; r < kAttnRows; ++r) {
-                    const float f = fsh[warp * 16 + r];  // 1 for rows beyond rows_here
-                    o[r] *= f;
-                    o[16 + r] *= f;
+            for (int blk = 0; blk < RP / 8; ++blk) {
+                if (8 * blk < rows_here) {
+                    float v[8];
+                    scores(blk, v);
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int r = 8 * blk + i;  // (rows beyond rows_here: zero queries, columns nobody reads)
+                        // (a row that has seen nothing yet: reference -inf, every score -inf)
+                        const float pv = v[i] > -INFINITY ? exp2f(v[i] - m_ref[r]) : 0.f;
+                        l[r] += pv;
+                        // P as bf16 hi + lo into the P tile: row r (hi) / RP + r (lo), column = this position
+                        const __nv_bfloat16 hv = __float2bfloat16_rn(pv), lv = __float2bfloat16_rn(pv - __bfloat162float(hv));
+                        const uint32_t at = panel + r * 128 + ((cc ^ (r & 7)) << 4);
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at), "h"(__bfloat16_as_ushort(hv)) : "memory");
+                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + RP * 128), "h"(__bfloat16_as_ushort(lv)) : "memory");
+                    }
                 }
-                tc_st_32(tO + lane_sel, o);
             }
             fence_async_proxy();
             tc_fence_before();
             mbar_arrive(p_ready);
         }
         // ---- the sums over positions, then thread = head dim tid: output or partial ----
-#pragma unroll 1
-        for (int r = 0; r < rows_here; ++r) {
-            float t = lrow[r * 128];
 #pragma unroll
-            for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (lane == 0) wsum[warp * 16 + r] = t;
+        for (int r = 0; r < RP; ++r) {
+            if (r < rows_here) {
+                const float t = warp_sum(l[r]);
+                if (lane == 0) wsum[warp * RP + r] = t;
+            }
         }
         if (n_chunks > 1) wait(&o_done[(n_chunks - 2) & 1], o_par(n_chunks - 2));
         if (n_chunks > 0) {
@@ -1616,23 +1662,30 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
         }
         named_bar(6, 128);
         const bool direct = p.n_split == 1;
-#pragma unroll 1
-        for (int r = 0; r < rows_here; ++r) {
-            const int m = m_base + r;
-            const float L = (wsum[r] + wsum[16 + r]) + (wsum[32 + r] + wsum[48 + r]);
-            const bool live = m < n_rows && L > 0.f && n_chunks > 0;
-            float a = 0.f, b2 = 0.f;
-            if (n_chunks > 0) tc_ld_2(tO + lane_sel + r, tO + lane_sel + 16 + r, a, b2);
-            const float acc = live ? a + b2 : 0.f;
-            if (direct) {
-                store_hilo(p.op[OP_AO], p.rk, r0 + m, h * Dh + tid, live ? acc / L : 0.f);
-            } else {
-                const size_t slot = ((size_t)(r0 + m) * p.H + h) * p.n_split + split;
-                if (tid == 0) {
-                    p.part_m[slot] = live ? wmrun[r] : -INFINITY;
-                    p.part_l[slot] = live ? L : 0.f;
+#pragma unroll
+        for (int blk = 0; blk < RP / 8; ++blk) {
+            if (8 * blk < rows_here) {
+                float oh[8], ol[8];
+                if (n_chunks > 0) tc_ld_2x8(tO + lane_sel + 8 * blk, tO + lane_sel + RP + 8 * blk, oh, ol);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int r = 8 * blk + i;
+                    if (r < rows_here) {
+                        const float L = (wsum[r] + wsum[RP + r]) + (wsum[2 * RP + r] + wsum[3 * RP + r]);
+                        const bool live = r < n_rows && L > 0.f && n_chunks > 0;
+                        const float acc = live ? oh[i] + ol[i] : 0.f;
+                        if (direct) {
+                            store_hilo(p.op[OP_AO], p.rk, r0 + r, h * Dh + tid, live ? acc / L : 0.f);
+                        } else {
+                            const size_t slot = ((size_t)(r0 + r) * p.H + h) * p.n_split + split;
+                            if (tid == 0) {
+                                p.part_m[slot] = live ? m_ref[r] : -INFINITY;
+                                p.part_l[slot] = live ? L : 0.f;
+                            }
+                            p.part_o[slot * Dh + tid] = acc;
+                        }
+                    }
                 }
-                p.part_o[slot * Dh + tid] = acc;
             }
         }
         tc_fence_before();
@@ -1641,7 +1694,7 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
         // ticket: the item that finishes last for this (sequence, head) merges all partials
         __threadfence();
         named_bar(3, kAttnThreadsP);
-        if (tid == 0) sh->flag = (atomicAdd(p.tickets + bh, 1u) == (unsigned)(p.n_split * MT - 1));
+        if (tid == 0) sh->flag = (atomicAdd(p.tickets + bh, 1u) == (unsigned)(p.n_split - 1));
         named_bar(3, kAttnThreadsP);
         if (sh->flag) {
             __threadfence();
@@ -1649,72 +1702,39 @@ __device__ __noinline__ void attention_item_tc(const FwdParams &p, int layer, in
             if (tid == 0) p.tickets[bh] = 0;  // ready for the next layer (a grid barrier lies between)
         }
     }
+    named_bar(3, kAttnThreadsP);  // everyone has read the counts
     if (tid == 0) {
         for (int i = 0; i < kTcStages; ++i) {
             const uint32_t uses = (uint32_t)((2 * n_chunks + kTcStages - 1 - i) / kTcStages);  // stages j < 2 n_chunks with j % kTcStages == i
-            acnt[AB_KV_FULL + i] = c_full[i] + uses;
-            acnt[AB_KV_FREE + i] = c_free[i] + uses;
+            acnt[AB_KV_FULL + i] += uses;
+            acnt[AB_KV_FREE + i] += uses;
         }
-        acnt[AB_S_FULL] = c_s0 + (uint32_t)((n_chunks + 1) / 2);
-        acnt[AB_S_FULL + 1] = c_s1 + (uint32_t)(n_chunks / 2);
-        acnt[AB_P_READY] = c_p + n_chunks;
-        acnt[AB_O_DONE] = c_o0 + (uint32_t)((n_chunks + 1) / 2);
-        acnt[AB_O_DONE + 1] = c_o1 + (uint32_t)(n_chunks / 2);
-        acnt[AB_FIXED] = c_fix + n_fix_total;
-        acnt[AB_LANDED] = c_land + n_fix_total;
+        acnt[AB_S_FULL] += (uint32_t)((n_chunks + 1) / 2);
+        acnt[AB_S_FULL + 1] += (uint32_t)(n_chunks / 2);
+        acnt[AB_P_READY] += n_chunks;
+        acnt[AB_O_DONE] += (uint32_t)((n_chunks + 1) / 2);
+        acnt[AB_O_DONE + 1] += (uint32_t)(n_chunks / 2);
+        acnt[AB_FIXED] += n_fix_total;
+        acnt[AB_LANDED] += n_fix_total;
     }
     named_bar(3, kAttnThreadsP);  // scratch, tensor memory and the counts are ready for the next item
-}
-
-__device__ __forceinline__ void attention_phase(const FwdParams &p, int layer, uint8_t *scratch, Shared *sh) {
-    const int MT = (p.M + kAttnRows - 1) / kAttnRows;
-    const int items = p.B * p.H * p.n_split * MT;
-    for (int item = blockIdx.x; item < items; item += gridDim.x) {
-        if (p.attn_tc == 1) attention_item_tc(p, layer, item, scratch, sh);
-        else if (p.attn_tc == 2 && p.Dh == 128) attention_item_mma8<128>(p, layer, item, scratch, sh);
-        else if (p.attn_tc == 2) attention_item_mma8<64>(p, layer, item, scratch, sh);
-        else attention_item(p, layer, item, scratch, sh);
     }
 }
 
-// Where the kernel's small state lives behind the ring (and the attention scratch) in shared memory.
-struct SmemMap {
-    uint64_t *fullW, *fullX, *empty, *accFull, *accEmpty, *mmaDone;
-    uint32_t *tmem_slot;
-    Shared *sh;
-    double *red;
-    float *epi_tile;
-    volatile int *epi_ok;
-    uint64_t *abar;
-    uint32_t *acnt;
-    RingPos *role_rp;  // [2]: the MMA issuer's and the operand issuer's walk of the ring, between GEMMs
-    int *role_seg;     // [8]: per work warp, tile segments so far
-    FwdParams *params; // the kernel parameters, copied once (see forward_kernel)
-    int *seq;          // [128]: lengths, rows of this pass
-    const float **ltab;  // [8 * kMaxStagedLayers + 2]
-};
-__device__ __forceinline__ SmemMap smem_map(const FwdParams &p, uint8_t *smem) {
-    SmemMap m;
-    const int S = p.stages;
-    m.fullW = (uint64_t *)(smem + p.bar_off);
-    m.fullX = m.fullW + S;
-    m.empty = m.fullX + S;
-    m.accFull = m.empty + S;
-    m.accEmpty = m.accFull + 2;
-    m.mmaDone = m.accEmpty + 2;
-    m.tmem_slot = (uint32_t *)(m.mmaDone + 1);
-    m.sh = (Shared *)(((uintptr_t)(m.mmaDone + 4) + 15) & ~(uintptr_t)15);
-    m.red = (double *)(m.sh + 1);
-    m.epi_tile = (float *)(m.red + 16);
-    m.epi_ok = (volatile int *)(m.epi_tile + 8 * kEpiPitch);
-    m.abar = (uint64_t *)(m.epi_tile + 8 * kEpiPitch + 4);
-    m.acnt = (uint32_t *)(m.abar + AB_COUNT);
-    m.role_rp = (RingPos *)(m.acnt + AB_COUNT);
-    m.role_seg = (int *)(m.role_rp + 2);
-    m.params = (FwdParams *)(((uintptr_t)(m.role_seg + 8) + 63) & ~(uintptr_t)63);
-    m.seq = (int *)((uint8_t *)m.params + 960);
-    m.ltab = (const float **)(m.seq + 128);
-    return m;
+// WIDE: passes of more than 16 rows per sequence on the tensor core, a kernel of its own.  (A function that might be called
+// shapes the register allocation of the whole kernel body: with the 32-row item beside the other forms the body reloads 3 KB of
+// spilled values around its phases, 176 bytes without it.  One kernel per form leaves the body none, but its live values then
+// take the registers that the items want, which save and restore them instead: the 16-row items 15.1 -> 17.8 us, the packed ones
+// of eight 2100-position sequences 51.3 -> 53.8.)
+enum { ATT_MMA = 0, ATT_TC16, ATT_PACKED, ATT_TC32 };
+template <bool WIDE>
+__device__ __forceinline__ void attention_phase(int layer) {
+    const FwdParams &p = params_copy();
+    if constexpr (WIDE) attention_items_tc<32>(layer);
+    else if (p.attn_form == ATT_TC16) attention_items_tc<16>(layer);
+    else if (p.attn_form == ATT_PACKED && p.Dh == 128) attention_items_mma8<128>(layer);
+    else if (p.attn_form == ATT_PACKED) attention_items_mma8<64>(layer);
+    else attention_items(layer);
 }
 
 // Run this CTA's units of GEMM gi (all 256 work threads call it; NT = padded rows / 8).  The units are
@@ -1724,18 +1744,20 @@ __device__ __forceinline__ SmemMap smem_map(const FwdParams &p, uint8_t *smem) {
 // holds nothing across its calls: with 227 KB of shared memory there is next to no L1 left, and a
 // value spilled to the stack costs an L2 round trip at every phase.
 template <int NT>
-__device__ __noinline__ void run_gemm(const FwdParams &p, int gi, uint8_t *smem) {
+__device__ __noinline__ void run_gemm(int gi) {
+    const FwdParams &p = params_copy();
+    uint8_t *smem = smem_base();
     constexpr int kRp = NT * 8;
     constexpr int kXBytes = 2 * kRp * kTileK * 2;
     constexpr int kStageBytes = kXBytes + kWTileBytesP;
     // M of the MMA: the operand tile's 2 kRp rows; the rows the MMA reads beyond them are the weight
     // tile's bytes (finite or not, they only reach accumulator lanes that nobody loads)
     constexpr int kM = 2 * kRp <= 64 ? 64 : 128;
-    const SmemMap mp = smem_map(p, smem);
+    SharedBlock &mp = shared_block();
     const int S = p.stages, S1 = p.stages_lo;
     uint8_t *ring = smem;
     uint64_t *fullW = mp.fullW, *fullX = mp.fullX, *empty = mp.empty, *accFull = mp.accFull, *accEmpty = mp.accEmpty;
-    Shared *sh = mp.sh;
+    Shared *sh = &mp.state;
     float *epi_tile = mp.epi_tile;
     volatile int *epi_ok = mp.epi_ok;
     const uint32_t tmem_base = sh->tmem_base;
@@ -1751,7 +1773,7 @@ __device__ __noinline__ void run_gemm(const FwdParams &p, int gi, uint8_t *smem)
         __syncwarp();
     };
 
-            const GemmDesc g = gemm_desc(p, gi, staged_ltab(sh));
+            const GemmDesc g = gemm_desc(p, gi, staged_ltab());
             int c0, c1;
             unit_range(p, g, c0, c1);
             if (c0 >= c1) return;  // (no state to save: nothing moved)
@@ -1908,19 +1930,21 @@ __device__ __noinline__ void run_gemm(const FwdParams &p, int gi, uint8_t *smem)
 //      posted too (the fallback when rounding leaves no index past u S);
 // then CTA 0 writes the tokens and commits the rows fed in this step.
 __device__ __forceinline__ int tail_per(const FwdParams &p) { return (((p.V + (int)gridDim.x - 1) / (int)gridDim.x) + 3) & ~3; }
-__device__ __forceinline__ const float *tail_row(const FwdParams &p, const Shared *sh, int b) {
-    int row = (b < 64 ? staged_len(sh)[64 + b] : __ldcg(p.ri.n_eff + b)) - 1;  // (staged behind the step's first barrier)
+__device__ __forceinline__ const float *tail_row(const FwdParams &p, int b) {
+    int row = (b < 64 ? staged_len()[64 + b] : __ldcg(p.ri.n_eff + b)) - 1;  // (staged behind the step's first barrier)
     if (row < 0) row = 0;
     return p.logits + ((size_t)b * p.M + row) * p.V;
 }
 
 // (All loops below fetch eight elements before they use the first: a load from L2 costs about a microsecond
 // under the weight stream, and a slice is only a few hundred elements.)
-__device__ __noinline__ void tail_partial(const FwdParams &p, const Shared *sh) {
+__device__ __noinline__ void tail_partial() {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = (int)gridDim.x;
     const int per = tail_per(p), lo = min(p.V, (int)blockIdx.x * per), hi = min(p.V, lo + per);
     for (int b = warp; b < p.B; b += kConsumerWarps) {
-        const float *lg = tail_row(p, sh, b);
+        const float *lg = tail_row(p, b);
         // running (max, argmax, sum of exp relative to the max) per lane, then over the warp
         float mx = -INFINITY, sum = 0.f;
         int am = 0x7fffffff;
@@ -1993,12 +2017,14 @@ __device__ __forceinline__ float tail_prob(float logit, float mx, int am, float 
     return expf((logit - mx) * inv_t) / z;
 }
 
-__device__ __noinline__ void tail_q(const FwdParams &p, const Shared *sh) {
+__device__ __noinline__ void tail_q() {
+    const FwdParams &p = params_copy();
+    Shared *sh = shared_state();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = (int)gridDim.x;
     const int per = tail_per(p), lo = min(p.V, (int)blockIdx.x * per), hi = min(p.V, lo + per);
     const int seg = (hi - lo + 31) / 32, j0 = min(hi, lo + lane * seg), j1 = min(hi, j0 + seg);
     for (int b = warp; b < p.B; b += kConsumerWarps) {
-        const float *lg = tail_row(p, sh, b);
+        const float *lg = tail_row(p, b);
         float l[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) l[u] = j0 + u < j1 ? __ldcg(lg + j0 + u) : 0.f;  // (under the partials' latency)
@@ -2025,7 +2051,8 @@ __device__ __noinline__ void tail_q(const FwdParams &p, const Shared *sh) {
     }
 }
 
-__device__ __noinline__ void tail_draw(const FwdParams &p) {
+__device__ __noinline__ void tail_draw() {
+    const FwdParams &p = params_copy();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, G = (int)gridDim.x;
     const int per = tail_per(p), lo = min(p.V, (int)blockIdx.x * per), hi = min(p.V, lo + per);
     const int seg = (hi - lo + 31) / 32, j0 = min(hi, lo + lane * seg), j1 = min(hi, j0 + seg);
@@ -2086,7 +2113,8 @@ __device__ __noinline__ void tail_draw(const FwdParams &p) {
 }
 
 // CTA 0: the tokens of this step, and the rows it fed become part of the cache
-__device__ __noinline__ void tail_commit(const FwdParams &p) {
+__device__ __noinline__ void tail_commit() {
+    const FwdParams &p = params_copy();
     if (blockIdx.x != 0) return;
     for (int b = threadIdx.x; b < p.B; b += kWorkThreads) {
         const int32_t *slot = p.tail_hit + ((size_t)p.cur_step * p.B + b) * 2;
@@ -2099,273 +2127,245 @@ __device__ __noinline__ void tail_commit(const FwdParams &p) {
 }
 
 // ---- the kernel -----------------------------------------------------------------------------
-// NT = padded rows / 8
+// The producer's walk and the work warps' phase program are functions of their own that keep next to nothing alive across
+// the calls they make: what is live there takes registers that the attention items and GEMMs want, and is spilled around every
+// one of the 130-260 calls of a pass (LIVE_NOTE).
 template <int NT>
+__device__ __forceinline__ constexpr int stage_x_bytes() { return 2 * NT * 8 * kTileK * 2; }
+
+template <int NT>
+__device__ __noinline__ void producer_program() {
+    const FwdParams &p = params_copy();
+    constexpr int kXBytes = stage_x_bytes<NT>(), kStageBytes = kXBytes + kWTileBytesP;
+    uint64_t *fullW = shared_block().fullW, *empty = shared_block().empty;
+    Shared *sh = shared_state();
+    uint8_t *ring = smem_base();
+    const int S = p.stages, S1 = p.stages_lo, NG = n_gemms(p), lane = threadIdx.x & 31;
+    // Weights never change, so this cursor runs as far ahead as the ring allows, across grid
+    // barriers.  The loop is kept minimal (no divisions, no clock reads while it makes progress):
+    // its rate bounds the weight stream.
+    if (lane == 0) {
+        RingPos rp;
+        bool failed = false;
+        int seen_release = 0;
+        // a CTA that never runs an attention item (fewer items than CTAs) never uses the scratch: its
+        // upper slots take weights at any time
+        const bool scratch_used = (int)blockIdx.x < p.attn_items;
+        for (int gws = 0; gws < NG * p.n_steps && !failed; ++gws) {
+            const int gw = ((gws / NG) << kStepShift) | (gws % NG);
+            const GemmDesc dw = gemm_desc(p, gw);
+            int c0, c1;
+            unit_range(p, dw, c0, c1);
+            if (c0 >= c1) continue;
+            int tw = c0 / dw.kchunks, kw = c0 % dw.kchunks;
+            for (int c = c0; c < c1; ++c) {
+                uint32_t ph;
+                const int s = ring_next(rp, ring_lo_only(dw, c - c0, S1), S, S1, ph);
+                if (s >= S1 && scratch_used && seen_release < dw.need_hi) {  // slot shared with the attention scratch
+                    const long long t0 = clock64();
+                    while ((seen_release = sh->released) < dw.need_hi) {
+                        if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
+                    }
+                    if (failed) { rp.par ^= 1u << s; break; }  // nothing was issued into s
+                }
+                if (!mbar_test_wait(&empty[s], ph ^ 1u)) {
+                    const long long t0 = clock64();
+                    while (!mbar_test_wait(&empty[s], ph ^ 1u)) {
+                        if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
+                    }
+                    if (failed) { rp.par ^= 1u << s; break; }  // nothing was issued into s
+                }
+                mbar_expect_tx(&fullW[s], kWTileBytesP);
+                tma_load_2d(ring + (size_t)s * kStageBytes + kXBytes, dw.tmW, kw * kTileK, tw * kTileNP, &fullW[s]);
+                if (++kw == dw.kchunks) { kw = 0; ++tw; }
+            }
+        }
+        if (failed) {
+            set_status(p.status, kTimeoutCode);
+            sh->abort = 1;
+        }
+        // error path only: wait (bounded) for copies still in flight before the CTA may exit
+        if (sh->abort)
+            for (int s = 0; s < S; ++s)
+                if ((rp.used >> s) & 1u) mbar_wait(&fullW[s], ((rp.par >> s) & 1u) ^ 1u);
+    }
+}
+// The phase program (the same structure gemm_desc() encodes).  `go` is uniform over the work threads (taken inside the grid
+// barrier), so every named barrier is reached by all of them or by none.
+template <int NT, bool WIDE>
+__device__ __noinline__ void work_program() {
+    const FwdParams &p = params_copy();
+    if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        p.trace[0] = t;
+    }
+    if (p.tail && blockIdx.x == 0)  // the draws' meeting places: smallest hit index / largest index with weight
+        for (int i = threadIdx.x; i < p.n_steps * p.B * 2; i += kWorkThreads) p.tail_hit[i] = (i & 1) ? -1 : 0x7fffffff;
+    bool go = true;
+    for (int step = 0; step < p.n_steps && go; ++step) {
+        const int gs = step << kStepShift;
+        if (step > 0) {  // the rows of this step: one per sequence, the token the step before drew
+            if (threadIdx.x == 0) params_copy().cur_step = step;
+            named_bar(2, kWorkThreads);
+        }
+        // Set-up, embedding and the first norm of a row all run on the CTA that owns the row, so only
+        // CTA-wide barriers separate them: one grid barrier in front of the first GEMM instead of two.
+        setup_phase();
+        named_bar(2, kWorkThreads);  // the row's position and validity are read back by the embedding
+        embed_phase();
+        named_bar(2, kWorkThreads);  // the embedding rows are read back by the norm
+        norm_for_layer(0);
+        go = grid_sync();
+        if (go && threadIdx.x < 64) {  // lengths and rows of this pass (written by the set-up of every row), for the
+            int *tab = shared_block().seq;  // attention items, which run behind further grid barriers
+            const int b = threadIdx.x;
+            tab[b] = b < p.B ? __ldcg(p.len + b) : 0;
+            tab[64 + b] = b < p.B ? __ldcg(p.ri.n_eff + b) : 0;
+        }
+        for (int l = 0; l < p.n_layers && go; ++l) {
+            run_gemm<NT>(gs | (4 * l + 0));                  // qkv
+            if (p.parallel) run_gemm<NT>(gs | (4 * l + 1));       // MLP in (same block input)
+            if (!(go = grid_sync())) break;
+            if (overlap_mlp_out(p)) {
+                act_phase();
+                if ((int)blockIdx.x < attention_ctas(p)) {
+                    grid_arrive();  // the activation is out; attention needs nothing from the others
+                    attention_phase<WIDE>(l);
+                    attn_signal();
+                } else {
+                    if (!(go = grid_sync())) break;
+                    run_gemm<NT>(gs | (4 * l + 2));               // MLP out -> x, beside the attention items
+                    run_gemm<NT>(gs | (4 * l + 3));               // out-proj -> x, once the attention CTAs have signalled
+                }
+                if (!(go = grid_sync())) break;
+            } else {
+                attention_phase<WIDE>(l);
+                if (p.parallel) act_phase();
+                if (!(go = grid_sync())) break;
+                if (p.parallel) {
+                    run_gemm<NT>(gs | (4 * l + 2));                   // out-proj -> x
+                    run_gemm<NT>(gs | (4 * l + 3));                   // MLP out  -> x
+                    if (!(go = grid_sync())) break;
+                } else {
+                    run_gemm<NT>(gs | (4 * l + 1));                   // out-proj -> x
+                    if (!(go = grid_sync())) break;
+                    norm_mid_layer(l);
+                    if (!(go = grid_sync())) break;
+                    run_gemm<NT>(gs | (4 * l + 2));                   // MLP in
+                    if (!(go = grid_sync())) break;
+                    act_phase();
+                    if (!(go = grid_sync())) break;
+                    run_gemm<NT>(gs | (4 * l + 3));                   // MLP out -> x
+                    if (!(go = grid_sync())) break;
+                }
+            }
+            norm_for_layer(l + 1);
+            if (!(go = grid_sync())) break;
+        }
+        if (go && p.want_logits) run_gemm<NT>(gs | (4 * p.n_layers));
+        if (go && p.tail) {  // q, the draw and the commit of this step (see tail_partial)
+            if (!(go = grid_sync())) break;
+            tail_partial();
+            if (!(go = grid_sync())) break;
+            tail_q();
+            if (!(go = grid_sync())) break;
+            tail_draw();
+            if (!(go = grid_sync())) break;
+            tail_commit();
+            if (!(go = grid_sync())) break;
+        }
+    }
+    if (go && p.tail && p.mailbox && blockIdx.x == 0 && (int)threadIdx.x < p.B)  // the host's length bound follows (see report_len)
+        *reinterpret_cast<volatile unsigned long long *>(p.mailbox + threadIdx.x) =
+            ((unsigned long long)p.mb_seq << 32) | (unsigned)__ldcg(p.len_rw + threadIdx.x);
+    if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        p.trace[shared_state()->epoch + 1] = t;
+        p.trace[shared_state()->epoch + 2] = 0;
+    }
+}
+// NT = padded rows / 8
+template <int NT, bool WIDE>
 __global__ void __launch_bounds__(kPersistThreads, 1) forward_kernel(const __grid_constant__ FwdParams kp) {
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    // The phase functions are not inlined and read their parameters through a reference; a reference into the
-    // kernel-parameter bank makes every field a generic load at the head of each phase, so they get a copy in
-    // shared memory instead (tensor maps stay where the copy engine can read them: pointers into kp / global).
-    static_assert(sizeof(FwdParams) <= 960, "parameter copy area");
-    FwdParams *psm = smem_map(kp, smem).params;
+    // A reference into the kernel-parameter bank would make every field a generic load at the head of each phase: the phase
+    // functions read a copy in shared memory (tensor maps stay where the copy engine can read them: pointers into kp / global).
+    SharedBlock &blk = shared_block();
     for (int i = threadIdx.x; i < (int)(sizeof(FwdParams) / 4); i += blockDim.x)
-        reinterpret_cast<uint32_t *>(psm)[i] = reinterpret_cast<const uint32_t *>(&kp)[i];
+        reinterpret_cast<uint32_t *>(blk.params)[i] = reinterpret_cast<const uint32_t *>(&kp)[i];
     __syncthreads();
-    if (threadIdx.x == 0) psm->tm_kv_ptr = &kp.tm_kv;
-    const FwdParams &p = *psm;  // (visible to everyone after the barrier below)
-    constexpr int kRp = NT * 8;
-    constexpr int kXBytes = 2 * kRp * kTileK * 2;  // operand tile (hi and lo rows), then the weight tile
-    constexpr int kStageBytes = kXBytes + kWTileBytesP;
-    const int S = p.stages, S1 = p.stages_lo;
-    uint8_t *ring = smem;
-    uint8_t *attn_scratch = smem + p.attn_smem_off;
-    uint64_t *fullW = (uint64_t *)(smem + p.bar_off);
-    uint64_t *fullX = fullW + S, *empty = fullX + S;
-    uint64_t *accFull = empty + S, *accEmpty = accFull + 2, *mmaDone = accEmpty + 2;
-    uint32_t *tmem_slot = (uint32_t *)(mmaDone + 1);
-    Shared *sh = (Shared *)(((uintptr_t)(mmaDone + 4) + 15) & ~(uintptr_t)15);
-    double *red = (double *)(sh + 1);
-    float *epi_tile = (float *)(red + 16);
-    uint64_t *abar = (uint64_t *)(epi_tile + 8 * kEpiPitch + 4);  // the tensor-core attention's barriers and counts
-    uint32_t *acnt = (uint32_t *)(abar + AB_COUNT);
-    RingPos *role_rp = (RingPos *)(acnt + AB_COUNT);  // the same places smem_map() gives
-    int *role_seg = (int *)(role_rp + 2);
-    int *seq_tab = smem_map(kp, smem).seq;
-    const float **ltab = smem_map(kp, smem).ltab;
+    if (threadIdx.x == 0) params_copy().tm_kv_ptr = &kp.tm_kv;
     if (kp.n_layers <= kMaxStagedLayers) {  // the layers' gain / bias pointers and the final norm's
         for (int i = threadIdx.x; i < 8 * kp.n_layers + 2; i += blockDim.x) {
             const int l = i >> 3, k = i & 7;
-            ltab[i] = l < kp.n_layers ? (&layer_desc(kp.md, l)->ln1_g)[k] : (k == 0 ? kp.md->lnf_g : kp.md->lnf_b);
+            blk.ltab[i] = l < kp.n_layers ? (&layer_desc(kp.md, l)->ln1_g)[k] : (k == 0 ? kp.md->lnf_g : kp.md->lnf_b);
         }
     }
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (warp == 0) {  // tensor memory for the accumulators; released by the same warp at the end
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&blk.tmem_slot)),
                      "n"(kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) {
-            mbar_init(&fullW[s], 1);
-            mbar_init(&fullX[s], 1);
-            mbar_init(&empty[s], 1);  // one tcgen05.commit per stage
+        for (int s = 0; s < kp.stages; ++s) {
+            mbar_init(&blk.fullW[s], 1);
+            mbar_init(&blk.fullX[s], 1);
+            mbar_init(&blk.empty[s], 1);  // one tcgen05.commit per stage
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(&accFull[b], 1);
-            mbar_init(&accEmpty[b], kEpiWarps);
+            mbar_init(&blk.accFull[b], 1);
+            mbar_init(&blk.accEmpty[b], kEpiWarps);
         }
-        mbar_init(mmaDone, 1);
+        mbar_init(&blk.mmaDone, 1);
         for (int i = 0; i < AB_COUNT; ++i) {
-            mbar_init(&abar[i], i == AB_P_READY ? 128 : i == AB_FIXED ? 64 : 1);  // landed: the MMA issuer alone
-            acnt[i] = 0;
+            mbar_init(&blk.abar[i], i == AB_P_READY ? 128 : i == AB_FIXED ? 64 : 1);  // landed: the MMA issuer alone
+            blk.acnt[i] = 0;
         }
-        role_rp[0] = RingPos();
-        role_rp[1] = RingPos();
-        for (int i = 0; i < 8; ++i) role_seg[i] = 0;
+        blk.role_rp[0] = RingPos();
+        blk.role_rp[1] = RingPos();
+        for (int i = 0; i < 8; ++i) blk.role_seg[i] = 0;
+        Shared *sh = &blk.state;
         sh->released = 0;
         sh->abort = 0;
         sh->go = 1;
+        sh->epoch = 0;
         sh->wait_limit = kp.wait_cycles > 0 ? kp.wait_cycles : kWaitCycles;
-        sh->attn_bar_off = (uint32_t)((uint8_t *)abar - (uint8_t *)sh);
-        sh->seq_off = (uint32_t)((uint8_t *)seq_tab - (uint8_t *)sh);
-        sh->ltab_off = kp.n_layers <= kMaxStagedLayers ? (uint32_t)((uint8_t *)ltab - (uint8_t *)sh) : 0u;
+        sh->ltab_staged = kp.n_layers <= kMaxStagedLayers;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    if (threadIdx.x == 0) sh->tmem_base = tmem_base;  // read after the next barrier only
-    const int NG = n_gemms(p);
+    if (threadIdx.x == 0) blk.state.tmem_base = blk.tmem_slot;  // read after the next barrier only
 
     if (warp == kConsumerWarps) {
-        // =============================== producer ===============================
-        // Weights never change, so this cursor runs as far ahead as the ring allows, across grid
-        // barriers.  The loop is kept minimal (no divisions, no clock reads while it makes progress):
-        // its rate bounds the weight stream.
-        if (lane == 0) {
-            RingPos rp;
-            bool failed = false;
-            int seen_release = 0;
-            // a CTA that never runs an attention item (fewer items than CTAs) never uses the scratch: its
-            // upper slots take weights at any time
-            const bool scratch_used = (int)blockIdx.x < p.B * p.H * p.n_split * ((p.M + kAttnRows - 1) / kAttnRows);
-            for (int gws = 0; gws < NG * p.n_steps && !failed; ++gws) {
-                const int gw = ((gws / NG) << kStepShift) | (gws % NG);
-                const GemmDesc dw = gemm_desc(p, gw);
-                int c0, c1;
-                unit_range(p, dw, c0, c1);
-                if (c0 >= c1) continue;
-                int tw = c0 / dw.kchunks, kw = c0 % dw.kchunks;
-                for (int c = c0; c < c1; ++c) {
-                    uint32_t ph;
-                    const int s = ring_next(rp, ring_lo_only(dw, c - c0, S1), S, S1, ph);
-                    if (s >= S1 && scratch_used && seen_release < dw.need_hi) {  // slot shared with the attention scratch
-                        const long long t0 = clock64();
-                        while ((seen_release = sh->released) < dw.need_hi) {
-                            if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
-                        }
-                        if (failed) { rp.par ^= 1u << s; break; }  // nothing was issued into s
-                    }
-                    if (!mbar_test_wait(&empty[s], ph ^ 1u)) {
-                        const long long t0 = clock64();
-                        while (!mbar_test_wait(&empty[s], ph ^ 1u)) {
-                            if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
-                        }
-                        if (failed) { rp.par ^= 1u << s; break; }  // nothing was issued into s
-                    }
-                    mbar_expect_tx(&fullW[s], kWTileBytesP);
-                    tma_load_2d(ring + (size_t)s * kStageBytes + kXBytes, dw.tmW, kw * kTileK, tw * kTileNP, &fullW[s]);
-                    if (++kw == dw.kchunks) { kw = 0; ++tw; }
-                }
-            }
-            if (failed) {
-                set_status(p.status, kTimeoutCode);
-                sh->abort = 1;
-            }
-            // error path only: wait (bounded) for copies still in flight before the CTA may exit
-            if (sh->abort)
-                for (int s = 0; s < S; ++s)
-                    if ((rp.used >> s) & 1u) mbar_wait(&fullW[s], ((rp.par >> s) & 1u) ^ 1u);
-        }
+        producer_program<NT>();
     } else {
         // =============================== work warps ===============================
-        int epoch = 0;  // grid barriers passed
-
-        if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            p.trace[0] = t;
-        }
-        // ---- phase program (the same structure gemm_desc() encodes) ----
-        // `go` is uniform over the work threads (taken inside the grid barrier), so every named barrier
-        // below is reached by all of them or by none.
-        auto norm_for_layer = [&](int l) {  // operand(s) of layer l's first GEMM(s), or of the LM head
-            if (l < p.n_layers) {
-                const float *const *lt = staged_ltab(sh);
-                const LayerDesc *ld = layer_desc(p.md, l);
-                const float *g1 = lt ? lt[8 * l + 0] : ld->ln1_g, *b1 = lt ? lt[8 * l + 1] : ld->ln1_b;
-                if (p.parallel)
-                    norm_phase(p, g1, b1, OP_XN1, lt ? lt[8 * l + 4] : ld->ln2_g, lt ? lt[8 * l + 5] : ld->ln2_b, OP_XN2, red);
-                else norm_phase(p, g1, b1, OP_XN1, nullptr, nullptr, 0, red);
-                grid_zero(p.qkv, p.R, 3 * p.d, 3 * p.d);
-                if (p.parallel) grid_zero(p.t_in, p.R, p.d_in, p.d_in);
-            } else if (p.want_logits) {
-                const float *const *lt = staged_ltab(sh);
-                norm_phase(p, lt ? lt[8 * p.n_layers] : p.md->lnf_g, lt ? lt[8 * p.n_layers + 1] : p.md->lnf_b, OP_XN1, nullptr,
-                           nullptr, 0, red);
-                grid_zero(p.logits, p.R, p.V, p.V);
-            }
-        };
-        if (p.tail && blockIdx.x == 0)  // the draws' meeting places: smallest hit index / largest index with weight
-            for (int i = threadIdx.x; i < p.n_steps * p.B * 2; i += kWorkThreads) p.tail_hit[i] = (i & 1) ? -1 : 0x7fffffff;
-        bool go = true;
-        for (int step = 0; step < p.n_steps && go; ++step) {
-            const int gs = step << kStepShift;
-            if (step > 0) {  // the rows of this step: one per sequence, the token the step before drew
-                if (threadIdx.x == 0) psm->cur_step = step;
-                named_bar(2, kWorkThreads);
-            }
-            // Set-up, embedding and the first norm of a row all run on the CTA that owns the row, so only
-            // CTA-wide barriers separate them: one grid barrier in front of the first GEMM instead of two.
-            setup_phase(p);
-            named_bar(2, kWorkThreads);  // the row's position and validity are read back by the embedding
-            embed_phase(p);
-            named_bar(2, kWorkThreads);  // the embedding rows are read back by the norm
-            norm_for_layer(0);
-            go = grid_sync(p, sh, epoch);
-            if (go && threadIdx.x < 64) {  // lengths and rows of this pass (written by the set-up of every row), for the
-                const int b = threadIdx.x;  // attention items, which run behind further grid barriers
-                seq_tab[b] = b < p.B ? __ldcg(p.len + b) : 0;
-                seq_tab[64 + b] = b < p.B ? __ldcg(p.ri.n_eff + b) : 0;
-            }
-            for (int l = 0; l < p.n_layers && go; ++l) {
-                run_gemm<NT>(p, gs | (4 * l + 0), smem);                  // qkv
-                if (p.parallel) run_gemm<NT>(p, gs | (4 * l + 1), smem);       // MLP in (same block input)
-                if (!(go = grid_sync(p, sh, epoch))) break;
-                if (overlap_mlp_out(p)) {
-                    act_phase(p);
-                    if ((int)blockIdx.x < attention_ctas(p)) {
-                        grid_arrive(p, sh, epoch);  // the activation is out; attention needs nothing from the others
-                        attention_phase(p, l, attn_scratch, sh);
-                        attn_signal(p, sh);
-                    } else {
-                        if (!(go = grid_sync(p, sh, epoch))) break;
-                        run_gemm<NT>(p, gs | (4 * l + 2), smem);               // MLP out -> x, beside the attention items
-                        run_gemm<NT>(p, gs | (4 * l + 3), smem);               // out-proj -> x, once the attention CTAs have signalled
-                    }
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                } else if (p.parallel) {
-                    attention_phase(p, l, attn_scratch, sh);
-                    act_phase(p);
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    run_gemm<NT>(p, gs | (4 * l + 2), smem);                   // out-proj -> x
-                    run_gemm<NT>(p, gs | (4 * l + 3), smem);                   // MLP out  -> x
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                } else {
-                    attention_phase(p, l, attn_scratch, sh);
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    run_gemm<NT>(p, gs | (4 * l + 1), smem);                   // out-proj -> x
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    const float *const *lt = staged_ltab(sh);
-                    const LayerDesc *ld = layer_desc(p.md, l);
-                    norm_phase(p, lt ? lt[8 * l + 4] : ld->ln2_g, lt ? lt[8 * l + 5] : ld->ln2_b, OP_XN1, nullptr, nullptr, 0, red);
-                    grid_zero(p.t_in, p.R, p.d_in, p.d_in);
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    run_gemm<NT>(p, gs | (4 * l + 2), smem);                   // MLP in
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    act_phase(p);
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                    run_gemm<NT>(p, gs | (4 * l + 3), smem);                   // MLP out -> x
-                    if (!(go = grid_sync(p, sh, epoch))) break;
-                }
-                norm_for_layer(l + 1);
-                if (!(go = grid_sync(p, sh, epoch))) break;
-            }
-            if (go && p.want_logits) run_gemm<NT>(p, gs | (4 * p.n_layers), smem);
-            if (go && p.tail) {  // q, the draw and the commit of this step (see tail_partial)
-                if (!(go = grid_sync(p, sh, epoch))) break;
-                tail_partial(p, sh);
-                if (!(go = grid_sync(p, sh, epoch))) break;
-                tail_q(p, sh);
-                if (!(go = grid_sync(p, sh, epoch))) break;
-                tail_draw(p);
-                if (!(go = grid_sync(p, sh, epoch))) break;
-                tail_commit(p);
-                if (!(go = grid_sync(p, sh, epoch))) break;
-            }
-        }
-        if (go && p.tail && p.mailbox && blockIdx.x == 0 && (int)threadIdx.x < p.B)  // the host's length bound follows (see report_len)
-            *reinterpret_cast<volatile unsigned long long *>(p.mailbox + threadIdx.x) =
-                ((unsigned long long)p.mb_seq << 32) | (unsigned)__ldcg(p.len_rw + threadIdx.x);
-        if (p.trace && blockIdx.x == 0 && threadIdx.x == 0) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            p.trace[epoch + 1] = t;
-            p.trace[epoch + 2] = 0;
-        }
-        if (warp == kXWarp && lane == 0 && sh->abort) {  // error path only: copies still in flight
-            const RingPos rp = role_rp[1];
-            for (int s = 0; s < S; ++s)
-                if ((rp.used >> s) & 1u) mbar_wait(&fullX[s], ((rp.par >> s) & 1u) ^ 1u);
+        work_program<NT, WIDE>();
+        if (warp == kXWarp && lane == 0 && blk.state.abort) {  // error path only: copies still in flight
+            const RingPos rp = blk.role_rp[1];
+            for (int s = 0; s < kp.stages; ++s)
+                if ((rp.used >> s) & 1u) mbar_wait(&blk.fullX[s], ((rp.par >> s) & 1u) ^ 1u);
         }
         if (warp == kMmaWarp) {  // nothing of this CTA may still be running on the tensor core
             if (lane == 0) {
-                tc_commit(mmaDone);
-                mbar_wait(mmaDone, 0);
+                tc_commit(&blk.mmaDone);
+                mbar_wait(&blk.mmaDone, 0);
             }
             __syncwarp();
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) leave_grid(p.gbar);
+    if (threadIdx.x == 0) leave_grid(kp.gbar);
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(blk.tmem_slot), "n"(kTmemCols) : "memory");
     }
 }
 

@@ -512,14 +512,12 @@ int run_attention(const ssd_model *m, ssd_kv *kv, int layer, const float *q, int
 
 inline int barriers_needed(const ssd_arch &a) { return (a.parallel_residual ? 5 : 8) * a.n_layers; }  // upper bound
 
-template <int NT>
+template <int NT, bool WIDE>
 int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStream_t st) {
     constexpr size_t stage = kWTileBytesP + 2 * NT * 8 * kTileK * 2;
-    size_t attn = align_up(attn_scratch_bytes(p.Dh), 128);
-    if (p.attn_tc == 1 && attn < (size_t)kTcScratchBytes) attn = kTcScratchBytes;
-    if (p.attn_tc == 2) attn = m8_scratch_bytes(p.Dh);
-    const size_t tail = 24 * 32 + 64 + 16 + sizeof(Shared) + 16 * sizeof(double) + kEpiBytes + 256;  // barriers, small state, epilogue tile
-    const size_t total = (size_t)kSmemBudget - 1024 - tail;
+    const size_t attn = WIDE ? tc_scratch_bytes(32) : p.attn_form == ATT_TC16 ? tc_scratch_bytes(16)
+                        : p.attn_form == ATT_PACKED ? m8_scratch_bytes(p.Dh) : align_up(attn_scratch_bytes(p.Dh), 128);
+    const size_t total = (size_t)kSmemBudget - 1024 - sizeof(SharedBlock);
     // upper slots share their bytes with the attention scratch; two slots never do where they fit
     // (one with the 48 KB stages of 64 rows, which only the prompt pass uses)
     size_t S2 = (attn + stage - 1) / stage;
@@ -534,13 +532,13 @@ int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStr
     p.stages = (int)(S1 + S2);
     p.stages_lo = (int)S1;
     p.attn_smem_off = (int)(S1 * stage);
-    p.bar_off = (int)align_up(S1 * stage + region2, 128);
-    const size_t smem = 1024 + (size_t)p.bar_off + tail;
+    const size_t smem = 1024 + S1 * stage + region2;
     static bool attr[64] = {false};  // the attribute belongs to the device's copy of the kernel
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SSD_E_CUDA;
     if (!attr[dev]) {
-        if (cudaFuncSetAttribute(forward_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget) !=
+        if (cudaFuncSetAttribute(forward_kernel<NT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kSmemBudget - (int)sizeof(SharedBlock)) !=
             cudaSuccess)
             return SSD_E_CUDA;
         attr[dev] = true;
@@ -571,23 +569,32 @@ int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStr
     }
     cfg.attrs = attrs;
     cfg.numAttrs = na;
-    if (cudaLaunchKernelExC(&cfg, (const void *)forward_kernel<NT>, args) != cudaSuccess) return SSD_E_CUDA;
+    if (cudaLaunchKernelExC(&cfg, (const void *)forward_kernel<NT, WIDE>, args) != cudaSuccess) return SSD_E_CUDA;
     g_launches.fetch_add(1, std::memory_order_relaxed);
     return SSD_OK;
 }
 
+template <int NT>
+int launch_forward_att(const FwdParams &p, const void *ws_base, size_t ws_bytes, cudaStream_t st) {
+    if (p.attn_form != ATT_TC32) return launch_forward_nt<NT, false>(p, ws_base, ws_bytes, st);
+    if constexpr (NT >= 3) return launch_forward_nt<NT, true>(p, ws_base, ws_bytes, st);  // (17 rows of a sequence and more)
+    return SSD_E_CAPACITY;
+}
 int launch_forward_rows(const FwdParams &p, int rows_k, const void *ws_base, size_t ws_bytes, cudaStream_t st) {
     switch (rows_k / 8) {
-        case 1: return launch_forward_nt<1>(p, ws_base, ws_bytes, st);
-        case 2: return launch_forward_nt<2>(p, ws_base, ws_bytes, st);
-        case 3: return launch_forward_nt<3>(p, ws_base, ws_bytes, st);
-        case 4: return launch_forward_nt<4>(p, ws_base, ws_bytes, st);
-        case 5: return launch_forward_nt<5>(p, ws_base, ws_bytes, st);
-        case 8: return launch_forward_nt<8>(p, ws_base, ws_bytes, st);
+        case 1: return launch_forward_att<1>(p, ws_base, ws_bytes, st);
+        case 2: return launch_forward_att<2>(p, ws_base, ws_bytes, st);
+        case 3: return launch_forward_att<3>(p, ws_base, ws_bytes, st);
+        case 4: return launch_forward_att<4>(p, ws_base, ws_bytes, st);
+        case 5: return launch_forward_att<5>(p, ws_base, ws_bytes, st);
+        case 8: return launch_forward_att<8>(p, ws_base, ws_bytes, st);
         default: break;
     }
     return SSD_E_CAPACITY;
 }
+
+// From this many positions per split the tensor-core items are the faster form for passes of more than eight rows.
+constexpr int kTcMinChunk = 1024;
 
 // The whole forward as one cooperative launch (bf16 models).
 int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int M, const int32_t *n_rows,
@@ -619,27 +626,28 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
     p.gbar = kv->gbar; p.tickets = w.tickets;
     int ctx = kv_bound(kv) + M;
     if (ctx > kv->S) ctx = kv->S;
-    // Tensor-core attention items stream 128 positions per ~2 us but cost ~8 us more to start than the
-    // warp-MMA items (64 positions per ~2 us): they pay off from about a thousand positions per split.
-    const int groups = kv->B * a.n_heads * ((M + 15) / 16);
-    p.attn_tc = 0;
+    // The form of the attention items: passes of at most eight rows per sequence (draft steps, decode steps, verification with
+    // K <= 7) take the items that carry hi and lo in one MMA tile; longer ones the tensor-core items where the splits are long
+    // enough for their start (head dimension 128), else the 16-row tiles on warp-level MMAs.
+    const int streams = kv->B * a.n_heads, tiles = streams * ((M + 15) / 16);
     p.kv_rows_per_layer = kv->B * 2 * a.n_heads * kv->S;
-    // Passes of at most eight rows per sequence (draft steps, decode steps, verification with K <= 7): the warp-MMA
-    // items that carry hi and lo in one tile.
-    const bool packed_form = M <= kM8Rows && (a.head_dim == 64 || a.head_dim == 128) && (g_attn_mode == 0 || g_attn_mode == 3);
-    if (packed_form) {
-        plan_split(groups, ctx, &p.chunk, &p.n_split, kAttnTile);
-        p.attn_tc = 2;
-    } else if (a.head_dim == 128 && kv->tm_rows_ok && g_attn_mode != 1 && g_attn_mode != 3) {
-        plan_split(groups, ctx, &p.chunk, &p.n_split, kTcChunk);
-        if (p.chunk >= 1024 || g_attn_mode == 2) {
-            p.attn_tc = 1;
-            p.tm_kv = kv->tm_rows;
-        }
+    int items_per_split = streams;
+    plan_split(streams, ctx, &p.chunk, &p.n_split, kTcChunk);
+    const bool tc_ok = a.head_dim == 128 && kv->tm_rows_ok && g_attn_mode != 1 && g_attn_mode != 3;
+    if (M <= kM8Rows && (a.head_dim == 64 || a.head_dim == 128) && (g_attn_mode == 0 || g_attn_mode == 3)) {
+        plan_split(streams, ctx, &p.chunk, &p.n_split, kAttnTile);
+        p.attn_form = ATT_PACKED;
+    } else if (tc_ok && (p.chunk >= kTcMinChunk || g_attn_mode == 2)) {
+        p.attn_form = M > 16 ? ATT_TC32 : ATT_TC16;
+        p.tm_kv = kv->tm_rows;
+    } else {
+        plan_split(tiles, ctx, &p.chunk, &p.n_split, kAttnTile);
+        p.attn_form = ATT_MMA;
+        items_per_split = tiles;
     }
-    if (!p.attn_tc) plan_split(groups, ctx, &p.chunk, &p.n_split, kAttnTile);
     {
-        const int items = groups * p.n_split, sms = g_num_sms > 0 ? g_num_sms : 148;
+        const int items = items_per_split * p.n_split, sms = g_num_sms > 0 ? g_num_sms : 148;
+        p.attn_items = items;
         p.attn_ctas = items < sms ? items : sms;
         p.overlap_out = (a.parallel_residual && 2 * p.attn_ctas <= sms) ? 1 : 0;
     }
