@@ -2165,6 +2165,7 @@ __device__ __noinline__ void producer_program() {
                     const long long t0 = clock64();
                     while ((seen_release = sh->released) < dw.need_hi) {
                         if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
+                        __nanosleep(100);  // (a tight poll takes issue slots and shared-memory cycles from the attention loop)
                     }
                     if (failed) { rp.par ^= 1u << s; break; }  // nothing was issued into s
                 }
