@@ -1285,6 +1285,18 @@ __device__ __forceinline__ void tc_ld_32(uint32_t taddr, float (&v)[32]) {
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+// 64 consecutive columns of this thread's lane in one round trip
+__device__ __forceinline__ void tc_ld_64(uint32_t taddr, float (&v)[64]) {
+    uint32_t r[64];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]), "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
+        : "r"(taddr)
+        : "memory");
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+}
 // eight columns from each of two places of this warp's lane quadrant, one round trip
 __device__ __forceinline__ void tc_ld_2x8(uint32_t ta, uint32_t tb, float (&a)[8], float (&b)[8]) {
     uint32_t r[16];
@@ -1334,6 +1346,13 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo, uint
 }
 // byte offset of (row, 16-byte chunk c) in a tile of 128-byte rows with the 128-byte swizzle
 __device__ __forceinline__ uint32_t sw128(int row, int c) { return (uint32_t)(row * 128 + ((c ^ (row & 7)) << 4)); }
+
+// 2^x by the special-function unit (results below 2^-126, which the references keep 2^-94 below a row's largest, become 0)
+__device__ __forceinline__ float exp2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 
 // (all of the first 128 threads) true in all of them if `mine` is true in any
 __device__ __forceinline__ bool softmax_vote(bool mine) {
@@ -1568,31 +1587,23 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             const uint32_t tSc = tS + 2 * RP * (c & 1) + lane_sel;
             wait(&s_full[c & 1], s_par(c));
             tc_fence_after();
-            // (the scores are read from tensor memory again for each use: a block of eight rows at a time in registers)
-            auto scores = [&](int blk, float (&v)[8]) {
-                float lo[8];
-                tc_ld_2x8(tSc + 8 * blk, tSc + RP + 8 * blk, v, lo);
-#pragma unroll
-                for (int i = 0; i < 8; ++i) v[i] = 8 * blk + i >= first ? v[i] + lo[i] : -INFINITY;
-            };
+            // all rows' scores in one tensor-memory round trip (they take 0.3 - 0.5 us each), kept in registers
+            float v[2 * RP];
+            if constexpr (RP == 16) tc_ld_32(tSc, v);
+            else tc_ld_64(tSc, v);
             bool over = false;
-#pragma unroll 1
-            for (int blk = 0; 8 * blk < rows_here; ++blk) {
-                float v[8];
-                scores(blk, v);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) over = over || (8 * blk + i < rows_here && v[i] > m_ref[8 * blk + i] + kTcMaxSlack);
+            for (int r = 0; r < RP; ++r) {
+                v[r] = r >= first ? v[r] + v[RP + r] : -INFINITY;
+                if (r % 4 == 0 && r >= rows_here) break;  // (rows in fours: the queries beyond rows_here are zeros)
+                over = over || (r < rows_here && v[r] > m_ref[r] + kTcMaxSlack);
             }
             if (softmax_vote(over)) {  // rare, and the first chunk: raise the references that are passed
-#pragma unroll 1
-                for (int blk = 0; 8 * blk < rows_here; ++blk) {
-                    float v[8];
-                    scores(blk, v);
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const float mx = warp_max(v[i]);
-                        if (lane == 0) wmax[warp * RP + 8 * blk + i] = mx;
-                    }
+                for (int r = 0; r < RP; ++r) {
+                    if (r >= rows_here) break;
+                    const float mx = warp_max(v[r]);
+                    if (lane == 0) wmax[warp * RP + r] = mx;
                 }
                 named_bar(6, 128);
                 if (tid < rows_here) {
@@ -1624,23 +1635,28 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             uint32_t panel = smem_u32(pt) + (uint32_t)((c % NP) * kQBytes + (tid >> 6) * kPanel + (tid & 7) * 2);
             uint32_t cc = (uint32_t)((tid & 63) >> 3);
             asm volatile("" : "+r"(panel), "+r"(cc));
+            // four rows' values before their stores: the stores keep the loads behind them from moving up
 #pragma unroll
-            for (int blk = 0; blk < RP / 8; ++blk) {
-                if (8 * blk < rows_here) {
-                    float v[8];
-                    scores(blk, v);
+            for (int r4 = 0; r4 < RP; r4 += 4) {
+                if (r4 >= rows_here) break;  // (rows beyond rows_here: columns nobody reads)
+                const float4 m4 = *reinterpret_cast<const float4 *>(m_ref + r4);
+                const float m[4] = {m4.x, m4.y, m4.z, m4.w};
+                __nv_bfloat16 hv[4], lv[4];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int r = 8 * blk + i;  // (rows beyond rows_here: zero queries, columns nobody reads)
-                        // (a row that has seen nothing yet: reference -inf, every score -inf)
-                        const float pv = v[i] > -INFINITY ? exp2f(v[i] - m_ref[r]) : 0.f;
-                        l[r] += pv;
-                        // P as bf16 hi + lo into the P tile: row r (hi) / RP + r (lo), column = this position
-                        const __nv_bfloat16 hv = __float2bfloat16_rn(pv), lv = __float2bfloat16_rn(pv - __bfloat162float(hv));
-                        const uint32_t at = panel + r * 128 + ((cc ^ (r & 7)) << 4);
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at), "h"(__bfloat16_as_ushort(hv)) : "memory");
-                        asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + RP * 128), "h"(__bfloat16_as_ushort(lv)) : "memory");
-                    }
+                for (int i = 0; i < 4; ++i) {
+                    // (a row that has seen nothing yet: reference -inf, every score -inf)
+                    const float pv = v[r4 + i] > -INFINITY ? exp2_approx(v[r4 + i] - m[i]) : 0.f;
+                    l[r4 + i] += pv;
+                    hv[i] = __float2bfloat16_rn(pv);
+                    lv[i] = __float2bfloat16_rn(pv - __bfloat162float(hv[i]));
+                }
+                // P as bf16 hi + lo into the P tile: row r (hi) / RP + r (lo), column = this position
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = r4 + i;
+                    const uint32_t at = panel + r * 128 + ((cc ^ (r & 7)) << 4);
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(at), "h"(__bfloat16_as_ushort(hv[i])) : "memory");
+                    asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + RP * 128), "h"(__bfloat16_as_ushort(lv[i])) : "memory");
                 }
             }
             fence_async_proxy();
