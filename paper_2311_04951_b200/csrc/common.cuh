@@ -52,6 +52,13 @@ __device__ __forceinline__ float warp_max(float v) {
     return v;
 }
 
+// max over the warp (an order-preserving map to signed integers, one reduction instruction); never of a NaN
+__device__ __forceinline__ float warp_max_redux(float v) {
+    const int b = __float_as_int(v);
+    const int m = __reduce_max_sync(0xffffffffu, b >= 0 ? b : b ^ 0x7fffffff);
+    return __int_as_float(m >= 0 ? m : m ^ 0x7fffffff);
+}
+
 // Block-wide reductions through shared scratch (>= 32 entries); every thread gets the result.
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T *scratch) {

@@ -1599,11 +1599,18 @@ __device__ __noinline__ void attention_items_tc(int layer) {
                 over = over || (r < rows_here && v[r] > m_ref[r] + kTcMaxSlack);
             }
             if (softmax_vote(over)) {  // rare, and the first chunk: raise the references that are passed
+                // (rolled, and from tensor memory again: straight-line code that runs once per item costs its instruction fetch)
+#pragma unroll 1
+                for (int blk = 0; 8 * blk < rows_here; ++blk) {
+                    float hi[8], lo[8];
+                    tc_ld_2x8(tSc + 8 * blk, tSc + RP + 8 * blk, hi, lo);
+                    float mine = -INFINITY;
 #pragma unroll
-                for (int r = 0; r < RP; ++r) {
-                    if (r >= rows_here) break;
-                    const float mx = warp_max(v[r]);
-                    if (lane == 0) wmax[warp * RP + r] = mx;
+                    for (int i = 0; i < 8; ++i) {
+                        const float mx = warp_max_redux(8 * blk + i >= first ? hi[i] + lo[i] : -INFINITY);
+                        mine = lane == i ? mx : mine;
+                    }
+                    if (lane < 8) wmax[warp * RP + 8 * blk + lane] = mine;
                 }
                 named_bar(6, 128);
                 if (tid < rows_here) {
@@ -1664,13 +1671,18 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             mbar_arrive(p_ready);
         }
         // ---- the sums over positions, then thread = head dim tid: output or partial ----
+        // (lane r of a warp ends up with row r's sum: RP - 1 exchanges instead of 5 RP)
 #pragma unroll
-        for (int r = 0; r < RP; ++r) {
-            if (r < rows_here) {
-                const float t = warp_sum(l[r]);
-                if (lane == 0) wsum[warp * RP + r] = t;
+        for (int hf = RP / 2; hf > 0; hf >>= 1) {
+            const bool up = lane & hf;
+#pragma unroll
+            for (int j = 0; j < hf; ++j) {
+                const float send = up ? l[j] : l[j + hf], keep = up ? l[j + hf] : l[j];
+                l[j] = keep + __shfl_xor_sync(0xffffffffu, send, hf);
             }
         }
+        if (RP == 16) l[0] += __shfl_xor_sync(0xffffffffu, l[0], 16);
+        if (lane < RP) wsum[warp * RP + lane] = l[0];
         if (n_chunks > 1) wait(&o_done[(n_chunks - 2) & 1], o_par(n_chunks - 2));
         if (n_chunks > 0) {
             wait(&o_done[(n_chunks - 1) & 1], o_par(n_chunks - 1));
@@ -1678,7 +1690,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
         }
         named_bar(6, 128);
         const bool direct = p.n_split == 1;
-#pragma unroll
+#pragma unroll 1
         for (int blk = 0; blk < RP / 8; ++blk) {
             if (8 * blk < rows_here) {
                 float oh[8], ol[8];

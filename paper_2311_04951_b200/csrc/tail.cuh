@@ -74,13 +74,6 @@ __device__ __forceinline__ void tail_load(const float *row, int base, int hi, fl
     }
 }
 
-// max over the warp (an order-preserving map to signed integers, one reduction instruction); never of a NaN
-__device__ __forceinline__ float warp_max_redux(float v) {
-    const int b = __float_as_int(v);
-    const int m = __reduce_max_sync(0xffffffffu, b >= 0 ? b : b ^ 0x7fffffff);
-    return __int_as_float(m >= 0 ? m : m ^ 0x7fffffff);
-}
-
 // (max, argmax, sum of exp relative to the max) of a part of a row
 struct PartStat {
     float mx;
