@@ -1249,8 +1249,8 @@ __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, boo
 // A row's softmax reference is the maximum of the first chunk it sees; it is only raised when a score passes it by more than
 // 2^32 (fp32 sums and bf16 hi + lo carry the factor without loss), which one barrier vote per chunk finds out: no maxima are
 // exchanged and O^T is not rescaled in the ordinary chunk.
-// Bound: the 64 KB of K and V a chunk fetches.  7B, 17 rows x 16384 positions: TC_OLD us a layer with two 16-row tiles that each
-// walk the cache and exchange maxima in every chunk, TC_NEW now, against 41 us of HBM time.
+// Bound: the 64 KB of K and V a chunk fetches.  7B, 17 rows x 16384 positions: 249 us a layer with two 16-row tiles that each
+// walk the cache and exchange maxima in every chunk, 97 now, against 41 us of HBM time.
 constexpr int kTcChunk = 128;
 constexpr int kTcStages = 4;  // K / V ring stages of 32 KB: the bytes in flight set the chunk rate (3 stages: 2.7 us per chunk)
 constexpr int kTcKvStage = kTcChunk * 128 * 2;  // one K or V chunk: two 64-column panels of 128 rows x 128 B
@@ -2157,7 +2157,7 @@ __device__ __noinline__ void tail_commit() {
 // ---- the kernel -----------------------------------------------------------------------------
 // The producer's walk and the work warps' phase program are functions of their own that keep next to nothing alive across
 // the calls they make: what is live there takes registers that the attention items and GEMMs want, and is spilled around every
-// one of the 130-260 calls of a pass (LIVE_NOTE).
+// one of the 130-260 calls of a pass (about a microsecond each where the line has left the little L1 there is).
 template <int NT>
 __device__ __forceinline__ constexpr int stage_x_bytes() { return 2 * NT * 8 * kTileK * 2; }
 

@@ -593,8 +593,11 @@ int launch_forward_rows(const FwdParams &p, int rows_k, const void *ws_base, siz
     return SSD_E_CAPACITY;
 }
 
-// From this many positions per split the tensor-core items are the faster form for passes of more than eight rows.
-constexpr int kTcMinChunk = 1024;
+// From this many positions per split the tensor-core items are the faster form for passes of more than eight rows: they cost
+// more to start (20 us against 12) and half as much per position (up to 16 rows; a quarter beyond, where the warp-MMA form needs
+// two row tiles).  7B layers, us, warp-MMA / tensor core: four sequences of 800 positions (one split) x 9 rows 165.1 / 163.1,
+// of 400 153.9 / 157.8; one sequence of 3200 (four splits) x 17 rows 175.4 / 165.0, of 1600 153.4 / 155.3.
+inline int tc_min_chunk(int M) { return M <= 16 ? 512 : 640; }
 
 // The whole forward as one cooperative launch (bf16 models).
 int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int M, const int32_t *n_rows,
@@ -637,7 +640,7 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
     if (M <= kM8Rows && (a.head_dim == 64 || a.head_dim == 128) && (g_attn_mode == 0 || g_attn_mode == 3)) {
         plan_split(streams, ctx, &p.chunk, &p.n_split, kAttnTile);
         p.attn_form = ATT_PACKED;
-    } else if (tc_ok && (p.chunk >= kTcMinChunk || g_attn_mode == 2)) {
+    } else if (tc_ok && (p.chunk >= tc_min_chunk(M) || g_attn_mode == 2)) {
         p.attn_form = M > 16 ? ATT_TC32 : ATT_TC16;
         p.tm_kv = kv->tm_rows;
     } else {
