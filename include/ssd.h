@@ -167,6 +167,16 @@ int kv_prefill(ssd_model *m, ssd_kv *kv, const int32_t *dev_tokens, const int32_
                void *dev_ws, size_t ws_bytes, void *stream);
 
 /*
+ * The prompt pass of a target and its draft: kv_prefill of both.  Where the draft is the target's first layers
+ * (ssd_model_share_prefix) and both caches are empty - the host's bound of every length is 0: fresh caches, or caches cut back
+ * to nothing and read with kv_lengths -, its keys and values are the target's first layers', and are copied instead of computed
+ * again.  (Section "So, what's the problem?": two models, two caches.)
+ */
+int kv_prefill_pair(ssd_model *target, ssd_kv *tkv, ssd_model *draft, ssd_kv *dkv, const int32_t *dev_tokens,
+                    const int32_t *dev_n_tokens, int max_tokens, void *dev_ws_target, size_t ws_target_bytes, void *dev_ws_draft,
+                    size_t ws_draft_bytes, void *stream);
+
+/*
  * One draft step (Section "Speculative Sampling": the small model is called a few times in a row to
  * propose tokens).  Feeds n_in[b] (1..rows_in) rows per sequence -- the tokens the draft cache has
  * not seen yet -- commits them to the draft cache, turns the LAST fed row's logits into

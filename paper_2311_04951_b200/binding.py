@@ -39,7 +39,7 @@ EXPORTS = ["ssd_model_create", "ssd_model_desc_bytes", "ssd_set_persistent", "ss
            "kv_commit", "kv_rollback", "spec_advance", "kv_lengths", "ssd_device_status",
            "verify_from_logits", "verify_from_logits_noalloc", "verify_scratch_bytes", "attention_rows", "ssd_last_logits", "ssd_set_trace", "ssd_read_trace", "ssd_launch_count",
            "ssd_gemm_profile", "ssd_gemm_profile_read", "ssd_strerror", "ssd_set_wait_limit", "ssd_wait_probe", "ssd_set_sampling", "draft_steps",
-           "ssd_prefill_workspace_bytes", "ssd_set_prefill_mode"]
+           "ssd_prefill_workspace_bytes", "ssd_set_prefill_mode", "kv_prefill_pair"]
 
 
 def lib_path() -> str:
@@ -77,6 +77,7 @@ def load():
     L.kv_destroy.argtypes = [vp]
     L.kv_destroy.restype = None
     L.kv_prefill.argtypes = [vp, vp, vp, vp, i32, vp, sz, vp]
+    L.kv_prefill_pair.argtypes = [vp, vp, vp, vp, vp, vp, i32, vp, sz, vp, sz, vp]
     L.draft_step.argtypes = [vp, vp, vp, i32, i32, vp, f32, vp, i32, vp, i32, vp, sz, vp, sz, vp]
     L.draft_steps.argtypes = [vp, vp, i32, vp, i32, i32, vp, f32, vp, i32, vp, i32, vp, sz, vp, sz, vp]
     L.target_verify.argtypes = [vp, vp, vp, i32, vp, vp, f32, vp, vp, i32, vp, vp, sz, vp]
@@ -239,6 +240,13 @@ def kv_prefill(model: Model, kv: KV, tokens: torch.Tensor, n_tokens: torch.Tenso
     assert tokens.dtype == torch.int32 and tokens.dim() == 2 and tokens.is_contiguous()
     _check(load().kv_prefill(model.h, kv.h, _p(tokens), _p(n_tokens), tokens.shape[1], _p(ws), ws.numel(), _stream()),
            "kv_prefill")
+
+
+def kv_prefill_pair(target: Model, tkv: KV, draft: Model, dkv: KV, tokens: torch.Tensor, n_tokens: torch.Tensor,
+                    ws_target: torch.Tensor, ws_draft: torch.Tensor) -> None:
+    assert tokens.dtype == torch.int32 and tokens.dim() == 2 and tokens.is_contiguous()
+    _check(load().kv_prefill_pair(target.h, tkv.h, draft.h, dkv.h, _p(tokens), _p(n_tokens), tokens.shape[1], _p(ws_target),
+                                  ws_target.numel(), _p(ws_draft), ws_draft.numel(), _stream()), "kv_prefill_pair")
 
 
 def draft_step(draft: Model, dkv: KV, tokens_in: torch.Tensor, tokens_stride: int, rows_in: int,

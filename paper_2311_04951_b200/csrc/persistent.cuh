@@ -156,7 +156,8 @@ struct GemmDesc {
     const float *bias;
 };
 
-__device__ __forceinline__ int n_gemms(const FwdParams &p) { return 4 * p.n_layers + (p.want_logits ? 1 : 0); }
+// (without logits the last layer ends with its keys and values: only its qkv projection is run)
+__device__ __forceinline__ int n_gemms(const FwdParams &p) { return p.want_logits ? 4 * p.n_layers + 1 : 4 * p.n_layers - 3; }
 // CTAs that run an attention item in a phase (each at most one when this is below the grid size).
 __device__ __forceinline__ int attention_ctas(const FwdParams &p) { return p.attn_ctas; }
 // Parallel-residual blocks with at most half of the CTAs on attention: the MLP-out GEMM depends on the
@@ -2254,8 +2255,13 @@ __device__ __noinline__ void work_program() {
         }
         for (int l = 0; l < p.n_layers && go; ++l) {
             run_gemm<NT>(gs | (4 * l + 0));                  // qkv
-            if (p.parallel) run_gemm<NT>(gs | (4 * l + 1));       // MLP in (same block input)
+            const bool kv_only = !p.want_logits && l + 1 == p.n_layers;
+            if (p.parallel && !kv_only) run_gemm<NT>(gs | (4 * l + 1));  // MLP in (same block input)
             if (!(go = grid_sync())) break;
+            if (kv_only) {
+                attention_phase<WIDE>(l);  // (its items append the rows)
+                break;
+            }
             if (overlap_mlp_out(p)) {
                 act_phase();
                 if ((int)blockIdx.x < attention_ctas(p)) {

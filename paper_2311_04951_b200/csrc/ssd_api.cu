@@ -1240,6 +1240,36 @@ int kv_prefill(ssd_model *m, ssd_kv *kv, const int32_t *dev_tokens, const int32_
     return SSD_OK;
 }
 
+// Whether `draft` is the first layers of `target` (the same tensors at the same places of the block).
+static bool is_prefix_of(const ssd_model *draft, const ssd_model *target) {
+    ssd_arch a = draft->a;
+    a.n_layers = target->a.n_layers;
+    const int n = T_L0 + PER_LAYER * draft->a.n_layers;
+    if (memcmp(&a, &target->a, sizeof(a)) != 0 || draft->a.n_layers > target->a.n_layers) return false;
+    for (int i = 0; i < n; ++i)
+        if (draft->w[i] != target->w[i]) return false;
+    return true;
+}
+
+int kv_prefill_pair(ssd_model *target, ssd_kv *tkv, ssd_model *draft, ssd_kv *dkv, const int32_t *dev_tokens,
+                    const int32_t *dev_n_tokens, int max_tokens, void *dev_ws_target, size_t ws_target_bytes, void *dev_ws_draft,
+                    size_t ws_draft_bytes, void *stream) {
+    if (!target || !tkv || !draft || !dkv || max_tokens < 0) return SSD_E_ARG;
+    const bool adopt = is_prefix_of(draft, target) && same_cache_shape(target, tkv) && same_cache_shape(draft, dkv) && tkv->B == dkv->B &&
+                       kv_bound(tkv) == 0 && kv_bound(dkv) == 0 && max_tokens <= dkv->S;
+    int rc = kv_prefill(target, tkv, dev_tokens, dev_n_tokens, max_tokens, dev_ws_target, ws_target_bytes, stream);
+    if (rc) return rc;
+    if (!adopt) return kv_prefill(draft, dkv, dev_tokens, dev_n_tokens, max_tokens, dev_ws_draft, ws_draft_bytes, stream);
+    if (max_tokens == 0) return SSD_OK;
+    cudaStream_t st = (cudaStream_t)stream;
+    const int row_bytes = (int)(draft->a.head_dim * dkv->esize);
+    LAUNCH(kv_adopt_kernel, dim3(ceil_div(max_tokens, 16), draft->a.n_heads, 2 * dkv->B * draft->a.n_layers), 256, 0, st, tkv->cache,
+           dkv->cache, tkv->len, dkv->B, tkv->S, dkv->S, row_bytes);
+    const unsigned seq = kv_note_op(dkv, max_tokens);
+    LAUNCH(kv_adopt_len_kernel, 1, 64, 0, st, tkv->len, tkv->status, dkv->len, dkv->status, dkv->B, dkv->S, dkv->mailbox_dev, seq);
+    return SSD_OK;
+}
+
 // ---- vocabulary-wide tail ----
 // A piece of a row (1 / 256 of it) is held in 1, 4 or 8 registers per lane: the smallest that the row fills, so that no slot is
 // worked on for nothing; from 65537 entries a piece is read in several steps of 8.

@@ -799,6 +799,29 @@ __global__ void kv_rollback_kernel(int32_t *len, const int32_t *new_len, int B, 
         report_len(mailbox, b, seq, v);
     }
 }
+// The cache of a layer-skip draft from its target's: both were empty and the target has been fed, so the draft's layers hold
+// the target's first layers' keys and values.  grid (16-row blocks of the longest prompt, H, 2 B layers), 16-byte pieces.
+__global__ void __launch_bounds__(256) kv_adopt_kernel(const uint8_t *src, uint8_t *dst, const int32_t *src_len, int B, int src_S,
+                                                       int dst_S, int row_bytes) {
+    const int plane = blockIdx.z, b = (plane >> 1) % B;   // plane = (layer B + b) 2 + K|V
+    const int rows = min(min(src_len[b], dst_S) - (int)blockIdx.x * 16, 16);
+    if (rows <= 0) return;
+    const size_t head = (size_t)plane * gridDim.y + blockIdx.y;
+    const uint4 *s = reinterpret_cast<const uint4 *>(src + (head * src_S + (size_t)blockIdx.x * 16) * row_bytes);
+    uint4 *d = reinterpret_cast<uint4 *>(dst + (head * dst_S + (size_t)blockIdx.x * 16) * row_bytes);
+    for (int i = threadIdx.x; i < rows * row_bytes / 16; i += 256) d[i] = s[i];
+}
+// ... and its lengths (one block of 64 threads)
+__global__ void kv_adopt_len_kernel(const int32_t *src_len, const int32_t *src_status, int32_t *len, int32_t *status, int B, int S,
+                                    unsigned long long *mailbox, unsigned seq) {
+    const int b = threadIdx.x;
+    if (b == 0 && *src_status != 0) set_status(status, *src_status);
+    if (b < B) {
+        const int v = min(src_len[b], S);
+        len[b] = v;
+        report_len(mailbox, b, seq, v);
+    }
+}
 // chunk c of a prompt pass: rows fed per sequence = clamp(n_tokens - c*C, 0, C)
 __global__ void prefill_rows_kernel(const int32_t *n_tokens, int chunk, int C, int32_t *n_rows, int B) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;

@@ -119,9 +119,14 @@ class Engine:
         if P > 1:
             body = prompts[:, :P - 1].contiguous()
             n = torch.full((self.batch,), P - 1, dtype=torch.int32, device=prompts.device)
-            B.kv_prefill(self.target, self.tkv, body, n, self._prompt_workspace(self.target, P - 1, self.ws_pre_t))
-            if self.dkv is not None:
-                B.kv_prefill(self.draft, self.dkv, body, n, self._prompt_workspace(self.draft, P - 1, self.ws_pre_d))
+            ws_t = self._prompt_workspace(self.target, P - 1, self.ws_pre_t)
+            if self.dkv is None:
+                B.kv_prefill(self.target, self.tkv, body, n, ws_t)
+            else:   # (the two passes follow one another on the stream: where the target's workspace is large enough, it serves both)
+                need = self.draft.prefill_workspace_bytes(self.batch, P - 1)
+                shared = ws_t is not self.ws_pre_t and 0 < need <= ws_t.numel()
+                ws_d = ws_t if shared else self._prompt_workspace(self.draft, P - 1, self.ws_pre_d)
+                B.kv_prefill_pair(self.target, self.tkv, self.draft, self.dkv, body, n, ws_t, ws_d)
         self.rows[:, 0] = prompts[:, P - 1]
         if self.dkv is not None:
             self.draft_in[:, 0] = prompts[:, P - 1]

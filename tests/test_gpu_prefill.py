@@ -175,3 +175,49 @@ def test_layer_skip_draft_takes_the_many_row_form(name, many_row_mode):
         assert kv.status() == 0 and kv.lengths().tolist() == n.tolist()
         caches.append(kv.cache_view().clone())
     assert torch.equal(caches[0][:arch.n_layers - 1], caches[1])
+
+
+@pytest.mark.parametrize("name,P", [("llama_bf16", 140), ("neox_bf16_h80", 140), ("neox_bf16", 21), ("gpt2_f32", 17), ("gpt2_bf16", 1)])
+def test_prompt_pass_of_a_target_and_its_layer_skip_draft(name, P):
+    """The draft's cache after the common pass is the one of a pass of its own: taken over from the target's (bit for bit) while
+    both are empty, computed when they are not (the few-row projections add their partial sums in no fixed order, so two
+    passes agree to rounding)."""
+    arch = ARCHS[name]
+    target = B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, 3, 6.0)))
+    draft = target.share_prefix(arch.n_layers - 1)
+    Bn, S, C = 3, 2 * P + 4, min(B.MAX_ROWS_PER_SEQ, B.MAX_ROWS // 3)
+    sizes = {m: max(m.prefill_workspace_bytes(Bn, P), m.workspace_bytes(Bn, C, S)) for m in (target, draft)}
+    ws = {m: B.device_buffer(n) for m, n in sizes.items()}
+    pair = {target: B.KV(target, Bn, S), draft: B.KV(draft, Bn, S + 12)}
+    alone = {target: B.KV(target, Bn, S), draft: B.KV(draft, Bn, S + 12)}
+    for seed in (36, 37):   # empty caches, then filled ones
+        prompts = torch.from_numpy(synth.gen_prompt(seed, Bn, P, arch.vocab)).cuda()
+        n = torch.tensor([P, max(P - 9, 1), 1], dtype=torch.int32, device="cuda")
+        n0 = B.launch_count()
+        B.kv_prefill_pair(target, pair[target], draft, pair[draft], prompts, n, ws[target], ws[draft])
+        n1 = B.launch_count()
+        for m in (target, draft):
+            B.kv_prefill(m, alone[m], prompts, n, ws[m])
+        if P > 1:
+            assert (n1 - n0 < B.launch_count() - n1) == (seed == 36)
+        for m in (target, draft):
+            assert pair[m].status() == 0 and pair[m].lengths().tolist() == alone[m].lengths().tolist()
+            got, ref = pair[m].cache_view(), alone[m].cache_view()
+            for b, v in enumerate(alone[m].lengths().tolist()):
+                _cache_close(arch, got[:, b, :, :, :v].float().cpu().numpy(), ref[:, b, :, :, :v].float().cpu().numpy())
+                if seed == 36:
+                    assert torch.equal(pair[draft].cache_view()[:, b, :, :, :v], pair[target].cache_view()[:-1, b, :, :, :v])
+
+
+def test_prompt_pass_of_a_target_and_a_draft_of_its_own():
+    arch = ARCHS["llama_bf16"]
+    models = [B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, s, 6.0))) for s in (3, 4)]
+    prompts = torch.from_numpy(synth.gen_prompt(38, 2, 20, arch.vocab)).cuda()
+    n = torch.tensor([20, 7], dtype=torch.int32, device="cuda")
+    ws = B.device_buffer(models[0].workspace_bytes(2, 8, 24))
+    pair, alone = [[B.KV(m, 2, 24) for m in models] for _ in range(2)]
+    B.kv_prefill_pair(models[0], pair[0], models[1], pair[1], prompts, n, ws, ws)
+    for m, kv, got in zip(models, alone, pair):
+        B.kv_prefill(m, kv, prompts, n, ws)
+        assert got.lengths().tolist() == kv.lengths().tolist() == [20, 7]
+        _cache_close(arch, *(k.cache_view()[:, 0, :, :, :20].float().cpu().numpy() for k in (got, kv)))
