@@ -34,6 +34,19 @@ constexpr int kPfStageBytes = 2 * kPfABytes + kPfWBytes;    // 64 KB
 constexpr int kPfThreads = 192;
 constexpr size_t kPfSmem = 1024 + (size_t)kPfStages * kPfStageBytes + 256;  // + barriers, TMEM slot, abort flag
 
+// eight values as bf16 hi + lo, 16 bytes each
+__device__ __forceinline__ void split_hilo8(const float (&y)[8], uint4 &hi, uint4 &lo) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 hv = __floats2bfloat162_rn(y[2 * i], y[2 * i + 1]);
+        h[i] = *reinterpret_cast<const uint32_t *>(&hv);
+        l[i] = pack_bf16x2(y[2 * i] - __low2float(hv), y[2 * i + 1] - __high2float(hv));
+    }
+    hi = make_uint4(h[0], h[1], h[2], h[3]);
+    lo = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
 struct PfGemmArgs {
     float *out;         // [R, ldo] fp32
     const float *bias;  // [N] or null
@@ -310,13 +323,74 @@ __global__ void __launch_bounds__(256) prefill_act_kernel(const float *__restric
     store_hilo4(hi, lo, (size_t)r * F + i, y);
 }
 
+// Rotary, the cache append and the attention kernels' queries: eight columns of one row's q, k or v per thread (16-byte loads
+// and stores).  Keys and values go to the cache in its bf16, queries - scaled to log2 units - become a bf16 hi / lo operand.
+// grid (ceil(3 d / 8 / 256), rows).
+// Memory-bound: 8184 rows x 7680, 419 MB: 121 us a column per thread, 91 so.
+struct PfAppendArgs {
+    const float *qkv;                // [R, 3 d]
+    __nv_bfloat16 *q_hi, *q_lo;      // [R, d]
+    __nv_bfloat16 *cache;            // this layer's slab [B][2][H][S][Dh]
+    int d, H, Dh, S, rotary_dim;
+    float q_scale;
+    RowInfo ri;
+};
+__device__ __forceinline__ void load8(const float *p, float (&v)[8]) {  // p 16-byte aligned
+    const float4 u = *reinterpret_cast<const float4 *>(p), w = *reinterpret_cast<const float4 *>(p + 4);
+    v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
+    v[4] = w.x; v[5] = w.y; v[6] = w.z; v[7] = w.w;
+}
+__global__ void __launch_bounds__(256) prefill_append_kernel(const PfAppendArgs a) {
+    const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 8;
+    if (c >= 3 * a.d) return;
+    const int which = c >= 2 * a.d ? 2 : c >= a.d ? 1 : 0, col = c - which * a.d, h = col / a.Dh, e = col % a.Dh;
+    const float *src = a.qkv + (size_t)r * 3 * a.d + c;
+    float x[8];
+    load8(src, x);
+    if (which < 2 && e < a.rotary_dim) {
+        const int half = a.rotary_dim >> 1;
+        const float *cos_r = a.ri.rope_cos + (size_t)r * half, *sin_r = a.ri.rope_sin + (size_t)r * half;
+        if ((half & 7) == 0) {  // the eight columns lie on one side of the split, their partners are eight columns too
+            const bool low = e < half;
+            const int j = low ? e : e - half;
+            float o[8], cs[8], sn[8];
+            load8(low ? src + half : src - half, o);
+            load8(cos_r + j, cs);
+            load8(sin_r + j, sn);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = low ? x[i] * cs[i] - o[i] * sn[i] : o[i] * sn[i] + x[i] * cs[i];
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (e + i >= a.rotary_dim) break;
+                const bool low = e + i < half;
+                const int j = low ? e + i : e + i - half;
+                const float o = low ? src[i + half] : src[i - half];
+                x[i] = low ? x[i] * cos_r[j] - o * sin_r[j] : o * sin_r[j] + x[i] * cos_r[j];
+            }
+        }
+    }
+    if (which == 0) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] *= a.q_scale;
+        uint4 hi, lo;
+        split_hilo8(x, hi, lo);
+        *reinterpret_cast<uint4 *>(a.q_hi + (size_t)r * a.d + col) = hi;
+        *reinterpret_cast<uint4 *>(a.q_lo + (size_t)r * a.d + col) = lo;
+    } else if (a.ri.valid[r]) {
+        const size_t plane = ((size_t)a.ri.seq[r] * 2 + (which - 1)) * a.H + h;
+        *reinterpret_cast<uint4 *>(a.cache + (plane * a.S + a.ri.pos[r]) * a.Dh + e) =
+            make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]), pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
+    }
+}
+
 // prefill_attn_kernel: causal attention of 64 query rows of one (sequence, head) over the cache, which already
 // holds this pass's keys / values (the append kernel has run).  Four warps of 16 rows each; K / V chunks of 64
 // positions go through two cp.async buffers shared by the four warps; per warp and chunk
 //   S [16 x 64] = Q (bf16 hi + lo) K^T,   running max / sum in registers (base-2 exponentials),
 //   O [16 x Dh] += P (bf16 hi + lo) V,
-// on mma.sync tiles (m16n8k16): the projections carry ~95 % of a prompt pass's arithmetic, so this step stays on
-// the warp-level path.  Row m of the sequence sees positions <= len + m.  The result goes to the out-projection
+// on mma.sync tiles (m16n8k16).  Taken for caches of 2^31 (layer, sequence, K | V, head, position) rows or more, which the
+// tensor-core form's map cannot address.  Row m of the sequence sees positions <= len + m.  The result goes to the out-projection
 // operand as bf16 hi + lo, row-major; rows that are not fed get zeros.
 constexpr int kPaRows = 64, kPaThreads = 128, kPaChunk = 64;
 inline size_t prefill_attn_smem(int Dh) {
@@ -324,13 +398,12 @@ inline size_t prefill_attn_smem(int Dh) {
 }
 
 struct PfAttnArgs {
-    const float *q;              // [B * M, d] position-encoded queries
+    const __nv_bfloat16 *q_hi, *q_lo;  // [B * M, d] position-encoded queries, in log2 units
     const __nv_bfloat16 *cache;  // this layer's slab [B][2][H][S][Dh]
     const int32_t *len;          // [B] committed lengths
     const int32_t *n_eff;        // [B] rows fed per sequence
     __nv_bfloat16 *out_hi, *out_lo;  // [B * M, d]
     int M, H, Dh, S, d;
-    float scale;
 };
 
 __global__ void __launch_bounds__(kPaThreads) prefill_attn_kernel(const PfAttnArgs a) {
@@ -348,7 +421,6 @@ __global__ void __launch_bounds__(kPaThreads) prefill_attn_kernel(const PfAttnAr
     const int rows_fed = max(0, min(kPaRows, n - m_base));
     const int p_end = rows_fed > 0 ? min(len + m_base + rows_fed, a.S) : 0;  // positions any row of this tile sees
     const int n_chunks = (p_end + kPaChunk - 1) / kPaChunk;
-    const float sc = a.scale * 1.4426950408889634f;
     const __nv_bfloat16 *kc = a.cache + ((size_t)(b * 2) * a.H + h) * a.S * Dh;
     const __nv_bfloat16 *vc = kc + (size_t)a.H * a.S * Dh;
 
@@ -369,25 +441,17 @@ __global__ void __launch_bounds__(kPaThreads) prefill_attn_kernel(const PfAttnAr
         cp_async_commit();
     };
     if (n_chunks > 0) load_chunk(0);
-    // Q rows of this tile as bf16 hi / lo
+    // Q rows of this tile
     for (int i = tid; i < kPaRows * vpr; i += kPaThreads) {
         const int ml = i / vpr, v8 = i % vpr, m = m_base + ml;
-        float qv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) qv[u] = 0.f;
+        uint4 hv = make_uint4(0, 0, 0, 0), lv = hv;
         if (m < n) {
-            const float *src = a.q + (size_t)(r0 + m) * a.d + h * Dh + v8 * 8;
-            const float4 x0 = *reinterpret_cast<const float4 *>(src), x1 = *reinterpret_cast<const float4 *>(src + 4);
-            qv[0] = x0.x; qv[1] = x0.y; qv[2] = x0.z; qv[3] = x0.w; qv[4] = x1.x; qv[5] = x1.y; qv[6] = x1.z; qv[7] = x1.w;
+            const size_t off = (size_t)(r0 + m) * a.d + h * Dh + v8 * 8;
+            hv = *reinterpret_cast<const uint4 *>(a.q_hi + off);
+            lv = *reinterpret_cast<const uint4 *>(a.q_lo + off);
         }
-        __nv_bfloat16 hq[8], lq[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            hq[u] = __float2bfloat16_rn(qv[u]);
-            lq[u] = __float2bfloat16_rn(qv[u] - __bfloat162float(hq[u]));
-        }
-        *reinterpret_cast<uint4 *>(Qhi + ml * pitch + v8 * 8) = *reinterpret_cast<uint4 *>(hq);
-        *reinterpret_cast<uint4 *>(Qlo + ml * pitch + v8 * 8) = *reinterpret_cast<uint4 *>(lq);
+        *reinterpret_cast<uint4 *>(Qhi + ml * pitch + v8 * 8) = hv;
+        *reinterpret_cast<uint4 *>(Qlo + ml * pitch + v8 * 8) = lv;
     }
 
     float o[16][4];
@@ -438,7 +502,7 @@ __global__ void __launch_bounds__(kPaThreads) prefill_attn_kernel(const PfAttnAr
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         const int pos = t0 + 8 * j + 2 * t + e;
-                        const float v = pos <= last ? s[j][2 * hrow + e] * sc : -INFINITY;
+                        const float v = pos <= last ? s[j][2 * hrow + e] : -INFINITY;
                         s[j][2 * hrow + e] = v;
                         mx = fmaxf(mx, v);
                     }
@@ -515,45 +579,41 @@ __global__ void __launch_bounds__(kPaThreads) prefill_attn_kernel(const PfAttnAr
     }
 }
 
-// prefill_attn_tc_kernel (head dim 128): the same causal attention on the 5th-generation tensor core, 128 query rows
+// prefill_attn_tc_kernel: the same causal attention on the 5th-generation tensor core, 128 query rows
 // of one (sequence, head) per CTA, 128 positions per chunk, scores, probabilities and output in tensor memory:
-//   S [128 rows x 128 positions] = Q (bf16 hi + lo, 128-byte-swizzled tiles in shared memory) x K chunk^T (straight
-//                                  from the TMA copy of the cache): 2 x 8 MMAs of K = 16 head dims;
-//   thread r of warps 0-3 owns query row r = tensor-memory lane r: it reads its row of S, keeps the row's running
-//   maximum and sum in registers (no exchange between threads), and writes P = exp2(S - max) back over the same
+//   S [128 rows x 128 positions] = Q (bf16 hi + lo, in log2 units) x K chunk^T, both straight from TMA copies into
+//                                  128-byte-swizzled tiles: 2 x Dh / 16 MMAs of K = 16 head dims;
+//   two threads (warps w and w + 4, 64 positions each) share query row r = tensor-memory lane r: they read its row of S, keep
+//   the row's running maximum (exchanged once per chunk) and their share of its sum in registers, and write P = exp2(S - max) back over the same
 //   columns as packed bf16 hi and lo (per group of 32 positions: 16 columns hi, 16 columns lo);
 //   O [128 rows x 128 head dims] += P (hi, then lo: the A operand read from tensor memory) x V chunk (the B operand,
 //                                  head dims contiguous: MN-major): 2 x 8 MMAs of K = 16 positions.
+// A tile is one or two panels of 64 head dims; the copies fill a shorter head up with zeros (K, V), which only P V multiplies.
+// V rows past the last visible position are whatever the cache holds there: they are cleared in the tile, for 0 x NaN is not 0.
+// Head 80, 8 x 1023 tokens: 458 us a layer on warp-level
+// MMAs, 241 here.
 // S is double-buffered (256 columns) so that the scores of chunk c + 1 are computed while the threads work on chunk
 // c; O takes 128 columns.  The running maximum is only raised when a chunk exceeds it by more than 2^8 (the sums and
-// O absorb the factor), so that rescaling O - a read and a write of the thread's 128 columns - is rare.
-// Warp 4 issues the MMAs, warp 5 the K / V copies (two stages each).  Every wait is bounded.
-constexpr int kPtRows = 128, kPtChunk = 128, kPtThreads = 192;
-constexpr int kPtQBytes = 2 * 128 * 128;             // one of hi / lo: two 64-column panels of 128 rows x 128 bytes
-constexpr int kPtKvBytes = 2 * 128 * 128;            // one K or V chunk, the same shape
-constexpr size_t kPtSmem = 1024 + 2 * kPtQBytes + 4 * kPtKvBytes + 256;
+// O absorb the factor), so that rescaling O - a read and a write of the thread's half of the columns - is rare.
+// Bound by the softmax arithmetic's latency: with one thread per row (one warp per scheduler) 8 x 1023 rows of head 80 took
+// 335 us a layer, with two 241.
+// Warp 8 issues the MMAs, warp 9 the Q, K and V copies (two stages of K and V).  Every wait is bounded.
+constexpr int kPtRows = 128, kPtChunk = 128, kPtThreads = 320;
+constexpr int kPtPanel = 128 * 128;                  // 64 head dims of 128 rows
+constexpr int kPtTile = 2 * kPtPanel;                // room of a Q (hi or lo), K or V tile
+constexpr size_t kPtSmem = 1024 + 6 * kPtTile + 256 + 4 * 128 * 4; // Q hi, Q lo, two K and two V chunks; barriers; maxima by chunk parity
 constexpr float kPtMaxSlack = 8.f;
 
 struct PtAttnArgs {
-    const float *q;              // [B * M, d] position-encoded queries
     const int32_t *len;          // [B] committed lengths
     const int32_t *n_eff;        // [B] rows fed per sequence
     __nv_bfloat16 *out_hi, *out_lo;  // [B * M, d]
-    int M, H, S, d;
-    int kv_row0;                 // first row of this layer in the cache seen as rows of 128 bf16
-    float scale;
+    int M, H, Dh, S, d;
+    int kv_row0;                 // first row of this layer in the cache seen as rows of one head
     long long wait_cycles;
     int32_t *status;
 };
 
-__device__ __forceinline__ void tc_st_16(uint32_t taddr, const uint32_t (&v)[16]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n"
-        "tcgen05.wait::st.sync.aligned;\n" ::"r"(taddr),
-        "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]),
-        "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15])
-        : "memory");
-}
 // 32 columns of this thread's lane; completion is awaited by tc_wait_st
 __device__ __forceinline__ void tc_st_32u_nowait(uint32_t taddr, const uint32_t (&v)[32]) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n" ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]) : "memory");
@@ -571,21 +631,25 @@ __device__ __forceinline__ void tc_mma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem,
 }
 
 __global__ void __launch_bounds__(kPtThreads, 1)
-prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArgs a) {
+prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const __grid_constant__ CUtensorMap tmQhi,
+                       const __grid_constant__ CUtensorMap tmQlo, const PtAttnArgs a) {
     extern __shared__ uint8_t pt_raw[];
     uint8_t *smem = (uint8_t *)(((uintptr_t)pt_raw + 1023) & ~(uintptr_t)1023);
-    uint8_t *qhi = smem, *qlo = smem + kPtQBytes, *kring = smem + 2 * kPtQBytes, *vring = kring + 2 * kPtKvBytes;
-    uint64_t *bars = (uint64_t *)(vring + 2 * kPtKvBytes);
+    uint8_t *qhi = smem, *qlo = smem + kPtTile, *kring = smem + 2 * kPtTile, *vring = kring + 2 * kPtTile;
+    uint64_t *bars = (uint64_t *)(vring + 2 * kPtTile);
     uint64_t *k_full = bars, *k_free = bars + 2, *v_full = bars + 4, *v_free = bars + 6, *s_full = bars + 8;
     // By chunk parity, like the score buffers: S of chunk c + 1 is issued before P V of chunk c, so a warp may be a whole
     // chunk ahead of the slowest one.  With one barrier its arrival for c + 1 would count for c, and its wait for P V of
     // the last chunk would pass on the phase before the previous chunk's.
     uint64_t *p_ready = bars + 10, *o_done = bars + 12;
-    uint32_t *tmem_slot = (uint32_t *)(bars + 14);
+    uint64_t *q_full = bars + 14;
+    uint32_t *tmem_slot = (uint32_t *)(bars + 15);
     volatile int *abort_flag = (volatile int *)(tmem_slot + 1);
+    volatile float *row_x = (volatile float *)(bars + 32);  // [chunk parity][half][row]: what the two threads of a row exchange
 
-    constexpr int Dh = 128;
-    const int mt = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+    const int Dh = a.Dh, panels = Dh > 64 ? 2 : 1;
+    // the longest row tiles first: a CTA's time goes with the positions its rows see
+    const int mt = (int)gridDim.x - 1 - (int)blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int len = a.len[b], n = a.n_eff[b];
     const int m_base = mt * kPtRows, r0 = b * a.M;
@@ -605,7 +669,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
     const int n_chunks = (p_end + kPtChunk - 1) / kPtChunk;
     const int krow0 = a.kv_row0 + ((b * 2) * a.H + h) * a.S, vrow0 = krow0 + a.H * a.S;
 
-    if (warp == 4) {
+    if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "n"(512)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -613,42 +677,13 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
     if (tid == 0) {
         for (int i = 0; i < 10; ++i) mbar_init(&bars[i], 1);
         for (int i = 0; i < 2; ++i) {
-            mbar_init(&p_ready[i], 128);
+            mbar_init(&p_ready[i], 256);
             mbar_init(&o_done[i], 1);
         }
+        mbar_init(q_full, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // Q rows of this tile as bf16 hi / lo (warps 0-3): consecutive threads take consecutive 8-column pieces of a row,
-    // all sixteen loads of a thread in flight together
-    if (tid < kPtRows) {
-        float4 x0[16], x1[16];
-#pragma unroll
-        for (int it = 0; it < 16; ++it) {
-            const int u = it * kPtRows + tid, row = u >> 4, g8 = u & 15, m = m_base + row;
-            x0[it] = x1[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (m < n) {
-                const float *src = a.q + (size_t)(r0 + m) * a.d + h * Dh + g8 * 8;
-                x0[it] = __ldg(reinterpret_cast<const float4 *>(src));
-                x1[it] = __ldg(reinterpret_cast<const float4 *>(src + 4));
-            }
-        }
-#pragma unroll
-        for (int it = 0; it < 16; ++it) {
-            const int u = it * kPtRows + tid, row = u >> 4, g8 = u & 15;
-            const float qv[8] = {x0[it].x, x0[it].y, x0[it].z, x0[it].w, x1[it].x, x1[it].y, x1[it].z, x1[it].w};
-            __nv_bfloat16 hq[8], lq[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                hq[e] = __float2bfloat16_rn(qv[e]);
-                lq[e] = __float2bfloat16_rn(qv[e] - __bfloat162float(hq[e]));
-            }
-            const uint32_t off = (uint32_t)(g8 >> 3) * 16384u + sw128(row, g8 & 7);
-            *reinterpret_cast<uint4 *>(qhi + off) = *reinterpret_cast<uint4 *>(hq);
-            *reinterpret_cast<uint4 *>(qlo + off) = *reinterpret_cast<uint4 *>(lq);
-        }
-    }
-    fence_async_proxy();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -667,50 +702,56 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
         }
     };
 
-    if (warp == 5) {
+    if (warp == 9) {
         if (lane == 0) {
             int issued_k = 0, issued_v = 0;
+            auto copy = [&](uint8_t *dst, const CUtensorMap *map, int x, int y, uint64_t *bar) {
+                mbar_expect_tx(bar, panels * kPtPanel);
+                for (int i = 0; i < panels; ++i) tma_load_2d(dst + i * kPtPanel, map, x + 64 * i, y, bar);
+            };
+            mbar_expect_tx(q_full, 2 * panels * kPtPanel);
+            for (int i = 0; i < panels; ++i) {
+                tma_load_2d(qhi + i * kPtPanel, &tmQhi, h * Dh + 64 * i, r0 + m_base, q_full);
+                tma_load_2d(qlo + i * kPtPanel, &tmQlo, h * Dh + 64 * i, r0 + m_base, q_full);
+            }
             for (int c = 0; c < n_chunks && !*abort_flag; ++c) {
                 const int s = c & 1;
                 if (c >= 2) wait(&k_free[s], ((c >> 1) - 1) & 1);
                 if (*abort_flag) break;
-                mbar_expect_tx(&k_full[s], kPtKvBytes);
-                tma_load_2d(kring + s * kPtKvBytes, &tmKV, 0, krow0 + c * kPtChunk, &k_full[s]);
-                tma_load_2d(kring + s * kPtKvBytes + 16384, &tmKV, 64, krow0 + c * kPtChunk, &k_full[s]);
+                copy(kring + s * kPtTile, &tmKV, 0, krow0 + c * kPtChunk, &k_full[s]);
                 ++issued_k;
                 if (c >= 2) wait(&v_free[s], ((c >> 1) - 1) & 1);
                 if (*abort_flag) break;
-                mbar_expect_tx(&v_full[s], kPtKvBytes);
-                tma_load_2d(vring + s * kPtKvBytes, &tmKV, 0, vrow0 + c * kPtChunk, &v_full[s]);
-                tma_load_2d(vring + s * kPtKvBytes + 16384, &tmKV, 64, vrow0 + c * kPtChunk, &v_full[s]);
+                copy(vring + s * kPtTile, &tmKV, 0, vrow0 + c * kPtChunk, &v_full[s]);
                 ++issued_v;
             }
-            if (*abort_flag) {  // error path only: copies still in flight into this CTA's shared memory
-                for (int c = max(0, issued_k - 2); c < issued_k; ++c) mbar_wait(&k_full[c & 1], (c >> 1) & 1);
-                for (int c = max(0, issued_v - 2); c < issued_v; ++c) mbar_wait(&v_full[c & 1], (c >> 1) & 1);
-            }
+            // no copy is in flight into this CTA's shared memory when it ends, whichever role has given up meanwhile
+            mbar_wait(q_full, 0);
+            for (int c = max(0, issued_k - 2); c < issued_k; ++c) mbar_wait(&k_full[c & 1], (c >> 1) & 1);
+            for (int c = max(0, issued_v - 2); c < issued_v; ++c) mbar_wait(&v_full[c & 1], (c >> 1) & 1);
         }
         __syncwarp();
-    } else if (warp == 4) {
+    } else if (warp == 8) {
         if (lane == 0) {
-            const uint32_t idS = umma_idesc_bf16(128, 128), idO = umma_idesc_bf16(128, 128) | (1u << 16);  // B of P V: MN-major
+            const uint32_t idS = umma_idesc_bf16(128, 128), idO = umma_idesc_bf16(128, 64 * panels) | (1u << 16);  // B of P V: MN-major
             auto issue_s = [&](int c) {
                 const int s = c & 1;
                 wait(&k_full[s], (c >> 1) & 1);
                 if (*abort_flag) return;
                 tc_fence_after();
-                const uint32_t ka = smem_u32(kring + s * kPtKvBytes), qa = smem_u32(qhi), ql = smem_u32(qlo);
+                const uint32_t ka = smem_u32(kring + s * kPtTile), qa = smem_u32(qhi);
+                for (int part = 0; part < 2; ++part)  // hi, then lo
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)  // k = 16 head dims per step; panel ks / 4
-                    tc_mma_bf16(tS + 128 * s, umma_desc(qa + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                                umma_desc(ka + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024), idS, ks ? 1u : 0u);
-#pragma unroll
-                for (int ks = 0; ks < 8; ++ks)
-                    tc_mma_bf16(tS + 128 * s, umma_desc(ql + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024),
-                                umma_desc(ka + (ks >> 2) * 16384 + (ks & 3) * 32, 16, 1024), idS, 1u);
+                    for (int ks = 0; ks < 8; ++ks) {  // k = 16 head dims per step; panel ks / 4
+                        if (16 * ks >= Dh) break;
+                        const uint32_t off = (ks >> 2) * kPtPanel + (ks & 3) * 32;
+                        tc_mma_bf16(tS + 128 * s, umma_desc(qa + part * kPtTile + off, 16, 1024), umma_desc(ka + off, 16, 1024), idS,
+                                    (part | ks) ? 1u : 0u);
+                    }
                 tc_commit(&s_full[s]);
                 tc_commit(&k_free[s]);
             };
+            wait(q_full, 0);
             issue_s(0);
             for (int c = 0; c < n_chunks && !*abort_flag; ++c) {
                 const int s = c & 1;
@@ -719,63 +760,72 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
                 wait(&v_full[s], (c >> 1) & 1);
                 if (*abort_flag) break;
                 tc_fence_after();
-                const uint32_t va = smem_u32(vring + s * kPtKvBytes), tP = tS + 128 * s;
+                const uint32_t va = smem_u32(vring + s * kPtTile), tP = tS + 128 * s;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)  // k = 16 positions per step: two 8-row groups of the V tile; P hi
-                    tc_mma_bf16_ta(tO, tP + 32 * (ks >> 1) + 8 * (ks & 1), umma_desc(va + ks * 2048, 16384, 1024), idO, (c | ks) ? 1u : 0u);
+                    tc_mma_bf16_ta(tO, tP + 32 * (ks >> 1) + 8 * (ks & 1), umma_desc(va + ks * 2048, kPtPanel, 1024), idO, (c | ks) ? 1u : 0u);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)  // P lo
-                    tc_mma_bf16_ta(tO, tP + 32 * (ks >> 1) + 16 + 8 * (ks & 1), umma_desc(va + ks * 2048, 16384, 1024), idO, 1u);
+                    tc_mma_bf16_ta(tO, tP + 32 * (ks >> 1) + 16 + 8 * (ks & 1), umma_desc(va + ks * 2048, kPtPanel, 1024), idO, 1u);
                 tc_commit(&o_done[s]);
                 tc_commit(&v_free[s]);
             }
         }
         __syncwarp();
     } else {
-        // ---------------- softmax and output: thread = query row = tensor-memory lane ----------------
-        const int m = m_base + tid;
+        // ---------------- softmax and output: two threads per query row = tensor-memory lane ----------------
+        const int row = tid & 127, half = tid >> 7;
+        const int m = m_base + row;
         const int last = m < n ? len + m : -1;  // last visible position
-        const uint32_t lane_sel = (uint32_t)(warp * 32) << 16;
-        const float sc = a.scale * 1.4426950408889634f;
+        const uint32_t lane_sel = (uint32_t)((warp & 3) * 32) << 16;
+        auto exchange = [&](int parity, float x) {  // the other thread's x (a barrier for the two warps of a lane quadrant)
+            row_x[(parity * 2 + half) * 128 + row] = x;
+            asm volatile("bar.sync %0, 64;" ::"r"(1 + (warp & 3)) : "memory");
+            return row_x[(parity * 2 + (half ^ 1)) * 128 + row];
+        };
         float m_run = -INFINITY, l_run = 0.f;
         for (int c = 0; c < n_chunks; ++c) {
-            const uint32_t tSc = tS + 128 * (c & 1) + lane_sel;
+            const uint32_t tSc = tS + 128 * (c & 1) + lane_sel + 64 * half;
             const int pos0 = c * kPtChunk;
             wait(&s_full[c & 1], (c >> 1) & 1);
             tc_fence_after();
-            // the row's 128 scores in two round trips, kept in registers for both passes
-            float v0[64], v1[64];
-            tc_ld_64(tSc, v0);
-            tc_ld_64(tSc + 64, v1);
-            float mc = -INFINITY;
+            float v[64];  // the thread's scores, kept in registers for both passes
+            tc_ld_64(tSc, v);
+            const int seen = last - (pos0 + 64 * half);  // the last of them that the row sees
+            if (!__all_sync(0xffffffffu, seen >= 63)) {
 #pragma unroll
-            for (int i = 0; i < 64; ++i) {
-                v0[i] = pos0 + i <= last ? v0[i] * sc : -INFINITY;
-                v1[i] = pos0 + 64 + i <= last ? v1[i] * sc : -INFINITY;
-                mc = fmaxf(mc, fmaxf(v0[i], v1[i]));
+                for (int i = 0; i < 64; ++i) v[i] = i <= seen ? v[i] : -INFINITY;
             }
+            float mc = v[0], mc1 = v[1], mc2 = v[2], mc3 = v[3];
+#pragma unroll
+            for (int i = 4; i < 64; i += 4) {
+                mc = fmaxf(mc, v[i]);
+                mc1 = fmaxf(mc1, v[i + 1]);
+                mc2 = fmaxf(mc2, v[i + 2]);
+                mc3 = fmaxf(mc3, v[i + 3]);
+            }
+            mc = fmaxf(fmaxf(mc, mc1), fmaxf(mc2, mc3));
+            mc = fmaxf(mc, exchange(c & 1, mc));
             const float m_new = (mc > m_run + kPtMaxSlack || m_run == -INFINITY) ? fmaxf(m_run, mc) : m_run;
             const float f = m_new > -INFINITY ? exp2f(m_run - m_new) : 1.f;  // 0 on the first non-empty chunk
             const float m_ref = m_new > -INFINITY ? m_new : 0.f;             // (all masked: every p is exp2(-inf) = 0)
-            float sum = 0.f;
-            auto emit = [&](const float (&v)[64], int half) {  // P of 64 positions: per 32 of them 16 columns hi, 16 lo
+            float sum = 0.f, sum1 = 0.f;
 #pragma unroll
-                for (int g = 0; g < 2; ++g) {
-                    uint32_t w[32];
+            for (int g = 0; g < 2; ++g) {  // P: per 32 positions 16 columns hi, 16 lo
+                uint32_t w[32];
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) {
-                        const float p0 = exp2f(v[32 * g + 2 * i] - m_ref), p1 = exp2f(v[32 * g + 2 * i + 1] - m_ref);
-                        sum += p0 + p1;
-                        const __nv_bfloat162 hv = __floats2bfloat162_rn(p0, p1);
-                        w[i] = *reinterpret_cast<const uint32_t *>(&hv);
-                        w[16 + i] = pack_bf16x2(p0 - __low2float(hv), p1 - __high2float(hv));
-                    }
-                    tc_st_32u_nowait(tSc + 64 * half + 32 * g, w);
+                for (int i = 0; i < 16; ++i) {
+                    const float p0 = exp2f(v[32 * g + 2 * i] - m_ref), p1 = exp2f(v[32 * g + 2 * i + 1] - m_ref);
+                    sum += p0;
+                    sum1 += p1;
+                    const __nv_bfloat162 hv = __floats2bfloat162_rn(p0, p1);
+                    w[i] = *reinterpret_cast<const uint32_t *>(&hv);
+                    w[16 + i] = pack_bf16x2(p0 - __low2float(hv), p1 - __high2float(hv));
                 }
-            };
-            emit(v0, 0);
-            emit(v1, 1);
+                tc_st_32u_nowait(tSc + 32 * g, w);
+            }
             tc_wait_st();
+            sum += sum1;
             l_run = l_run * f + sum;
             m_run = m_new;
             // the accumulated O row moves to the new maximum, once P V of the previous chunk has written it; the
@@ -784,7 +834,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
                 wait(&o_done[(c - 1) & 1], ((c - 1) >> 1) & 1);
                 tc_fence_after();
 #pragma unroll 1
-                for (int g = 0; g < 4; ++g) {
+                for (int g = half * panels; g < (half + 1) * panels; ++g) {  // its half of the columns, 32 at a time
                     float o[32];
                     tc_ld_32(tO + lane_sel + 32 * g, o);
 #pragma unroll
@@ -792,32 +842,40 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
                     tc_st_32(tO + lane_sel + 32 * g, o);
                 }
             }
+            if (pos0 + kPtChunk > p_end) {  // (the last chunk)
+                wait(&v_full[c & 1], (c >> 1) & 1);
+                if (pos0 + row >= p_end && half < panels && !*abort_flag)
+                    for (int i = 0; i < 8; ++i)  // (the swizzle stays within a row's 128 bytes)
+                        *reinterpret_cast<uint4 *>(vring + (c & 1) * kPtTile + half * kPtPanel + row * 128 + i * 16) =
+                            make_uint4(0, 0, 0, 0);
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
             tc_fence_before();
             mbar_arrive(&p_ready[c & 1]);
         }
         wait(&o_done[(n_chunks - 1) & 1], ((n_chunks - 1) >> 1) & 1);
         tc_fence_after();
         {
+            const float l = l_run + exchange(n_chunks & 1, l_run);
             const bool store = m < a.M && !*abort_flag;  // (the loads are warp-wide: every lane takes them)
-            const float inv = (m < n && l_run > 0.f) ? 1.f / l_run : 0.f;
+            const float inv = (m < n && l > 0.f) ? 1.f / l : 0.f;
             const size_t base = (size_t)(r0 + (store ? m : 0)) * a.d + h * Dh;
 #pragma unroll 1
-            for (int g = 0; g < 2; ++g) {
-                float o[64];
-                tc_ld_64(tO + lane_sel + 64 * g, o);
+            for (int g = half * panels; g < (half + 1) * panels; ++g) {
+                if (32 * g >= Dh) break;
+                float o[32];
+                tc_ld_32(tO + lane_sel + 32 * g, o);
                 if (store) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {  // eight head dims: 16 bytes of hi, 16 bytes of lo
-                        uint32_t hw[4], lw[4];
+                    for (int i = 0; i < 4; ++i) {  // eight head dims: 16 bytes of hi, 16 bytes of lo
+                        if (32 * g + 8 * i >= Dh) break;
+                        float y[8];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const float y0 = o[8 * i + 2 * e] * inv, y1 = o[8 * i + 2 * e + 1] * inv;
-                            const __nv_bfloat162 hv = __floats2bfloat162_rn(y0, y1);
-                            hw[e] = *reinterpret_cast<const uint32_t *>(&hv);
-                            lw[e] = pack_bf16x2(y0 - __low2float(hv), y1 - __high2float(hv));
-                        }
-                        *reinterpret_cast<uint4 *>(a.out_hi + base + 64 * g + 8 * i) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                        *reinterpret_cast<uint4 *>(a.out_lo + base + 64 * g + 8 * i) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                        for (int e = 0; e < 8; ++e) y[e] = o[8 * i + e] * inv;
+                        uint4 hv, lv;
+                        split_hilo8(y, hv, lv);
+                        *reinterpret_cast<uint4 *>(a.out_hi + base + 32 * g + 8 * i) = hv;
+                        *reinterpret_cast<uint4 *>(a.out_lo + base + 32 * g + 8 * i) = lv;
                     }
                 }
             }
@@ -825,7 +883,7 @@ prefill_attn_tc_kernel(const __grid_constant__ CUtensorMap tmKV, const PtAttnArg
         tc_fence_before();
     }
     __syncthreads();
-    if (warp == 4) {
+    if (warp == 8) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512) : "memory");
     }

@@ -196,7 +196,7 @@ struct ssd_kv {
     unsigned *gbar;  // grid barrier counter and its neighbours (header ints 32 .. 48)
     uint8_t *cache;
     size_t layer_bytes, esize;
-    CUtensorMap tm_rows;  // bf16 caches of head dim 128: every (layer, sequence, K|V, head, position) row, box 64 x 128
+    CUtensorMap tm_rows;  // bf16 caches, head dim % 16 == 0: every (layer, sequence, K|V, head, position) row, box 64 x 128
     bool tm_rows_ok;
     int len_ub;   // host-side upper bound of the committed lengths
     int last_rows;  // rows the last forward left uncommitted (upper bound bookkeeping)
@@ -831,8 +831,8 @@ constexpr int kWideMinRows = 256;   // below this the few-row kernel's passes ar
 struct WideWs {
     RowInfo ri;
     int32_t *n_rows_tmp;
-    float *x, *qkv, *qrot, *t_in;
-    Operand xn1, xn2, ao, act;
+    float *x, *qkv, *t_in;
+    Operand q, xn1, xn2, ao, act;
     int rows_pad;
     size_t bytes;
 };
@@ -858,7 +858,6 @@ WideWs carve_wide(const ssd_model *m, int B, int C, uint8_t *base) {
     w.n_rows_tmp = (int32_t *)take(sizeof(int32_t) * B);
     w.x = (float *)take(sizeof(float) * R * d);
     w.qkv = (float *)take(sizeof(float) * R * 3 * d);
-    w.qrot = (float *)take(sizeof(float) * R * d);
     w.t_in = (float *)take(sizeof(float) * R * m->d_in);
     auto operand = [&](size_t ld, bool needed) {  // rows padded to whole 128-row tiles; hi and lo apart
         Operand o;
@@ -868,6 +867,7 @@ WideWs carve_wide(const ssd_model *m, int B, int C, uint8_t *base) {
         o.lo = (__nv_bfloat16 *)take(2 * Rp * ld);
         return o;
     };
+    w.q = operand(d, true);
     w.xn1 = operand(d, true);
     w.xn2 = operand(d, a.parallel_residual != 0);
     w.ao = operand(d, true);
@@ -879,8 +879,7 @@ WideWs carve_wide(const ssd_model *m, int B, int C, uint8_t *base) {
 
 bool wide_path_ok(const ssd_model *m) {
     const ssd_arch &a = m->a;
-    return a.dtype == 1 && g_prefill_mode != 1 && a.head_dim % 16 == 0 && a.d_model % 8 == 0 && a.d_ff % 8 == 0 && m->d_in % 4 == 0 &&
-           !m->tm256.empty();
+    return a.dtype == 1 && g_prefill_mode != 1 && a.head_dim % 16 == 0 && a.d_model % 8 == 0 && a.d_ff % 8 == 0 && m->d_in % 4 == 0 && !m->tm256.empty();
 }
 
 // out[R, ldo] (+)= X[R, Kd] W[N, Kd]^T + bias over 128 x 256 output tiles
@@ -937,31 +936,33 @@ int forward_wide(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride
         if ((rc = gemm_wide(st, tm + 0, w.xn1, Rp, R, d, 3 * d, w.qkv, 3 * d, b_qkv, false, kv->status))) return rc;
         if (a.parallel_residual)
             if ((rc = gemm_wide(st, tm + 2, w.xn2, Rp, R, d, m->d_in, w.t_in, m->d_in, b_in, false, kv->status))) return rc;
-        RopeArgs ra;
-        ra.qkv = w.qkv; ra.q_out = w.qrot;
-        ra.cache = kv->cache + (size_t)l * kv->layer_bytes;
-        ra.d = d; ra.H = a.n_heads; ra.Dh = a.head_dim; ra.S = kv->S;
-        ra.rotary_dim = a.pos == 1 ? a.rotary_dim : 0;
-        ra.ri = w.ri;
-        LAUNCH(rope_append_kernel<__nv_bfloat16>, R, 256, 0, st, ra);
-        PfAttnArgs at;
-        at.q = w.qrot;
-        at.cache = (const __nv_bfloat16 *)(kv->cache + (size_t)l * kv->layer_bytes);
-        at.len = kv->len; at.n_eff = w.ri.n_eff;
-        at.out_hi = w.ao.hi; at.out_lo = w.ao.lo;
-        at.M = C; at.H = a.n_heads; at.Dh = a.head_dim; at.S = kv->S; at.d = d;
-        at.scale = 1.0f / sqrtf((float)a.head_dim);
-        if (a.head_dim == 128 && kv->tm_rows_ok && g_prefill_mode != 3) {  // tensor-core form
+        PfAppendArgs ap;
+        ap.qkv = w.qkv; ap.q_hi = w.q.hi; ap.q_lo = w.q.lo;
+        ap.cache = (__nv_bfloat16 *)(kv->cache + (size_t)l * kv->layer_bytes);
+        ap.d = d; ap.H = a.n_heads; ap.Dh = a.head_dim; ap.S = kv->S;
+        ap.rotary_dim = a.pos == 1 ? a.rotary_dim : 0;
+        ap.q_scale = 1.4426950408889634f / sqrtf((float)a.head_dim);
+        ap.ri = w.ri;
+        LAUNCH(prefill_append_kernel, dim3(ceil_div(3 * d, 2048), R), 256, 0, st, ap);
+        if (kv->tm_rows_ok && g_prefill_mode != 3) {  // tensor-core form
             PtAttnArgs pt;
-            pt.q = w.qrot; pt.len = kv->len; pt.n_eff = w.ri.n_eff;
+            CUtensorMap qh, ql;
+            if (make_map(&qh, w.q.hi, Rp, d, kPtRows) || make_map(&ql, w.q.lo, Rp, d, kPtRows)) return SSD_E_CUDA;
+            pt.len = kv->len; pt.n_eff = w.ri.n_eff;
             pt.out_hi = w.ao.hi; pt.out_lo = w.ao.lo;
-            pt.M = C; pt.H = a.n_heads; pt.S = kv->S; pt.d = d;
+            pt.M = C; pt.H = a.n_heads; pt.Dh = a.head_dim; pt.S = kv->S; pt.d = d;
             pt.kv_row0 = l * (kv->B * 2 * a.n_heads * kv->S);
-            pt.scale = at.scale;
             pt.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : kWaitCycles;
             pt.status = kv->status;
-            LAUNCH(prefill_attn_tc_kernel, dim3(ceil_div(C, kPtRows), a.n_heads, B), kPtThreads, kPtSmem, st, kv->tm_rows, pt);
+            LAUNCH(prefill_attn_tc_kernel, dim3(ceil_div(C, kPtRows), a.n_heads, B), kPtThreads, kPtSmem, st, kv->tm_rows, qh, ql,
+                   pt);
         } else {
+            PfAttnArgs at;
+            at.q_hi = w.q.hi; at.q_lo = w.q.lo;
+            at.cache = ap.cache;
+            at.len = kv->len; at.n_eff = w.ri.n_eff;
+            at.out_hi = w.ao.hi; at.out_lo = w.ao.lo;
+            at.M = C; at.H = a.n_heads; at.Dh = a.head_dim; at.S = kv->S; at.d = d;
             LAUNCH(prefill_attn_kernel, dim3(ceil_div(C, kPaRows), a.n_heads, B), kPaThreads, prefill_attn_smem(a.head_dim), st,
                    at);
         }
@@ -1163,8 +1164,8 @@ int kv_init(const ssd_model *m, int batch, int max_len, void *dev_buf, size_t by
     kv->tm_rows_ok = false;
     {
         const long long rows = (long long)m->a.n_layers * batch * 2 * m->a.n_heads * max_len;
-        if (m->a.dtype == 1 && m->a.head_dim == 128 && rows < (1ll << 31))
-            kv->tm_rows_ok = make_map(&kv->tm_rows, kv->cache, (int)rows, 128, kTcChunk) == SSD_OK;
+        if (m->a.dtype == 1 && m->a.head_dim % 16 == 0 && rows < (1ll << 31))
+            kv->tm_rows_ok = make_map(&kv->tm_rows, kv->cache, (int)rows, m->a.head_dim, kTcChunk) == SSD_OK;
     }
     if (cudaMemsetAsync(dev_buf, 0, kv_header_bytes(batch), (cudaStream_t)stream) != cudaSuccess) {
         kv_destroy(kv);

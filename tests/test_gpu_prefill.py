@@ -177,6 +177,38 @@ def test_layer_skip_draft_takes_the_many_row_form(name, many_row_mode):
     assert torch.equal(caches[0][:arch.n_layers - 1], caches[1])
 
 
+def _odd(arch, **kw):
+    return arch.replace(dtype=synth.DT_BF16, **kw)
+
+
+# head dims of one and two 64-column panels with and without a remainder; rotary widths whose halves are not whole 16-byte
+# pieces; MLP widths that end inside a 128- or 256-column weight tile, and a SwiGLU tile that reaches past both halves
+ODD = {
+    "head16-rot12-gelu200": _odd(synth.neox_like(2, 144, 9, 200, 300), rotary_dim=12),
+    "head48-swiglu136": _odd(synth.llama_like(2, 144, 3, 136, 300)),
+    "head80-rot20-gelu264": _odd(synth.neox_like(2, 160, 2, 264, 300), rotary_dim=20),
+    "head96-rot24-gelu128": _odd(synth.neox_like(2, 192, 2, 128, 300), rotary_dim=24),
+    "head112-swiglu392": _odd(synth.llama_like(2, 224, 2, 392, 300)),
+}
+
+
+@pytest.mark.parametrize("name", list(ODD))
+@pytest.mark.parametrize("P", [127, 129, 257])
+def test_many_row_prompt_pass_at_odd_head_and_mlp_widths(name, P, many_row_mode):
+    """Around the 128-position chunk and the 128-row tile, over a cache that holds NaNs wherever nothing was stored (a position
+    that no row sees must not reach the output, not even times zero)."""
+    arch = ODD[name]
+    ws_np = gu.scaled_weights(synth, arch, 3, 6.0)
+    model = B.Model(arch, B.upload_weights(arch, ws_np))
+    S, lens = P + 8, np.array([P, P - 63], np.int32)
+    prompts = synth.gen_prompt(35, 2, P, arch.vocab)
+    kv = B.KV(model, 2, S)
+    kv.cache_view().fill_(float("nan"))
+    B.kv_prefill(model, kv, torch.from_numpy(prompts).cuda(), torch.from_numpy(lens).cuda(),
+                 B.device_buffer(model.prefill_workspace_bytes(2, P)))
+    _check_against_oracle(arch, od.Model(arch, ws_np), model, kv, prompts, lens, S)
+
+
 @pytest.mark.parametrize("name,P", [("llama_bf16", 140), ("neox_bf16_h80", 140), ("neox_bf16", 21), ("gpt2_f32", 17), ("gpt2_bf16", 1)])
 def test_prompt_pass_of_a_target_and_its_layer_skip_draft(name, P):
     """The draft's cache after the common pass is the one of a pass of its own: taken over from the target's (bit for bit) while
