@@ -237,8 +237,10 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 }
 
 // Row norm for the many-row pass: one CTA of 256 threads per row, the row held in registers (float4 per thread,
-// up to 8192 columns; wider rows are re-read), statistics in fp64, one or two outputs (bf16 hi + lo, row-major)
-// from the same statistics.
+// up to 8192 columns; wider rows are re-read), statistics in fp64 in one exchange, one or two outputs (bf16 hi + lo, row-major)
+// from the same statistics.  The mean is subtracted as an fp32 pair, so a large common offset costs nothing; the rest is fp32
+// arithmetic (the result is split to 16 bits next): converting each value to fp64 and back took most of the kernel.
+// Memory-bound: 8184 x 2560, two outputs, 252 MB: 109 us with the values in fp64 and two exchanges, 64 so.
 struct PfNormArgs {
     const float *x;
     int d, kind;  // 0 LayerNorm, 1 RMSNorm
@@ -258,32 +260,40 @@ __device__ __forceinline__ void store_hilo4(__nv_bfloat16 *hi, __nv_bfloat16 *lo
     *reinterpret_cast<uint2 *>(lo + idx) = lv;
 }
 __global__ void __launch_bounds__(256) prefill_norm_kernel(const PfNormArgs a) {  // d % 4 == 0
-    __shared__ double red[32];
+    __shared__ double red[16];
     const int r = blockIdx.x, q4 = a.d >> 2;
     const float4 *x4 = reinterpret_cast<const float4 *>(a.x + (size_t)r * a.d);
     float4 v[8];
     double s = 0.0, ss = 0.0;
+    auto add = [&](const float4 &w) {
+        s += ((double)w.x + (double)w.y) + ((double)w.z + (double)w.w);
+        ss += ((double)w.x * w.x + (double)w.y * w.y) + ((double)w.z * w.z + (double)w.w * w.w);
+    };
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int i = threadIdx.x + 256 * k;
         v[k] = i < q4 ? x4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        s += ((double)v[k].x + (double)v[k].y) + ((double)v[k].z + (double)v[k].w);
     }
-    for (int i = threadIdx.x + 2048; i < q4; i += 256) {
-        const float4 w = x4[i];
-        s += ((double)w.x + (double)w.y) + ((double)w.z + (double)w.w);
-    }
-    double mean = 0.0;
-    if (a.kind == 0) mean = block_sum(s, red) / a.d;
-    auto sq = [&](const float4 &w) {
-        const double c0 = w.x - mean, c1 = w.y - mean, c2 = w.z - mean, c3 = w.w - mean;
-        return (c0 * c0 + c1 * c1) + (c2 * c2 + c3 * c3);
-    };
 #pragma unroll
     for (int k = 0; k < 8; ++k)
-        if (threadIdx.x + 256 * k < q4) ss += sq(v[k]);
-    for (int i = threadIdx.x + 2048; i < q4; i += 256) ss += sq(x4[i]);
-    const double rstd = rsqrt(block_sum(ss, red) / a.d + (double)a.eps);
+        if (256 * k < q4) add(v[k]);
+    for (int i = threadIdx.x + 2048; i < q4; i += 256) add(x4[i]);
+    s = warp_sum(s);
+    ss = warp_sum(ss);
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = s;
+        red[8 + (threadIdx.x >> 5)] = ss;
+    }
+    __syncthreads();
+    s = ss = 0.0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        s += red[w];
+        ss += red[8 + w];
+    }
+    const double mean = a.kind == 0 ? s / a.d : 0.0;
+    const double var = ss / a.d - mean * mean;
+    const float mu = (float)mean, mu_lo = (float)(mean - (double)mu), rs = (float)rsqrt((var > 0.0 ? var : 0.0) + (double)a.eps);
 #pragma unroll
     for (int n = 0; n < 2; ++n) {
         if (n >= a.n_norms) break;
@@ -293,10 +303,10 @@ __global__ void __launch_bounds__(256) prefill_norm_kernel(const PfNormArgs a) {
             const float4 g = __ldg(g4 + i);
             const float4 bb = b4 ? __ldg(b4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
             float4 y;
-            y.x = (float)(((double)w.x - mean) * rstd * (double)g.x + (double)bb.x);
-            y.y = (float)(((double)w.y - mean) * rstd * (double)g.y + (double)bb.y);
-            y.z = (float)(((double)w.z - mean) * rstd * (double)g.z + (double)bb.z);
-            y.w = (float)(((double)w.w - mean) * rstd * (double)g.w + (double)bb.w);
+            y.x = ((w.x - mu) - mu_lo) * rs * g.x + bb.x;
+            y.y = ((w.y - mu) - mu_lo) * rs * g.y + bb.y;
+            y.z = ((w.z - mu) - mu_lo) * rs * g.z + bb.z;
+            y.w = ((w.w - mu) - mu_lo) * rs * g.w + bb.w;
             store_hilo4(a.hi[n], a.lo[n], (size_t)r * a.d + 4 * (size_t)i, y);
         };
 #pragma unroll
