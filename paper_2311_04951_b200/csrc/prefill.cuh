@@ -2,20 +2,24 @@
 // sampling starts).  With hundreds or thousands of rows per forward the linear layers are compute-bound: this
 // file holds the two kernels that differ from the few-row path - a tiled tcgen05 GEMM over 128 activation rows
 // x 256 weight rows per CTA, and a causal attention over row tiles whose keys / values all sit in the cache -
-// the row-wise steps (set-up, embedding, norms, activation, rotary + append) are the stepwise path's kernels,
+// with the norm and the rotary / append / query steps at memory speed; set-up and embedding are the stepwise path's kernels,
 // which take any number of rows.
 //
 // prefill_gemm_kernel:  out[r, n] += sum_k (Xhi[r, k] + Xlo[r, k]) * W[n, k]
-//   * output tiles of 128 rows x 256 columns, dealt round-robin to one CTA per SM; 192 threads: warp 0 = TMA
-//     producer, warp 1 = MMA issuer, warps 2-5 = epilogue (one tensor-memory lane quadrant each); two accumulators
-//     in tensor memory (2 x 256 columns), so a tile's epilogue runs under the next tile's products;
+//   * output tiles of 128 rows x 256 columns, dealt round-robin to one CTA per SM; 320 threads: warp 0 = TMA
+//     producer, warp 1 = MMA issuer, warps 2-9 = epilogue (a tensor-memory lane quadrant and half of the columns each:
+//     with four warps the 128 x 256 GELUs of a tile took longer than the next tile's products: 929 us where eight take
+//     690, 8184 rows x 2560 -> 10240); two accumulators in tensor memory (2 x 256 columns), so a tile's epilogue runs under the next tile's products;
 //   * a stage of the shared-memory ring = the activation rows' hi tile and lo tile (128 rows x 64 k, bf16) and
 //     the weight tile (256 rows x 64 k), all by 2-D tensor-map copies with the 128-byte swizzle, 64 KB;
 //   * per stage eight tcgen05.mma (M = 128, N = 256, K = 16): four k-steps with the hi tile, four with the lo
 //     tile, into ONE fp32 accumulator in tensor memory: W hi + W lo is the fp32-activation product to ~2^-17,
 //     the same arithmetic as the few-row path (the price is half the tensor throughput);
 //   * the tile is owned by this CTA alone (no split over k), so the epilogue writes accumulator + bias over the
-//     output, or adds them to it (the residual stream), with plain loads and stores.
+//     output, adds them to it (the residual stream), or - the MLP's input projection - applies the activation and writes the
+//     next projection's bf16 hi / lo operand, all with plain loads and stores under the next tile's products.  For SwiGLU a
+//     weight tile is 128 gate rows and the 128 up rows of the same columns.  (8184 rows x 2560 -> 10240: 690 us; with the
+//     fp32 pre-activations written and read back by a kernel of its own 640 + 138.)
 // Every wait is bounded; on time-out the kernel records SSD_E_TIMEOUT, drains its copies and returns.
 #pragma once
 #include <cuda.h>
@@ -31,7 +35,7 @@ constexpr int kPfTileM = 128, kPfTileN = 256, kPfStages = 3;
 constexpr int kPfABytes = kPfTileM * kTileK * 2;            // 16 KB: one of hi / lo
 constexpr int kPfWBytes = kPfTileN * kTileK * 2;            // 32 KB
 constexpr int kPfStageBytes = 2 * kPfABytes + kPfWBytes;    // 64 KB
-constexpr int kPfThreads = 192;
+constexpr int kPfEpiWarps = 8, kPfThreads = 64 + 32 * kPfEpiWarps;
 constexpr size_t kPfSmem = 1024 + (size_t)kPfStages * kPfStageBytes + 256;  // + barriers, TMEM slot, abort flag
 
 // eight values as bf16 hi + lo, 16 bytes each
@@ -47,11 +51,16 @@ __device__ __forceinline__ void split_hilo8(const float (&y)[8], uint4 &hi, uint
     lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
+enum { PF_WRITE = 0,   // out = X W^T + bias
+       PF_ADD,         // out += X W^T + bias (the residual stream)
+       PF_GELU,        // act = GELU(X W^T + bias), as bf16 hi + lo
+       PF_SWIGLU };    // act = SiLU(gate) * up
 struct PfGemmArgs {
     float *out;         // [R, ldo] fp32
     const float *bias;  // [N] or null
-    int accumulate;     // 1: out += X W^T + bias (the residual stream); 0: out = X W^T + bias
-    int ldo, N, Kd, R;
+    int mode;           // PF_*
+    int ldo, N, Kd, R;  // N = output columns (SwiGLU: half of W's rows)
+    __nv_bfloat16 *act_hi, *act_lo;  // PF_GELU / PF_SWIGLU: [R, N] row-major
     long long wait_cycles;  // bound of every wait that takes work
     int32_t *status;
 };
@@ -70,7 +79,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int kchunks = (a.Kd + kTileK - 1) / kTileK;
-    const int tiles_m = (a.R + kPfTileM - 1) / kPfTileM, tiles_n = (a.N + kPfTileN - 1) / kPfTileN;
+    const int cols = a.mode == PF_SWIGLU ? kPfTileN / 2 : kPfTileN;  // output columns of a tile
+    const int tiles_m = (a.R + kPfTileM - 1) / kPfTileM, tiles_n = (a.N + cols - 1) / cols;
     const int n_tiles = tiles_m * tiles_n;
     // this CTA's tiles: blockIdx.x, + gridDim.x, ...; row tiles vary fastest, so the CTAs that run together share
     // weight tiles in L2 (the activations of all rows stay there anyway)
@@ -87,7 +97,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&acc_full[i], 1);
-            mbar_init(&acc_empty[i], 4);  // one arrival per epilogue warp
+            mbar_init(&acc_empty[i], kPfEpiWarps);  // one arrival per epilogue warp
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -102,7 +112,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
         if (lane == 0) {
             bool ok = true;
             for (int tile = blockIdx.x; ok && tile < n_tiles; tile += gridDim.x) {
-                const int m0 = (tile % tiles_m) * kPfTileM, n0 = (tile / tiles_m) * kPfTileN;
+                const int m0 = (tile % tiles_m) * kPfTileM, n0 = (tile / tiles_m) * cols;
                 for (int kc = 0; kc < kchunks; ++kc, ++issued) {
                     const int s = issued % kPfStages;
                     if (*abort_flag ||
@@ -115,6 +125,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
                     tma_load_2d(st, &tmXhi, kc * kTileK, m0, &full[s]);
                     tma_load_2d(st + kPfABytes, &tmXlo, kc * kTileK, m0, &full[s]);
                     tma_load_2d(st + 2 * kPfABytes, &tmW, kc * kTileK, n0, &full[s]);
+                    if (a.mode == PF_SWIGLU)  // (the map's box is 128 rows: gate above, up here)
+                        tma_load_2d(st + 2 * kPfABytes + kPfWBytes / 2, &tmW, kc * kTileK, a.N + n0, &full[s]);
                 }
             }
             if (!ok) {
@@ -160,12 +172,12 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
         __syncwarp();
     } else {
         // epilogue: accumulator row r sits in tensor-memory lane r; warp w reaches lanes 32 (w % 4) ..
-        const int quad = warp & 3;
+        const int quad = warp & 3, part = (warp - 2) >> 2;
         const bool vec = ((uintptr_t)a.out & 15) == 0 && (a.ldo & 3) == 0 && (!a.bias || ((uintptr_t)a.bias & 15) == 0);
         int j = 0;
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++j) {
             const int buf = j & 1;
-            const int m0 = (tile % tiles_m) * kPfTileM, n0 = (tile / tiles_m) * kPfTileN;
+            const int m0 = (tile % tiles_m) * kPfTileM, n0 = (tile / tiles_m) * cols;
             const int row = m0 + quad * 32 + lane;
             // (the wait ends early once another role has given up)
             bool landed = false;
@@ -181,40 +193,79 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
                 break;
             }
             tc_fence_after();
-            float *orow = a.out + (size_t)row * a.ldo + n0;
+            if (a.mode >= PF_GELU) {
+                const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * kPfTileN);
+                const size_t orow = (size_t)row * a.N + n0;
 #pragma unroll 1
-            for (int cb = 0; cb < kPfTileN / 32; ++cb) {
-                if (n0 + cb * 32 >= a.N) break;
-                float v[32];
-                tc_ld_32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * kPfTileN + cb * 32), v);
-                if (row < a.R) {
-                    if (vec && n0 + cb * 32 + 31 < a.N) {
-                        if (a.bias) {
+                for (int cb = part * (cols / 64); cb < (part + 1) * (cols / 64); ++cb) {
+                    if (n0 + cb * 32 >= a.N) break;
+                    float v[32], u[32];
+                    tc_ld_32(acc + cb * 32, v);
+                    if (a.mode == PF_SWIGLU) tc_ld_32(acc + kPfTileN / 2 + cb * 32, u);
+                    if (row < a.R) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const float4 bv = __ldg(reinterpret_cast<const float4 *>(a.bias + n0 + cb * 32 + 4 * i));
-                                v[4 * i] += bv.x; v[4 * i + 1] += bv.y; v[4 * i + 2] += bv.z; v[4 * i + 3] += bv.w;
+                        for (int i = 0; i < 4; ++i) {   // eight columns: 16 bytes of hi, 16 bytes of lo (N is a multiple of 8)
+                            const int c0 = n0 + cb * 32 + 8 * i;
+                            if (c0 >= a.N) break;
+                            float y[8], bg[8] = {}, bu[8] = {};
+                            if (a.bias) {
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) bg[e] = __ldg(a.bias + c0 + e);
+                                if (a.mode == PF_SWIGLU) {
+#pragma unroll
+                                    for (int e = 0; e < 8; ++e) bu[e] = __ldg(a.bias + a.N + c0 + e);
+                                }
                             }
-                        }
-                        if (a.accumulate) {
-                            float4 o[8];
+                            if (a.mode == PF_GELU) {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) o[i] = *reinterpret_cast<const float4 *>(orow + cb * 32 + 4 * i);
+                                for (int e = 0; e < 8; ++e) y[e] = gelu_erf(v[8 * i + e] + bg[e]);
+                            } else {
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                v[4 * i] += o[i].x; v[4 * i + 1] += o[i].y; v[4 * i + 2] += o[i].z; v[4 * i + 3] += o[i].w;
+                                for (int e = 0; e < 8; ++e) y[e] = silu(v[8 * i + e] + bg[e]) * (u[8 * i + e] + bu[e]);
                             }
+                            uint4 hv, lv;
+                            split_hilo8(y, hv, lv);
+                            *reinterpret_cast<uint4 *>(a.act_hi + orow + cb * 32 + 8 * i) = hv;
+                            *reinterpret_cast<uint4 *>(a.act_lo + orow + cb * 32 + 8 * i) = lv;
                         }
+                    }
+                }
+            } else {
+                float *orow = a.out + (size_t)row * a.ldo + n0;
+#pragma unroll 1
+                for (int cb = part * (kPfTileN / 64); cb < (part + 1) * (kPfTileN / 64); ++cb) {
+                    if (n0 + cb * 32 >= a.N) break;
+                    float v[32];
+                    tc_ld_32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * kPfTileN + cb * 32), v);
+                    if (row < a.R) {
+                        if (vec && n0 + cb * 32 + 31 < a.N) {
+                            if (a.bias) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            *reinterpret_cast<float4 *>(orow + cb * 32 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-                    } else {
-                        for (int i = 0; i < 32; ++i) {
-                            const int col = n0 + cb * 32 + i;
-                            if (col < a.N) {
-                                float y = v[i] + (a.bias ? a.bias[col] : 0.f);
-                                if (a.accumulate) y += orow[cb * 32 + i];
-                                orow[cb * 32 + i] = y;
+                                for (int i = 0; i < 8; ++i) {
+                                    const float4 bv = __ldg(reinterpret_cast<const float4 *>(a.bias + n0 + cb * 32 + 4 * i));
+                                    v[4 * i] += bv.x; v[4 * i + 1] += bv.y; v[4 * i + 2] += bv.z; v[4 * i + 3] += bv.w;
+                                }
+                            }
+                            if (a.mode == PF_ADD) {
+                                float4 o[8];
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) o[i] = *reinterpret_cast<const float4 *>(orow + cb * 32 + 4 * i);
+#pragma unroll
+                                for (int i = 0; i < 8; ++i) {
+                                    v[4 * i] += o[i].x; v[4 * i + 1] += o[i].y; v[4 * i + 2] += o[i].z; v[4 * i + 3] += o[i].w;
+                                }
+                            }
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)
+                                *reinterpret_cast<float4 *>(orow + cb * 32 + 4 * i) = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+                        } else {
+                            for (int i = 0; i < 32; ++i) {
+                                const int col = n0 + cb * 32 + i;
+                                if (col < a.N) {
+                                    float y = v[i] + (a.bias ? a.bias[col] : 0.f);
+                                    if (a.mode == PF_ADD) y += orow[cb * 32 + i];
+                                    orow[cb * 32 + i] = y;
+                                }
                             }
                         }
                     }
@@ -222,7 +273,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_consta
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);  // this warp has read its quadrant of the buffer
+            if (lane == 0) mbar_arrive(&acc_empty[buf]);  // this warp has read its part of the buffer
         }
         tc_fence_before();
     }
@@ -316,27 +367,10 @@ __global__ void __launch_bounds__(256) prefill_norm_kernel(const PfNormArgs a) {
     }
 }
 
-// act[r, i] = GELU(t[r, i])  or  SiLU(t[r, i]) * t[r, F + i], four columns per thread; grid (ceil(F / 1024), R); F % 4 == 0
-__global__ void __launch_bounds__(256) prefill_act_kernel(const float *__restrict__ t, int ld_t, int F, int swiglu,
-                                                          __nv_bfloat16 *hi, __nv_bfloat16 *lo) {
-    const int r = blockIdx.y, i = 4 * (blockIdx.x * 256 + threadIdx.x);
-    if (i >= F) return;
-    const float *tr = t + (size_t)r * ld_t;
-    const float4 u = *reinterpret_cast<const float4 *>(tr + i);
-    float4 y;
-    if (swiglu) {
-        const float4 w = *reinterpret_cast<const float4 *>(tr + F + i);
-        y = make_float4(silu(u.x) * w.x, silu(u.y) * w.y, silu(u.z) * w.z, silu(u.w) * w.w);
-    } else {
-        y = make_float4(gelu_erf(u.x), gelu_erf(u.y), gelu_erf(u.z), gelu_erf(u.w));
-    }
-    store_hilo4(hi, lo, (size_t)r * F + i, y);
-}
-
-// Rotary, the cache append and the attention kernels' queries: eight columns of one row's q, k or v per thread (16-byte loads
-// and stores).  Keys and values go to the cache in its bf16, queries - scaled to log2 units - become a bf16 hi / lo operand.
-// grid (ceil(3 d / 8 / 256), rows).
-// Memory-bound: 8184 rows x 7680, 419 MB: 121 us a column per thread, 91 so.
+// Rotary, the cache append and the attention kernels' queries: eight columns of one row per thread (16-byte loads and stores).
+// prefill_append_kernel puts keys and values into the cache in its bf16, prefill_query_kernel scales the queries to log2 units
+// and makes a bf16 hi / lo operand of them.  grid (ceil(2 d / 8 / 256), rows) and (ceil(d / 8 / 256), rows).
+// Memory-bound: 8184 rows x 7680, 419 MB: 121 us in one kernel with a column per thread, 60 + 31 so.
 struct PfAppendArgs {
     const float *qkv;                // [R, 3 d]
     __nv_bfloat16 *q_hi, *q_lo;      // [R, d]
@@ -350,15 +384,11 @@ __device__ __forceinline__ void load8(const float *p, float (&v)[8]) {  // p 16-
     v[0] = u.x; v[1] = u.y; v[2] = u.z; v[3] = u.w;
     v[4] = w.x; v[5] = w.y; v[6] = w.z; v[7] = w.w;
 }
-__global__ void __launch_bounds__(256) prefill_append_kernel(const PfAppendArgs a) {
-    const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 8;
-    if (c >= 3 * a.d) return;
-    const int which = c >= 2 * a.d ? 2 : c >= a.d ? 1 : 0, col = c - which * a.d, h = col / a.Dh, e = col % a.Dh;
-    const float *src = a.qkv + (size_t)r * 3 * a.d + c;
-    float x[8];
+// eight columns of row r from `src` (the head's column e first), turned by the row's position
+__device__ __forceinline__ void load8_rotary(const PfAppendArgs &a, const float *src, int r, int e, int rotary_dim, float (&x)[8]) {
     load8(src, x);
-    if (which < 2 && e < a.rotary_dim) {
-        const int half = a.rotary_dim >> 1;
+    if (e < rotary_dim) {
+        const int half = rotary_dim >> 1;
         const float *cos_r = a.ri.rope_cos + (size_t)r * half, *sin_r = a.ri.rope_sin + (size_t)r * half;
         if ((half & 7) == 0) {  // the eight columns lie on one side of the split, their partners are eight columns too
             const bool low = e < half;
@@ -372,7 +402,7 @@ __global__ void __launch_bounds__(256) prefill_append_kernel(const PfAppendArgs 
         } else {
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                if (e + i >= a.rotary_dim) break;
+                if (e + i >= rotary_dim) break;
                 const bool low = e + i < half;
                 const int j = low ? e + i : e + i - half;
                 const float o = low ? src[i + half] : src[i - half];
@@ -380,18 +410,28 @@ __global__ void __launch_bounds__(256) prefill_append_kernel(const PfAppendArgs 
             }
         }
     }
-    if (which == 0) {
+}
+__global__ void __launch_bounds__(256) prefill_append_kernel(const PfAppendArgs a) {
+    const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 8;
+    if (c >= 2 * a.d || !a.ri.valid[r]) return;
+    const int is_v = c >= a.d ? 1 : 0, col = c - is_v * a.d, h = col / a.Dh, e = col % a.Dh;
+    float x[8];
+    load8_rotary(a, a.qkv + (size_t)r * 3 * a.d + a.d + c, r, e, is_v ? 0 : a.rotary_dim, x);
+    const size_t plane = ((size_t)a.ri.seq[r] * 2 + is_v) * a.H + h;
+    *reinterpret_cast<uint4 *>(a.cache + (plane * a.S + a.ri.pos[r]) * a.Dh + e) =
+        make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]), pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
+}
+__global__ void __launch_bounds__(256) prefill_query_kernel(const PfAppendArgs a) {
+    const int r = blockIdx.y, c = (blockIdx.x * 256 + threadIdx.x) * 8;
+    if (c >= a.d) return;
+    float x[8];
+    load8_rotary(a, a.qkv + (size_t)r * 3 * a.d + c, r, c % a.Dh, a.rotary_dim, x);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] *= a.q_scale;
-        uint4 hi, lo;
-        split_hilo8(x, hi, lo);
-        *reinterpret_cast<uint4 *>(a.q_hi + (size_t)r * a.d + col) = hi;
-        *reinterpret_cast<uint4 *>(a.q_lo + (size_t)r * a.d + col) = lo;
-    } else if (a.ri.valid[r]) {
-        const size_t plane = ((size_t)a.ri.seq[r] * 2 + (which - 1)) * a.H + h;
-        *reinterpret_cast<uint4 *>(a.cache + (plane * a.S + a.ri.pos[r]) * a.Dh + e) =
-            make_uint4(pack_bf16x2(x[0], x[1]), pack_bf16x2(x[2], x[3]), pack_bf16x2(x[4], x[5]), pack_bf16x2(x[6], x[7]));
-    }
+    for (int i = 0; i < 8; ++i) x[i] *= a.q_scale;
+    uint4 hi, lo;
+    split_hilo8(x, hi, lo);
+    *reinterpret_cast<uint4 *>(a.q_hi + (size_t)r * a.d + c) = hi;
+    *reinterpret_cast<uint4 *>(a.q_lo + (size_t)r * a.d + c) = lo;
 }
 
 // prefill_attn_kernel: causal attention of 64 query rows of one (sequence, head) over the cache, which already

@@ -831,7 +831,7 @@ constexpr int kWideMinRows = 256;   // below this the few-row kernel's passes ar
 struct WideWs {
     RowInfo ri;
     int32_t *n_rows_tmp;
-    float *x, *qkv, *t_in;
+    float *x, *qkv;
     Operand q, xn1, xn2, ao, act;
     int rows_pad;
     size_t bytes;
@@ -858,7 +858,6 @@ WideWs carve_wide(const ssd_model *m, int B, int C, uint8_t *base) {
     w.n_rows_tmp = (int32_t *)take(sizeof(int32_t) * B);
     w.x = (float *)take(sizeof(float) * R * d);
     w.qkv = (float *)take(sizeof(float) * R * 3 * d);
-    w.t_in = (float *)take(sizeof(float) * R * m->d_in);
     auto operand = [&](size_t ld, bool needed) {  // rows padded to whole 128-row tiles; hi and lo apart
         Operand o;
         o.f32 = nullptr; o.hi = nullptr; o.lo = nullptr; o.ld = (int)ld;
@@ -879,25 +878,28 @@ WideWs carve_wide(const ssd_model *m, int B, int C, uint8_t *base) {
 
 bool wide_path_ok(const ssd_model *m) {
     const ssd_arch &a = m->a;
-    return a.dtype == 1 && g_prefill_mode != 1 && a.head_dim % 16 == 0 && a.d_model % 8 == 0 && a.d_ff % 8 == 0 && m->d_in % 4 == 0 && !m->tm256.empty();
+    return a.dtype == 1 && g_prefill_mode != 1 && a.head_dim % 16 == 0 && a.d_model % 8 == 0 && a.d_ff % 8 == 0 && !m->tm256.empty();
 }
 
-// out[R, ldo] (+)= X[R, Kd] W[N, Kd]^T + bias over 128 x 256 output tiles
-int gemm_wide(cudaStream_t st, const CUtensorMap *tw, const Operand &X, int rows_pad, int R, int Kd, int N, float *out,
-              int ldo, const float *bias, bool accumulate, int32_t *status) {
+// X[R, Kd] W[N, Kd]^T + bias over 128 x 256 output tiles, written to / added to `out`, or through the activation into `act`
+// (then N = the activation's columns; for PF_SWIGLU tw has 128-row boxes)
+int gemm_wide(cudaStream_t st, const CUtensorMap *tw, const Operand &X, int rows_pad, int R, int Kd, int N, int mode, float *out,
+              int ldo, const float *bias, const Operand *act, int32_t *status) {
     CUtensorMap th, tl;
     if (make_map(&th, X.hi, rows_pad, Kd, kPfTileM) || make_map(&tl, X.lo, rows_pad, Kd, kPfTileM)) return SSD_E_CUDA;
     PfGemmArgs g;
-    g.out = out; g.bias = bias; g.accumulate = accumulate ? 1 : 0;
+    g.out = out; g.bias = bias; g.mode = mode;
     g.ldo = ldo; g.N = N; g.Kd = Kd; g.R = R; g.status = status;
+    g.act_hi = act ? act->hi : nullptr; g.act_lo = act ? act->lo : nullptr;
     g.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : kWaitCycles;
-    const int n_tiles = ceil_div(N, kPfTileN) * ceil_div(R, kPfTileM), sms = g_num_sms > 0 ? g_num_sms : 148;
+    const int cols = mode == PF_SWIGLU ? kPfTileN / 2 : kPfTileN;
+    const int n_tiles = ceil_div(N, cols) * ceil_div(R, kPfTileM), sms = g_num_sms > 0 ? g_num_sms : 148;
     LAUNCH(prefill_gemm_kernel, n_tiles < sms ? n_tiles : sms, kPfThreads, kPfSmem, st, *tw, th, tl, g);
     return SSD_OK;
 }
 
 // One decoder forward over B x C prompt rows: fills the cache (no logits).  The steps of the stepwise forward with
-// many-row kernels: the projections write (q, k, v and the MLP input) or add to (the residual stream) their output
+// many-row kernels: the projections write (q, k, v), add to (the residual stream) or activate (the MLP input) their output
 // together with the bias, so nothing is pre-loaded.
 int forward_wide(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride, int C, const int32_t *n_rows,
                  const WideWs &w, cudaStream_t st) {
@@ -933,9 +935,11 @@ int forward_wide(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride
             n1.hi[1] = w.xn2.hi; n1.lo[1] = w.xn2.lo;
         }
         LAUNCH(prefill_norm_kernel, R, 256, 0, st, n1);
-        if ((rc = gemm_wide(st, tm + 0, w.xn1, Rp, R, d, 3 * d, w.qkv, 3 * d, b_qkv, false, kv->status))) return rc;
-        if (a.parallel_residual)
-            if ((rc = gemm_wide(st, tm + 2, w.xn2, Rp, R, d, m->d_in, w.t_in, m->d_in, b_in, false, kv->status))) return rc;
+        auto mlp_in = [&](const Operand &x) {
+            return a.act == 1 ? gemm_wide(st, &m->tm[4 * l + 2], x, Rp, R, d, F, PF_SWIGLU, nullptr, 0, b_in, &w.act, kv->status)
+                              : gemm_wide(st, tm + 2, x, Rp, R, d, F, PF_GELU, nullptr, 0, b_in, &w.act, kv->status);
+        };
+        if ((rc = gemm_wide(st, tm + 0, w.xn1, Rp, R, d, 3 * d, PF_WRITE, w.qkv, 3 * d, b_qkv, nullptr, kv->status))) return rc;
         PfAppendArgs ap;
         ap.qkv = w.qkv; ap.q_hi = w.q.hi; ap.q_lo = w.q.lo;
         ap.cache = (__nv_bfloat16 *)(kv->cache + (size_t)l * kv->layer_bytes);
@@ -943,7 +947,8 @@ int forward_wide(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride
         ap.rotary_dim = a.pos == 1 ? a.rotary_dim : 0;
         ap.q_scale = 1.4426950408889634f / sqrtf((float)a.head_dim);
         ap.ri = w.ri;
-        LAUNCH(prefill_append_kernel, dim3(ceil_div(3 * d, 2048), R), 256, 0, st, ap);
+        LAUNCH(prefill_append_kernel, dim3(ceil_div(2 * d, 2048), R), 256, 0, st, ap);
+        LAUNCH(prefill_query_kernel, dim3(ceil_div(d, 2048), R), 256, 0, st, ap);
         if (kv->tm_rows_ok && g_prefill_mode != 3) {  // tensor-core form
             PtAttnArgs pt;
             CUtensorMap qh, ql;
@@ -966,14 +971,14 @@ int forward_wide(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride
             LAUNCH(prefill_attn_kernel, dim3(ceil_div(C, kPaRows), a.n_heads, B), kPaThreads, prefill_attn_smem(a.head_dim), st,
                    at);
         }
-        if ((rc = gemm_wide(st, tm + 1, w.ao, Rp, R, d, d, w.x, d, b_o, true, kv->status))) return rc;
+        if (a.parallel_residual && (rc = mlp_in(w.xn2))) return rc;
+        if ((rc = gemm_wide(st, tm + 1, w.ao, Rp, R, d, d, PF_ADD, w.x, d, b_o, nullptr, kv->status))) return rc;
         if (!a.parallel_residual) {
             PfNormArgs n2 = norm_args((const float *)lw(m, l, L_LN2G), (const float *)lw(m, l, L_LN2B), w.xn1);
             LAUNCH(prefill_norm_kernel, R, 256, 0, st, n2);
-            if ((rc = gemm_wide(st, tm + 2, w.xn1, Rp, R, d, m->d_in, w.t_in, m->d_in, b_in, false, kv->status))) return rc;
+            if ((rc = mlp_in(w.xn1))) return rc;
         }
-        LAUNCH(prefill_act_kernel, dim3(ceil_div(F, 1024), R), 256, 0, st, w.t_in, m->d_in, F, a.act == 1, w.act.hi, w.act.lo);
-        if ((rc = gemm_wide(st, tm + 3, w.act, Rp, R, F, d, w.x, d, b_out, true, kv->status))) return rc;
+        if ((rc = gemm_wide(st, tm + 3, w.act, Rp, R, F, d, PF_ADD, w.x, d, b_out, nullptr, kv->status))) return rc;
     }
     kv->last_rows = C;
     return SSD_OK;
