@@ -261,3 +261,24 @@ def test_fp32_forward_in_one_kernel_matches_oracle_and_stepwise(arch, lens, M):
         gu.assert_logits_close(res[0][0][b], oc.feed(rows[b], advance=False))
         n = int(lens[b]) + M
         assert np.abs(res[0][1][:, b, :, :, :n] - oc.kv[:, :, :, :n]).max() <= 1e-3
+
+
+@pytest.mark.parametrize("d,H", [(128, 2), (2048, 16), (2176, 17), (4224, 33)])
+def test_embedding_rows_in_sixteen_byte_pieces_and_unaligned(d, H):
+    """A part of a thread's pieces, exactly one each, some with two, a second round; and a table two bytes off a 16-byte
+    boundary, which is read a value at a time.  (Weights scaled as their fan-in asks: x6 at d = 256.)"""
+    arch = synth.llama_like(1, d, H, 128, 128)
+    ws_np = gu.scaled_weights(synth, arch, 3, 6.0 * (256 / d) ** 0.5)
+    rows = synth.gen_prompt(8, 2, 3, arch.vocab)
+    omodel = od.Model(arch, ws_np)
+    for shift in (0, 1):
+        tensors = B.upload_weights(arch, ws_np)
+        buf = torch.empty(tensors[0].numel() + 8, dtype=tensors[0].dtype, device="cuda")
+        tensors[0] = buf[shift:shift + tensors[0].numel()].view_as(tensors[0]).copy_(tensors[0])
+        assert tensors[0].data_ptr() % 16 == 2 * shift
+        model = B.Model(arch, tensors)
+        kv = B.KV(model, 2, 16)
+        got = gpu_logits(model, kv, model.new_workspace(2, 3, 16), rows, 2)
+        assert kv.status() == 0
+        for b in range(2):
+            gu.assert_logits_close(got[b], omodel.new_cache(16).feed(rows[b], advance=False))
