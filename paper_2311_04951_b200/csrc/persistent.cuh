@@ -2247,7 +2247,6 @@ __device__ __noinline__ void work_program() {
         for (int i = threadIdx.x; i < p.n_steps * p.B * 2; i += kWorkThreads) p.tail_hit[i] = (i & 1) ? -1 : 0x7fffffff;
     bool go = true;
     for (int step = 0; step < p.n_steps && go; ++step) {
-        const int gs = step << kStepShift;
         if (step > 0) {  // the rows of this step: one per sequence, the token the step before drew
             if (threadIdx.x == 0) params_copy().cur_step = step;
             named_bar(2, kWorkThreads);
@@ -2267,9 +2266,10 @@ __device__ __noinline__ void work_program() {
             tab[64 + b] = b < p.B ? __ldcg(p.ri.n_eff + b) : 0;
         }
         for (int l = 0; l < p.n_layers && go; ++l) {
-            run_gemm<NT>(gs | (4 * l + 0));                  // qkv
+            asm volatile("" : "+r"(l));  // (no induction variables beside it: each would be one more value kept across the calls)
+            run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 0));                  // qkv
             const bool kv_only = !p.want_logits && l + 1 == p.n_layers;
-            if (p.parallel && !kv_only) run_gemm<NT>(gs | (4 * l + 1));  // MLP in (same block input)
+            if (p.parallel && !kv_only) run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 1));  // MLP in (same block input)
             if (!(go = grid_sync())) break;
             if (kv_only) {
                 attention_phase<WIDE>(l);  // (its items append the rows)
@@ -2283,8 +2283,8 @@ __device__ __noinline__ void work_program() {
                     attn_signal();
                 } else {
                     if (!(go = grid_sync())) break;
-                    run_gemm<NT>(gs | (4 * l + 2));               // MLP out -> x, beside the attention items
-                    run_gemm<NT>(gs | (4 * l + 3));               // out-proj -> x, once the attention CTAs have signalled
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));               // MLP out -> x, beside the attention items
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));               // out-proj -> x, once the attention CTAs have signalled
                 }
                 if (!(go = grid_sync())) break;
             } else {
@@ -2292,26 +2292,26 @@ __device__ __noinline__ void work_program() {
                 if (p.parallel) act_phase();
                 if (!(go = grid_sync())) break;
                 if (p.parallel) {
-                    run_gemm<NT>(gs | (4 * l + 2));                   // out-proj -> x
-                    run_gemm<NT>(gs | (4 * l + 3));                   // MLP out  -> x
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));                   // out-proj -> x
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));                   // MLP out  -> x
                     if (!(go = grid_sync())) break;
                 } else {
-                    run_gemm<NT>(gs | (4 * l + 1));                   // out-proj -> x
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 1));                   // out-proj -> x
                     if (!(go = grid_sync())) break;
                     norm_mid_layer(l);
                     if (!(go = grid_sync())) break;
-                    run_gemm<NT>(gs | (4 * l + 2));                   // MLP in
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));                   // MLP in
                     if (!(go = grid_sync())) break;
                     act_phase();
                     if (!(go = grid_sync())) break;
-                    run_gemm<NT>(gs | (4 * l + 3));                   // MLP out -> x
+                    run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));                   // MLP out -> x
                     if (!(go = grid_sync())) break;
                 }
             }
             norm_for_layer(l + 1);
             if (!(go = grid_sync())) break;
         }
-        if (go && p.want_logits) run_gemm<NT>(gs | (4 * p.n_layers));
+        if (go && p.want_logits) run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * p.n_layers));
         if (go && p.tail) {  // q, the draw and the commit of this step (see tail_partial)
             if (!(go = grid_sync())) break;
             tail_partial();
