@@ -63,19 +63,21 @@ __device__ __noinline__ void attention_items_mma8(int layer) {
     constexpr int RPI = 32 / GPR;
     const int lr = lane / GPR, lc = lane % GPR;
     const uint32_t wst_u = smem_u32(wst) + (uint32_t)(lr * ROWB);
+    // The loop issues more instructions than its MMAs leave room for, so a row costs two copies and one minimum (a bounds test,
+    // a select and a byte count per row, with 64-bit offsets: 54.3 us a layer for eight sequences of 2100 positions, 51.7 so).
     auto issue = [&](int i) {  // block warp + 8 i of this warp into stage i % NS
         const int blk = warp + 8 * i, pos0 = p_begin + blk * kM8Block + lr;
         const uint32_t st = wst_u + (uint32_t)((i % NS) * STAGE);
-        const size_t off0 = (size_t)pos0 * DH + lc * 8;
+        if (blk < nb) {
+            const int past = (c1 - 1 - pos0) * DH;  // rows past the range repeat its last row: finite, and masked
+            const __nv_bfloat16 *ks = kc + pos0 * DH + lc * 8, *vs = vc + pos0 * DH + lc * 8;
 #pragma unroll 4
-        for (int it = 0; it < kM8Block / RPI; ++it) {
-            const int r = it * RPI + lr;
-            const bool in = blk < nb && pos0 + it * RPI < c1;
-            const size_t off = in ? off0 + (size_t)it * RPI * DH : 0;
-            const uint32_t so = st + (uint32_t)(it * RPI * ROWB + ((lc ^ (r & 7)) << 4));
-            const uint32_t nbytes = in ? 16u : 0u;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(so), "l"(kc + off), "r"(nbytes) : "memory");
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(so + kM8Block * ROWB), "l"(vc + off), "r"(nbytes) : "memory");
+            for (int it = 0; it < kM8Block / RPI; ++it) {
+                const int off = min(it * RPI * DH, past);
+                const uint32_t so = st + (uint32_t)(it * RPI * ROWB + ((lc ^ ((it * RPI + lr) & 7)) << 4));
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(so), "l"(ks + off) : "memory");
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(so + kM8Block * ROWB), "l"(vs + off) : "memory");
+            }
         }
         cp_async_commit();
     };
