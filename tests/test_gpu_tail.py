@@ -225,3 +225,50 @@ def test_tail_at_the_edges_of_the_row_pieces(V, top_k, top_p):
                 assert np.abs(p[b, i] - ref).max() <= gu.P_ATOL
             assert abs(float(p[b, i].astype(np.float64).sum()) - 1.0) < 1e-5
         gu.check_decisions_on_own_rows(p[b], q[b], rows[b, 1:], u[b, :K], u[b, K], int(n_acc[b]), int(nxt[b]))
+
+
+@pytest.mark.parametrize("top_k", [0, 37])
+@pytest.mark.parametrize("V", [33, 8193, 32000, 65537])
+@pytest.mark.parametrize("u_draw", [1.0, float("nan"), float("inf"), -0.25, 1.0 - 2.0 ** -24, 0.0])
+def test_every_uniform_draws_a_token(u_draw, V, top_k):
+    """A uniform outside [0, 1) - a float64 one close to 1 rounds to 1.0 - still writes a token: the last index with weight > 0
+    from 1 on and for a NaN, the first one below 0; in the residual draw (sequence 0) and in the bonus draw (sequence 1).
+    The end of the row weighs nothing."""
+    K = 1
+    logits = synth.gen_logits(91 + V, 2 * (K + 1), V, 1.5).reshape(2, K + 1, V)
+    logits[:, :, V - V // 3:] = -np.inf
+    q = np.stack([osamp.filter_top_k_top_p(osamp.softmax_t(synth.gen_logits(92 + b, 1, V, 1.5)[0], 1.0), top_k) for b in range(2)])[:, None]
+    p_ref = np.stack([osamp.filter_top_k_top_p(osamp.softmax_t(logits[b, 0], 1.0), top_k) for b in range(2)])
+    x = [int(np.argmax(q[0, 0])), int(np.argmax(p_ref[1]))]
+    u = np.array([[2.0 * p_ref[0, x[0]] / q[0, 0, x[0]] + 1.0, u_draw], [0.0, u_draw]], np.float32)  # refused; accepted
+    B.set_sampling(top_k, 1.0)
+    try:
+        n_acc, nxt, p = run_tail(logits, np.array([[0, x[0]], [0, x[1]]], np.int32), q, u, 1.0)
+    finally:
+        B.set_sampling(0, 1.0)
+    assert n_acc.tolist() == [0, 1]
+    for b, w in ((0, osamp.residual(p[0, 0], q[0, 0])), (1, p[1, 1])):
+        live = np.nonzero(w > 0)[0]
+        if not u_draw < 1.0:
+            assert nxt[b] == live[-1]
+        elif u_draw <= 0.0:
+            assert nxt[b] == live[0]
+        else:
+            assert w[nxt[b]] > 0 and w[nxt[b]:].astype(np.float64).sum() >= 0.5 * 2.0 ** -24 * w.astype(np.float64).sum()
+
+
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("u", [1.0, float("nan")])
+def test_a_draft_step_draws_a_token_for_a_uniform_of_one(u, fused):
+    """As above for the draft's draw, in the stand-alone tail and in the one inside the forward kernel."""
+    arch = synth.neox_like(2, 128, 4, 256, 640)
+    m = B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, 21, 7.0)))
+    kv, ws = B.KV(m, 1, 16), m.new_workspace(1, 1, 16)
+    tok = torch.full((1, 1), -7, dtype=torch.int32, device="cuda")
+    q = torch.zeros(1, 1, arch.vocab, device="cuda")
+    x, uu = torch.tensor([[5]], dtype=torch.int32, device="cuda"), torch.tensor([[u]], device="cuda")
+    if fused:
+        B.draft_steps(m, kv, 1, x, 1, 1, None, 1.0, uu, 1, tok, 1, q, arch.vocab, ws)
+    else:
+        B.draft_step(m, kv, x, 1, 1, None, 1.0, uu, 1, tok, 1, q, arch.vocab, ws)
+    assert int(tok.item()) == int(torch.nonzero(q[0, 0] > 0).max()) and kv.status() == 0
