@@ -222,7 +222,9 @@ int draft_steps(ssd_model *draft, ssd_kv *dkv, int n_steps, const int32_t *dev_t
  * max(0, p_i - q_i) renormalised (from p_i if that residual is all zero); if all K are
  * accepted draw it from p_{K+1}; both draws by inverse CDF with u_{K+1}.
  *   dev_q           fp32 [batch, K, vocab] draft distributions (ignored when K == 0)
- *   dev_u           fp32 [batch, K+1]: K acceptance uniforms, then the resampling uniform
+ *   dev_u           fp32 [batch, K+1]: K acceptance uniforms, then the resampling uniform; in [0,1).  Every draw writes a
+ *                   token: from 1 on (a float64 uniform may round to it) and for a NaN the last index with weight > 0,
+ *                   below 0 the first
  *   dev_n_accepted  int32 [batch] out
  *   dev_next_token  int32 out at [b * next_token_stride]
  *   dev_p_debug     fp32 [batch, K+1, vocab] out or NULL: the p rows the decisions used

@@ -488,6 +488,7 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
 struct DrawSmem {
     double tot[kTailWarps], incl[kTailWarps];  // the warps' sums, and their running sums
     double cta[2];              // this CTA's total, by draw (a kernel draws at most twice)
+    int last[kTailWarps], cta_last;  // largest index with weight > 0
     float w[32 * 8];            // the owner warp's entries, handed from its load order to index order
 };
 
@@ -496,6 +497,8 @@ struct DrawSmem {
 // called again by the warp whose piece the draw falls into.  That warp is found without a vote: piece boundaries are the
 // same fp64 numbers on both sides (a piece ends where the next one starts), so exactly one piece holds u * S.  Inside it
 // a zero-weight index is never drawn; if rounding leaves no index, the piece's largest with weight > 0 is taken.
+// Outside [0, 1) no piece holds u * S: below 0 the first index with weight > 0 is drawn, from 1 on (and for a NaN, or an
+// infinite S) the last one.
 // Returns the index in every lane of that warp and -1 elsewhere; *total = S everywhere (S <= 0: nothing was drawn).
 template <int IT, typename WeightFn>
 __device__ __forceinline__ int cluster_draw(WeightFn weights, int V, float u, DrawSmem *ds, cg::cluster_group &cl, int slot,
@@ -535,7 +538,25 @@ __device__ __forceinline__ int cluster_draw(WeightFn weights, int V, float u, Dr
     *total = S;
     if (!(S > 0.0)) return -1;
     const double beg = c_beg + w_beg, end = c_beg + w_end;  // (the last warp's end is c_beg + T, where the next CTA begins)
-    const double target = (double)u * S;
+    double target = (double)u * S;
+    if (!(target < S)) {  // the same in all threads of the cluster
+        int mine = -1;
+        for (int b = lo; b < hi; b += kStep) {
+            weights(b, w);
+#pragma unroll
+            for (int k = 0; k < IT; ++k)
+                if (w[k] > 0.f) mine = b + 32 * k + lane;
+        }
+        mine = __reduce_max_sync(0xffffffffu, mine);
+        if (lane == 0) ds->last[warp] = mine;
+        __syncthreads();
+        const int cta_last = __reduce_max_sync(0xffffffffu, ds->last[lane]);
+        if (threadIdx.x == 0) ds->cta_last = cta_last;
+        cl.sync();
+        const int last = __reduce_max_sync(0xffffffffu, lane < kTailCluster ? *cl.map_shared_rank(&ds->cta_last, lane) : -1);
+        return mine == last ? last : -1;
+    }
+    if (target < 0.0) target = 0.0;
     if (!(beg <= target && target < end)) return -1;  // the same in all lanes
     double run = beg;
     int hit = -1, last = -1;
