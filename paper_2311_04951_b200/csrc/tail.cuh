@@ -91,7 +91,7 @@ __device__ __forceinline__ PartStat join_parts(PartStat a, float inv_t) {
     for (int o = W / 2; o > 0; o >>= 1) am = min(am, __shfl_xor_sync(0xffffffffu, am, o));
     double s = 0.0;
     if (inv_t != 0.f) {
-        s = a.mx > -INFINITY ? a.s * (double)expf((a.mx - m) * inv_t) : 0.0;
+        s = a.mx > -INFINITY ? a.s * (double)expf((a.mx - m) * inv_t) : a.s;  // (nothing, or NaN)
 #pragma unroll
         for (int o = W / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     }
@@ -157,12 +157,13 @@ __device__ __forceinline__ void cluster_stats(const float *logits, int rows, int
         }
         am = __reduce_min_sync(0xffffffffu, am);
         double s = 0.0;
-        if (inv_t != 0.f && m > -INFINITY) {
+        if (inv_t != 0.f) {
             float part = 0.f;
             if (!one) tail_load<IT>(lg, lo, hi, -INFINITY, l);
+            const float ref = m > -INFINITY ? m : 0.f;  // (a piece of NaNs has no maximum, but they reach the row's sum)
             for (int b = lo;;) {
 #pragma unroll
-                for (int u = 0; u < IT; ++u) part += expf((l[u] - m) * inv_t);  // exp(-inf) = 0
+                for (int u = 0; u < IT; ++u) part += expf((l[u] - ref) * inv_t);  // exp(-inf) = 0
                 b += kStep;
                 if (b >= hi) break;
                 tail_load<IT>(lg, b, hi, -INFINITY, l);
@@ -338,8 +339,8 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         const float m = warp_max_redux(mx);
         const int am = __reduce_min_sync(0xffffffffu, mx == m ? at : 0x7fffffff);
         float part = 0.f;
-        if (m > -INFINITY)
-            for (int j = lo + lane; j < hi; j += 32) part += expf((entry(j) - m) * inv_t);
+        const float ref = m > -INFINITY ? m : 0.f;  // (as in cluster_stats)
+        for (int j = lo + lane; j < hi; j += 32) part += expf((entry(j) - ref) * inv_t);
         const double s = warp_sum((double)part);
         if (lane == 0) {
             PartStat t;
@@ -478,7 +479,7 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         float *p = a.p_out + row * V;
         for (int j = lo + lane; j < hi; j += 32) {
             const float pr = cached ? mine[j] : prob_of(__ldcg(lg + j), st, inv_t, j);
-            p[j] = pr >= f.thr ? pr / f.mass : 0.f;   // (as prob_f)
+            p[j] = f.mass == 0.f ? pr : pr >= f.thr ? pr / f.mass : 0.f;   // (as prob_f)
         }
     }
     cl.sync();  // nobody leaves while its shared memory is read

@@ -272,3 +272,26 @@ def test_a_draft_step_draws_a_token_for_a_uniform_of_one(u, fused):
     else:
         B.draft_step(m, kv, x, 1, 1, None, 1.0, uu, 1, tok, 1, q, arch.vocab, ws)
     assert int(tok.item()) == int(torch.nonzero(q[0, 0] > 0).max()) and kv.status() == 0
+
+
+@pytest.mark.parametrize("top_k", [0, 50])
+@pytest.mark.parametrize("V,n_bad", [(8192, 32), (8192, 256), (32000, 512), (66000, 1056)])
+def test_a_run_of_nans_makes_the_whole_row_not_a_number(V, n_bad, top_k):
+    """NaN logits that fill a whole warp's piece of the row (which then has no maximum) reach the row's sum like single ones:
+    every probability of the row is NaN, its draft token is refused and the token of the largest finite logit is emitted; the
+    neighbouring sequence is not touched."""
+    logits, rows, q, u = make_case(4000 + V, 2, 1, V, 1.0, True)
+    q = np.stack([osamp.filter_top_k_top_p(q[b, 0], top_k) for b in range(2)])[:, None]
+    rows[:, 1] = [int(np.argmax(q[b, 0])) for b in range(2)]
+    bad = np.zeros(V, bool)
+    bad[n_bad * 3:n_bad * 4] = True
+    logits[0, :, bad] = np.nan
+    B.set_sampling(top_k, 1.0)
+    try:
+        n_acc, nxt, p = run_tail(logits, rows, q, u, 1.0)
+    finally:
+        B.set_sampling(0, 1.0)
+    assert np.isnan(p[0]).all() and n_acc[0] == 0
+    assert nxt[0] == int(np.argmax(np.where(bad, -np.inf, logits[0, 0])))
+    assert np.isfinite(p[1]).all()
+    gu.check_decisions_on_own_rows(p[1], q[1], rows[1, 1:], u[1, :1], u[1, 1], int(n_acc[1]), int(nxt[1]))
