@@ -395,7 +395,7 @@ struct alignas(16) Shared {
 };
 // The phase functions find their state at fixed shared-memory addresses: nothing is passed to them and nothing is kept in
 // registers across their calls for it, and a field is one shared-memory load with an immediate address.
-constexpr int kAttnBars = 15;
+constexpr int kAttnBars = 16;
 struct alignas(128) SharedBlock {
     uint8_t params[(sizeof(FwdParams) + 63) / 64 * 64];  // the kernel parameters, copied once (see forward_kernel)
     Shared state;
@@ -1278,9 +1278,10 @@ __host__ __device__ constexpr int tc_scratch_bytes(int rp) {  // ring, Q tile, P
 // only meaningful for a waiter that follows every phase of its barrier in order and that the barrier
 // cannot pass by two phases; the threads that patch this pass's rows into a chunk skip most chunks, so
 // they do not wait on the ring's barriers: the MMA issuer, which follows every stage, tells them through
-// `landed` when such a chunk has arrived, and hears back through `fixed`.  (The vote keeps the softmax warps within a chunk
-// of each other, so that p_ready may be one barrier.)
-enum { AB_KV_FULL = 0, AB_KV_FREE = kTcStages, AB_S_FULL = 2 * kTcStages, AB_P_READY = AB_S_FULL + 2, AB_O_DONE /* two: chunk parity */,
+// `landed` when such a chunk has arrived, and hears back through `fixed`.  p_ready goes by chunk parity, as the P tiles do:
+// with two tiles the softmax may hand over P of chunk c + 1 before the issuer has looked for P of chunk c, and on one barrier
+// that wait would be passed by two phases (and run to its limit).
+enum { AB_KV_FULL = 0, AB_KV_FREE = kTcStages, AB_S_FULL = 2 * kTcStages, AB_P_READY = AB_S_FULL + 2, AB_O_DONE = AB_P_READY + 2 /* two each: chunk parity */,
        AB_FIXED = AB_O_DONE + 2, AB_LANDED, AB_COUNT };
 constexpr float kTcMaxSlack = 32.f;
 
@@ -1433,6 +1434,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
     // P V of chunk c completes phase c >> 1 of o_done[c & 1]
     auto o_par = [&](int c) { return (acnt[AB_O_DONE + (c & 1)] + (uint32_t)(c >> 1)) & 1u; };
     auto s_par = [&](int c) { return (acnt[AB_S_FULL + (c & 1)] + (uint32_t)(c >> 1)) & 1u; };
+    auto p_par = [&](int c) { return (acnt[AB_P_READY + (c & 1)] + (uint32_t)(c >> 1)) & 1u; };
     auto full_par = [&](int j) { return (acnt[AB_KV_FULL + j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u; };          // stage j has landed
     auto free_par = [&](int j) { return ((acnt[AB_KV_FREE + j % kTcStages] + (uint32_t)(j / kTcStages)) & 1u) ^ 1u; };   // its slot was released
     int n_fix_total = 0;
@@ -1521,7 +1523,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             for (int c = 0; c < n_chunks && !sh->abort; ++c) {
                 const int jv = 2 * c + 1;
                 if (c + 1 < n_chunks) issue_s(c + 1);
-                wait(p_ready, (acnt[AB_P_READY] + c) & 1u);
+                wait(&p_ready[c & 1], p_par(c));
                 wait(&kv_full[jv % kTcStages], full_par(jv));
                 if (sh->abort) break;
                 tc_fence_after();
@@ -1682,7 +1684,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             }
             fence_async_proxy();
             tc_fence_before();
-            mbar_arrive(p_ready);
+            mbar_arrive(&p_ready[c & 1]);
         }
         // ---- the sums over positions, then thread = head dim tid: output or partial ----
         // (lane r of a warp ends up with row r's sum: RP - 1 exchanges instead of 5 RP)
@@ -1753,7 +1755,8 @@ __device__ __noinline__ void attention_items_tc(int layer) {
         }
         acnt[AB_S_FULL] += (uint32_t)((n_chunks + 1) / 2);
         acnt[AB_S_FULL + 1] += (uint32_t)(n_chunks / 2);
-        acnt[AB_P_READY] += n_chunks;
+        acnt[AB_P_READY] += (uint32_t)((n_chunks + 1) / 2);
+        acnt[AB_P_READY + 1] += (uint32_t)(n_chunks / 2);
         acnt[AB_O_DONE] += (uint32_t)((n_chunks + 1) / 2);
         acnt[AB_O_DONE + 1] += (uint32_t)(n_chunks / 2);
         acnt[AB_FIXED] += n_fix_total;
@@ -2370,7 +2373,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1) forward_kernel(const __gri
         }
         mbar_init(&blk.mmaDone, 1);
         for (int i = 0; i < AB_COUNT; ++i) {
-            mbar_init(&blk.abar[i], i == AB_P_READY ? 128 : i == AB_FIXED ? 64 : 1);  // landed: the MMA issuer alone
+            mbar_init(&blk.abar[i], i == AB_P_READY || i == AB_P_READY + 1 ? 128 : i == AB_FIXED ? 64 : 1);  // landed: the MMA issuer alone
             blk.acnt[i] = 0;
         }
         blk.role_rp[0] = RingPos();
