@@ -20,16 +20,19 @@
 #include "tail.cuh"
 #include "prefill.cuh"
 #include "f32_forward.cuh"
+#include "device_table.h"
 
 using namespace ssd;
 
 namespace {
 
 std::atomic<uint64_t> g_launches{0};
-int g_num_sms = 0;
-int g_l2_window = 0;  // bytes of L2 that may hold persisting lines (0: the device has none / the limit could not be set)
-bool g_attr_done = false;
-std::mutex g_mu;
+
+struct DeviceInfo {
+    int num_sms;
+    int l2_window;  // bytes of L2 that may hold persisting lines (0: the device has none / the limit could not be set)
+};
+DeviceTable<DeviceInfo> g_devices;
 
 // ---- optional per-launch timing of the kernel that streams the weights (forward_kernel for bf16
 //      models in single-kernel mode, otherwise every gemm launch) ----
@@ -133,12 +136,8 @@ size_t attn_smem(int Dh) {
     return (size_t)MR * (Dh + kAttnTile + 3) * 4 + 2 * (size_t)kAttnTile * (Dh + 16 / sizeof(T)) * sizeof(T);
 }
 
-int init_device_once() {
-    std::lock_guard<std::mutex> lk(g_mu);
-    if (g_attr_done) return SSD_OK;
-    int dev = 0;
-    CUDA_OK(cudaGetDevice(&dev));
-    CUDA_OK(cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev));
+int init_device(int dev, DeviceInfo &info) {
+    CUDA_OK(cudaDeviceGetAttribute(&info.num_sms, cudaDevAttrMultiProcessorCount, dev));
     {   // room in L2 for persisting lines (a limit of this process's context, gone with it)
         int max_persist = 0, max_window = 0;
         cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, dev);
@@ -146,7 +145,7 @@ int init_device_once() {
         size_t want = 32u << 20;
         if ((size_t)max_persist < want) want = (size_t)max_persist;
         if (want > 0 && cudaDeviceSetLimit(cudaLimitPersistingL2CacheSize, want) == cudaSuccess)
-            g_l2_window = (int)(want < (size_t)max_window ? want : (size_t)max_window);
+            info.l2_window = (int)(want < (size_t)max_window ? want : (size_t)max_window);
         (void)cudaGetLastError();
     }
     int rc = 0;
@@ -164,15 +163,30 @@ int init_device_once() {
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 8>, attn_smem<__nv_bfloat16, 8>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 16>, attn_smem<__nv_bfloat16, 16>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 32>, attn_smem<__nv_bfloat16, 32>(128));
-    rc |= set_smem(row_filter_kernel, (size_t)kFilterCache * 4);
     rc |= set_smem(forward_f32_kernel<8>, kFfMaxSmem);
     rc |= set_smem(forward_f32_kernel<kMaxRowsPerSeq>, kFfMaxSmem);
     rc |= set_smem(prefill_gemm_kernel, kPfSmem);
     rc |= set_smem(prefill_attn_kernel, prefill_attn_smem(128));
     rc |= set_smem(prefill_attn_tc_kernel, kPtSmem);
-    if (rc) return SSD_E_CUDA;
-    g_attr_done = true;
-    return SSD_OK;
+    return rc ? SSD_E_CUDA : SSD_OK;
+}
+// The current device's entry: kernel attributes set, SM count and L2 window known.
+int device_info(const DeviceInfo **out) {
+    int dev = 0;
+    CUDA_OK(cudaGetDevice(&dev));
+    return g_devices.get(dev, [dev](DeviceInfo &info) { return init_device(dev, info); }, out) ? SSD_E_CUDA : SSD_OK;
+}
+int num_sms() {
+    const DeviceInfo *info;
+    return device_info(&info) == SSD_OK ? info->num_sms : 148;
+}
+// Let `kernel` take `bytes` of shared memory on the current device.
+template <typename K>
+int allow_smem(DeviceTable<bool> &devices, K kernel, size_t bytes) {
+    int dev = 0;
+    CUDA_OK(cudaGetDevice(&dev));
+    const bool *unused;
+    return devices.get(dev, [&](bool &) { return set_smem(kernel, bytes); }, &unused) ? SSD_E_CUDA : SSD_OK;
 }
 
 }  // namespace
@@ -425,7 +439,8 @@ int gemm(const GemmCall &c, const void *W, const CUtensorMap *tw, const Operand 
         g.stages = 0;
         g.status = status;
         long long total = (long long)g.n_tiles * g.kchunks;
-        int grid = (int)(total < g_num_sms ? total : g_num_sms);
+        const int sms = num_sms();
+        int grid = (int)(total < sms ? total : sms);
         switch (c.Rp / 8) {
             case 1: rc = launch_gemm_nt<1>(c.st, *tw, th, tl, g, grid); break;
             case 2: rc = launch_gemm_nt<2>(c.st, *tw, th, tl, g, grid); break;
@@ -448,7 +463,7 @@ int gemm(const GemmCall &c, const void *W, const CUtensorMap *tw, const Operand 
 // aim is one round of items over the SMs: as many splits as keep groups * splits <= #SMs.
 void plan_split(int groups, int ctx, int *chunk, int *n_split, int tile = kAttnTile) {
     if (ctx < 1) ctx = 1;
-    const int sms = g_num_sms > 0 ? g_num_sms : 148;
+    const int sms = num_sms();
     int ns = ctx <= 256 ? 1 : sms / (groups > 0 ? groups : 1);
     int max_by_len = ceil_div(ctx, 2 * kAttnTile);  // at least 128 positions per split
     if (ns > max_by_len) ns = max_by_len;
@@ -533,23 +548,18 @@ int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStr
     p.stages_lo = (int)S1;
     p.attn_smem_off = (int)(S1 * stage);
     const size_t smem = 1024 + S1 * stage + region2;
-    static bool attr[64] = {false};  // the attribute belongs to the device's copy of the kernel
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SSD_E_CUDA;
-    if (!attr[dev]) {
-        if (cudaFuncSetAttribute(forward_kernel<NT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemBudget - (int)sizeof(SharedBlock)) !=
-            cudaSuccess)
-            return SSD_E_CUDA;
-        attr[dev] = true;
-    }
+    const DeviceInfo *info;
+    int rc = device_info(&info);
+    if (rc) return rc;
+    static DeviceTable<bool> devices;
+    if ((rc = allow_smem(devices, forward_kernel<NT, WIDE>, (size_t)kSmemBudget - sizeof(SharedBlock)))) return rc;
     void *args[] = {&p};
     // The workspace (residual stream, GEMM outputs and operands: a few MB that every phase re-reads and that the
     // GEMMs reduce into) is marked persisting in L2 for this launch, so that the weight stream does not push it
     // out between the phase that writes a buffer and the phase that reads it.
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
-    cfg.gridDim = dim3(g_num_sms);
+    cfg.gridDim = dim3(info->num_sms);
     cfg.blockDim = dim3(kPersistThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -558,10 +568,10 @@ int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStr
     attrs[na].id = cudaLaunchAttributeCooperative;
     attrs[na].val.cooperative = 1;
     ++na;
-    if (g_l2_window > 0 && ws_base && ws_bytes > 0) {
+    if (info->l2_window > 0 && ws_base && ws_bytes > 0) {
         attrs[na].id = cudaLaunchAttributeAccessPolicyWindow;
         attrs[na].val.accessPolicyWindow.base_ptr = const_cast<void *>(ws_base);
-        attrs[na].val.accessPolicyWindow.num_bytes = ws_bytes < (size_t)g_l2_window ? ws_bytes : (size_t)g_l2_window;
+        attrs[na].val.accessPolicyWindow.num_bytes = ws_bytes < (size_t)info->l2_window ? ws_bytes : (size_t)info->l2_window;
         attrs[na].val.accessPolicyWindow.hitRatio = 1.0f;
         attrs[na].val.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
         attrs[na].val.accessPolicyWindow.missProp = cudaAccessPropertyStreaming;
@@ -649,7 +659,7 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
         items_per_split = tiles;
     }
     {
-        const int items = items_per_split * p.n_split, sms = g_num_sms > 0 ? g_num_sms : 148;
+        const int items = items_per_split * p.n_split, sms = num_sms();
         p.attn_items = items;
         p.attn_ctas = items < sms ? items : sms;
         p.overlap_out = (a.parallel_residual && 2 * p.attn_ctas <= sms) ? 1 : 0;
@@ -658,7 +668,7 @@ int forward_persistent(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_
     p.wait_cycles = g_wait_cycles;
     p.n_steps = 1;
     if (dl) {
-        if (g_num_sms > kMaxCtas) return SSD_E_CAPACITY;
+        if (num_sms() > kMaxCtas) return SSD_E_CAPACITY;
         p.n_steps = dl->n_steps; p.tail = 1; p.inv_t = dl->inv_t;
         p.u = dl->u; p.u_stride = dl->u_stride;
         p.tok_out = dl->tok_out; p.tok_out_stride = dl->tok_out_stride;
@@ -724,7 +734,10 @@ int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride,
     if (want_logits && a.vocab > widest) widest = a.vocab;
     int grid = ceil_div(widest, kFfWarps);
     if (grid < kv->B * a.n_heads) grid = kv->B * a.n_heads;
-    if (grid > g_num_sms) grid = g_num_sms;
+    const DeviceInfo *info;
+    const int rc = device_info(&info);
+    if (rc) return rc;
+    if (grid > info->num_sms) grid = info->num_sms;
     const void *k = M <= 8 ? (const void *)forward_f32_kernel<8> : (const void *)forward_f32_kernel<kMaxRowsPerSeq>;
     CUDA_OK(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kFfThreads), args, smem, st));
     g_launches.fetch_add(1, std::memory_order_relaxed);
@@ -893,7 +906,7 @@ int gemm_wide(cudaStream_t st, const CUtensorMap *tw, const Operand &X, int rows
     g.act_hi = act ? act->hi : nullptr; g.act_lo = act ? act->lo : nullptr;
     g.wait_cycles = g_wait_cycles > 0 ? g_wait_cycles : kWaitCycles;
     const int cols = mode == PF_SWIGLU ? kPfTileN / 2 : kPfTileN;
-    const int n_tiles = ceil_div(N, cols) * ceil_div(R, kPfTileM), sms = g_num_sms > 0 ? g_num_sms : 148;
+    const int n_tiles = ceil_div(N, cols) * ceil_div(R, kPfTileM), sms = num_sms();
     LAUNCH(prefill_gemm_kernel, n_tiles < sms ? n_tiles : sms, kPfThreads, kPfSmem, st, *tw, th, tl, g);
     return SSD_OK;
 }
@@ -1022,7 +1035,8 @@ int ssd_model_create(const ssd_arch *arch, const void *const *dev_weights, int n
     }
     const int fb = T_L0 + PER_LAYER * arch->n_layers;
     if (!need(fb) || (!arch->tie_lm_head && !need(fb + 2))) return SSD_E_ARG;
-    if ((rc = init_device_once())) return rc;
+    const DeviceInfo *info;
+    if ((rc = device_info(&info))) return rc;
     ssd_model *m = new (std::nothrow) ssd_model();
     if (!m) return SSD_E_ARG;
     m->a = *arch;
@@ -1286,6 +1300,9 @@ static bool restricted(float temperature, int V) {  // (a greedy row is its own 
 }
 static int run_row_filter(const float *logits, int B, int M, int V, const int32_t *n_eff, float temperature, RowStat *stats,
                           RowFilter *filt, float *p_out, cudaStream_t st) {
+    static DeviceTable<bool> devices;  // (on supplied logits the tail may be a program's first call on the device)
+    const int rc = allow_smem(devices, row_filter_kernel, (size_t)kFilterCache * 4);
+    if (rc) return rc;
     FilterArgs f;
     f.logits = logits; f.M = M; f.V = V; f.n_eff = n_eff; f.inv_t = 1.0f / temperature;
     f.top_k = g_top_k; f.top_p = g_top_p;
@@ -1401,8 +1418,6 @@ int verify_from_logits(const float *dev_logits, int batch, int K, int vocab, con
         return SSD_E_ARG;
     if (K > 0 && !dev_q) return SSD_E_ARG;
     if (scratch_bytes < verify_scratch_bytes(batch, K)) return SSD_E_CAPACITY;
-    const int rc = init_device_once();  // (may be a program's first call)
-    if (rc) return rc;
     return run_verify_tail(dev_logits, batch, K, vocab, dev_rows, dev_q, dev_u, temperature, dev_n_accepted,
                            dev_next_token, next_token_stride, dev_p_debug, nullptr, (RowStat *)dev_scratch,
                            (RowFilter *)((uint8_t *)dev_scratch + align_up(sizeof(RowStat) * (size_t)batch * (K + 1), 256)),
