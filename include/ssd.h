@@ -170,7 +170,9 @@ int kv_prefill(ssd_model *m, ssd_kv *kv, const int32_t *dev_tokens, const int32_
  * The prompt pass of a target and its draft: kv_prefill of both.  Where the draft is the target's first layers
  * (ssd_model_share_prefix) and both caches are empty - the host's bound of every length is 0: fresh caches, or caches cut back
  * to nothing and read with kv_lengths -, its keys and values are the target's first layers', and are copied instead of computed
- * again.  (Section "So, what's the problem?": two models, two caches.)
+ * again (not while the stream is being captured: a replay may find them filled).  If the device then finds a length that the
+ * host's bound excludes (the slab was written by other means), that sequence's draft cache is left alone and the draft's status
+ * word becomes SSD_E_ARG.  (Section "So, what's the problem?": two models, two caches.)
  */
 int kv_prefill_pair(ssd_model *target, ssd_kv *tkv, ssd_model *draft, ssd_kv *dkv, const int32_t *dev_tokens,
                     const int32_t *dev_n_tokens, int max_tokens, void *dev_ws_target, size_t ws_target_bytes, void *dev_ws_draft,

@@ -1275,8 +1275,11 @@ int kv_prefill_pair(ssd_model *target, ssd_kv *tkv, ssd_model *draft, ssd_kv *dk
                     const int32_t *dev_n_tokens, int max_tokens, void *dev_ws_target, size_t ws_target_bytes, void *dev_ws_draft,
                     size_t ws_draft_bytes, void *stream) {
     if (!target || !tkv || !draft || !dkv || max_tokens < 0) return SSD_E_ARG;
-    const bool adopt = is_prefix_of(draft, target) && same_cache_shape(target, tkv) && same_cache_shape(draft, dkv) && tkv->B == dkv->B &&
-                       kv_bound(tkv) == 0 && kv_bound(dkv) == 0 && max_tokens <= dkv->S;
+    // (a recorded call may be replayed on caches that are not empty)
+    cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
+    CUDA_OK(cudaStreamIsCapturing((cudaStream_t)stream, &recording));
+    const bool adopt = recording == cudaStreamCaptureStatusNone && is_prefix_of(draft, target) && same_cache_shape(target, tkv) &&
+                       same_cache_shape(draft, dkv) && tkv->B == dkv->B && kv_bound(tkv) == 0 && kv_bound(dkv) == 0 && max_tokens <= dkv->S;
     int rc = kv_prefill(target, tkv, dev_tokens, dev_n_tokens, max_tokens, dev_ws_target, ws_target_bytes, stream);
     if (rc) return rc;
     if (!adopt) return kv_prefill(draft, dkv, dev_tokens, dev_n_tokens, max_tokens, dev_ws_draft, ws_draft_bytes, stream);
@@ -1284,9 +1287,10 @@ int kv_prefill_pair(ssd_model *target, ssd_kv *tkv, ssd_model *draft, ssd_kv *dk
     cudaStream_t st = (cudaStream_t)stream;
     const int row_bytes = (int)(draft->a.head_dim * dkv->esize);
     LAUNCH(kv_adopt_kernel, dim3(ceil_div(max_tokens, 16), draft->a.n_heads, 2 * dkv->B * draft->a.n_layers), 256, 0, st, tkv->cache,
-           dkv->cache, tkv->len, dkv->B, tkv->S, dkv->S, row_bytes);
+           dkv->cache, tkv->len, dkv->len, max_tokens, dkv->B, tkv->S, dkv->S, row_bytes);
     const unsigned seq = kv_note_op(dkv, max_tokens);
-    LAUNCH(kv_adopt_len_kernel, 1, 64, 0, st, tkv->len, tkv->status, dkv->len, dkv->status, dkv->B, dkv->S, dkv->mailbox_dev, seq);
+    LAUNCH(kv_adopt_len_kernel, 1, 64, 0, st, tkv->len, tkv->status, dkv->len, dkv->status, max_tokens, dkv->B, dkv->S, dkv->mailbox_dev,
+           seq);
     return SSD_OK;
 }
 
@@ -1482,7 +1486,13 @@ int kv_lengths(ssd_kv *kv, int32_t *host_out, void *stream) {
     CUDA_OK(cudaStreamSynchronize(st));
     int mx = 0;
     for (int b = 0; b < kv->B; ++b) mx = host_out[b] > mx ? host_out[b] : mx;
-    kv->len_ub = mx;  // the bound is exact again
+    // The bound is exact again, whatever the words say (a copy of another cache's slab changes lengths without a kernel that
+    // reports them): the lengths just read become the report of an operation of their own.
+    const unsigned seq = kv_note_op(kv, 0);
+    if (kv->mailbox)
+        for (int b = 0; b < kv->B; ++b)
+            reinterpret_cast<volatile unsigned long long *>(kv->mailbox)[b] = ((unsigned long long)seq << 32) | (unsigned)host_out[b];
+    kv->len_ub = mx;
     return SSD_OK;
 }
 

@@ -822,10 +822,13 @@ __global__ void kv_rollback_kernel(int32_t *len, const int32_t *new_len, int B, 
     }
 }
 // The cache of a layer-skip draft from its target's: both were empty and the target has been fed, so the draft's layers hold
-// the target's first layers' keys and values.  grid (16-row blocks of the longest prompt, H, 2 B layers), 16-byte pieces.
-__global__ void __launch_bounds__(256) kv_adopt_kernel(const uint8_t *src, uint8_t *dst, const int32_t *src_len, int B, int src_S,
-                                                       int dst_S, int row_bytes) {
+// the target's first layers' keys and values.  The host knows that from its bounds; a sequence whose lengths say otherwise
+// (someone wrote the slab) is left as it is, and the draft's status says SSD_E_ARG.
+// grid (16-row blocks of the longest prompt, H, 2 B layers), 16-byte pieces.
+__global__ void __launch_bounds__(256) kv_adopt_kernel(const uint8_t *src, uint8_t *dst, const int32_t *src_len, const int32_t *dst_len,
+                                                       int max_tokens, int B, int src_S, int dst_S, int row_bytes) {
     const int plane = blockIdx.z, b = (plane >> 1) % B;   // plane = (layer B + b) 2 + K|V
+    if (dst_len[b] != 0 || src_len[b] > max_tokens) return;
     const int rows = min(min(src_len[b], dst_S) - (int)blockIdx.x * 16, 16);
     if (rows <= 0) return;
     const size_t head = (size_t)plane * gridDim.y + blockIdx.y;
@@ -834,12 +837,14 @@ __global__ void __launch_bounds__(256) kv_adopt_kernel(const uint8_t *src, uint8
     for (int i = threadIdx.x; i < rows * row_bytes / 16; i += 256) d[i] = s[i];
 }
 // ... and its lengths (one block of 64 threads)
-__global__ void kv_adopt_len_kernel(const int32_t *src_len, const int32_t *src_status, int32_t *len, int32_t *status, int B, int S,
-                                    unsigned long long *mailbox, unsigned seq) {
+__global__ void kv_adopt_len_kernel(const int32_t *src_len, const int32_t *src_status, int32_t *len, int32_t *status, int max_tokens,
+                                    int B, int S, unsigned long long *mailbox, unsigned seq) {
     const int b = threadIdx.x;
     if (b == 0 && *src_status != 0) set_status(status, *src_status);
     if (b < B) {
-        const int v = min(src_len[b], S);
+        const bool empty = len[b] == 0 && src_len[b] <= max_tokens;
+        if (!empty) set_status(status, -1);
+        const int v = empty ? min(src_len[b], S) : len[b];
         len[b] = v;
         report_len(mailbox, b, seq, v);
     }

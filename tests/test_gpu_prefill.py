@@ -253,3 +253,73 @@ def test_prompt_pass_of_a_target_and_a_draft_of_its_own():
         B.kv_prefill(m, kv, prompts, n, ws)
         assert got.lengths().tolist() == kv.lengths().tolist() == [20, 7]
         _cache_close(arch, *(k.cache_view()[:, 0, :, :, :20].float().cpu().numpy() for k in (got, kv)))
+
+
+def _layer_skip_pair():
+    arch = synth.llama_like(3, 256, 4, 512, 512)
+    target = B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, 51, 6.0)))
+    return arch, target, target.share_prefix(1)
+
+
+def _prompt(seed, n, vocab):
+    return torch.from_numpy(synth.gen_prompt(seed, 2, n, vocab)).cuda(), torch.full((2,), n, dtype=torch.int32, device="cuda")
+
+
+def _rows_close(kv, ref, n):
+    got, want = (k.cache_view()[..., :n, :].float() for k in (kv, ref))
+    assert ((got - want).abs() <= gu.LOGIT_ATOL + gu.LOGIT_RTOL * want.abs().amax(-1, keepdim=True)).all()
+
+
+def test_prompt_pair_after_a_slab_copy_does_not_take_the_cache_for_an_empty_one():
+    """Lengths that a copy of another cache's slab brought (no kernel reported them) and kv_lengths has read: the draft's
+    prompt is computed, not taken over from a target cache that holds more than it."""
+    arch, target, draft = _layer_skip_pair()
+    S = 96
+    ws_t, ws_d = target.new_workspace(2, 8, S), draft.new_workspace(2, 8, S)
+    first, second = _prompt(1, 20, arch.vocab), _prompt(2, 12, arch.vocab)
+    full, tkv, dkv, alone = B.KV(target, 2, S), B.KV(target, 2, S), B.KV(draft, 2, S), B.KV(draft, 2, S)
+    B.kv_prefill(target, full, *first, ws_t)
+    zero = torch.zeros(2, dtype=torch.int32, device="cuda")
+    B.kv_rollback(tkv, zero)
+    B.kv_rollback(dkv, zero)
+    torch.cuda.synchronize()
+    tkv.buf.copy_(full.buf)
+    assert tkv.lengths().tolist() == [20, 20] and dkv.lengths().tolist() == [0, 0]
+    B.kv_prefill_pair(target, tkv, draft, dkv, *second, ws_t, ws_d)
+    assert tkv.lengths().tolist() == [32, 32] and dkv.lengths().tolist() == [12, 12]
+    assert tkv.status() == 0 and dkv.status() == 0
+    B.kv_prefill(draft, alone, *second, ws_d)
+    _rows_close(dkv, alone, 12)
+
+
+def test_prompt_pair_over_a_slab_written_behind_the_library_is_refused():
+    """The same copy without kv_lengths: the host's bound still says empty; the device sees that it is not."""
+    arch, target, draft = _layer_skip_pair()
+    S = 96
+    ws_t, ws_d = target.new_workspace(2, 8, S), draft.new_workspace(2, 8, S)
+    full, tkv, dkv = B.KV(target, 2, S), B.KV(target, 2, S), B.KV(draft, 2, S)
+    B.kv_prefill(target, full, *_prompt(1, 20, arch.vocab), ws_t)
+    tkv.buf.copy_(full.buf)
+    B.kv_prefill_pair(target, tkv, draft, dkv, *_prompt(2, 12, arch.vocab), ws_t, ws_d)
+    assert tkv.lengths().tolist() == [32, 32] and tkv.status() == 0
+    assert dkv.status() == -1 and dkv.lengths().tolist() == [0, 0]
+
+
+def test_recorded_prompt_pair_extends_both_caches_at_every_replay():
+    """A pair call recorded on empty caches and replayed twice: the second replay's prompt follows the first one's in both."""
+    arch, target, draft = _layer_skip_pair()
+    S, n = 96, 12
+    ws_t, ws_d = target.new_workspace(2, 8, S), draft.new_workspace(2, 8, S)
+    prompt = _prompt(3, n, arch.vocab)
+    tkv, dkv, alone = B.KV(target, 2, S), B.KV(draft, 2, S), B.KV(draft, 2, S)
+    for _ in range(2):
+        B.kv_prefill(draft, alone, *prompt, ws_d)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        B.kv_prefill_pair(target, tkv, draft, dkv, *prompt, ws_t, ws_d)
+    graph.replay()
+    graph.replay()
+    assert tkv.lengths().tolist() == dkv.lengths().tolist() == [2 * n, 2 * n]
+    assert tkv.status() == 0 and dkv.status() == 0
+    _rows_close(dkv, alone, 2 * n)
