@@ -1623,7 +1623,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
                     float mine = -INFINITY;
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
-                        const float mx = warp_max_redux(8 * blk + i >= first ? hi[i] + lo[i] : -INFINITY);
+                        const float mx = warp_max_redux(8 * blk + i >= first ? fmaxf(hi[i] + lo[i], -INFINITY) : -INFINITY);  // (no NaN)
                         mine = lane == i ? mx : mine;
                     }
                     if (lane < 8) wmax[warp * RP + 8 * blk + lane] = mine;
@@ -1667,8 +1667,8 @@ __device__ __noinline__ void attention_items_tc(int layer) {
                 __nv_bfloat16 hv[4], lv[4];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
-                    // (a row that has seen nothing yet: reference -inf, every score -inf)
-                    const float pv = v[r4 + i] > -INFINITY ? exp2_approx(v[r4 + i] - m[i]) : 0.f;
+                    // (a row that has seen nothing yet: reference -inf, every score -inf; a NaN score reaches the row's sum)
+                    const float pv = v[r4 + i] != -INFINITY ? exp2_approx(v[r4 + i] - m[i]) : 0.f;
                     l[r4 + i] += pv;
                     hv[i] = __float2bfloat16_rn(pv);
                     lv[i] = __float2bfloat16_rn(pv - __bfloat162float(hv[i]));

@@ -153,3 +153,36 @@ def _forward_over_seeded_cache(arch, lens, M, mode, scale=6.0):
         g, r = cache[:, b, :, :, n0:n1], oc.kv[:, :, :, n0:n1]
         assert (np.abs(g - r) <= gu.LOGIT_RTOL * np.abs(r) + gu.LOGIT_ATOL).all()
         assert np.array_equal(cache[:, b, :, :, :n0], fill_f[:, b, :, :, :n0])   # committed rows untouched
+
+
+@pytest.mark.parametrize("M", [9, 20])      # up to 16 rows, and more
+def test_a_key_that_is_not_a_number_is_not_passed_over(M):
+    """One NaN among the keys a head sees: its scores are NaN, so the head contributes nothing to any row, in the tensor-core
+    items as in the warp-MMA ones (one split of one tile in both)."""
+    from tests import gpu_util as gu
+    arch = synth.llama_like(2, 256, 2, 512, 512)
+    model = B.Model(arch, B.upload_weights(arch, gu.scaled_weights(synth, arch, 11, 6.0)))
+    dev, n, S = "cuda", 40, 128
+    rows = torch.from_numpy(synth.gen_prompt(13, 1, M, arch.vocab)).to(dev)
+    fill = synth.gen_kv_fill(12, (arch.n_layers, 1, 2, arch.n_heads, S, arch.head_dim), arch.dtype)
+    got = {}
+    for mode in (1, 2):
+        for bad in (False, True):
+            kv, ws = B.KV(model, 1, S), model.new_workspace(1, M, S)
+            kv.cache_view().copy_(torch.from_numpy(fill.view(np.int16)).to(dev).view(torch.bfloat16))
+            if bad:
+                kv.cache_view()[0, 0, 0, 1, 5, 3] = float("nan")
+            B.kv_commit(kv, torch.tensor([n], dtype=torch.int32, device=dev))
+            kv.lengths()
+            out = [torch.zeros(1, dtype=torch.int32, device=dev) for _ in range(2)]
+            q, u = torch.full((1, M - 1, arch.vocab), 1.0 / arch.vocab, device=dev), torch.full((1, M), 0.5, device=dev)
+            B.set_attention_mode(mode)
+            try:
+                B.target_verify(model, kv, rows, M - 1, q, u, 1.0, out[0], out[1], 1, None, ws)
+                got[mode, bad] = B.last_logits(model, 1, M, ws).cpu().numpy()[0]
+            finally:
+                B.set_attention_mode(0)
+            assert kv.status() == 0
+    gu.assert_logits_close(got[2, False], got[1, False])
+    assert np.isfinite(got[1, True]).all() and np.abs(got[1, True] - got[1, False]).max() > 0.1
+    gu.assert_logits_close(got[2, True], got[1, True])
