@@ -24,13 +24,22 @@
 namespace ssd {
 
 constexpr int kFfThreads = 512, kFfWarps = kFfThreads / 32;
-constexpr int kFfRows = 8;              // activation rows a warp sums at a time
+constexpr int kFfRows = 8;              // activation rows a warp sums at a time, query rows an attention item walks its positions for
 constexpr int kFfMaxLayers = 32;        // (their tensors' addresses ride in the kernel parameters)
 constexpr int kFfMaxSmem = 200 * 1024;
 constexpr int kFfChunk = 256;           // positions per attention step
-// An item walks its positions alone: beyond this many the stepwise path's split over CTAs is the faster form
-// (a 256-position step costs about 3 us, the split path's three launches about 20).
-constexpr int kFfMaxCtx = 1536;
+// An item walks its positions alone (6.5 us per 256 of them and layer at head 64, 20 at head 128, half as much again per further
+// block of eight rows); beyond this many the stepwise path, which splits them over CTAs, is the faster form.  What the one kernel
+// saves elsewhere grows with the rows of the pass and with the width.  us a layer, one kernel / stepwise: head 128, d 512, one
+// row at 700 positions 91 / 92, at 1000 117 / 97; five rows at 1000 128 / 147; head 64, d 64, nine rows at 700 89 / 99, at
+// 1300 122 / 104.
+// (From 32 items on the split path's share of an SM is no smaller.)
+inline int ff_max_ctx(int d, int Dh, int H, int B, int M) {
+    if (B * H >= 32) return 1536;
+    const double one = 64.0 / Dh * (1280.0 + (d > 256 ? 0.5 * (d - 256) : 0.0)), per_row = 30.0 + 0.3 * d * 64.0 / Dh;
+    const double most = (one + per_row * (B * M - 1)) / (1.0 + 0.6 * ((M - 1) / kFfRows));
+    return most < 1536.0 ? (int)most : 1536;
+}
 
 struct FfLayer {
     const float *ln1_g, *ln1_b, *w_qkv, *b_qkv, *w_o, *b_o, *ln2_g, *ln2_b, *w_in, *b_in, *w_out, *b_out;
@@ -59,7 +68,7 @@ struct FfParams {
 inline size_t ff_smem(int d, int F, int M, int Dh) {
     const size_t gemm = (size_t)kFfRows * (d > F ? d : F) * 4;
     const size_t groups = kFfThreads / Dh;
-    const size_t attn = ((size_t)M * Dh + (size_t)M * kFfChunk + 3 * (size_t)M + groups * M * Dh) * 4;
+    const size_t attn = ((size_t)M * Dh + (size_t)kFfRows * kFfChunk + 3 * (size_t)kFfRows + groups * kFfRows * Dh) * 4;
     return gemm > attn ? gemm : attn;
 }
 
@@ -253,12 +262,12 @@ __device__ __forceinline__ void ff_stage(const FfParams &p, int rb, const float 
     __syncthreads();
 }
 
-// Attention of one (sequence, head): rotary, append, scores, softmax, P V.  MR bounds the rows per sequence.
-template <int MR>
+// Attention of one (sequence, head): rotary, append, then scores, softmax and P V for eight rows at a time (their sums live in
+// registers: arrays for all 32 rows a pass may have went through the stack, 50 us per 256 positions where eight rows take 8).
 __device__ __forceinline__ void ff_attention(const FfParams &p, int layer, int item, bool append_only, float *smem) {
     const int b = item / p.H, h = item % p.H, Dh = p.Dh, d = p.d, M = p.M, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = p.ri.n_eff[b], len = p.len[b], r0 = b * M, half = p.rotary_dim / 2;
-    float *qs = smem, *sc = qs + M * Dh, *fac = sc + M * kFfChunk, *run_m = fac + M, *run_l = run_m + M, *red = run_l + M;
+    float *qs = smem, *sc = qs + M * Dh, *fac = sc + kFfRows * kFfChunk, *run_m = fac + kFfRows, *run_l = run_m + kFfRows, *red = run_l + kFfRows;
     float *kc = p.cache + (size_t)layer * p.layer_elems + ((size_t)(b * 2) * p.H + h) * p.S * Dh;
     float *vc = kc + (size_t)p.H * p.S * Dh;
     for (int i = tid; i < M * Dh; i += kFfThreads) {
@@ -279,47 +288,49 @@ __device__ __forceinline__ void ff_attention(const FfParams &p, int layer, int i
         }
     }
     if (append_only) return;
-    if (tid < M) { run_m[tid] = -INFINITY; run_l[tid] = 0.f; }
     const int groups = kFfThreads / Dh, ge = tid % Dh, gi = tid / Dh;
-    float o[MR];
+#pragma unroll 1
+    for (int m0 = 0; m0 < M; m0 += kFfRows) {
+    const int rows = min(kFfRows, M - m0), nb = max(0, min(n - m0, kFfRows)), end = nb > 0 ? len + m0 + nb : 0;
+    if (tid < kFfRows) { run_m[tid] = -INFINITY; run_l[tid] = 0.f; }
+    float o[kFfRows];
 #pragma unroll
-    for (int m = 0; m < MR; ++m) o[m] = 0.f;
-    const int end = len + n;
-    __syncthreads();  // the appended rows are read back through the cache
+    for (int m = 0; m < kFfRows; ++m) o[m] = 0.f;
+    __syncthreads();  // (the first time:) the appended rows are read back through the cache
     for (int t0 = 0; t0 < end; t0 += kFfChunk) {
         const int np = min(kFfChunk, end - t0);
         // scores: four lanes per position, each a quarter of the head in 16-byte pieces
         for (int pp = tid >> 2; pp < ((np + 7) & ~7); pp += kFfThreads / 4) {
             const int quarter = tid & 3;
-            float s[MR];
+            float s[kFfRows];
 #pragma unroll
-            for (int m = 0; m < MR; ++m) s[m] = 0.f;
+            for (int m = 0; m < kFfRows; ++m) s[m] = 0.f;
             if (pp < np) {
                 const float4 *k4 = reinterpret_cast<const float4 *>(kc + (size_t)(t0 + pp) * Dh);
 #pragma unroll 4
                 for (int i = quarter; i < Dh / 4; i += 4) {
                     const float4 k = k4[i];
 #pragma unroll
-                    for (int m = 0; m < MR; ++m) {
-                        if (m < n) {
-                            const float4 q = reinterpret_cast<const float4 *>(qs + m * Dh)[i];
+                    for (int m = 0; m < kFfRows; ++m) {
+                        if (m < nb) {
+                            const float4 q = reinterpret_cast<const float4 *>(qs + (m0 + m) * Dh)[i];
                             s[m] = fmaf(q.x, k.x, fmaf(q.y, k.y, fmaf(q.z, k.z, fmaf(q.w, k.w, s[m]))));
                         }
                     }
                 }
             }
 #pragma unroll
-            for (int m = 0; m < MR; ++m) {
-                if (m < n) {
+            for (int m = 0; m < kFfRows; ++m) {
+                if (m < nb) {
                     float v = s[m];
                     v += __shfl_xor_sync(0xffffffffu, v, 1);
                     v += __shfl_xor_sync(0xffffffffu, v, 2);
-                    if (quarter == (m & 3) && pp < np) sc[m * kFfChunk + pp] = t0 + pp <= len + m ? v : -INFINITY;
+                    if (quarter == (m & 3) && pp < np) sc[m * kFfChunk + pp] = t0 + pp <= len + m0 + m ? v : -INFINITY;
                 }
             }
         }
         __syncthreads();
-        for (int m = warp; m < n; m += kFfWarps) {  // running softmax statistics: one warp per row
+        for (int m = warp; m < nb; m += kFfWarps) {  // running softmax statistics: one warp per row
             float v[kFfChunk / 32], mx = run_m[m];
             const float old = mx;
 #pragma unroll
@@ -346,35 +357,36 @@ __device__ __forceinline__ void ff_attention(const FfParams &p, int layer, int i
         __syncthreads();
         if (gi < groups) {
 #pragma unroll
-            for (int m = 0; m < MR; ++m)
-                if (m < n) o[m] *= fac[m];
+            for (int m = 0; m < kFfRows; ++m)
+                if (m < nb) o[m] *= fac[m];
 #pragma unroll 4
             for (int pp = gi; pp < np; pp += groups) {
                 const float v = vc[(size_t)(t0 + pp) * Dh + ge];
 #pragma unroll
-                for (int m = 0; m < MR; ++m)
-                    if (m < n) o[m] = fmaf(sc[m * kFfChunk + pp], v, o[m]);
+                for (int m = 0; m < kFfRows; ++m)
+                    if (m < nb) o[m] = fmaf(sc[m * kFfChunk + pp], v, o[m]);
             }
         }
         __syncthreads();  // the scores are overwritten by the next step
     }
     if (gi < groups) {
 #pragma unroll
-        for (int m = 0; m < MR; ++m)
-            if (m < n) red[((size_t)gi * M + m) * Dh + ge] = o[m];
+        for (int m = 0; m < kFfRows; ++m)
+            if (m < nb) red[(gi * kFfRows + m) * Dh + ge] = o[m];
     }
     __syncthreads();
-    for (int i = tid; i < M * Dh; i += kFfThreads) {
+    for (int i = tid; i < rows * Dh; i += kFfThreads) {
         const int m = i / Dh, e = i % Dh;
         float v = 0.f;
-        if (m < n) {
-            for (int k = 0; k < groups; ++k) v += red[((size_t)k * M + m) * Dh + e];
+        if (m < nb) {
+            for (int k = 0; k < groups; ++k) v += red[(k * kFfRows + m) * Dh + e];
             const float L = run_l[m];
             v = L > 0.f ? v / L : 0.f;
         }
-        p.ao[(size_t)(r0 + m) * d + h * Dh + e] = v;
+        p.ao[(size_t)(r0 + m0 + m) * d + h * Dh + e] = v;
     }
     __syncthreads();
+    }
 }
 
 // The steps of a pass.  Sequential layer: qkv | attention | out-projection | MLP in | MLP out; parallel-residual layer: qkv, MLP in |
@@ -417,7 +429,6 @@ __device__ __forceinline__ void ff_out(const FfParams &p, const FfStep &s, int n
     }
 }
 
-template <int MR>
 __device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatile int &ok) {
     const float4 *xs4 = reinterpret_cast<const float4 *>(xs);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, r8 = lane >> 2;
@@ -475,7 +486,7 @@ __device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatil
         const bool last = i >= 5 * (p.n_layers - 1) && !p.want_logits;  // of the last layer only the keys and values are wanted
         bool fetched = true;                                            // this warp's first columns
         if (s.kind == FS_ATTN) {
-            for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention<MR>(p, i / 5, item, last, xs);
+            for (int item = blockIdx.x; item < p.B * p.H; item += gridDim.x) ff_attention(p, i / 5, item, last, xs);
             if (last) return;
         } else if (!(last && s.kind == FS_IN)) {
 #pragma unroll 1
@@ -526,11 +537,10 @@ __device__ __forceinline__ void ff_forward(const FfParams &p, float *xs, volatil
 // (The same kernel as one cluster of 16 CTAs, with the cluster's hardware barrier instead of the counter in L2, gains what the
 // barriers cost and loses it again to 16 SMs' share of the projections: 124 us for four layers and 5 rows against 128 on 64
 // CTAs, 31 against 30 for one layer and one row.)
-template <int MR>
 __global__ void __launch_bounds__(kFfThreads, 1) forward_f32_kernel(const __grid_constant__ FfParams p) {
     extern __shared__ __align__(16) float ff_smem_[];
     __shared__ volatile int ok;
-    ff_forward<MR>(p, ff_smem_, ok);
+    ff_forward(p, ff_smem_, ok);
     __syncthreads();
     if (threadIdx.x == 0) leave_grid(p.gbar);
 }

@@ -163,8 +163,7 @@ int init_device(int dev, DeviceInfo &info) {
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 8>, attn_smem<__nv_bfloat16, 8>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 16>, attn_smem<__nv_bfloat16, 16>(128));
     rc |= set_smem(attn_partial_kernel<__nv_bfloat16, 32>, attn_smem<__nv_bfloat16, 32>(128));
-    rc |= set_smem(forward_f32_kernel<8>, kFfMaxSmem);
-    rc |= set_smem(forward_f32_kernel<kMaxRowsPerSeq>, kFfMaxSmem);
+    rc |= set_smem(forward_f32_kernel, kFfMaxSmem);
     rc |= set_smem(prefill_gemm_kernel, kPfSmem);
     rc |= set_smem(prefill_attn_kernel, prefill_attn_smem(128));
     rc |= set_smem(prefill_attn_tc_kernel, kPtSmem);
@@ -698,7 +697,7 @@ bool single_kernel_path(const ssd_model *m) {
 // fp32 models whose row blocks fit shared memory, with contexts that one CTA walks quickly (see f32_forward.cuh)
 bool f32_kernel_path(const ssd_model *m, ssd_kv *kv, int M) {
     const ssd_arch &a = m->a;
-    return a.dtype == 0 && g_persistent && a.n_layers <= kFfMaxLayers && a.d_ff % 4 == 0 && kv_bound(kv) + M <= kFfMaxCtx &&
+    return a.dtype == 0 && g_persistent && a.n_layers <= kFfMaxLayers && a.d_ff % 4 == 0 && kv_bound(kv) + M <= ff_max_ctx(a.d_model, a.head_dim, a.n_heads, kv->B, M) &&
            ff_smem(a.d_model, a.d_ff, M, a.head_dim) <= (size_t)kFfMaxSmem && m->aligned16;
 }
 
@@ -738,8 +737,7 @@ int forward_f32(ssd_model *m, ssd_kv *kv, const int32_t *tokens, int tok_stride,
     const int rc = device_info(&info);
     if (rc) return rc;
     if (grid > info->num_sms) grid = info->num_sms;
-    const void *k = M <= 8 ? (const void *)forward_f32_kernel<8> : (const void *)forward_f32_kernel<kMaxRowsPerSeq>;
-    CUDA_OK(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kFfThreads), args, smem, st));
+    CUDA_OK(cudaLaunchCooperativeKernel((const void *)forward_f32_kernel, dim3(grid), dim3(kFfThreads), args, smem, st));
     g_launches.fetch_add(1, std::memory_order_relaxed);
     kv->last_rows = M;
     return SSD_OK;

@@ -282,3 +282,34 @@ def test_embedding_rows_in_sixteen_byte_pieces_and_unaligned(d, H):
         assert kv.status() == 0
         for b in range(2):
             gu.assert_logits_close(got[b], omodel.new_cache(16).feed(rows[b], advance=False))
+
+
+@pytest.mark.parametrize("arch,M,lens", [
+    (synth.llama_like(2, 256, 2, 512, 300, dtype=synth.DT_F32), 1, (630, 650)),       # head 128: up to 640 positions for one row
+    (synth.neox_like(2, 64, 1, 128, 130, dtype=synth.DT_F32), 9, (1000, 1100)),       # head 64, nine rows: up to 1045
+    (synth.neox_like(1, 256, 32, 128, 130, dtype=synth.DT_F32), 2, (1500, 1540)),     # 32 heads: up to 1536
+])
+def test_fp32_passes_leave_the_one_kernel_form_where_its_items_walk_too_long(arch, M, lens):
+    """A pass below the crossover is one launch and the tail's, one beyond it the stepwise path's many; both give the same
+    logits as the other form."""
+    ws_np = gu.scaled_weights(synth, arch, 41, 4.0)
+    model = B.Model(arch, B.upload_weights(arch, ws_np))
+    rows = synth.gen_prompt(43, 1, M, arch.vocab)
+    S = max(lens) + M + 6
+    fill = torch.from_numpy(synth.gen_kv_fill(12, (arch.n_layers, 1, 2, arch.n_heads, S, arch.head_dim), arch.dtype)).cuda()
+    for n, one in zip(lens, (True, False)):
+        res, launches = [], []
+        for on in (True, False):
+            B.set_persistent(on)
+            try:
+                kv, ws = B.KV(model, 1, S), model.new_workspace(1, M, S)
+                kv.cache_view().copy_(fill)
+                B.kv_commit(kv, torch.tensor([n], dtype=torch.int32, device="cuda"))
+                assert kv.lengths().tolist() == [n]
+                n0 = B.launch_count()
+                res.append(gpu_logits(model, kv, ws, rows, M - 1))
+                launches.append(B.launch_count() - n0)
+                assert kv.status() == 0
+            finally:
+                B.set_persistent(True)
+        assert (launches[0] < launches[1]) == one and np.abs(res[0] - res[1]).max() <= 1e-3
