@@ -1300,6 +1300,17 @@ constexpr int kTailSmallV = 32 * kTailCluster * kTailWarps, kTailMediumV = 4 * k
 static bool restricted(float temperature, int V) {  // (a greedy row is its own restriction)
     return temperature > 0.f && ((g_top_k > 0 && g_top_k < V) || (g_top_p > 0.f && g_top_p < 1.f));
 }
+// Whether the rows of a verification are worth a cluster each and a launch of their own (row_stats_kernel), instead of one
+// cluster that walks a sequence's K + 1 rows in front of its accept scan.  The walk costs `row` us a row, whatever the batch; the
+// second launch and its hand-over cost about as much as 10 us of it, and what the rows apart gain shrinks as the clusters of
+// all sequences fill the GPU.  us a call, together / apart: 50304 entries, sampled, exported, one sequence: 5 rows 23 / 19,
+// 17 rows 54 / 21; 8 sequences x 17 rows 54 / 43; 5 rows of 32000, not exported, 13 / 15; 5 rows of 100000 27 / 21.
+static bool rows_apart(int B, int K, int V, bool sampled, bool exported) {
+    const float step = V <= kTailSmallV ? 0.3f : V <= kTailMediumV ? 0.4f : 0.65f * (float)ceil_div(V, 8 * kTailSmallV);
+    const float row = step * (sampled ? 2.f : 1.f) * (exported ? 2.f : 1.f);
+    const int most = V <= kTailMediumV ? 5 : 10;  // sequences
+    return B < most && (float)(K + 1) * row * (float)(most - B) > 10.f * (float)most;
+}
 static int run_row_filter(const float *logits, int B, int M, int V, const int32_t *n_eff, float temperature, RowStat *stats,
                           RowFilter *filt, float *p_out, cudaStream_t st) {
     static DeviceTable<bool> devices;  // (on supplied logits the tail may be a program's first call on the device)
@@ -1397,9 +1408,21 @@ static int run_verify_tail(const float *logits, int B, int K, int V, const int32
     v.inv_t = temperature > 0.f ? 1.0f / temperature : 0.f;
     v.n_accepted = n_acc; v.next_token = next; v.next_stride = next_stride;
     v.p_debug = p_debug; v.keep = keep; v.stats = stats; v.filt = filt;
-    if (restricted(temperature, V)) {
-        const int rc = run_row_filter(logits, B, K + 1, V, nullptr, temperature, stats, filt, p_debug, st);
-        if (rc) return rc;
+    const bool apart = !restricted(temperature, V) && stats && rows_apart(B, K, V, temperature > 0.f, p_debug != nullptr);
+    if (apart || restricted(temperature, V)) {
+        if (apart) {
+            FilterArgs f;
+            memset(&f, 0, sizeof(f));
+            f.logits = logits; f.M = K + 1; f.V = V; f.inv_t = v.inv_t;
+            f.stats = stats; f.filt = filt; f.p_out = p_debug;
+            const dim3 grid(kTailCluster * (K + 1), B);
+            if (V <= kTailSmallV) { LAUNCH(row_stats_kernel<1>, grid, kTailThreads, 0, st, f); }
+            else if (V <= kTailMediumV) { LAUNCH(row_stats_kernel<4>, grid, kTailThreads, 0, st, f); }
+            else { LAUNCH(row_stats_kernel<8>, grid, kTailThreads, 0, st, f); }
+        } else {
+            const int rc = run_row_filter(logits, B, K + 1, V, nullptr, temperature, stats, filt, p_debug, st);
+            if (rc) return rc;
+        }
         if (V <= kTailSmallV) { LAUNCH((verify_kernel<true, 1>), B * kTailCluster, kTailThreads, 0, st, v); }
         else if (V <= kTailMediumV) { LAUNCH((verify_kernel<true, 4>), B * kTailCluster, kTailThreads, 0, st, v); }
         else { LAUNCH((verify_kernel<true, 8>), B * kTailCluster, kTailThreads, 0, st, v); }

@@ -485,6 +485,39 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     cl.sync();  // nobody leaves while its shared memory is read
 }
 
+// The unrestricted counterpart, a cluster of eight per row: grid (kTailCluster M, B).  Taken where one cluster per sequence would
+// walk the rows for longer than a second launch costs (see rows_apart in the host code).
+template <int IT>
+__global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThreads) row_stats_kernel(FilterArgs a) {
+    __shared__ StatSmem ss;
+    cg::cluster_group cl = cg::this_cluster();
+    const int i = blockIdx.x / kTailCluster, b = blockIdx.y, V = a.V, rank = (int)cl.block_rank(), lane = threadIdx.x & 31;
+    const size_t row = (size_t)b * a.M + i;
+    const float *lg = a.logits + row * V;
+    float l[IT];
+    cluster_stats<IT>(lg, 1, V, a.inv_t, &ss, cl, l);
+    const RowStat st = ss.row[0];
+    if (rank == 0 && threadIdx.x == 0) {
+        a.stats[row] = st;
+        a.filt[row].thr = a.filt[row].mass = 0.f;
+    }
+    if (a.p_out) {
+        int lo, hi;
+        tail_piece(V, rank, lo, hi);
+        const bool one = hi - lo <= 32 * IT;
+        float *p = a.p_out + row * V;
+        for (int base = lo; base < hi; base += 32 * IT) {
+            if (!one) tail_load<IT>(lg, base, hi, 0.f, l);
+#pragma unroll
+            for (int k = 0; k < IT; ++k) {
+                const int j = base + lane + 32 * k;
+                if (j < hi) p[j] = prob_of(l[k], st, a.inv_t, j);
+            }
+        }
+    }
+    cl.sync();  // nobody leaves while its shared memory is read
+}
+
 // ---- inverse-CDF draw -------------------------------------------------------------------------------
 struct DrawSmem {
     double tot[kTailWarps], incl[kTailWarps];  // the warps' sums, and their running sums

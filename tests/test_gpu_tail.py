@@ -295,3 +295,26 @@ def test_a_run_of_nans_makes_the_whole_row_not_a_number(V, n_bad, top_k):
     assert nxt[0] == int(np.argmax(np.where(bad, -np.inf, logits[0, 0])))
     assert np.isfinite(p[1]).all()
     gu.check_decisions_on_own_rows(p[1], q[1], rows[1, 1:], u[1, :1], u[1, 1], int(n_acc[1]), int(nxt[1]))
+
+
+@pytest.mark.parametrize("T", [0.0, 0.8])
+@pytest.mark.parametrize("V,Bn,K,want_p", [
+    (1000, 1, 4, True), (8192, 1, 31, True), (8193, 4, 31, True), (32769, 2, 12, True), (50304, 1, 8, False), (50304, 9, 16, True),
+    (65537, 2, 7, False), (131100, 3, 5, True),
+])
+def test_rows_in_clusters_of_their_own_give_the_same_bits(V, Bn, K, want_p, T):
+    """The same verification with its rows walked by one cluster (the entry point without scratch always does) and, from some
+    number of rows on, with a cluster per row in a launch before: equal decisions and p rows, bit for bit."""
+    logits, rows, q, u = make_case(5000 + V, Bn, K, V, T, True)
+    n0 = B.launch_count()
+    n_acc, nxt, p = run_tail(logits, rows, q, u, T, want_p)
+    launches = B.launch_count() - n0
+    dev = "cuda"
+    out = [torch.full((Bn,), -7, dtype=torch.int32, device=dev) for _ in range(2)]
+    p1 = torch.zeros(Bn, K + 1, V, device=dev) if want_p else None
+    B.verify_from_logits_noalloc(torch.from_numpy(logits).to(dev), K, torch.from_numpy(rows).to(dev),
+                                 torch.from_numpy(q).to(dev), torch.from_numpy(u).to(dev), T, out[0], out[1], 1, p1)
+    assert launches == (1 if (V, Bn) in ((1000, 1), (50304, 9)) or T == 0.0 and V in (8193, 50304, 65537) else 2)
+    assert out[0].cpu().numpy().tolist() == n_acc.tolist() and out[1].cpu().numpy().tolist() == nxt.tolist()
+    if want_p:
+        assert np.array_equal(p1.cpu().numpy(), p)
