@@ -77,22 +77,6 @@ __device__ __forceinline__ T block_sum(T v, T *scratch) {
     return t;
 }
 
-__device__ __forceinline__ float block_max(float v, float *scratch) {
-    int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    v = warp_max(v);
-    __syncthreads();
-    if (lane == 0) scratch[w] = v;
-    __syncthreads();
-    float t = (threadIdx.x < nw) ? scratch[threadIdx.x] : -INFINITY;
-    if (w == 0) {
-        t = warp_max(t);
-        if (lane == 0) scratch[0] = t;
-    }
-    __syncthreads();
-    t = scratch[0];
-    return t;
-}
-
 // Per-row bookkeeping of one forward, filled by setup_rows_kernel.
 struct RowInfo {
     int32_t *seq;    // [R] sequence of row r

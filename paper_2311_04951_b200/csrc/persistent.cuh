@@ -325,24 +325,10 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t adesc, uin
         "}\n" ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// 16 lanes x 32 columns of the accumulator (the 16-lane x 256-bit shape, four times along the columns).
-// Thread (g = lane / 4, t = lane % 4) receives, for column block k = 0..3: v[4k], v[4k+1] = lane g,
+// 16 lanes x 64 columns of the accumulator (the 16-lane x 256-bit shape, eight times along the columns).
+// Thread (g = lane / 4, t = lane % 4) receives, for column block k = 0..7: v[4k], v[4k+1] = lane g,
 // columns 8k + 2t, 8k + 2t + 1 and v[4k+2], v[4k+3] = lane g + 8, the same columns.  The wait is part
 // of the same statement so that no use of the results can be scheduled before it.
-__device__ __forceinline__ void tc_ld_16x32(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
-        : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// the same shape eight times along the columns: 16 lanes x 64 columns in one round trip
 __device__ __forceinline__ void tc_ld_16x64(uint32_t taddr, float (&v)[32]) {
     uint32_t r[32];
     asm volatile(
@@ -660,7 +646,6 @@ __device__ __noinline__ void norm_phase(const float *g1, const float *b1, int op
 // The norm in front of layer l's first GEMM(s) - or of the LM head - and the zeroing of what they accumulate into.
 __device__ __noinline__ void norm_for_layer(int l) {
     const FwdParams &p = params_copy();
-    Shared *sh = shared_state();
     const float *const *lt = staged_ltab();
     if (l < p.n_layers) {
         const LayerDesc *ld = layer_desc(p.md, l);
@@ -678,7 +663,6 @@ __device__ __noinline__ void norm_for_layer(int l) {
 // ... and between the two halves of a sequential block.
 __device__ __noinline__ void norm_mid_layer(int l) {
     const FwdParams &p = params_copy();
-    Shared *sh = shared_state();
     const float *const *lt = staged_ltab();
     const LayerDesc *ld = layer_desc(p.md, l);
     norm_phase(lt ? lt[8 * l + 4] : ld->ln2_g, lt ? lt[8 * l + 5] : ld->ln2_b, OP_XN1, nullptr, nullptr, 0);
@@ -1241,10 +1225,6 @@ __device__ __noinline__ void attention_items(int layer) {
     }
 }
 
-__device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, bool valid) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-
 #include "attn_mma8.cuh"
 
 // ---- attention on tcgen05 (head dim 128) ----------------------------------------------------------
@@ -1268,7 +1248,6 @@ __device__ __forceinline__ void cp_async16_zfill(void *dst, const void *src, boo
 constexpr int kTcChunk = 128;
 constexpr int kTcStages = 4;  // K / V ring stages of 32 KB: the bytes in flight set the chunk rate (3 stages: 2.7 us per chunk)
 constexpr int kTcKvStage = kTcChunk * 128 * 2;  // one K or V chunk: two 64-column panels of 128 rows x 128 B
-__host__ __device__ constexpr int tc_rows_pad(int M) { return M <= 16 ? 16 : 32; }
 __host__ __device__ constexpr int tc_p_tiles(int rp) { return rp == 16 ? 2 : 1; }   // P tiles used in turn
 __host__ __device__ constexpr int tc_scratch_bytes(int rp) {  // ring, Q tile, P tiles, maxima and sums of four warps, references and factors
     return kTcStages * kTcKvStage + (1 + tc_p_tiles(rp)) * 2 * rp * 256 + 10 * rp * 4;
@@ -1325,19 +1304,6 @@ __device__ __forceinline__ void tc_ld_2x8(uint32_t ta, uint32_t tb, float (&a)[8
         : "memory");
 #pragma unroll
     for (int i = 0; i < 8; ++i) { a[i] = __uint_as_float(r[i]); b[i] = __uint_as_float(r[8 + i]); }
-}
-// one column from each of two places of this warp's lane quadrant
-__device__ __forceinline__ void tc_ld_2(uint32_t ta, uint32_t tb, float &a, float &b) {
-    uint32_t x, y;
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%2];\n"
-        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%1}, [%3];\n"
-        "tcgen05.wait::ld.sync.aligned;\n"
-        : "=r"(x), "=r"(y)
-        : "r"(ta), "r"(tb)
-        : "memory");
-    a = __uint_as_float(x);
-    b = __uint_as_float(y);
 }
 __device__ __forceinline__ void tc_st_32(uint32_t taddr, const float (&v)[32]) {
     asm volatile(
