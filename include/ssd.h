@@ -152,7 +152,7 @@ void kv_destroy(ssd_kv *kv);
  *  - bf16 models whose workspace holds ssd_prefill_workspace_bytes(m, batch, c) for some c with
  *    batch * c >= 256 rows take the many-row form: equal passes of up to 8192 / batch rows per sequence
  *    (the largest the workspace fits), every linear layer as a tiled tcgen05 GEMM over 128 rows x 256
- *    weight rows per CTA with the activations as bf16 hi + lo, causal attention over 64-row tiles
+ *    weight rows per CTA with the activations as bf16 hi + lo, causal attention over 128-row tiles
  *    against the cache.  Compute-bound; the arithmetic is that of the few-row passes up to fp32
  *    summation order.
  *  - otherwise chunks through the few-row forward: as many rows per sequence as SSD_MAX_ROWS / batch,
@@ -313,8 +313,10 @@ size_t verify_scratch_bytes(int batch, int K);
  * same tail for such callers.
  *
  * The tail is one kernel that keeps what its rows hand to each other in shared memory, so the call needs no
- * device memory of its own.  Inputs and outputs are the caller's.
- *   - batch * (K + 1) > SSD_NOALLOC_MAX_ROWS is refused with SSD_E_CAPACITY; nothing is launched.
+ * device memory of its own.  Inputs and outputs are the caller's.  (verify_from_logits gives many rows, exports and wide
+ * vocabularies a cluster per row, which needs its scratch; this call walks them one after the other.)
+ *   - batch * (K + 1) > SSD_NOALLOC_MAX_ROWS is refused with SSD_E_CAPACITY; nothing is launched (a limit of the
+ *     interface, kept for its callers: the kernel has none).
  *   - The call never calls cudaMalloc / cudaFree or any allocating routine.
  *   - SSD_E_UNIMPL while a sampling restriction is set (its threshold search needs scratch).
  * Results are identical to verify_from_logits.

@@ -10,8 +10,8 @@
 // vocabulary fills); what the warps find meets once in shared memory and once, through distributed shared memory, across
 // the cluster, always combined in the same order.  What bounds it is instruction issue on the cluster's few SMs and that
 // chain of exchanges, not the bytes: hence one kernel per verification, which carries the statistics of ALL rows of a
-// sequence through one exchange (one sequence, 5 rows of 32000: 21.6 us a call back to back with a cluster per row and a
-// second launch for the draw, now 14.3).
+// sequence through one exchange (one sequence, 5 rows of 32000: 20.8 us a call back to back with a cluster per row and a
+// second launch for the draw, 12.3 so), as long as the rows that follow one another cost less than a second launch.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -209,8 +209,8 @@ __device__ __forceinline__ void cluster_stats(const float *logits, int rows, int
 // A row is a cluster of TWO CTAs, its probabilities computed once and kept in their shared memory (up to kFilterCache of
 // them each): the histograms of two CTAs are joined with three remote loads per thread, where eight CTAs took 9 us per
 // pass for it and left most of 48 rows waiting for SMs.
-// 8 sequences x 6 rows x 50304 entries, top-k 50 and top-p 0.9, whole call: 573 us with byte-wide bins and fp64 atomics on
-// eight CTAs, 193 with these bins on eight, 55 on two.
+// 8 sequences x 6 rows x 50304 entries, top-k 50 and top-p 0.9, whole call: 565 us with byte-wide bins and fp64 atomics on
+// eight CTAs, 193 with these bins on eight, 53 on two.
 constexpr int kBins = 1024;
 constexpr int kFilterCluster = 2;
 constexpr int kFilterCache = 44 * 1024;     // probabilities a CTA keeps (176 KB)

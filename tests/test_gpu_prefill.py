@@ -132,7 +132,7 @@ def test_prompt_longer_than_the_cache_is_refused(many_row_mode):
 
 def test_many_row_prompt_pass_is_run_to_run_identical():
     """Nothing in the many-row pass depends on an order of arrival: the projections own their output tiles and a query
-    row's softmax and output belong to one thread.  Repeated passes over the same prompts must agree bit for bit (the
+    row's softmax and output belong to two threads that exchange one maximum per chunk.  Repeated passes over the same prompts must agree bit for bit (the
     tensor-core attention runs its warps up to a chunk apart; with several chunks per row tile and many CTAs a
     hand-over that miscounts shows up as other bits within a few passes)."""
     arch = synth.llama_like(2, 4096, 32, 512, 512)

@@ -2,11 +2,11 @@
 
 Some users of this library cannot allocate device memory around a call: a serving runtime that
 owns a fixed arena and forbids cudaMalloc once it is up, a decode loop where an allocation would
-stall the device, a binding that can forward pointers but not own buffers.  For them the library
-keeps the small scratch of the tail kernels in a fixed array of its own.  This test calls that
-entry point through the C ABI twice in a row (second call: other sizes and values, so leftovers of
-the first would show) and requires exactly the outputs of the ordinary entry point; it also checks
-that a request beyond the array's size is refused.  Collected last on purpose."""
+stall the device, a binding that can forward pointers but not own buffers.  For them the tail is one
+kernel that needs no scratch.  This test calls that entry point through the C ABI twice in a row
+(second call: other sizes and values, so leftovers of the first would show) and requires exactly the
+outputs of the ordinary entry point; it also checks that a request beyond the interface's limit of
+rows is refused.  Collected last on purpose."""
 import numpy as np
 import pytest
 import torch
