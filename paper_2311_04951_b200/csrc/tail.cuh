@@ -477,9 +477,11 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     }
     if (a.p_out) {
         float *p = a.p_out + row * V;
+        // (as prob_f; a row without mass is one of NaNs.  A test for that in the loop cost 2 of 36 us, 15 rows of 32000)
+        const float thr = f.mass == 0.f ? 0.f : f.thr, kept_mass = f.mass == 0.f ? 1.f : f.mass;
         for (int j = lo + lane; j < hi; j += 32) {
             const float pr = cached ? mine[j] : prob_of(__ldcg(lg + j), st, inv_t, j);
-            p[j] = f.mass == 0.f ? pr : pr >= f.thr ? pr / f.mass : 0.f;   // (as prob_f)
+            p[j] = pr < thr ? 0.f : pr / kept_mass;
         }
     }
     cl.sync();  // nobody leaves while its shared memory is read
@@ -573,7 +575,7 @@ __device__ __forceinline__ int cluster_draw(WeightFn weights, int V, float u, Dr
     if (!(S > 0.0)) return -1;
     const double beg = c_beg + w_beg, end = c_beg + w_end;  // (the last warp's end is c_beg + T, where the next CTA begins)
     double target = (double)u * S;
-    if (!(target < S)) {  // the same in all threads of the cluster
+    if (__builtin_expect(!(target < S), 0)) {  // the same in all threads of the cluster
         int mine = -1;
         for (int b = lo; b < hi; b += kStep) {
             weights(b, w);
