@@ -524,7 +524,6 @@ __global__ void __cluster_dims__(kTailCluster, 1, 1) __launch_bounds__(kTailThre
 struct DrawSmem {
     double tot[kTailWarps], incl[kTailWarps];  // the warps' sums, and their running sums
     double cta[2];              // this CTA's total, by draw (a kernel draws at most twice)
-    int last[kTailWarps], cta_last;  // largest index with weight > 0
     float w[32 * 8];            // the owner warp's entries, handed from its load order to index order
 };
 
@@ -575,25 +574,16 @@ __device__ __forceinline__ int cluster_draw(WeightFn weights, int V, float u, Dr
     if (!(S > 0.0)) return -1;
     const double beg = c_beg + w_beg, end = c_beg + w_end;  // (the last warp's end is c_beg + T, where the next CTA begins)
     double target = (double)u * S;
-    if (__builtin_expect(!(target < S), 0)) {  // the same in all threads of the cluster
-        int mine = -1;
-        for (int b = lo; b < hi; b += kStep) {
-            weights(b, w);
-#pragma unroll
-            for (int k = 0; k < IT; ++k)
-                if (w[k] > 0.f) mine = b + 32 * k + lane;
-        }
-        mine = __reduce_max_sync(0xffffffffu, mine);
-        if (lane == 0) ds->last[warp] = mine;
-        __syncthreads();
-        const int cta_last = __reduce_max_sync(0xffffffffu, ds->last[lane]);
-        if (threadIdx.x == 0) ds->cta_last = cta_last;
-        cl.sync();
-        const int last = __reduce_max_sync(0xffffffffu, lane < kTailCluster ? *cl.map_shared_rank(&ds->cta_last, lane) : -1);
-        return mine == last ? last : -1;
+    bool owner;
+    if (target < S) {
+        target = target < 0.0 ? 0.0 : target;
+        owner = beg <= target && target < end;
+    } else {  // (the same in all threads of the cluster) the last piece that weighs anything, walked to its end
+        const unsigned warps = __ballot_sync(0xffffffffu, ds->tot[lane] > 0.0), ctas = __ballot_sync(0xffffffffu, one_cta > 0.0);
+        owner = __clz(ctas) == 31 - rank && __clz(warps) == 31 - warp;
+        target = INFINITY;
     }
-    if (target < 0.0) target = 0.0;
-    if (!(beg <= target && target < end)) return -1;  // the same in all lanes
+    if (!owner) return -1;  // the same in all lanes
     double run = beg;
     int hit = -1, last = -1;
     for (int b = lo; b < hi && hit < 0; b += kStep) {
