@@ -268,12 +268,11 @@ __device__ __noinline__ void attention_items_mma8(int layer) {
     }
     if (!direct) {
         // ticket: the item that finishes last for this (sequence, head) merges all partials
-        __threadfence();
+        // (one release and one acquire for the CTA, as in the grid barrier)
         named_bar(3, kAttnThreadsP);
-        if (tid == 0) sh->flag = (atomicAdd(p.tickets + bh, 1u) == (unsigned)(p.n_split - 1));
+        if (tid == 0) sh->flag = (atomic_add_acq_rel(p.tickets + bh, 1u) == (unsigned)(p.n_split - 1));
         named_bar(3, kAttnThreadsP);
         if (sh->flag) {
-            __threadfence();
             merge_splits(p, r0, h, DH);
             if (tid == 0) p.tickets[bh] = 0;  // ready for the next layer (a grid barrier lies between)
         }

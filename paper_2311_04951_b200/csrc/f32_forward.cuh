@@ -85,8 +85,7 @@ __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, vola
     ++epoch;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        red_release_add(p.gbar, 1u);
+        red_release_add(p.gbar, 1u);  // (one release and one acquire: the CTA barriers pass them on)
         const unsigned target = epoch * gridDim.x;
         if (ld_acquire(p.gbar) < target) {
             const long long t0 = clock64();
@@ -98,7 +97,6 @@ __device__ __forceinline__ bool ff_sync(const FfParams &p, unsigned &epoch, vola
                 }
             }
         }
-        __threadfence();
         ff_stamp(p, epoch);
     }
     __syncthreads();
