@@ -532,21 +532,17 @@ int launch_forward_nt(FwdParams p, const void *ws_base, size_t ws_bytes, cudaStr
     const size_t attn = WIDE ? tc_scratch_bytes(32) : p.attn_form == ATT_TC16 ? tc_scratch_bytes(16)
                         : p.attn_form == ATT_PACKED ? m8_scratch_bytes(p.Dh) : align_up(attn_scratch_bytes(p.Dh), 128);
     const size_t total = (size_t)kSmemBudget - 1024 - sizeof(SharedBlock);
-    // upper slots share their bytes with the attention scratch; two slots never do where they fit
-    // (one with the 48 KB stages of 64 rows, which only the prompt pass uses)
-    size_t S2 = (attn + stage - 1) / stage;
-    size_t region2 = S2 * stage;
-    if (region2 + 2 * stage > total) {
-        S2 = attn / stage;
-        region2 = attn;
-    }
-    if (region2 + stage > total) return SSD_E_CAPACITY;
-    size_t S1 = (total - region2) / stage;
-    if (S1 + S2 > 32) S1 = 32 - S2;  // one parity bit per slot
-    p.stages = (int)(S1 + S2);
+    // As many slots as there is room for; the upper ones share their bytes with the attention scratch, which may reach beyond the
+    // last of them, and at least one does not.  (Two that never do, where that cost a slot: five slots instead of four under a
+    // 40-row pass of 7B, 5510 -> 5446 us, and under 9 rows of 2.7B, 1878 -> 1837.)
+    if (attn + stage > total) return SSD_E_CAPACITY;
+    size_t S = total / stage, S1 = (total - attn) / stage;
+    if (S > 32) S = 32;  // one parity bit per slot
+    if (S1 > S) S1 = S;
+    p.stages = (int)S;
     p.stages_lo = (int)S1;
     p.attn_smem_off = (int)(S1 * stage);
-    const size_t smem = 1024 + S1 * stage + region2;
+    const size_t smem = 1024 + (S * stage > S1 * stage + attn ? S * stage : S1 * stage + attn);
     const DeviceInfo *info;
     int rc = device_info(&info);
     if (rc) return rc;
