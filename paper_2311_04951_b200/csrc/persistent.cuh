@@ -148,7 +148,7 @@ struct GemmDesc {
     const __nv_bfloat16 *xop;  // tiled operand
     int N, Kd, n_tiles, kchunks;
     int need;  // grid barriers that must have completed before its operand exists
-    int need_hi;  // ... before its tiles may use the ring slots shared with the attention scratch
+    int need_hi;  // grid barriers that this CTA must have arrived at before its tiles may use the ring slots shared with the attention scratch
     int kind;     // 0 qkv, 1 o, 2 in, 3 out, 4 LM head
     unsigned wait_attn;  // attention CTAs that must have signalled before its operand exists (0: a grid barrier covers it)
     float *out;
@@ -375,7 +375,8 @@ __device__ __forceinline__ int ring_next(RingPos &r, bool lo_only, int S, int S1
 __device__ __forceinline__ bool ring_lo_only(const GemmDesc &g, int j, int S1) { return g.kind == 1 && j < S1; }
 
 struct alignas(16) Shared {
-    volatile int released;  // grid barriers completed so far
+    volatile int arrived;   // grid barriers this CTA has arrived at: its scratch is free of the phase in front of the last of them
+    volatile int passed;    // grid barriers seen to be complete
     volatile int abort;     // some wait in this CTA gave up
     volatile int go;        // snapshot of !abort taken inside the grid barrier: uniform for all work threads
     int epoch;              // grid barriers passed (thread 0's)
@@ -432,61 +433,75 @@ __device__ __forceinline__ bool mbar_spin_or_abort(uint64_t *bar, uint32_t parit
     return true;
 }
 
-// Grid barrier for the 256 work threads of every CTA.  Returns false (the same value in every work
-// thread of the CTA) once a wait has timed out anywhere in this CTA; the caller then stops.
-// One release and one acquire, both thread 0's: the CTA barriers around them pass them on to the other threads.  A fence per
-// thread in front and one behind the poll made two more trips to L2 of every barrier (7B verification 3486 -> 3371 us, 1.4B
-// 945 -> 899).
+// Poll (bounded) until grid barrier number `epoch` is complete; one thread.
+__device__ __forceinline__ bool grid_poll(const FwdParams &p, Shared *sh, int epoch) {
+    const unsigned target = (unsigned)epoch * gridDim.x;
+    if (ld_acquire(p.gbar) < target) {
+        const long long t0 = clock64();
+        while (ld_acquire(p.gbar) < target)
+            if (sh->abort || clock64() - t0 > sh->wait_limit) return false;
+    }
+    sh->passed = epoch;
+    return true;
+}
+__device__ __forceinline__ void grid_stamp(const FwdParams &p, int epoch) {
+    if (p.trace && blockIdx.x == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+        p.trace[epoch] = t;
+    }
+}
+
+// Arrival of the 256 work threads at the next grid barrier; what they wrote before it is published.
+// One release (and where the barrier is waited for, one acquire), both thread 0's: the CTA barriers around them pass them on to
+// the other threads.  A fence per thread in front and one behind the poll made two more trips to L2 of every barrier (7B
+// verification 3486 -> 3371 us, 1.4B 945 -> 899).
+__device__ __forceinline__ bool grid_arrive_work(const FwdParams &p, Shared *sh) {
+    fence_async_proxy();  // this thread's operand writes must be seen by other CTAs' TMA reads
+    named_bar(1, kWorkThreads);
+    if (threadIdx.x != 0) return true;
+    const int epoch = ++sh->epoch;
+    bool ok = sh->abort == 0;
+    __threadfence_block();  // (the producer reads `arrived` without a barrier)
+    sh->arrived = epoch;
+    // (the count is the sum of all arrivals: nobody arrives at a barrier before the one in front of it is complete)
+    if (ok && sh->passed < epoch - 1) ok = grid_poll(p, sh, epoch - 1);
+    if (ok) red_release_add(p.gbar, 1u);
+    return ok;
+}
+// Grid barrier.  Returns false (the same value in every work thread of the CTA) once a wait has timed out anywhere in this CTA;
+// the caller then stops.
 __device__ __noinline__ bool grid_sync() {
     const FwdParams &p = params_copy();
     Shared *sh = shared_state();
-    fence_async_proxy();  // this thread's operand writes must be seen by other CTAs' TMA reads
-    named_bar(1, kWorkThreads);
+    bool ok = grid_arrive_work(p, sh);
     if (threadIdx.x == 0) {
-        const int epoch = ++sh->epoch;
-        bool ok = sh->abort == 0;
-        if (ok) {
-            red_release_add(p.gbar, 1u);
-            const unsigned target = (unsigned)epoch * gridDim.x;
-            if (ld_acquire(p.gbar) < target) {
-                const long long t0 = clock64();
-                while (ld_acquire(p.gbar) < target) {
-                    if (clock64() - t0 > sh->wait_limit) { ok = false; break; }
-                }
-            }
-        }
+        ok = ok && grid_poll(p, sh, sh->epoch);
         if (!ok) {
             set_status(p.status, kTimeoutCode);
             sh->abort = 1;
         }
         sh->go = ok ? 1 : 0;
-        __threadfence_block();  // (the producer reads `released` without a barrier)
-        sh->released = epoch;
-        if (p.trace && blockIdx.x == 0) {
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            p.trace[epoch] = t;
-        }
+        grid_stamp(p, sh->epoch);
     }
     named_bar(1, kWorkThreads);
     return sh->go != 0;
 }
 
-// Arrival at the next grid barrier without waiting for it (for a CTA whose next work does not depend on
-// what the others publish there).  Its own writes are published like at a full barrier.
+// Arrival without a wait: in front of a GEMM, whose operand issuer is the only one that needs the other CTAs' work and waits for the
+// barrier itself (gemm_desc's `need`), while the other roles set themselves up; and of a CTA whose next work does not depend on
+// what the others publish there.  The barrier behind that work waits for this one first where nobody has (a time-out in between
+// is found there as well).
 __device__ __noinline__ void grid_arrive() {
     const FwdParams &p = params_copy();
     Shared *sh = shared_state();
-    fence_async_proxy();
-    named_bar(1, kWorkThreads);
+    const bool ok = grid_arrive_work(p, sh);
     if (threadIdx.x == 0) {
-        const int epoch = ++sh->epoch;
-        if (sh->abort == 0) red_release_add(p.gbar, 1u);
-        if (p.trace && blockIdx.x == 0) {  // (the stamp of a barrier this CTA does not wait at: its arrival)
-            unsigned long long t;
-            asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-            p.trace[epoch] = t;
+        if (!ok) {
+            set_status(p.status, kTimeoutCode);
+            sh->abort = 1;
         }
+        grid_stamp(p, sh->epoch);  // (where the operand issuer waits for it, its stamp replaces this one)
     }
 }
 
@@ -1828,8 +1843,17 @@ __device__ __noinline__ void run_gemm(int gi) {
                 }
                 __syncwarp();
             } else if (warp == kXWarp) {
-                // operand tiles of this GEMM (their phase has been released: this runs after its barrier)
+                // operand tiles of this GEMM, once the barrier behind the phase that makes them is complete
                 bool ready = true;
+                if (lane == 0 && !sh->abort && sh->passed < g.need) {
+                    ready = grid_poll(p, sh, g.need);
+                    if (ready) {
+                        grid_stamp(p, g.need);
+                    } else {
+                        set_status(p.status, kTimeoutCode);
+                        sh->abort = 1;
+                    }
+                }
                 if (lane == 0 && !sh->abort && g.wait_attn) {
                     // the attention output is complete once every attention CTA of this layer has signalled
                     const unsigned *cnt = attn_done(p);
@@ -2162,7 +2186,7 @@ __device__ __forceinline__ void producer_program() {
     if (lane == 0) {
         RingPos rp;
         bool failed = false;
-        int seen_release = 0;
+        int seen_arrival = 0;
         // a CTA that never runs an attention item (fewer items than CTAs) never uses the scratch: its
         // upper slots take weights at any time
         const bool scratch_used = (int)blockIdx.x < p.attn_items;
@@ -2176,9 +2200,9 @@ __device__ __forceinline__ void producer_program() {
             for (int c = c0; c < c1; ++c) {
                 uint32_t ph;
                 const int s = ring_next(rp, ring_lo_only(dw, c - c0, S1), S, S1, ph);
-                if (s >= S1 && scratch_used && seen_release < dw.need_hi) {  // slot shared with the attention scratch
+                if (s >= S1 && scratch_used && seen_arrival < dw.need_hi) {  // slot shared with the attention scratch
                     const long long t0 = clock64();
-                    while ((seen_release = sh->released) < dw.need_hi) {
+                    while ((seen_arrival = sh->arrived) < dw.need_hi) {
                         if (sh->abort || clock64() - t0 > sh->wait_limit) { failed = true; break; }
                         __nanosleep(100);  // (a tight poll takes issue slots and shared-memory cycles from the attention loop)
                     }
@@ -2255,7 +2279,7 @@ __device__ __forceinline__ void work_program() {
                     attention_phase<WIDE>(l);
                     attn_signal();
                 } else {
-                    if (!(go = grid_sync())) break;
+                    grid_arrive();
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));               // MLP out -> x, beside the attention items
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));               // out-proj -> x, once the attention CTAs have signalled
                 }
@@ -2263,7 +2287,7 @@ __device__ __forceinline__ void work_program() {
             } else {
                 attention_phase<WIDE>(l);
                 if (p.parallel) act_phase();
-                if (!(go = grid_sync())) break;
+                grid_arrive();
                 if (p.parallel) {
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));                   // out-proj -> x
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));                   // MLP out  -> x
@@ -2272,17 +2296,17 @@ __device__ __forceinline__ void work_program() {
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 1));                   // out-proj -> x
                     if (!(go = grid_sync())) break;
                     norm_mid_layer(l);
-                    if (!(go = grid_sync())) break;
+                    grid_arrive();
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 2));                   // MLP in
                     if (!(go = grid_sync())) break;
                     act_phase();
-                    if (!(go = grid_sync())) break;
+                    grid_arrive();
                     run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * l + 3));                   // MLP out -> x
                     if (!(go = grid_sync())) break;
                 }
             }
             norm_for_layer(l + 1);
-            if (!(go = grid_sync())) break;
+            grid_arrive();
         }
         if (go && p.want_logits) run_gemm<NT>((params_copy().cur_step << kStepShift) | (4 * p.n_layers));
         if (go && p.tail) {  // q, the draw and the commit of this step (see tail_partial)
@@ -2350,7 +2374,8 @@ __global__ void __launch_bounds__(kPersistThreads, 1) forward_kernel(const __gri
         blk.role_rp[1] = RingPos();
         for (int i = 0; i < 8; ++i) blk.role_seg[i] = 0;
         Shared *sh = &blk.state;
-        sh->released = 0;
+        sh->arrived = 0;
+        sh->passed = 0;
         sh->abort = 0;
         sh->go = 1;
         sh->epoch = 0;
