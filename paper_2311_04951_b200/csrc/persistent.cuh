@@ -1906,6 +1906,18 @@ __device__ __noinline__ void run_gemm(int gi) {
                     const bool has_k0 = (t > tile0) || (c0 % g.kchunks == 0);
                     const float *bias = (has_k0 && g.bias) ? g.bias : nullptr;
                     const int g8 = lane >> 2, t4 = lane & 3;
+                    // a thread's four columns are the same in every row: their bias is taken once per tile
+                    const int c4 = (threadIdx.x & 63) * 4, n = t * kTileNP + c4;
+                    float *col = g.out + n;
+                    float4 bb = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (bias && n + 3 < g.N && vec_ok) {
+                        bb = __ldg(reinterpret_cast<const float4 *>(bias + n));
+                    } else if (bias) {
+                        if (n < g.N) bb.x = __ldg(bias + n);
+                        if (n + 1 < g.N) bb.y = __ldg(bias + n + 1);
+                        if (n + 2 < g.N) bb.z = __ldg(bias + n + 2);
+                        if (n + 3 < g.N) bb.w = __ldg(bias + n + 3);
+                    }
                     // Block q of 8 rows sits in accumulator lanes 32 q .. 32 q + 15 (M = 64) or 16 q .. 16 q + 15
                     // (M = 128); a warp reaches the 32 lanes of its own quadrant only.
 #pragma unroll 1
@@ -1925,22 +1937,21 @@ __device__ __noinline__ void run_gemm(int gi) {
                             }
                         }
                         named_bar(5, kEpiWarps * 32);
-                        const int rows_here = min(8, p.R - 8 * q);
-                        for (int i = threadIdx.x; i < rows_here * (kTileNP / 4); i += kEpiWarps * 32) {
-                            const int rr = i / (kTileNP / 4), c4 = (i % (kTileNP / 4)) * 4, n = t * kTileNP + c4;
-                            if (n >= g.N) continue;
-                            float4 v = *reinterpret_cast<const float4 *>(epi_tile + rr * kEpiPitch + c4);
-                            float *dst = g.out + (size_t)(8 * q + rr) * g.ldo + n;
-                            if (vec_ok && n + 3 < g.N) {
-                                if (bias) {
-                                    const float4 bb = __ldg(reinterpret_cast<const float4 *>(bias + n));
-                                    v.x += bb.x; v.y += bb.y; v.z += bb.z; v.w += bb.w;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const int rr = (threadIdx.x >> 6) + 2 * k, row = 8 * q + rr;
+                            if (row < p.R && n < g.N) {
+                                float4 v = *reinterpret_cast<const float4 *>(epi_tile + rr * kEpiPitch + c4);
+                                v.x += bb.x; v.y += bb.y; v.z += bb.z; v.w += bb.w;
+                                float *dst = col + (size_t)row * g.ldo;
+                                if (vec_ok && n + 3 < g.N) {
+                                    red_add_v4(dst, v);
+                                } else {
+                                    atomicAdd(dst, v.x);
+                                    if (n + 1 < g.N) atomicAdd(dst + 1, v.y);
+                                    if (n + 2 < g.N) atomicAdd(dst + 2, v.z);
+                                    if (n + 3 < g.N) atomicAdd(dst + 3, v.w);
                                 }
-                                red_add_v4(dst, v);
-                            } else {
-                                const float e[4] = {v.x, v.y, v.z, v.w};
-                                for (int u = 0; u < 4; ++u)
-                                    if (n + u < g.N) atomicAdd(dst + u, e[u] + (bias ? __ldg(bias + n + u) : 0.f));
                             }
                         }
                         named_bar(5, kEpiWarps * 32);  // the tile is free for the next block
