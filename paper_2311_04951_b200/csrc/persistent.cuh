@@ -272,6 +272,9 @@ __device__ __forceinline__ unsigned atomic_add_acq_rel(unsigned *p, unsigned v) 
     return old;
 }
 __device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async;" ::: "memory"); }
+// ... for shared memory alone (some 40 cycles; the general form about half a microsecond) and for global memory alone
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // Tile row of the hi part of row r (the lo part is 8 further): rows come in blocks of 8, each block
 // as 8 hi rows followed by 8 lo rows, so that an accumulator load hands both to one thread.
@@ -457,7 +460,10 @@ __device__ __forceinline__ void grid_stamp(const FwdParams &p, int epoch) {
 // the other threads.  A fence per thread in front and one behind the poll made two more trips to L2 of every barrier (7B
 // verification 3486 -> 3371 us, 1.4B 945 -> 899).
 __device__ __forceinline__ bool grid_arrive_work(const FwdParams &p, Shared *sh) {
-    fence_async_proxy();  // this thread's operand writes must be seen by other CTAs' TMA reads
+    // What this thread did in shared memory is over before the producer's copies may land there.  (Its writes to global memory reach
+    // other CTAs' bulk copies through the release below, the operand issuer's acquire and that thread's proxy fence; a fence for
+    // global memory here, in every thread, cost each barrier half a microsecond: norms included, 2.7B verification 1855 -> 1780 us.)
+    fence_async_shared();
     named_bar(1, kWorkThreads);
     if (threadIdx.x != 0) return true;
     const int epoch = ++sh->epoch;
@@ -525,7 +531,6 @@ __device__ __forceinline__ unsigned *attn_done(const FwdParams &p) { return p.gb
 __device__ __noinline__ void attn_signal() {
     const FwdParams &p = params_copy();
     Shared *sh = shared_state();
-    fence_async_proxy();  // the attention output is read by other CTAs' bulk copies
     named_bar(1, kWorkThreads);
     if (threadIdx.x == 0 && sh->abort == 0) red_release_add(attn_done(p), 1u);
 }
@@ -546,7 +551,6 @@ __device__ __forceinline__ void block_sum2_work(double &a, double &b, double *re
     a = ta;
     b = tb;
 }
-__device__ __forceinline__ void prefetch_l1(const void *ptr) { asm volatile("prefetch.global.L1 [%0];" ::"l"(ptr)); }
 
 // zero a [R, n] fp32 buffer (row pitch ld), spread over the whole grid
 __device__ __forceinline__ void grid_zero(float *dst, int R, int n, int ld) {
@@ -567,17 +571,15 @@ __device__ __forceinline__ void grid_zero(float *dst, int R, int n, int ld) {
 }
 
 // Norm of every row of x into hi/lo operand buffers (one or two gain/bias sets from the same
-// statistics); one CTA per row.  The row (Q float4 per thread) stays in registers between the
-// statistics and the write pass, and all loads of a pass are issued before the first use, so the
-// phase costs about two L2 round trips instead of one per element.  Q is a template parameter so
+// statistics); one CTA per row.  Bound by latency: a barrier, the row, its sums, the operand.  The row (Q float4 per thread)
+// stays in registers between the statistics and the write pass, and gains and biases are loaded with it: fetched under the
+// statistics into L1 - of which there is next to none - they were a second trip of 1.2-2 us behind them (with the barriers' cheaper fence a 7B
+// layer 101.5 -> 99.2 us, a 1.4B layer 34.5 -> 31.8).  Q is a template parameter so
 // that a call executes only the code its row width needs: the instructions of a phase are not in
 // the instruction cache when it starts (the kernel is far larger than that cache), and every KB of
 // straight-line code costs a fraction of a microsecond to fetch.
 __device__ __forceinline__ void norm_emit(const FwdParams &p, int r, int i, const float4 v, float mu, float rs,
-                                          const float *g, const float *b, int op) {
-    const float4 gg = __ldg(reinterpret_cast<const float4 *>(g) + i);
-    float4 bb = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (b) bb = __ldg(reinterpret_cast<const float4 *>(b) + i);
+                                          const float4 gg, const float4 bb, int op) {
     const float y0 = (v.x - mu) * rs * gg.x + bb.x, y1 = (v.y - mu) * rs * gg.y + bb.y;
     const float y2 = (v.z - mu) * rs * gg.z + bb.z, y3 = (v.w - mu) * rs * gg.w + bb.w;
     const __nv_bfloat162 h01 = __floats2bfloat162_rn(y0, y1), h23 = __floats2bfloat162_rn(y2, y3);
@@ -591,29 +593,27 @@ __device__ __forceinline__ void norm_emit(const FwdParams &p, int r, int i, cons
     *reinterpret_cast<uint2 *>(hi) = hv;
     *reinterpret_cast<uint2 *>(lo) = lv;
 }
+__device__ __forceinline__ float4 norm_vec(const float *v, int i, int n4) {  // (no bias: zeros)
+    return v && i < n4 ? __ldg(reinterpret_cast<const float4 *>(v) + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
 
-template <int Q>  // float4 per thread held in registers: rows up to Q * 1024 wide; wider rows are re-read
+// Q: float4 per thread, rows up to Q * 1024 wide.  Wider rows (TAIL: beyond 5120) are read again, with what goes with them.
+template <int Q, bool TWO, bool TAIL>
 __device__ __noinline__ void norm_rows(const float *g1, const float *b1, int op1, const float *g2, const float *b2, int op2) {
     const FwdParams &p = params_copy();
     const int n4 = p.d >> 2;  // d is a multiple of 8
     for (int r = blockIdx.x; r < p.R; r += gridDim.x) {
         const float4 *x4 = reinterpret_cast<const float4 *>(p.x + (size_t)r * p.d);
-        float4 xv[Q];
+        float4 xv[Q], gv[Q], bv[Q], hv[TWO ? Q : 1], cv[TWO ? Q : 1];
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int i = threadIdx.x + q * kWorkThreads;
             xv[q] = i < n4 ? __ldcg(x4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        // the gain / bias vectors were last read a whole pass of weights ago: fetch them now, under the
-        // statistics, instead of as a second trip to DRAM after them
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            const int i = threadIdx.x + q * kWorkThreads;
-            if (i < n4) {
-                prefetch_l1(reinterpret_cast<const float4 *>(g1) + i);
-                if (b1) prefetch_l1(reinterpret_cast<const float4 *>(b1) + i);
-                if (g2) prefetch_l1(reinterpret_cast<const float4 *>(g2) + i);
-                if (b2) prefetch_l1(reinterpret_cast<const float4 *>(b2) + i);
+            gv[q] = norm_vec(g1, i, n4);
+            bv[q] = norm_vec(b1, i, n4);
+            if constexpr (TWO) {
+                hv[q] = norm_vec(g2, i, n4);
+                cv[q] = norm_vec(b2, i, n4);
             }
         }
         double s1 = 0.0, s2 = 0.0;
@@ -622,11 +622,13 @@ __device__ __noinline__ void norm_rows(const float *g1, const float *b1, int op1
             s1 += (double)xv[q].x + (double)xv[q].y + (double)xv[q].z + (double)xv[q].w;
             s2 += (double)xv[q].x * xv[q].x + (double)xv[q].y * xv[q].y + (double)xv[q].z * xv[q].z + (double)xv[q].w * xv[q].w;
         }
+        if constexpr (TAIL) {
 #pragma unroll 1
-        for (int i = threadIdx.x + Q * kWorkThreads; i < n4; i += kWorkThreads) {
-            const float4 v = __ldcg(x4 + i);
-            s1 += (double)v.x + (double)v.y + (double)v.z + (double)v.w;
-            s2 += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+            for (int i = threadIdx.x + Q * kWorkThreads; i < n4; i += kWorkThreads) {
+                const float4 v = __ldcg(x4 + i);
+                s1 += (double)v.x + (double)v.y + (double)v.z + (double)v.w;
+                s2 += (double)v.x * v.x + (double)v.y * v.y + (double)v.z * v.z + (double)v.w * v.w;
+            }
         }
         block_sum2_work(s1, s2, shared_block().red);
         double mean = 0.0, var;
@@ -638,29 +640,37 @@ __device__ __noinline__ void norm_rows(const float *g1, const float *b1, int op1
             var = s2 * p.inv_d;
         }
         const float mu = (float)mean, rs = (float)rsqrt(var + (double)p.eps);
-#pragma unroll 1
-        for (int e = 0; e < (g2 ? 2 : 1); ++e) {  // (rolled: the second gain set reuses the first one's code)
-            const float *g = e ? g2 : g1, *b = e ? b2 : b1;
-            const int op = e ? op2 : op1;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const int i = threadIdx.x + q * kWorkThreads;
-                if (i < n4) norm_emit(p, r, i, xv[q], mu, rs, g, b, op);
+        for (int q = 0; q < Q; ++q) {
+            const int i = threadIdx.x + q * kWorkThreads;
+            if (i < n4) {
+                norm_emit(p, r, i, xv[q], mu, rs, gv[q], bv[q], op1);
+                if constexpr (TWO) norm_emit(p, r, i, xv[q], mu, rs, hv[q], cv[q], op2);
             }
+        }
+        if constexpr (TAIL) {
 #pragma unroll 1
-            for (int i = threadIdx.x + Q * kWorkThreads; i < n4; i += kWorkThreads)
-                norm_emit(p, r, i, __ldcg(x4 + i), mu, rs, g, b, op);
+            for (int i = threadIdx.x + Q * kWorkThreads; i < n4; i += kWorkThreads) {
+                const float4 v = __ldcg(x4 + i);
+                norm_emit(p, r, i, v, mu, rs, norm_vec(g1, i, n4), norm_vec(b1, i, n4), op1);
+                if constexpr (TWO) norm_emit(p, r, i, v, mu, rs, norm_vec(g2, i, n4), norm_vec(b2, i, n4), op2);
+            }
         }
     }
 }
 
+template <bool TWO>
+__device__ __forceinline__ void norm_widths(const float *g1, const float *b1, int op1, const float *g2, const float *b2, int op2) {
+    const int n4 = params_copy().d >> 2;
+    if (n4 <= kWorkThreads) norm_rows<1, TWO, false>(g1, b1, op1, g2, b2, op2);
+    else if (n4 <= 2 * kWorkThreads) norm_rows<2, TWO, false>(g1, b1, op1, g2, b2, op2);
+    else if (n4 <= 3 * kWorkThreads) norm_rows<3, TWO, false>(g1, b1, op1, g2, b2, op2);
+    else if (n4 <= 4 * kWorkThreads) norm_rows<4, TWO, false>(g1, b1, op1, g2, b2, op2);
+    else norm_rows<5, TWO, true>(g1, b1, op1, g2, b2, op2);
+}
 __device__ __noinline__ void norm_phase(const float *g1, const float *b1, int op1, const float *g2, const float *b2, int op2) {
-    const FwdParams &p = params_copy();
-    const int n4 = p.d >> 2;
-    if (n4 <= kWorkThreads) norm_rows<1>(g1, b1, op1, g2, b2, op2);
-    else if (n4 <= 2 * kWorkThreads) norm_rows<2>(g1, b1, op1, g2, b2, op2);
-    else if (n4 <= 4 * kWorkThreads) norm_rows<4>(g1, b1, op1, g2, b2, op2);
-    else norm_rows<8>(g1, b1, op1, g2, b2, op2);
+    if (g2) norm_widths<true>(g1, b1, op1, g2, b2, op2);
+    else norm_widths<false>(g1, b1, op1, nullptr, nullptr, 0);
 }
 
 // The norm in front of layer l's first GEMM(s) - or of the LM head - and the zeroing of what they accumulate into.
@@ -1869,7 +1879,7 @@ __device__ __noinline__ void run_gemm(int gi) {
                     }
                 }
                 if (lane == 0 && ready && !sh->abort) {
-                    fence_async_proxy();  // that phase's generic-proxy writes -> visible to the bulk copies
+                    fence_async_global();  // that phase's generic-proxy writes -> visible to the bulk copies
                     int kx = c0 % g.kchunks;
                     for (int c = c0; c < c1; ++c) {
                         uint32_t ph;
