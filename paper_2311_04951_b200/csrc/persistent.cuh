@@ -1469,7 +1469,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
         *reinterpret_cast<uint4 *>(panel + sw128(RP + m, v8 & 7)) = *reinterpret_cast<uint4 *>(lq);
     }
     // (P rows that no softmax thread writes meet output columns that nobody reads)
-    fence_async_proxy();
+    fence_async_shared();
     named_bar(3, kAttnThreadsP);
 
     if (warp == 5) {
@@ -1580,7 +1580,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
             }
             if (!here) wait(landed, (acnt[AB_LANDED] + (uint32_t)n_fixed) & 1u);
             ++n_fixed;
-            fence_async_proxy();
+            fence_async_shared();
             mbar_arrive(fixed);
         }
     } else {
@@ -1677,7 +1677,7 @@ __device__ __noinline__ void attention_items_tc(int layer) {
                     asm volatile("st.shared.b16 [%0], %1;" ::"r"(at + RP * 128), "h"(__bfloat16_as_ushort(lv[i])) : "memory");
                 }
             }
-            fence_async_proxy();
+            fence_async_shared();  // (the general form, per chunk and thread: 17 rows x 16384 positions 100 -> 87 us a layer)
             tc_fence_before();
             mbar_arrive(&p_ready[c & 1]);
         }
