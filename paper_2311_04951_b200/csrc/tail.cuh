@@ -216,6 +216,13 @@ constexpr int kFilterCluster = 2;
 constexpr int kFilterCache = 44 * 1024;     // probabilities a CTA keeps (176 KB)
 constexpr int kFilterBatch = 8;
 constexpr double kMassUnit = 4611686018427387904.0;  // 2^62
+// Up to kPickK tokens the threshold is found among candidates instead of by histograms over the row: the k-th largest of a CTA's
+// 1024 threads' maxima is a lower bound of the k-th largest logit, and little more than k tokens of a CTA reach it.  A pass of
+// the histograms computes a probability, its mass in fp64 and a bin for every entry of the row, 4-10 us each; picking compares
+// every entry once.  Same counts and masses of the same tokens (integers, so in any order): the same bits.  Rows with more than
+// kPickMax candidates (ties, many equal entries), without a finite sum or with a bound below 1e-30 go the general way.
+// 8 sequences x 6 rows x 50304 entries, top-k 50 and top-p 0.9, whole call: 53 -> 29 us.
+constexpr int kPickK = 96, kPickMax = 256;
 struct FilterHist {
     unsigned cnt[kBins], mlo[kBins], mhi[kBins];
 };
@@ -227,6 +234,13 @@ struct FilterSmem {
     int first, last;            // first bin that meets the target, last bin that holds anything
     unsigned above_cnt;         // of the chosen bin: what lies above it, and its own mass
     unsigned long long above_mass, sel_mass;
+    // few tokens to keep: this CTA's candidates, both CTAs' together, the thresholds' patterns and what weighs at least as much
+    float low;
+    int n_cand;
+    float cand[kPickMax];
+    float all[kPickMax];
+    unsigned best[2];
+    unsigned long long best_mass[2];
 };
 __host__ __device__ constexpr size_t filter_smem(int V) {  // dynamic shared memory: the CTA's probabilities
     const size_t n = (size_t)((V + kFilterCluster - 1) / kFilterCluster) + 32 * kTailWarps;
@@ -335,6 +349,20 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         }
     }
     auto entry = [&](int j) { return cached ? mine[j] : __ldcg(lg + j); };
+    const bool use_k = a.top_k > 0 && a.top_k < V, use_p = a.top_p > 0.f && a.top_p < 1.f;
+    const bool pick = use_k && a.top_k <= kPickK && cached && inv_t > 0.f;
+    if (pick) {  // a bound from the threads' maxima, on the upper half of their patterns' bits (a little lower: still a bound)
+        const unsigned bits = __float_as_uint(mx), key = bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
+        unsigned bound = 0;
+#pragma unroll 1
+        for (unsigned bit = 0x80000000u; bit >= 0x10000u; bit >>= 1)
+            if (__syncthreads_count(key >= (bound | bit)) >= a.top_k) bound |= bit;
+        if (tid == 0) {
+            fs->low = __uint_as_float(bound ^ ((bound >> 31) ? 0x80000000u : 0xffffffffu));
+            fs->n_cand = 0;
+            fs->best[0] = fs->best[1] = 0;
+        }
+    }
     {
         const float m = warp_max_redux(mx);
         const int am = __reduce_min_sync(0xffffffffu, mx == m ? at : 0x7fffffff);
@@ -359,6 +387,80 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     cl.sync();
     const RowStat st = row_stat(join_parts<kFilterCluster>(*cl.map_shared_rank(&fs->cta, lane % kFilterCluster), inv_t));
     const unsigned kmax = __float_as_uint(prob_of(st.mx, st, inv_t, st.amax));
+    auto mass_of = [](float p) { return __double2ull_rz((double)fminf(p, 2.f) * kMassUnit); };
+    auto write_stats = [&](const RowFilter &f) {
+        if (rank == 0 && tid == 0) {
+            a.stats[(size_t)b * n_rows + i] = st;
+            a.filt[(size_t)b * n_rows + i] = f;
+        }
+    };
+    if (pick) {
+        const float low = fmaxf(fs->low, cl.map_shared_rank(fs, rank ^ 1)->low);
+        // (an entry 1e-4 below the bound in the exponent has the smaller probability whatever the roundings)
+        const float cut = (low - st.mx) * inv_t - 1e-4f;
+        bool few = low > -INFINITY && st.z > 0.f && st.z < INFINITY && prob_of(low, st, inv_t, -1) >= 1e-30f;
+        if (few) {
+            for (int j = lo + lane; j < hi; j += 32) {
+                const float x = mine[j];
+                if ((x - st.mx) * inv_t >= cut) {
+                    const int at_ = atomicAdd(&fs->n_cand, 1);
+                    if (at_ < kPickMax) fs->cand[at_] = prob_of(x, st, inv_t, j);
+                }
+            }
+        }
+        cl.sync();
+        const FilterSmem *o0 = cl.map_shared_rank(fs, 0), *o1 = cl.map_shared_rank(fs, 1);
+        const int n0 = o0->n_cand, n = n0 + o1->n_cand;
+        if (few && n >= a.top_k && n <= kPickMax) {
+            float v = 0.f;
+            if (tid < n) {
+                v = tid < n0 ? o0->cand[tid] : o1->cand[tid - n0];
+                fs->all[tid] = v;
+            }
+            __syncthreads();
+            int c = 0;                  // tokens at least as probable, and their mass
+            unsigned long long m = 0;
+            if (tid < n) {
+                for (int j = 0; j < n; ++j) {
+                    const float w = fs->all[j];
+                    if (w >= v) { ++c; m += mass_of(w); }
+                }
+                if (c >= a.top_k) atomicMax(&fs->best[0], __float_as_uint(v));
+            }
+            __syncthreads();
+            RowFilter f;
+            f.thr = __uint_as_float(fs->best[0]);
+            if (tid < n && v == f.thr) fs->best_mass[0] = m;  // (the same value by whoever holds it)
+            __syncthreads();
+            const unsigned long long kept = fs->best_mass[0];
+            unsigned long long mass = kept;
+            if (use_p) {
+                const unsigned long long target = __double2ull_ru((double)a.top_p * (double)kept);
+                if (tid < n && v >= f.thr && m >= target) atomicMax(&fs->best[1], __float_as_uint(v));
+                __syncthreads();
+                f.thr = __uint_as_float(fs->best[1]);
+                if (tid < n && v == f.thr) fs->best_mass[1] = m;
+                __syncthreads();
+                mass = fs->best_mass[1];
+            }
+            f.mass = (float)((double)mass / kMassUnit);
+            write_stats(f);
+            if (a.p_out) {
+                float *p = a.p_out + row * V;
+                for (int j = lo + lane; j < hi; j += 32) {
+                    const float x = mine[j];
+                    float out = 0.f;
+                    if ((x - st.mx) * inv_t >= cut) {
+                        const float pr = prob_of(x, st, inv_t, j);
+                        out = pr < f.thr ? 0.f : pr / f.mass;
+                    }
+                    p[j] = out;
+                }
+            }
+            cl.sync();  // nobody leaves while its shared memory is read
+            return;
+        }
+    }
 
     // ---- histogram of the keys in [d_lo, d_lo + bins << shift) with p >= p_min (open_end: the last bin takes all beyond) ----
     auto count = [&](FilterHist &h, unsigned d_lo, int shift, int bins, bool open_end, float p_min, bool first) {
@@ -388,7 +490,7 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
                 m = 0;
             }
             ++c;
-            m += __double2ull_rz((double)fminf(p, 2.f) * kMassUnit);
+            m += mass_of(p);
         }
         bin_add(h, bin, c, m);
     };
@@ -433,7 +535,6 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     f.thr = 0.f;
     f.mass = 0.f;
     double mass = 0.0;
-    const bool use_k = a.top_k > 0 && a.top_k < V, use_p = a.top_p > 0.f && a.top_p < 1.f;
     unsigned long long kept = ~0ull;  // mass of what top-k keeps
     if (use_k) {
         const unsigned want = (unsigned)a.top_k;
@@ -471,10 +572,7 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         mass = (double)(kr.above_mass + kr.sel_mass) / kMassUnit;
     }
     f.mass = (float)mass;
-    if (rank == 0 && tid == 0) {
-        a.stats[(size_t)b * n_rows + i] = st;
-        a.filt[(size_t)b * n_rows + i] = f;
-    }
+    write_stats(f);
     if (a.p_out) {
         float *p = a.p_out + row * V;
         // (as prob_f; a row without mass is one of NaNs.  A test for that in the loop cost 2 of 36 us, 15 rows of 32000)

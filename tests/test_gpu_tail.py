@@ -227,6 +227,39 @@ def test_tail_at_the_edges_of_the_row_pieces(V, top_k, top_p):
         gu.check_decisions_on_own_rows(p[b], q[b], rows[b, 1:], u[b, :K], u[b, K], int(n_acc[b]), int(nxt[b]))
 
 
+@pytest.mark.parametrize("top_k", [1, 96, 97])  # the last k of the picked form, the first of the histograms
+@pytest.mark.parametrize("V", [130, 1025, 32000])
+def test_few_kept_tokens_are_picked_or_searched_alike(V, top_k):
+    """Up to 96 kept tokens are picked among those that reach a bound; rows that give no usable bound or too many candidates
+    (a constant row, more than 256 equal maxima, fewer finite entries than tokens to keep) take the histograms as every row
+    does beyond 96.  All follow the oracle's restriction of the row's probabilities, ties at the threshold included."""
+    T, K, Bn, top_p = 0.7, 3, 2, 0.9
+    logits, rows, q, u = make_case(4000 + V, Bn, K, V, T, True)
+    logits[0, 1] = 0.25
+    logits[0, 2] = np.round(logits[0, 2] * 4) / 4                  # ties everywhere
+    logits[0, 3, :min(V, 300)] = logits[0, 3].max() + 1            # more equal maxima than candidates
+    logits[1, 0, 60:] = -np.inf                                    # fewer finite entries than tokens to keep
+    logits[1, 1, :min(V - 1, 50)] += 40                            # the kept ones in one warp's piece
+    logits[1, 2] *= 50
+    q = np.stack([[osamp.filter_top_k_top_p(q[b, i], top_k, top_p) for i in range(K)] for b in range(Bn)])
+    rows[:, 1:] = synth.draw_tokens_from_rows(79, q.reshape(Bn * K, V)).reshape(Bn, K)
+    B.set_sampling(top_k, top_p)
+    try:
+        n_acc, nxt, p = run_tail(logits, rows, q, u, T)
+    finally:
+        B.set_sampling(0, 1.0)
+    for b in range(Bn):
+        for i in range(K + 1):
+            raw = osamp.softmax_t(logits[b, i], T)
+            ref = osamp.filter_top_k_top_p(raw, top_k, top_p)
+            odd = raw[(p[b, i] > 0) != (ref > 0)]
+            if odd.size:      # only values at the threshold, within the rounding of the probabilities (as at the row's edges above)
+                assert np.ptp(odd) <= 1e-6 * odd.max()
+            else:
+                assert np.abs(p[b, i] - ref).max() <= gu.P_ATOL
+        gu.check_decisions_on_own_rows(p[b], q[b], rows[b, 1:], u[b, :K], u[b, K], int(n_acc[b]), int(nxt[b]))
+
+
 @pytest.mark.parametrize("top_k", [0, 37])
 @pytest.mark.parametrize("V", [33, 8193, 32000, 65537])
 @pytest.mark.parametrize("u_draw", [1.0, float("nan"), float("inf"), -0.25, 1.0 - 2.0 ** -24, 0.0])
