@@ -11,7 +11,7 @@
 //     first 1024 weights of the warp's first column are fetched into registers BEFORE the barrier in front of the phase;
 //   * attention: one CTA per (sequence, head): four lanes per position for the scores, a thread per (head column, position
 //     group) for P V; the CTA appends the pass's keys / values itself, so nothing else has to wait for them.
-// Generation with the four-layer 256-wide model (K = 4, 16 iterations): 13.7 ms as one launch per step, 5.6 as one
+// Generation with the four-layer 256-wide model (K = 4, 16 iterations): 13.7 ms as one launch per step, 5.3 as one
 // per forward.
 // Results as the stepwise path's up to fp32 summation order.  Every barrier wait is bounded.
 #pragma once

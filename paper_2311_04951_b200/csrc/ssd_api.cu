@@ -599,9 +599,10 @@ int launch_forward_rows(const FwdParams &p, int rows_k, const void *ws_base, siz
 }
 
 // From this many positions per split the tensor-core items are the faster form for passes of more than eight rows: they cost
-// more to start (20 us against 12) and half as much per position (up to 16 rows; a quarter beyond, where the warp-MMA form needs
-// two row tiles).  7B layers, us, warp-MMA / tensor core: four sequences of 800 positions (one split) x 9 rows 165.1 / 163.1,
-// of 400 153.9 / 157.8; one sequence of 3200 (four splits) x 17 rows 175.4 / 165.0, of 1600 153.4 / 155.3.
+// more to start (18 us against 12, 28 beyond 16 rows) and half as much per position (up to 16 rows; a quarter beyond, where the
+// warp-MMA form needs two row tiles).  7B passes, us, warp-MMA / tensor core: four sequences x 9 rows of 600 positions (one split)
+// 4255 / 4223, of 450 4162 / 4176; one sequence x 17 rows of 2400 (four splits) 4590 / 4329, of 1400 4136 / 4183, two of 1000
+// (two splits) 4598 / 4717.
 inline int tc_min_chunk(int M) { return M <= 16 ? 512 : 640; }
 
 // The whole forward as one cooperative launch (bf16 models).

@@ -162,6 +162,33 @@ def test_single_kernel_forward_equals_stepwise_forward(name):
         assert (np.abs(a - c) <= gu.LOGIT_RTOL * np.abs(c) + gu.LOGIT_ATOL).all()
 
 
+@pytest.mark.parametrize("family,d", [("neox", 1040), ("llama", 2064), ("neox", 3088), ("llama", 4112), ("neox", 5136), ("llama", 5136)])
+def test_norms_just_beyond_a_row_width_equal_the_stepwise_ones(family, d):
+    """A norm holds 1024 columns per register step, up to five steps, with one or two gain sets; rows a little wider than each
+    (and than all five, whose rest is read again), against the stepwise path: one layer of heads of 16, same tolerances as the
+    comparison of the two paths above."""
+    like = synth.neox_like if family == "neox" else synth.llama_like
+    arch = like(1, d, d // 16, 128, 136)
+    ws_np = gu.scaled_weights(synth, arch, 3, 1.0)
+    model = B.Model(arch, B.upload_weights(arch, ws_np))
+    S, K = 16, 2
+    prompts, rows = synth.gen_prompt(4, 1, 5, arch.vocab), synth.gen_prompt(5, 1, K + 1, arch.vocab)
+    res = []
+    for persistent in (True, False):
+        B.set_persistent(persistent)
+        try:
+            kv = B.KV(model, 1, S)
+            ws = model.new_workspace(1, 8, S)
+            B.kv_prefill(model, kv, torch.from_numpy(prompts).to("cuda"), torch.tensor([5], dtype=torch.int32, device="cuda"), ws)
+            lg = gpu_logits(model, kv, ws, rows, K)
+            assert kv.status() == 0
+            res.append((lg, kv.cache_view().float().cpu().numpy()[:, :, :, :, :5 + K + 1]))
+        finally:
+            B.set_persistent(True)
+    assert np.abs(res[0][0] - res[1][0]).max() < 1e-2
+    assert (np.abs(res[0][1] - res[1][1]) <= gu.LOGIT_RTOL * np.abs(res[1][1]) + gu.LOGIT_ATOL).all()
+
+
 @pytest.mark.parametrize("Bn,M", [(1, 9), (1, 17), (3, 11), (8, 5), (2, 32), (8, 8)])
 def test_row_counts_of_the_single_kernel_gemms(Bn, M):
     """The forward kernel is instantiated per padded row count (8, 16, 24, 32, 40, 64 rows: operand tiles of
