@@ -1310,14 +1310,18 @@ static bool rows_apart(int B, int K, int V, bool sampled, bool exported) {
 }
 static int run_row_filter(const float *logits, int B, int M, int V, const int32_t *n_eff, float temperature, RowStat *stats,
                           RowFilter *filt, float *p_out, cudaStream_t st) {
-    static DeviceTable<bool> devices;  // (on supplied logits the tail may be a program's first call on the device)
-    const int rc = allow_smem(devices, row_filter_kernel, (size_t)kFilterCache * 4);
-    if (rc) return rc;
+    static DeviceTable<bool> devices[2];  // (on supplied logits the tail may be a program's first call on the device)
     FilterArgs f;
     f.logits = logits; f.M = M; f.V = V; f.n_eff = n_eff; f.inv_t = 1.0f / temperature;
     f.top_k = g_top_k; f.top_p = g_top_p;
     f.stats = stats; f.filt = filt; f.p_out = p_out;
-    LAUNCH(row_filter_kernel, dim3((n_eff ? 1 : M) * kFilterCluster, B), kTailThreads, filter_smem(V), st, f);
+    const dim3 grid((n_eff ? 1 : M) * kFilterCluster, B);
+    const bool pick = filter_picks(f);
+    const int rc = pick ? allow_smem(devices[1], row_filter_kernel<true>, (size_t)kFilterCache * 4)
+                        : allow_smem(devices[0], row_filter_kernel<false>, (size_t)kFilterCache * 4);
+    if (rc) return rc;
+    if (pick) { LAUNCH(row_filter_kernel<true>, grid, kTailThreads, filter_smem(V), st, f); }
+    else { LAUNCH(row_filter_kernel<false>, grid, kTailThreads, filter_smem(V), st, f); }
     return SSD_OK;
 }
 

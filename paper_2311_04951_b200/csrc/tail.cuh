@@ -217,11 +217,16 @@ constexpr int kFilterCache = 44 * 1024;     // probabilities a CTA keeps (176 KB
 constexpr int kFilterBatch = 8;
 constexpr double kMassUnit = 4611686018427387904.0;  // 2^62
 // Up to kPickK tokens the threshold is found among candidates instead of by histograms over the row: the k-th largest of a CTA's
-// 1024 threads' maxima is a lower bound of the k-th largest logit, and little more than k tokens of a CTA reach it.  A pass of
-// the histograms computes a probability, its mass in fp64 and a bin for every entry of the row, 4-10 us each; picking compares
-// every entry once.  Same counts and masses of the same tokens (integers, so in any order): the same bits.  Rows with more than
-// kPickMax candidates (ties, many equal entries), without a finite sum or with a bound below 1e-30 go the general way.
-// 8 sequences x 6 rows x 50304 entries, top-k 50 and top-p 0.9, whole call: 53 -> 29 us.
+// 1024 threads' maxima is a lower bound of the k-th largest logit, and some 2 k tokens of the two CTAs reach it (at k = 96 about
+// 195 of the 256 that there is room for; beyond 96 ever more rows would not fit).  A pass of the histograms computes a
+// probability, its mass in fp64 and a bin for every entry of the row, 4-10 us each; picking compares every entry once.
+// Same counts and masses of the same tokens (integers, so in any order): the same bits.  Rows with more than kPickMax candidates
+// (ties, a run of large entries in one warp's piece), without a finite sum or with a bound below 1e-30 go the general way; what
+// lies below a bound is not counted there, which pays for the search.
+// us a call, histograms / picked, top-p 0.9 and rows exported: 8 sequences x 6 rows x 50304 entries, k = 1 53.5 / 24.9, 20 28.9,
+// 50 28.9, 96 31.0 (the same around -100 and 300); 17 x 12 rows of 32000, k = 50, 103.7 / 52.4.  Rows that go back to the histograms:
+// constant 67.8 / 63.7, 30 finite entries 78.1 / 73.2, a NaN 57.1 / 55.5, sorted 59.3 / 57.5, 300 equal maxima 57.5 / 57.5
+// (17 x 12 rows of 32000 111.4 / 117.0).
 constexpr int kPickK = 96, kPickMax = 256;
 struct FilterHist {
     unsigned cnt[kBins], mlo[kBins], mhi[kBins];
@@ -234,11 +239,15 @@ struct FilterSmem {
     int first, last;            // first bin that meets the target, last bin that holds anything
     unsigned above_cnt;         // of the chosen bin: what lies above it, and its own mass
     unsigned long long above_mass, sel_mass;
-    // few tokens to keep: this CTA's candidates, both CTAs' together, the thresholds' patterns and what weighs at least as much
+    // few tokens to keep: per warp the bits that are set in all and in any of its threads' maxima, the largest of these and the
+    // smallest that reaches the bound; the bound and how many of the CTA's maxima reach it; its candidates, both CTAs' together with their
+    // masses, the thresholds' patterns and what weighs at least as much
+    unsigned key_and[kTailWarps], key_or[kTailWarps], key_top[kTailWarps], key_low[kTailWarps];
     float low;
-    int n_cand;
+    int n_low, n_cand;
     float cand[kPickMax];
     float all[kPickMax];
+    unsigned long long all_mass[kPickMax];
     unsigned best[2];
     unsigned long long best_mass[2];
 };
@@ -317,6 +326,11 @@ struct FilterArgs {
     RowFilter *filt;
     float *p_out;         // [B, M, V] or null
 };
+inline bool filter_picks(const FilterArgs &a) {
+    return a.top_k > 0 && a.top_k <= kPickK && a.top_k < a.V && a.inv_t > 0.f && filter_smem(a.V) > 0;
+}
+// PICK: with the search among candidates in front (see kPickK); without it, nothing of it is in the general way's way.
+template <bool PICK>
 __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailThreads) row_filter_kernel(FilterArgs a) {
     extern __shared__ float fcache[];
     __shared__ FilterSmem sm;
@@ -330,7 +344,7 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     const float *lg = a.logits + row * V;
     int lo, hi;
     row_piece(V, kFilterCluster * kTailWarps, rank * kTailWarps + warp, lo, hi);
-    const bool cached = filter_smem(V) > 0;
+    const bool cached = PICK || filter_smem(V) > 0;
     int cta_lo, unused;
     row_piece(V, kFilterCluster * kTailWarps, rank * kTailWarps, cta_lo, unused);
     float *mine = fcache - cta_lo;   // entry j of the row at mine[j]
@@ -349,19 +363,38 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         }
     }
     auto entry = [&](int j) { return cached ? mine[j] : __ldcg(lg + j); };
-    const bool use_k = a.top_k > 0 && a.top_k < V, use_p = a.top_p > 0.f && a.top_p < 1.f;
-    const bool pick = use_k && a.top_k <= kPickK && cached && inv_t > 0.f;
-    if (pick) {  // a bound from the threads' maxima, on the upper half of their patterns' bits (a little lower: still a bound)
-        const unsigned bits = __float_as_uint(mx), key = bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u);
-        unsigned bound = 0;
+    int n_low = 0;
+    if constexpr (PICK) {
+        // The bound, from the order-preserving patterns of the threads' maxima: the largest if it is there top_k times; else, from the
+        // top, the bits in which they differ at all, until little more than top_k of them reach it.  So it is as close wherever
+        // the logits lie: on the patterns' upper halves, rows around 300 had too many candidates.
+        const bool any = mx > -INFINITY;
+        const unsigned bits = __float_as_uint(mx), key = any ? bits ^ ((bits >> 31) ? 0xffffffffu : 0x80000000u) : 0u;
+        const unsigned wa = __reduce_and_sync(0xffffffffu, any ? key : 0xffffffffu), wo = __reduce_or_sync(0xffffffffu, key);
+        const unsigned wt = __reduce_max_sync(0xffffffffu, key);
+        if (lane == 0) { fs->key_and[warp] = wa; fs->key_or[warp] = wo; fs->key_top[warp] = wt; }
+        unsigned bound = 0xffffffffu;
+        n_low = __syncthreads_count(any);
+        if (n_low >= a.top_k) {
+            bound = __reduce_max_sync(0xffffffffu, fs->key_top[lane]);
+            const int n_top = __syncthreads_count(key == bound);
+            if (n_top >= a.top_k) {
+                n_low = n_top;
+            } else {
+                bound = __reduce_and_sync(0xffffffffu, fs->key_and[lane]);
+                unsigned rest = bound ^ __reduce_or_sync(0xffffffffu, fs->key_or[lane]);
+                const int enough = a.top_k + (a.top_k >> 5) + 2;
 #pragma unroll 1
-        for (unsigned bit = 0x80000000u; bit >= 0x10000u; bit >>= 1)
-            if (__syncthreads_count(key >= (bound | bit)) >= a.top_k) bound |= bit;
-        if (tid == 0) {
-            fs->low = __uint_as_float(bound ^ ((bound >> 31) ? 0x80000000u : 0xffffffffu));
-            fs->n_cand = 0;
-            fs->best[0] = fs->best[1] = 0;
+                while (rest && n_low > enough) {
+                    const unsigned bit = 0x80000000u >> __clz(rest);
+                    rest ^= bit;
+                    const int n = __syncthreads_count(key >= (bound | bit));
+                    if (n >= a.top_k) { bound |= bit; n_low = n; }
+                }
+            }
         }
+        const unsigned wl = __reduce_min_sync(0xffffffffu, any && key >= bound ? key : 0xffffffffu);
+        if (lane == 0) fs->key_low[warp] = wl;
     }
     {
         const float m = warp_max_redux(mx);
@@ -383,6 +416,15 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
     if (warp == 0) {
         const PartStat t = join_parts<32>(fs->warp[lane], inv_t);
         if (lane == 0) fs->cta = t;
+        if constexpr (PICK) {
+            const unsigned k = __reduce_min_sync(0xffffffffu, fs->key_low[lane]);
+            if (lane == 0) {
+                fs->low = k == 0xffffffffu ? -INFINITY : __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
+                fs->n_low = n_low;
+                fs->n_cand = 0;
+                fs->best[0] = fs->best[1] = 0;
+            }
+        }
     }
     cl.sync();
     const RowStat st = row_stat(join_parts<kFilterCluster>(*cl.map_shared_rank(&fs->cta, lane % kFilterCluster), inv_t));
@@ -394,37 +436,53 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
             a.filt[(size_t)b * n_rows + i] = f;
         }
     };
-    if (pick) {
-        const float low = fmaxf(fs->low, cl.map_shared_rank(fs, rank ^ 1)->low);
+    const bool use_k = PICK || (a.top_k > 0 && a.top_k < V), use_p = a.top_p > 0.f && a.top_p < 1.f;
+    float cut = -INFINITY;  // entries whose exponent lies below it are out whatever the search finds
+    if constexpr (PICK) {
+        const FilterSmem *o = cl.map_shared_rank(fs, rank ^ 1);
+        const float low = fmaxf(fs->low, o->low);
         // (an entry 1e-4 below the bound in the exponent has the smaller probability whatever the roundings)
-        const float cut = (low - st.mx) * inv_t - 1e-4f;
-        bool few = low > -INFINITY && st.z > 0.f && st.z < INFINITY && prob_of(low, st, inv_t, -1) >= 1e-30f;
-        if (few) {
-            for (int j = lo + lane; j < hi; j += 32) {
-                const float x = mine[j];
-                if ((x - st.mx) * inv_t >= cut) {
-                    const int at_ = atomicAdd(&fs->n_cand, 1);
-                    if (at_ < kPickMax) fs->cand[at_] = prob_of(x, st, inv_t, j);
+        if (low > -INFINITY && st.z > 0.f && st.z < INFINITY && prob_of(low, st, inv_t, -1) >= 1e-30f) cut = (low - st.mx) * inv_t - 1e-4f;
+        const int n_min = (fs->low == low ? fs->n_low : 0) + (o->low == low ? o->n_low : 0);
+        int n = kPickMax + 1;
+        if (cut > -INFINITY && n_min <= kPickMax) {  // (the same on both CTAs)
+            for (int base = lo; base < hi; base += 128) {
+                float x[4];
+                bool some = false;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int j = base + 32 * u + lane;
+                    x[u] = j < hi ? mine[j] : -INFINITY;
+                    some |= (x[u] - st.mx) * inv_t >= cut;
+                }
+                if (some) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        if ((x[u] - st.mx) * inv_t >= cut) {
+                            const int at_ = atomicAdd(&fs->n_cand, 1);
+                            if (at_ < kPickMax) fs->cand[at_] = prob_of(x[u], st, inv_t, base + 32 * u + lane);
+                        }
+                    }
                 }
             }
+            cl.sync();
+            n = fs->n_cand + o->n_cand;
         }
-        cl.sync();
         const FilterSmem *o0 = cl.map_shared_rank(fs, 0), *o1 = cl.map_shared_rank(fs, 1);
-        const int n0 = o0->n_cand, n = n0 + o1->n_cand;
-        if (few && n >= a.top_k && n <= kPickMax) {
+        if (n <= kPickMax) {
+            const int n0 = o0->n_cand;
             float v = 0.f;
             if (tid < n) {
                 v = tid < n0 ? o0->cand[tid] : o1->cand[tid - n0];
                 fs->all[tid] = v;
+                fs->all_mass[tid] = mass_of(v);
             }
             __syncthreads();
             int c = 0;                  // tokens at least as probable, and their mass
             unsigned long long m = 0;
             if (tid < n) {
-                for (int j = 0; j < n; ++j) {
-                    const float w = fs->all[j];
-                    if (w >= v) { ++c; m += mass_of(w); }
-                }
+                for (int j = 0; j < n; ++j)
+                    if (fs->all[j] >= v) { ++c; m += fs->all_mass[j]; }
                 if (c >= a.top_k) atomicMax(&fs->best[0], __float_as_uint(v));
             }
             __syncthreads();
@@ -470,7 +528,14 @@ __global__ void __cluster_dims__(kFilterCluster, 1, 1) __launch_bounds__(kTailTh
         for (int j = lo + lane; j < hi; j += 32) {
             float p;
             if (first || !cached) {
-                p = prob_of(entry(j), st, inv_t, j);
+                const float x = entry(j);
+                if constexpr (PICK) {
+                    if ((x - st.mx) * inv_t < cut) {  // (below the threshold, whatever it is: never counted, exported as zero)
+                        mine[j] = 0.f;
+                        continue;
+                    }
+                }
+                p = prob_of(x, st, inv_t, j);
                 if (cached) mine[j] = p;
             } else {
                 p = mine[j];

@@ -287,6 +287,38 @@ def test_few_kept_tokens_are_picked_or_searched_alike(V, top_k):
         gu.check_decisions_on_own_rows(p[b], q[b], rows[b, 1:], u[b, :K], u[b, K], int(n_acc[b]), int(nxt[b]))
 
 
+def test_picked_rows_cost_the_same_wherever_the_logits_lie():
+    """The candidate bound does not hang on the logits' absolute size: rows around 300 gave more than 256 candidates each, went the
+    general way after all and took twice the time of rows around 0."""
+    Bn, K, V, T, top_k = 8, 5, 32000, 0.8, 50
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(9)
+    base = torch.empty(Bn, K + 1, V, device="cuda").normal_(0.0, 2.0, generator=gen)
+    q = torch.softmax(base[:, :K], -1).contiguous()
+    rows, u = torch.zeros(Bn, K + 1, dtype=torch.int32, device="cuda"), torch.full((Bn, K + 1), 0.5, device="cuda")
+    n_acc, nxt = torch.zeros(Bn, dtype=torch.int32, device="cuda"), torch.zeros(Bn, dtype=torch.int32, device="cuda")
+    scratch = torch.empty(B.verify_scratch_bytes(Bn, K), dtype=torch.uint8, device="cuda")
+
+    def best(logits):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ms = []
+        for _ in range(8):
+            ev[0].record()
+            for _ in range(20):
+                B.verify_from_logits(logits, K, rows, q, u, T, n_acc, nxt, 1, None, scratch)
+            ev[1].record()
+            torch.cuda.synchronize()
+            ms.append(ev[0].elapsed_time(ev[1]))
+        return min(ms)
+
+    B.set_sampling(top_k, 0.9)
+    try:
+        near = best(base)
+        assert max(best(base + 300.0), best(base - 100.0)) <= 1.4 * near
+    finally:
+        B.set_sampling(0, 1.0)
+
+
 @pytest.mark.parametrize("top_k", [0, 37])
 @pytest.mark.parametrize("V", [33, 8193, 32000, 65537])
 @pytest.mark.parametrize("u_draw", [1.0, float("nan"), float("inf"), -0.25, 1.0 - 2.0 ** -24, 0.0])
