@@ -162,14 +162,21 @@ def test_single_kernel_forward_equals_stepwise_forward(name):
         assert (np.abs(a - c) <= gu.LOGIT_RTOL * np.abs(c) + gu.LOGIT_ATOL).all()
 
 
-@pytest.mark.parametrize("family,d", [("neox", 1040), ("llama", 2064), ("neox", 3088), ("llama", 4112), ("neox", 5136), ("llama", 5136)])
+@pytest.mark.parametrize("family,d", [("neox", 1040), ("llama", 2064), ("neox", 3088), ("llama", 4112), ("neox", 5136), ("llama", 5136),
+                                      ("neox", 6160), ("llama", 7184)])
 def test_norms_just_beyond_a_row_width_equal_the_stepwise_ones(family, d):
     """A norm holds 1024 columns per register step, up to five steps, with one or two gain sets; rows a little wider than each
-    (and than all five, whose rest is read again), against the stepwise path: one layer of heads of 16, same tolerances as the
-    comparison of the two paths above."""
+    (and than all five, whose rest is read again, in one, two and three steps), against the stepwise path: one layer of heads of
+    16, same tolerances as the comparison of the two paths above.  The columns beyond the last full step have gains and biases of
+    their own, different in each norm: leaving them out, or taking one norm's for the other's, moves a projection by 0.1 and more."""
     like = synth.neox_like if family == "neox" else synth.llama_like
     arch = like(1, d, d // 16, 128, 136)
     ws_np = gu.scaled_weights(synth, arch, 3, 1.0)
+    for name, gain, bias in (("l0.ln1", 3.0, 1.5), ("l0.ln2", -2.0, -1.5), ("lnf", 2.0, 1.0)):
+        for end, value in (("_g", gain), ("_b", bias)):
+            w = ws_np[synth.tensor_names(arch).index(name + end)]
+            if w is not None:
+                w[-16:] = value
     model = B.Model(arch, B.upload_weights(arch, ws_np))
     S, K = 16, 2
     prompts, rows = synth.gen_prompt(4, 1, 5, arch.vocab), synth.gen_prompt(5, 1, K + 1, arch.vocab)
