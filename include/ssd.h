@@ -340,12 +340,14 @@ int ssd_last_logits(const ssd_model *m, int batch, int rows_per_seq, const void 
                     float *dev_out, void *stream);
 
 /* Profiling aid for the single-kernel forward, whose phases no external profiler can separate:
- * when enabled, one CTA stamps the GPU's nanosecond timer at kernel start, after every grid
- * barrier and at its end.  ssd_read_trace copies the stamps of the last forward that used this
+ * when enabled, one CTA stamps the GPU's nanosecond timer at kernel start, at every grid
+ * barrier - when it is complete, or where that CTA does not wait for it when the CTA arrives - and at
+ * its end.  ssd_read_trace copies the stamps of the last forward that used this
  * workspace (same batch / rows_per_seq) to the host; consecutive differences are phase durations
- * in the order: set-up, embedding, then per layer [qkv(+MLP-in), attention, out-proj(+MLP-out),
- * statistics] (parallel residual) or [qkv, attention, out-proj, statistics, MLP-in, MLP-out,
- * statistics] (sequential), then the LM head.  Synchronises the stream.  Off by default. */
+ * in the order: set-up with embedding and first norm, then per layer [qkv + MLP-in, attention +
+ * activation, out-proj + MLP-out, norms] (parallel residual; with few attention items [qkv + MLP-in,
+ * activation, attention beside MLP-out and out-proj, norms]) or [qkv, attention, out-proj, norm, MLP-in,
+ * activation, MLP-out, norm] (sequential), then the LM head.  Synchronises the stream.  Off by default. */
 int ssd_set_trace(int enable);
 int ssd_read_trace(const ssd_model *m, int batch, int rows_per_seq, const void *dev_ws, size_t ws_bytes,
                    uint64_t *host_out, int max_entries, int *n_out, void *stream);

@@ -35,7 +35,8 @@
 // across calls, because a spilled value or a read through the parameter bank would be a trip to L2 at
 // the head of every one of the pass's ~130-260 phases (227 KB of shared memory leave next to no L1).
 // Every wait (mbarrier, grid barrier) is bounded; on time-out SSD_E_TIMEOUT is recorded, the CTA
-// stops taking work, waits (bounded) for its copies in flight, drains the tensor core, frees its
+// does no more GEMM work and stops at the next grid barrier that it waits at (an arrival takes no
+// snapshot of the outcome), waits (bounded) for its copies in flight, drains the tensor core, frees its
 // tensor memory and returns.  A parity wait is used only where the waiter follows every phase of its
 // barrier in order and the barrier cannot pass it by two phases.
 #pragma once
@@ -117,7 +118,7 @@ struct alignas(64) FwdParams {
     // their bytes with the attention scratch (at attn_smem_off = stages_lo * stage bytes) and are used
     // only between attention phases.
     int stages, stages_lo, attn_smem_off;
-    unsigned long long *trace;  // optional: CTA 0 stamps the global timer after every grid barrier
+    unsigned long long *trace;  // optional: CTA 0 stamps the global timer at every grid barrier (see grid_stamp)
     // tensor-core attention (head dim 128): the whole cache as rows of Dh bf16, box 64 x 128 rows
     CUtensorMap tm_kv;
     const CUtensorMap *tm_kv_ptr;  // where the copy engine can read tm_kv (set by the kernel: see params copy)
@@ -382,7 +383,7 @@ struct alignas(16) Shared {
     volatile int passed;    // grid barriers seen to be complete
     volatile int abort;     // some wait in this CTA gave up
     volatile int go;        // snapshot of !abort taken inside the grid barrier: uniform for all work threads
-    int epoch;              // grid barriers passed (thread 0's)
+    int epoch;              // grid barriers arrived at (thread 0's)
     int flag;
     long long wait_limit;   // cycles after which a wait that takes work gives up (the drain waits of the error path keep kWaitCycles)
     uint32_t tmem_base;     // base address of this CTA's tensor memory
@@ -447,6 +448,8 @@ __device__ __forceinline__ bool grid_poll(const FwdParams &p, Shared *sh, int ep
     sh->passed = epoch;
     return true;
 }
+// CTA 0's stamp of a barrier: its completion where a thread of that CTA waits for it (grid_sync, or the operand issuer of the GEMM
+// behind an arrival), else the CTA's arrival.
 __device__ __forceinline__ void grid_stamp(const FwdParams &p, int epoch) {
     if (p.trace && blockIdx.x == 0) {
         unsigned long long t;
@@ -461,8 +464,9 @@ __device__ __forceinline__ void grid_stamp(const FwdParams &p, int epoch) {
 // verification 3486 -> 3371 us, 1.4B 945 -> 899).
 __device__ __forceinline__ bool grid_arrive_work(const FwdParams &p, Shared *sh) {
     // What this thread did in shared memory is over before the producer's copies may land there.  (Its writes to global memory reach
-    // other CTAs' bulk copies through the release below, the operand issuer's acquire and that thread's proxy fence; a fence for
-    // global memory here, in every thread, cost each barrier half a microsecond: norms included, 2.7B verification 1855 -> 1780 us.)
+    // other CTAs' bulk copies through the release below, the operand issuer's acquire and that thread's proxy fence.  The general
+    // fence here, in every thread, costs each barrier half a microsecond: a layer of the 7B verification 100.7 us instead of 99.5,
+    // at batch 8 159.7 / 158.2, of the 7B's draft there 47.1 / 44.5, of 2.7B 54.9 / 54.1.)
     fence_async_shared();
     named_bar(1, kWorkThreads);
     if (threadIdx.x != 0) return true;
@@ -494,9 +498,10 @@ __device__ __noinline__ bool grid_sync() {
     return sh->go != 0;
 }
 
-// Arrival without a wait: in front of a GEMM, whose operand issuer is the only one that needs the other CTAs' work and waits for the
-// barrier itself (gemm_desc's `need`), while the other roles set themselves up; and of a CTA whose next work does not depend on
-// what the others publish there.  The barrier behind that work waits for this one first where nobody has (a time-out in between
+// Arrival without a wait: in front of a GEMM, whose operand issuer waits for the barrier itself (gemm_desc's `need`) while the other
+// roles set themselves up - the epilogue needs the other CTAs' zeroing of its output, but has nothing to reduce before operand
+// copies, MMAs and commit have passed the issuer's wait on to it; and of a CTA whose next work does not depend on what the
+// others publish there.  The barrier behind that work waits for this one first where nobody has (a time-out in between
 // is found there as well).
 __device__ __noinline__ void grid_arrive() {
     const FwdParams &p = params_copy();
@@ -526,7 +531,7 @@ __device__ __forceinline__ void leave_grid(unsigned *gbar) {
 // Count of attention CTAs that have finished their items, over the layers of this pass (cleared with the
 // barrier counter).  With few attention items in a parallel-residual block the CTAs
 // without an item run the MLP-out GEMM beside the attention and go straight on to the out-projection:
-// its operand issuer waits for this count instead of a grid barrier.
+// its operand issuer waits for this count as well as for the barrier behind the activation, which says nothing of the attention.
 __device__ __forceinline__ unsigned *attn_done(const FwdParams &p) { return p.gbar + 8; }
 __device__ __noinline__ void attn_signal() {
     const FwdParams &p = params_copy();
@@ -572,9 +577,9 @@ __device__ __forceinline__ void grid_zero(float *dst, int R, int n, int ld) {
 
 // Norm of every row of x into hi/lo operand buffers (one or two gain/bias sets from the same
 // statistics); one CTA per row.  Bound by latency: a barrier, the row, its sums, the operand.  The row (Q float4 per thread)
-// stays in registers between the statistics and the write pass, and gains and biases are loaded with it: fetched under the
-// statistics into L1 - of which there is next to none - they were a second trip of 1.2-2 us behind them (with the barriers' cheaper fence a 7B
-// layer 101.5 -> 99.2 us, a 1.4B layer 34.5 -> 31.8).  Q is a template parameter so
+// stays in registers between the statistics and the write pass, and gains and biases are loaded with it: prefetched into L1 -
+// of which there is next to none - under the statistics, they were a second trip behind them (a layer of 1.4B 32.9 -> 32.5 us, of
+// its draft 21.1 -> 20.4, of 12B 115.5 -> 114.4; of 7B and 2.7B 0.1-0.2).  Q is a template parameter so
 // that a call executes only the code its row width needs: the instructions of a phase are not in
 // the instruction cache when it starts (the kernel is far larger than that cache), and every KB of
 // straight-line code costs a fraction of a microsecond to fetch.
@@ -599,8 +604,8 @@ __device__ __forceinline__ float4 norm_vec(const float *v, int i, int n4) {  // 
 
 // Entry i of the table of gains and biases: eight per layer (norm 1 at 0, norm 2 at 4), then the final norm's two.  The norms find
 // their vectors by that one number: as six arguments through three functions they were reloaded from the stack at the head of
-// every norm (with the zeroing in front of the norm, so that nothing is kept across it: 7B verification 3235 -> 3220 us, at
-// batch 8 5134 -> 5067, 1.4B 836 -> 808).
+// every norm (with the zeroing in front of the norm, so that nothing is kept across it: 7B verification 3252 -> 3238 us, at
+// batch 8 5128 -> 5061, 1.4B 833 -> 807).
 __device__ __forceinline__ const float *norm_ptr(const FwdParams &p, int i) {
     const float *const *lt = staged_ltab();
     if (lt) return lt[i];
@@ -608,7 +613,10 @@ __device__ __forceinline__ const float *norm_ptr(const FwdParams &p, int i) {
     return l < p.n_layers ? (&layer_desc(p.md, l)->ln1_g)[i & 7] : (i & 1) ? p.md->lnf_b : p.md->lnf_g;
 }
 
-// Q: float4 per thread, rows up to Q * 1024 wide.  Wider rows (TAIL: beyond 5120) are read again, with what goes with them.
+// Q: float4 per thread, rows up to Q * 1024 wide.  Wider rows (TAIL: beyond 5120) are read again, with what goes with them.  Eight
+// steps in registers instead - the second set's vectors behind the sums, as all four do not fit - were the longer way up to 7168
+// columns and no shorter beyond (eight layers, us, five / eight: two sets, d = 5632 1247 / 1284, 7168 1828 / 1860, 8192 2307 / 2324;
+// one set, 5632 1331 / 1345, 7168 1926 / 1927, 8192 2375 / 2366).
 // set: where the vectors stand in the pointer table (see norm_ptr); TWO: norm 2 of the same layer as well.
 template <int Q, bool TWO, bool TAIL>
 __device__ __noinline__ void norm_rows(int set) {
@@ -1283,7 +1291,7 @@ __device__ __noinline__ void attention_items(int layer) {
 // 2^32 (fp32 sums and bf16 hi + lo carry the factor without loss), which one barrier vote per chunk finds out: no maxima are
 // exchanged and O^T is not rescaled in the ordinary chunk.
 // Bound: the 64 KB of K and V a chunk fetches.  7B, 17 rows x 16384 positions: 249 us a layer with two 16-row tiles that each
-// walk the cache and exchange maxima in every chunk, 97 now, against 41 us of HBM time.
+// walk the cache and exchange maxima in every chunk, 84 now, against 41 us of HBM time.
 constexpr int kTcChunk = 128;
 constexpr int kTcStages = 4;  // K / V ring stages of 32 KB: the bytes in flight set the chunk rate (3 stages: 2.7 us per chunk)
 constexpr int kTcKvStage = kTcChunk * 128 * 2;  // one K or V chunk: two 64-column panels of 128 rows x 128 B
@@ -1456,7 +1464,10 @@ __device__ __noinline__ void attention_items_tc(int layer) {
     };
     const int n_early = min(kTcStages, 2 * n_chunks);
     if (warp == 5 && lane == 0 && !sh->abort) {
-        fence_async_proxy();  // the previous user of these slots wrote them through the generic proxy
+        // Shared AND global memory: the previous user of these slots wrote them through the generic proxy, and so did the items of an
+        // earlier step of this launch with the cache rows that the copies read (they reach this thread through the grid
+        // barriers, which fence shared memory alone).
+        fence_async_proxy();
         for (int j = 0; j < n_early; ++j) issue_kv(j);
     }
     // ---- set-up: Q tile (rotary applied, in log2 units; RP hi rows, RP lo rows) ----

@@ -59,9 +59,9 @@ class Engine:
         self.batch, self.max_len, self.K, self.T = batch, max_len, K, float(temperature)
         self.K_max = K
         # Draft loop as ONE draft_steps call (one launch that ends every step inside the kernel) or as one
-        # draft_step call per token.  Measured on B200 the two are within a few per cent of each other (the
-        # in-kernel tail costs grid barriers where the other path costs two small launches); the per-token form
-        # is the default because it is the faster one at batch 1.
+        # draft_step call per token.  The per-token form is the default because it is the faster one (the in-kernel
+        # tail costs five grid barriers and commits behind the last, where the other path costs two small launches):
+        # one launch is 6 - 17 us a step longer at the 7B, 1.4B and 2.7B workloads' batches, 39 at 1.4B and batch 8.
         self.fused_draft = False
         self.prompt_ws_cap = 4 << 30      # bytes of temporary workspace the prompt pass may take
         V = target.arch.vocab
