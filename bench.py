@@ -42,8 +42,8 @@ NOMINAL_HBM_GBS = 8000.0
 # An entry is dropped (None) when the kernel has changed since its capture.
 NCU_TRAFFIC = {
     # workload: (captured workload, dram bytes of the captured launch, layers captured)
-    "llama-7b-b8": ("llama-7b-l4-b8", 3.1158e9, 4),        # profiles/forward_kernel_llama-7b-l4-b8_verify.md
-    "llama-7b-l4-b8": ("llama-7b-l4-b8", 3.1158e9, 4),
+    "llama-7b-b8": ("llama-7b-l4-b8", 3.1130e9, 4),        # profiles/forward_kernel_llama-7b-l4-b8_verify.md
+    "llama-7b-l4-b8": ("llama-7b-l4-b8", 3.1130e9, 4),
 }
 
 # bench workloads: name -> preset (+ overrides)
